@@ -99,6 +99,27 @@ cudaError_t launch_pdl(Ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block, 
   return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
 }
 
+// As launch_pdl, in clusters of `cluster` CTAs along x (the grid a multiple of it).
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(Ctx* ctx, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, unsigned cluster,
+                               Args&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = ctx->stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = ctx->pdl ? 1 : 0;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Args&&>(args)...);
+}
+
 // Device-side error recording: keeps the first non-zero code.
 __device__ __forceinline__ void record_error(int* status, int code) {
   if (status) atomicCAS(status, 0, code);
@@ -202,9 +223,14 @@ inline void set_pair_blocks(PairArgs& a, float eps, uint64_t query) {
 int launch_pair_simt(Ctx* ctx, const PairArgs& a);
 // INT4 g128 weight [d_out, d_in/2] + fp16 scales -> bf16 [d_out, d_in].
 int launch_dequant_int4(Ctx* ctx, const void* Wq, const void* Ws, void* Wb, int64_t d_out, int d_in);
-// Row count from which the INT4 pair forward expands W to bf16 first instead of dequantising per M-tile.
-constexpr int64_t INT4_STAGED_MIN_ROWS = 1024;
+// Fewer rows than this take the few-row kernel (W read once, rows on the MMA's N side; INT4 dequantised in it).
+constexpr int64_t FEW_ROWS = 256;
+// Row count from which an INT4 pair forward takes row scales and layer groups (the library's contract).
+constexpr int64_t INT4_ROWSCALE_MIN_ROWS = 1024;
 int launch_pair_tc(Ctx* ctx, const PairArgs& a);
+// The few-row kernel serves fewer than FEW_ROWS rows whose outputs (every block padded to 16 rows) fit one tile.
+bool pair_fr_supported(const PairArgs& a);
+int launch_pair_fr(Ctx* ctx, const PairArgs& a);
 // Plain product D[M, N] (fp32) = A[M, K] * B[N, K]^T with 16-bit A, B (K-major), on tcgen05.
 // Low-rank term of the tensor-core pair forward (see k_aug.cu):
 //   LOWRANK_EPILOGUE  (C + c_b Z_b) p summed in the epilogue (fp32 tables)

@@ -11,7 +11,6 @@ namespace zoact {
 namespace pairtc {
 int dispatch_bf16(Ctx* ctx, int mode, int rt, int ydtype, const TmaSet& tm, const Params& p);
 int dispatch_fp16(Ctx* ctx, int mode, int rt, int ydtype, const TmaSet& tm, const Params& p);
-int dispatch_w4(Ctx* ctx, int mode, int rt, int ydtype, const CUtensorMap& a, const Params& p);
 int dispatch2_bf16(Ctx* ctx, int mode, int rt, int ydtype, const TmaSet& tm, const Params& p);
 int dispatch2_fp16(Ctx* ctx, int mode, int rt, int ydtype, const TmaSet& tm, const Params& p);
 int dispatch2_w4(Ctx* ctx, int mode, int ydtype, const TmaSet& tm, const Params& p);
@@ -77,7 +76,6 @@ int encode_tmap_2d_16bit(CUtensorMap* map, const void* base, int dtype, int64_t 
   return res == CUDA_SUCCESS ? ZOACT_OK : ZOACT_ERR_INVALID_ARG;
 }
 
-// Unswizzled boxes of 8- or 16-bit integers (INT4 packed weights, fp16 scales read as raw bits).
 int encode_tmap_2d_int(CUtensorMap* map, const void* base, int elem_bytes, int64_t rows, int64_t cols, int box_cols,
                        int box_rows) {
   EncodeTiledFn fn = get_encode_fn();
@@ -136,16 +134,16 @@ bool pair_rowscale_supported(const Ctx* ctx, int64_t rows, int shared, int xdtyp
   const char* lsel = std::getenv("ZOACT_LOWRANK");
   if ((sel && std::strcmp(sel, "1cta") == 0) || (lsel && std::strcmp(lsel, "epilogue") == 0)) return false;
   if (wtype == ZOACT_DT_INT4_G128) {
-    // INT4 reaches the CTA-pair kernel expanded to bf16 (from 1024 rows, or ZOACT_INT4=staged) or with
-    // ZOACT_INT4=kernel; below 1024 rows the one-CTA kernel dequantises it
+    // INT4: from 1024 rows, or with ZOACT_INT4=staged or =kernel
     const char* isel = std::getenv("ZOACT_INT4");
-    return rows >= INT4_STAGED_MIN_ROWS || (isel && (std::strcmp(isel, "staged") == 0 || std::strcmp(isel, "kernel") == 0));
+    return rows >= INT4_ROWSCALE_MIN_ROWS || (isel && (std::strcmp(isel, "staged") == 0 || std::strcmp(isel, "kernel") == 0));
   }
   return true;
 }
 
 int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   using namespace pairtc;
+  if (pair_fr_supported(a)) return launch_pair_fr(ctx, a);
   // ranks above 32 have no epilogue tables: the low-rank term must ride the MMA, which needs stacked rows
   const bool big_r = a.r > 32;
   if (big_r && !ctx->may_allocate) return ZOACT_ERR_UNSUPPORTED;
@@ -174,8 +172,8 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
     b.rows = (int64_t)a.nb * a.T;
     return launch_pair_tc(ctx, b);
   }
-  // INT4 weights.  Below 1024 rows the one-CTA kernel dequantises in the kernel; from 1024 rows W is expanded
-  // to bf16 once per call and the bf16 kernel runs (the default: measured faster, see pair_tc2_kernel.cuh).
+  // INT4 weights: the few-row kernel dequantises in the kernel; from FEW_ROWS rows W is expanded to bf16 once
+  // per call and the bf16 kernel runs (the default: measured faster, see pair_tc2_kernel.cuh).
   // ZOACT_INT4=kernel runs stacked rows from 256 on the CTA-pair kernel with its own dequantising warps
   // (bf16 or fp32 output, d_in a multiple of 1024); ZOACT_INT4=staged expands W at every row count.
   const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
@@ -183,7 +181,6 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   const char* lsel = std::getenv("ZOACT_LOWRANK");
   const bool lr_epi = lsel && std::strcmp(lsel, "epilogue") == 0;
   const char* isel = std::getenv("ZOACT_INT4");
-  const bool int4_staged = isel && std::strcmp(isel, "staged") == 0;   // expansion at any row count
   const bool int4_kernel = isel && std::strcmp(isel, "kernel") == 0;   // CTA-pair in-kernel dequantisation
   // (the scales' tensor map wants rows of a multiple of 16 bytes: d_in a multiple of 1024)
   auto al16 = [](const void* q) { return q == nullptr || ((uintptr_t)q & 15u) == 0; };
@@ -192,8 +189,7 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
                       al16(a.w_scales) && al16(a.w_scales2) &&
                       (a.ydtype == ZOACT_DT_BF16 || a.ydtype == ZOACT_DT_FP32) && !one_cta && !lr_epi &&
                       int4_kernel;
-  if (a.wtype == ZOACT_DT_INT4_G128 && !w4_two &&
-      (a.rows >= INT4_STAGED_MIN_ROWS || big_r || (int4_staged && ctx->may_allocate))) {
+  if (a.wtype == ZOACT_DT_INT4_G128 && !w4_two) {
     // staged INT4: expand W (and W2) to bf16 in context scratch, then the bf16 kernel (timed together)
     const size_t bytes = (size_t)a.d_out * a.d_in * 2;
     void* wb = scratch(ctx, SLOT_WDQ0, bytes);
@@ -229,15 +225,15 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   TmaSet tm;
   int st = encode_tmap_2d_16bit(&tm.a, a.X, a.xdtype, a.rows, a.d_in, BM);
   if (st) return st;
-  // CTA pairs (256-row tiles) once there are enough rows to fill them (INT4: where w4_two allows)
-  const bool two = (w4 ? w4_two : a.rows >= 2 * BM && !one_cta);
+  // CTA pairs (256-row tiles) once there are enough rows to fill them
+  const bool two = w4 || (a.rows >= 2 * BM && !one_cta);
   // CTA pairs: always 256-wide tiles.  A 256 x bn x 16 MMA measured the same time for bn = 192, 224 and 256, so
   // a tile costs the same at any of these widths and the widest needs the fewest waves (the Llama-3-8B MLP step:
   // 0.645 ms at 256 and at 224, 0.709 at 192; the OPT stack: 145.7 ms at 256, 149.1 at 224).
   const int bn = (gated || w4 || two) ? BN : choose_bn(a.rows, a.d_out, ctx->sm_count);
   const int b_box = gated ? BN / 2 : (two ? bn / 2 : bn);
   tm.s = tm.s2 = tm.a;
-  if (w4 && two) {
+  if (w4) {
     // packed rows and their scales by TMA, dequantised in shared memory by the kernel's own warps
     st = encode_tmap_2d_int(&tm.b, a.W, 1, a.d_out, a.d_in / 2, BK / 2, BM);
     if (st) return st;
@@ -251,8 +247,6 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
       st = encode_tmap_2d_int(&tm.s2, a.w_scales2, 2, a.d_out, a.d_in / 128, 8, BM);
       if (st) return st;
     }
-  } else if (w4) {
-    tm.b = tm.b2 = tm.a;                 // W arrives through the dequantising warps, not TMA
   } else {
     st = encode_tmap_2d_16bit(&tm.b, a.W, a.wtype, a.d_out, a.d_in, b_box);
     if (st) return st;
@@ -267,7 +261,7 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   int lmode = LOWRANK_EPILOGUE;
   const bool distinct = gated && a.P2 != a.P;
   int slots = 1;
-  if ((!w4 || two) && ctx->may_allocate && (big_r || !lr_epi)) {
+  if (ctx->may_allocate && (big_r || !lr_epi)) {
     // stacked rows: the whole term on the tensor cores -- one K slot when every tile lies in one evaluation
     // block, else S slots (block index mod S) with S the most blocks a tile can span; shared inputs keep
     // +-Z p in the epilogue (C p on the tensor cores)
@@ -446,20 +440,11 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   }
   p.status = ctx->d_status;
   const int mode = gated ? MODE_GATED : MODE_PAIR;
-  if (w4) {
-    p.Wq = static_cast<const uint8_t*>(a.W);
-    p.Ws = static_cast<const __half*>(a.w_scales);
-    p.Wq2 = static_cast<const uint8_t*>(a.W2);
-    p.Ws2 = static_cast<const __half*>(a.w_scales2);
-    st = timing_begin(ctx);
-    if (st) return st;
-    st = two ? dispatch2_w4(ctx, mode, a.ydtype, tm, p) : dispatch_w4(ctx, mode, rt, a.ydtype, tm.a, p);
-    if (st) return st;
-    return timing_end(ctx);
-  }
   st = timing_begin(ctx);
   if (st) return st;
-  if (two)
+  if (w4)
+    st = dispatch2_w4(ctx, mode, a.ydtype, tm, p);
+  else if (two)
     st = a.xdtype == ZOACT_DT_BF16 ? dispatch2_bf16(ctx, mode, rt, a.ydtype, tm, p)
                                    : dispatch2_fp16(ctx, mode, rt, a.ydtype, tm, p);
   else

@@ -18,8 +18,7 @@ static int launch_two_w4(Ctx* ctx, const TmaSet& tm, const Params& p) {
 }
 
 int dispatch2_w4(Ctx* ctx, int mode, int ydtype, const TmaSet& tm, const Params& p) {
-  if (p.y_staged != STAGE_ALL || p.aug_mode != LOWRANK_ALL_ON_TC || !p.Wq || !p.Ws) return ZOACT_ERR_UNSUPPORTED;
-  if (mode == MODE_GATED && (!p.Wq2 || !p.Ws2)) return ZOACT_ERR_UNSUPPORTED;
+  if (p.y_staged != STAGE_ALL || p.aug_mode != LOWRANK_ALL_ON_TC) return ZOACT_ERR_UNSUPPORTED;
   if (ydtype == ZOACT_DT_FP32)
     return mode == MODE_GATED ? launch_two_w4<float, MODE_GATED>(ctx, tm, p) : launch_two_w4<float, MODE_PAIR>(ctx, tm, p);
   if (ydtype == ZOACT_DT_BF16)

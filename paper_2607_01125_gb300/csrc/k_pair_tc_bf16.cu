@@ -6,10 +6,10 @@ namespace pairtc {
 
 template <typename TO, int RT, int MODE>
 static int launch_one(Ctx* ctx, const TmaSet& tm, const Params& p) {
-  auto kern = pair_tc_kernel<TO, RT, MODE, 1, false>;
+  auto kern = pair_tc_kernel<TO, RT, MODE, 1>;
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES));
   const int grid = p.num_tiles < ctx->sm_count ? p.num_tiles : ctx->sm_count;
-  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3(grid), dim3(num_threads(false)), SMEM_BYTES, tm, p)); ++ctx->n_launch;
+  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3(grid), dim3(NUM_THREADS), SMEM_BYTES, tm, p)); ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
 }

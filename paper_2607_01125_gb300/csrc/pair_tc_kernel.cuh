@@ -36,17 +36,6 @@
 // term there (stacked rows whose tiles lie in one block) the epilogue only
 // converts and stores; with C p there the epilogue adds c_b Z_b p from Z tables,
 // once for both signs of a shared-input pair (y+- = acc +- eps Z p).
-//
-// INT4 weights (W4): the frozen W is symmetric INT4 in groups of 128 along d_in
-// with fp16 scales.  Four more warps (448 threads in all) dequantise it: per
-// K-block each thread loads 2 rows x 32 packed bytes and their scales with
-// plain global loads (prefetched one K-block ahead), turns every nibble q into
-// bf16 q * s (magic-number conversion 0x4300 | (q ^ 8) = 128 + q + 8, minus
-// 136, times the scale, in bf16x2 arithmetic) and writes the 128-byte-swizzled
-// bf16 tile straight into the MMA's shared-memory stage, then fences the
-// async proxy and arrives on the stage's barrier.  Only X comes by TMA.  With
-// 14 warps the registers per thread drop to 128, so the epilogue works on
-// 8-column chunks.
 #pragma once
 #include "internal.h"
 #include "philox.cuh"
@@ -75,9 +64,7 @@ __host__ __device__ constexpr int gated_slots(int rt) {
 }
 constexpr int EPI_WARPS = 8;
 constexpr int EPI_THREADS = 32 * EPI_WARPS;
-constexpr int DQ_THREADS = 128;                     // INT4 dequantisation warps
-__host__ __device__ constexpr int num_threads(bool w4) { return 64 + EPI_THREADS + (w4 ? DQ_THREADS : 0); }
-__host__ __device__ constexpr int epi_base(bool w4) { return 64 + (w4 ? DQ_THREADS : 0); }
+constexpr int NUM_THREADS = 64 + EPI_THREADS;
 constexpr int TMEM_COLS = 512;
 constexpr int SMEM_BYTES = 1024 /*align slack*/ + STAGES * STAGE_BYTES + TBL_FLOATS * 4 + 256;
 constexpr int GROUP_M = 8;
@@ -134,10 +121,8 @@ struct Params {
   int64_t ldy;       // plain mode: row stride of D
   int vec_ok;        // C, C2, P, P2 and ldy allow 16-byte vector access
   int bn;            // N-tile width of pair / plain tiles (multiple of 32, <= BN); gated tiles use BN
-  // INT4 weights: packed [d_out, d_in/2] bytes and fp16 scales [d_out, d_in/128]
-  const uint8_t* Wq;
+  // INT4 weights of few rows: fp16 scales [d_out, d_in/128]
   const __half* Ws;
-  const uint8_t* Wq2;
   const __half* Ws2;
   int* status;
   // fused loss pair (STAGE_LOSS): target [T, d_out] of Y's type through tm.y / tm.y16 (or none: mean of
@@ -372,65 +357,6 @@ __device__ __forceinline__ void tmem_ldN(uint32_t taddr, float* v) {
   else tc::tmem_ld8(taddr, v);
 }
 
-// ---- INT4 dequantisation into a 128-byte-swizzled bf16 B tile ----
-// 8 nibbles (elements k..k+7, low nibble first) scaled by s -> 8 bf16 (16 bytes).
-__device__ __forceinline__ uint4 dequant8(uint32_t w, __nv_bfloat162 s2) {
-  const uint32_t x = w ^ 0x88888888u;                 // nibble q -> q + 8 in [0, 15]
-  const __nv_bfloat162 c136 = __floats2bfloat162_rn(136.0f, 136.0f);
-  uint32_t out[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const uint32_t lo = (x >> (8 * i)) & 0xFu, hi = (x >> (8 * i + 4)) & 0xFu;
-    uint32_t v = 0x43004300u | lo | (hi << 16);       // bf16 pair (128 + q + 8)
-    __nv_bfloat162 h = *reinterpret_cast<__nv_bfloat162*>(&v);
-    h = __hmul2(__hsub2(h, c136), s2);                // q exactly, then q * s rounded to bf16
-    out[i] = *reinterpret_cast<uint32_t*>(&h);
-  }
-  return make_uint4(out[0], out[1], out[2], out[3]);
-}
-
-// Row `row` (0..255) of the B tile of K-block kb: source row, packed bytes and scale.
-struct DqRow {
-  uint4 q0, q1;       // 32 packed bytes = 64 elements
-  __half s;
-  bool valid;
-};
-
-template <int MODE>
-__device__ __forceinline__ DqRow dq_load(const Params& prm, int n_blk, int row, int kb) {
-  DqRow d;
-  const uint8_t* Wq = prm.Wq;
-  const __half* Ws = prm.Ws;
-  int n;
-  if (MODE == MODE_GATED) {
-    n = n_blk * (BN / 2) + (row & (BN / 2 - 1));
-    if (row >= BN / 2) { Wq = prm.Wq2; Ws = prm.Ws2; }
-  } else {
-    n = n_blk * BN + row;
-  }
-  d.valid = n < prm.d_out;
-  if (d.valid) {
-    const uint4* src = reinterpret_cast<const uint4*>(Wq + (int64_t)n * (prm.d_in / 2) + kb * (BK / 2));
-    d.q0 = __ldg(src);
-    d.q1 = __ldg(src + 1);
-    d.s = Ws[(int64_t)n * (prm.d_in / 128) + (kb * BK) / 128];
-  } else {
-    d.q0 = d.q1 = make_uint4(0x88888888u, 0x88888888u, 0x88888888u, 0x88888888u);   // q = 0
-    d.s = __float2half_rn(0.f);
-  }
-  return d;
-}
-
-__device__ __forceinline__ void dq_store(uint8_t* btile, int row, const DqRow& d) {
-  const __nv_bfloat16 sb = __float2bfloat16_rn(__half2float(d.s));
-  const __nv_bfloat162 s2 = __halves2bfloat162(sb, sb);
-  uint8_t* rowp = btile + row * 128;
-  const uint32_t w[8] = {d.q0.x, d.q0.y, d.q0.z, d.q0.w, d.q1.x, d.q1.y, d.q1.z, d.q1.w};
-#pragma unroll
-  for (int c = 0; c < 8; ++c)
-    *reinterpret_cast<uint4*>(rowp + ((c ^ (row & 7)) << 4)) = dequant8(w[c], s2);
-}
-
 // The epilogue's wait for a finished accumulator, taken by one thread and
 // shared through a named barrier so that all epilogue threads leave (or
 // continue) together even if the wait gives up.
@@ -660,12 +586,12 @@ __device__ __forceinline__ bool epi_pair_tile(const Params& prm, SS* ss, float* 
   return true;
 }
 
-template <typename TO, int RT, int MODE, int AB_BF16, bool W4>
-__global__ void __launch_bounds__(num_threads(W4), 1)
+template <typename TO, int RT, int MODE, int AB_BF16>
+__global__ void __launch_bounds__(NUM_THREADS, 1)
 pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
-  // epilogue chunk width (columns per tcgen05.ld): 8 where the registers are scarce (INT4's 14 warps,
-  // the gated pair's two accumulators and two projections)
-  constexpr int CW = (W4 || MODE == MODE_GATED) ? 8 : 16;
+  // epilogue chunk width (columns per tcgen05.ld): 8 where the registers are scarce (the gated pair's two
+  // accumulators and two projections)
+  constexpr int CW = MODE == MODE_GATED ? 8 : 16;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   float* tbl = reinterpret_cast<float*>(smem + STAGES * STAGE_BYTES);
@@ -677,8 +603,7 @@ pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      // full: the producer's expect_tx arrival, plus one arrival per dequantising thread (INT4)
-      tc::mbar_init(tc::smem_u32(&ss->full[s]), W4 ? 1 + DQ_THREADS : 1);
+      tc::mbar_init(tc::smem_u32(&ss->full[s]), 1);
       tc::mbar_init(tc::smem_u32(&ss->empty[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -689,8 +614,8 @@ pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
     ss->abort_flag = 0;
     tc::fence_mbar_init();
     tc::prefetch_tmap(&tm.a);
-    if (!W4) tc::prefetch_tmap(&tm.b);
-    if (!W4 && MODE == MODE_GATED) tc::prefetch_tmap(&tm.b2);
+    tc::prefetch_tmap(&tm.b);
+    if (MODE == MODE_GATED) tc::prefetch_tmap(&tm.b2);
     if (prm.aug_kb > 0) {
       tc::prefetch_tmap(&tm.aa);
       tc::prefetch_tmap(&tm.ba);
@@ -709,7 +634,7 @@ pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
   pdl_trigger();
 
   const int num_m = prm.num_m, num_n = prm.num_n, num_k = prm.num_k;
-  const int total_k = num_k + (W4 ? 0 : prm.aug_kb);   // main K-blocks, then the low-rank ones
+  const int total_k = num_k + prm.aug_kb;   // main K-blocks, then the low-rank ones
   const int bn = MODE == MODE_GATED ? BN : prm.bn;  // this launch's N-tile width
 
   if (warp == 0) {
@@ -725,16 +650,14 @@ pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
         for (int kb = 0; kb < total_k; ++kb) {
           if (!tc::mbar_wait(tc::smem_u32(&ss->empty[stage]), phase ^ 1u, abort_flag, prm.status)) { ok = false; break; }
           const uint32_t full = tc::smem_u32(&ss->full[stage]);
-          tc::mbar_arrive_expect_tx(full, W4 ? A_BYTES : (MODE == MODE_GATED ? STAGE_BYTES : A_BYTES + bn * BK * 2));
+          tc::mbar_arrive_expect_tx(full, MODE == MODE_GATED ? STAGE_BYTES : A_BYTES + bn * BK * 2);
           const uint32_t sa = tc::smem_u32(smem + stage * STAGE_BYTES);
           const uint32_t sb = sa + A_BYTES;
           const bool aug = kb >= num_k;
           int kx = kb * BK, kxb = kb * BK, yb = 0;
           if (aug) aug_coords(prm, (int64_t)m_blk * BM, BM, kb - num_k, kx, kxb, yb);
           tc::tma_load_2d(sa, aug ? &tm.aa : &tm.a, kx, m_blk * BM, full);
-          if (W4) {
-            // B arrives from the dequantising warps
-          } else if (MODE == MODE_GATED) {
+          if (MODE == MODE_GATED) {
             tc::tma_load_2d(sb, aug ? &tm.ba : &tm.b, kxb, yb + n_blk * (BN / 2), full);
             tc::tma_load_2d(sb + B_BYTES / 2, aug ? &tm.ba2 : &tm.b2, kxb, yb + n_blk * (BN / 2), full);
           } else {
@@ -793,47 +716,9 @@ pair_tc_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
         tc::mbar_wait_drain(tc::smem_u32(&ss->drain), 0, 100000000ull);
       }
     }
-  } else if (W4 && warp < 2 + DQ_THREADS / 32) {
-    // ---------------- INT4 dequantisation (warps 2..5) ----------------
-    const int dtid = threadIdx.x - 64;             // 0..127: rows 2*dtid and 2*dtid + 1 of each B tile
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    bool have = false;
-    DqRow cur0, cur1;
-    // walk the same (tile, K-block) sequence as the producer, one K-block of loads ahead
-    int tile = blockIdx.x, kb = 0;
-    if (tile < prm.num_tiles) {
-      int m_blk, n_blk;
-      tile_coords(tile, num_m, num_n, m_blk, n_blk);
-      cur0 = dq_load<MODE>(prm, n_blk, 2 * dtid, 0);
-      cur1 = dq_load<MODE>(prm, n_blk, 2 * dtid + 1, 0);
-      have = true;
-    }
-    while (have && ok) {
-      // next K-block's loads first
-      int nt = tile, nkb = kb + 1;
-      if (nkb == num_k) { nkb = 0; nt += gridDim.x; }
-      DqRow nxt0, nxt1;
-      const bool more = nt < prm.num_tiles;
-      if (more) {
-        int m_blk, n_blk;
-        tile_coords(nt, num_m, num_n, m_blk, n_blk);
-        nxt0 = dq_load<MODE>(prm, n_blk, 2 * dtid, nkb);
-        nxt1 = dq_load<MODE>(prm, n_blk, 2 * dtid + 1, nkb);
-      }
-      if (!tc::mbar_wait(tc::smem_u32(&ss->empty[stage]), phase ^ 1u, abort_flag, prm.status)) { ok = false; break; }
-      uint8_t* btile = smem + stage * STAGE_BYTES + A_BYTES;
-      dq_store(btile, 2 * dtid, cur0);
-      dq_store(btile, 2 * dtid + 1, cur1);
-      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // generic writes -> tensor-core reads
-      tc::mbar_arrive(tc::smem_u32(&ss->full[stage]));
-      if (++stage == STAGES) { stage = 0; phase ^= 1u; }
-      tile = nt; kb = nkb; cur0 = nxt0; cur1 = nxt1; have = more;
-    }
   } else {
     // ---------------- epilogue (8 warps) ----------------
-    const int etid = threadIdx.x - epi_base(W4);    // 0..255
+    const int etid = threadIdx.x - 64;    // 0..255
     const int half = etid >> 7;                     // which half of the tile's columns
     const int quad = warp & 3;                      // TMEM lane quadrant this warp may access
     const int row_in_tile = quad * 32 + lane;

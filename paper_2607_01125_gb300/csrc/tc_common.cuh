@@ -322,6 +322,9 @@ __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint4 v) {
 // elements, box = box_rows x 64 columns, 128-byte swizzle, zero fill outside).
 int encode_tmap_2d_16bit(CUtensorMap* map, const void* base, int dtype, int64_t rows, int64_t cols,
                          int box_rows);
+// Host: unswizzled boxes of 8- or 16-bit integers (INT4 packed weights, fp16 scales read as raw bits).
+int encode_tmap_2d_int(CUtensorMap* map, const void* base, int elem_bytes, int64_t rows, int64_t cols, int box_cols,
+                       int box_rows);
 // Host: encode an output tensor map for bulk stores: row-major [rows, cols] of
 // ydtype (FP32/BF16/FP16), box = box_rows x box_cols, 128-byte swizzle when
 // swizzle128 (box_cols * element size must then be 128) else none.

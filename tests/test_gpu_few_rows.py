@@ -1,0 +1,117 @@
+"""The few-row pair forward (fewer than 256 rows of X) at the edges of its tiles, against the fp64 oracle.
+
+Tolerances, per element: fp32 accumulation 8 sqrt(d_in) 2^-24 sum |terms| (the K ranges of a cluster are added in a
+fixed order, so the bound of one sum holds), the 16-bit split of the low-rank term above 32 ranks (2^-14 of its
+|terms|), INT4 weights rounded once to bf16 (2^-9 of sum |x w|).  Gated outputs: the same bound on gate and up, through
+|d silu| <= 1.1, plus __expf / __fdividef in SiLU (2^-20 of the product).
+"""
+import numpy as np
+import pytest
+import torch
+
+import paper_2607_01125_gb300 as zo
+from oracle import layers, philox
+from synth import normal, quantize_int4_g128
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = zo.Context(0)
+    yield c
+    assert c.device_status() == 0
+    c.close()
+
+
+def np64(t):
+    return t.detach().double().cpu().numpy()
+
+
+def _layer(d_in, d_out, r, wtype, seed, lid, U=None):
+    U = normal((d_in, r), seed + 1, DEV) / np.sqrt(d_in) if U is None else U
+    C = normal((d_out * r,), seed + 2, DEV, std=0.3)
+    Wf = normal((d_out, d_in), seed, DEV, std=0.02)
+    if wtype == "int4":
+        packed, scales = quantize_int4_g128(Wf)
+        L = zo.make_layer(packed, U, C, lid, w_scales=scales, wtype=zo.DT_INT4_G128, d_in=d_in)
+        return L, layers.dequant_int4_g128(packed.cpu().numpy(), scales.float().cpu().numpy(), d_in), U, C
+    W = Wf.to({"bf16": torch.bfloat16, "fp16": torch.float16}[wtype])
+    return zo.make_layer(W, U, C, lid), np64(W), U, C
+
+
+def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4):
+    """Blocks of outputs and the bound of their error."""
+    Xn, Un, Cn = np64(X), np64(U), np64(C).reshape(W.shape[0], r)
+    out, bound = [], []
+    for b, (c, q) in enumerate(pts):
+        x = Xn if shared else Xn[b * T:(b + 1) * T]
+        Tb = Cn + c * philox.perturbation(seed, lid, q, W.shape[0], r)
+        out.append(x @ W.T + (x @ Un) @ Tb.T)
+        base = np.abs(x) @ np.abs(W).T
+        lr = np.abs(x @ Un) @ np.abs(Tb).T + (np.abs(x) @ np.abs(Un)) @ np.abs(Tb).T * 2.0 ** -10
+        bound.append(8 * np.sqrt(W.shape[1]) * 2.0 ** -24 * (base + lr) + (2.0 ** -14 * lr if r > 32 else 0.0) +
+                     (2.0 ** -9 * base if int4 else 0.0) + 1e-6)
+    return np.concatenate(out), np.concatenate(bound)
+
+
+@pytest.mark.parametrize("wtype,d_in,d_out,T,r,shared,nb,gated", [
+    ("bf16", 64, 8, 1, 1, False, 2, False),         # one K-block, two rows, eight outputs
+    ("bf16", 1000, 520, 37, 5, False, 2, False),    # ragged K and N tiles, rank 5
+    ("bf16", 4096, 1024, 16, 16, False, 2, False),  # eight K ranges; 32 rows
+    ("fp16", 2048, 136, 127, 32, False, 2, False),  # 254 rows
+    ("bf16", 8200, 256, 17, 16, True, 2, False),    # shared input, K ending inside a block
+    ("fp16", 512, 264, 255, 8, True, 2, False),     # the most rows
+    ("bf16", 512, 384, 14, 16, False, 17, False),   # 17 blocks of 14 rows
+    ("bf16", 1024, 200, 9, 32, True, 5, True),      # gated, shared, five blocks
+    ("bf16", 4096, 640, 100, 16, False, 2, True),   # gated, 200 rows: one CTA per SM, rows in several chunks
+    ("bf16", 4096, 256, 64, 32, False, 2, True),
+    ("bf16", 512, 264, 60, 40, False, 2, False),    # rank above 32: extra K-blocks
+    ("fp16", 576, 264, 21, 70, False, 3, True),
+    ("int4", 128, 8, 1, 4, False, 2, False),        # one scale group
+    ("int4", 14336, 512, 64, 32, False, 2, False),  # eight K ranges, odd ones starting inside a scale group
+    ("int4", 1152, 264, 100, 16, False, 2, False),  # 9 groups; 200 rows
+    ("int4", 2048, 136, 255, 3, True, 2, False),
+    ("int4", 1024, 200, 40, 16, False, 2, True),
+    ("int4", 1024, 520, 120, 32, True, 3, True),    # gated, rank 32: one CTA per SM
+])
+def test_few_rows(ctx, wtype, d_in, d_out, T, r, shared, nb, gated):
+    seed, eps = 11, 0.5
+    pts = [(eps, 7), (-eps, 7)] if nb == 2 else [(0.0, 0)] + [(eps * (1 + j) / nb, j) for j in range(nb - 1)]
+    L, W, U, C = _layer(d_in, d_out, r, wtype, 100, 3)
+    dt = torch.float16 if wtype == "fp16" else torch.bfloat16
+    X = normal(((T if shared else nb * T), d_in), 5, DEV, dtype=dt)
+    ref, bound = _ref(W, U, C, X, T, shared, pts, seed, 3, r, wtype == "int4")
+    if gated:
+        L2, W2, U2, C2 = _layer(d_in, d_out, r, wtype, 200, 4)      # its own basis: a second projection
+        u, ub = _ref(W2, U2, C2, X, T, shared, pts, seed, 4, r, wtype == "int4")
+        g = layers.silu(ref)
+        bound = 1.1 * bound * np.abs(u) + np.abs(g) * ub + 1.1 * bound * ub + 2.0 ** -20 * np.abs(g * u)
+        ref = g * u
+    for ydt in (torch.float32, dt):
+        outs = []
+        for _ in range(2):
+            Y = torch.full((nb * T, d_out), float("nan"), dtype=ydt, device=DEV)
+            if gated:
+                zo.zoact_multi_forward_gated(ctx, L, L2, X, T, shared, pts, seed, Y)
+            else:
+                zo.zoact_multi_forward(ctx, L, X, T, shared, pts, seed, Y)
+            torch.cuda.synchronize()
+            assert ctx.device_status() == 0
+            outs.append(Y)
+        assert torch.equal(outs[0], outs[1])             # the K ranges are added in a fixed order
+        rnd = {torch.float32: 0.0, torch.bfloat16: 2.0 ** -8, torch.float16: 2.0 ** -11}[ydt]
+        err = np.abs(np64(outs[0]) - ref)
+        assert np.all(err <= bound + rnd * np.abs(ref)), (ydt, float((err - bound - rnd * np.abs(ref)).max()))
+
+
+def test_few_rows_two_signs_equal_at_zero_eps(ctx):
+    # both signs of a stacked pair with equal inputs go through the same accumulator columns' arithmetic
+    d_in, d_out, T, r = 2048, 264, 33, 16
+    L, W, U, C = _layer(d_in, d_out, r, "bf16", 300, 1)
+    x = normal((T, d_in), 6, DEV, dtype=torch.bfloat16)
+    Y = torch.empty(2 * T, d_out, dtype=torch.float32, device=DEV)
+    zo.zoact_pair_forward(ctx, L, torch.cat([x, x]), T, False, 0.0, 1, 2, Y)
+    torch.cuda.synchronize()
+    assert torch.equal(Y[:T], Y[T:])
