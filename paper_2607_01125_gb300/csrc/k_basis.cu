@@ -10,9 +10,9 @@
 //      S = Y^T Y (64 x 64 output tiles; fp32 over 32-row slabs, fp64 across
 //      slabs and row chunks), Cholesky S = R^T R and R^-1 in one block (fp64,
 //      in global memory), Q = Y R^-1; done twice for orthogonality.
-//   4. Rayleigh-Ritz: S = Q^T G Q (fp64), Jacobi in one block (fp64): cyclic in
-//      shared memory for k <= 64, parallel round-robin pairs in global memory
-//      above; eigenpairs sorted by value, U = Q V[:, :r], each column flipped so
+//   4. Rayleigh-Ritz: S = Q^T G Q (fp64), Jacobi (fp64): two-sided in one block's
+//      shared memory for k <= 64, one-sided on the Cholesky factor over the whole
+//      chip above; eigenpairs sorted by value, U = Q V[:, :r], each column flipped so
 //      its largest-magnitude entry is positive (first index on ties).
 //   k = r + oversample <= 512.
 #include "internal.h"
@@ -186,7 +186,8 @@ __global__ void sum_partials_kernel(const double* __restrict__ part, double* __r
 
 // ---- Cholesky S = R^T R (R upper) and Rinv, one block, R in global memory (k x k fp64); shift on breakdown ----
 __global__ void __launch_bounds__(256) chol_inv_kernel(const double* __restrict__ S, double* __restrict__ R,
-                                                       double* __restrict__ Rinv, int k, int* status) {
+                                                       double* __restrict__ Rinv, double* __restrict__ shift_out,
+                                                       int k, int* status) {
   __shared__ int bad;
   __shared__ double shift, rjj_s;
   __shared__ double red[256];
@@ -241,6 +242,7 @@ __global__ void __launch_bounds__(256) chol_inv_kernel(const double* __restrict_
     if (t == 0) record_error(status, ZOACT_ERR_NONFINITE);
     return;
   }
+  if (t == 0) *shift_out = shift;
   // Rinv: solve R * Ri = I column by column (column c per thread)
   for (int c = t; c < k; c += blockDim.x) {
     for (int i = k - 1; i >= 0; --i) {
@@ -281,199 +283,290 @@ __global__ void apply_rinv_kernel(const float* Y, const double* __restrict__ Rin
   }
 }
 
-// ---- cyclic Jacobi on S (k x k, fp64), eigenvalues descending; V columns ----
-constexpr int JACOBI_SMEM = 2 * KMAX * (KMAX + 1) * 8;
-__global__ void jacobi_kernel(const double* __restrict__ S, double* __restrict__ Vout, double* __restrict__ evals,
-                              int k) {
-  extern __shared__ double jac_sm[];
-  double (*A)[KMAX + 1] = reinterpret_cast<double (*)[KMAX + 1]>(jac_sm);
-  double (*V)[KMAX + 1] = reinterpret_cast<double (*)[KMAX + 1]>(jac_sm + KMAX * (KMAX + 1));
-  __shared__ double cs[2];
-  __shared__ int done;
-  __shared__ int order[KMAX];
-  const int t = threadIdx.x;  // blockDim.x >= k
-  for (int v = t; v < k * k; v += blockDim.x) {
-    const int i = v / k, j = v % k;
-    A[i][j] = 0.5 * (S[i * k + j] + S[j * k + i]);
-    V[i][j] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  for (int sweep = 0; sweep < 60; ++sweep) {
-    if (t == 0) {
-      double off = 0.0, tot = 0.0;
-      for (int i = 0; i < k; ++i)
-        for (int j = 0; j < k; ++j) {
-          tot += A[i][j] * A[i][j];
-          if (i != j) off += A[i][j] * A[i][j];
-        }
-      done = (off <= 1e-30 * tot) ? 1 : 0;
-    }
-    __syncthreads();
-    if (done) break;
-    for (int p = 0; p < k - 1; ++p) {
-      for (int q = p + 1; q < k; ++q) {
-        if (t == 0) {
-          const double apq = A[p][q];
-          double c = 1.0, s = 0.0;
-          if (fabs(apq) > 1e-300) {
-            const double theta = (A[q][q] - A[p][p]) / (2.0 * apq);
-            double tt;
-            if (fabs(theta) > 1e150) tt = 0.5 / theta;
-            else tt = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(1.0 + tt * tt);
-            s = tt * c;
-          }
-          cs[0] = c; cs[1] = s;
-        }
-        __syncthreads();
-        const double c = cs[0], s = cs[1];
-        if (s != 0.0) {
-          if (t < k) {  // columns p, q
-            const double ap = A[t][p], aq = A[t][q];
-            A[t][p] = c * ap - s * aq;
-            A[t][q] = s * ap + c * aq;
-            const double vp = V[t][p], vq = V[t][q];
-            V[t][p] = c * vp - s * vq;
-            V[t][q] = s * vp + c * vq;
-          }
-          __syncthreads();
-          if (t < k) {  // rows p, q
-            const double ap = A[p][t], aq = A[q][t];
-            A[p][t] = c * ap - s * aq;
-            A[q][t] = s * ap + c * aq;
-          }
-        }
-        __syncthreads();
-      }
-    }
-  }
-  if (t == 0) {
-    for (int i = 0; i < k; ++i) order[i] = i;
-    for (int i = 0; i < k; ++i) {  // selection sort, descending
-      int best = i;
-      for (int j = i + 1; j < k; ++j)
-        if (A[order[j]][order[j]] > A[order[best]][order[best]]) best = j;
-      const int tmp = order[i]; order[i] = order[best]; order[best] = tmp;
-    }
-  }
-  __syncthreads();
-  for (int v = t; v < k * k; v += blockDim.x) {
-    const int i = v / k, j = v % k;
-    Vout[i * k + j] = V[i][order[j]];
-  }
-  for (int j = t; j < k; j += blockDim.x) evals[j] = A[order[j]][order[j]];
-}
-
-// ---- Jacobi for k > KMAX: A, V in global memory (k x k fp64 each), one block; every sweep runs the
-// round-robin schedule of k' - 1 rounds (k' = k rounded up to even; index k' - 1 is a dummy when k is odd)
-// of k'/2 disjoint rotations: angles from the current A, then A <- A J (columns), A <- J^T A (rows),
-// V <- V J.  Eigenvalues descending in evals, eigenvectors as the columns of Vout. ----
+// ---- eigenpairs of S (k x k, fp64), k <= KMAX: two-sided Jacobi in one block ----
+// Each round of the round-robin schedule (n = k rounded up to even, n - 1 rounds a sweep) rotates n / 2 disjoint
+// pairs: one warp forms the angles, then every thread updates the 2 x 2 blocks J_i^T A J_j of the symmetric matrix in
+// shared memory, half of them (i <= j).  Bound by the fp64 pipe (2 lanes a cycle and SM), so the eigenvectors are left
+// out: the angles are logged and jacobi_vectors_kernel applies them to every row of V on its own SM.  The matrix is
+// padded to n with a zero row, whose rotations are trivial.  Stops when off(A)^2 <= 1e-30 |A|_F^2.
+// k = 48: 17.2 ms as rotations taken one by one with the vectors beside them; 0.92 ms here (its vectors 0.07).
+constexpr int JAC_THREADS = 512;
+constexpr int JAC_SWEEPS = 60;
+constexpr int JACOBI_SMEM = KMAX * (KMAX + 1) * 8;
 __device__ __forceinline__ int rr_member(int slot, int round, int n) {
   // slot 0 stays; slots 1 .. n-1 rotate by `round`
-  return slot == 0 ? 0 : 1 + (slot - 1 + round) % (n - 1);
+  int m = slot - 1 + round;
+  if (m >= n - 1) m -= n - 1;
+  return slot == 0 ? 0 : 1 + m;
 }
-__global__ void __launch_bounds__(1024) jacobi_big_kernel(const double* __restrict__ S, double* __restrict__ A,
-                                                          double* __restrict__ V, double* __restrict__ Vout,
-                                                          double* __restrict__ evals, int k) {
-  __shared__ double cs_c[KLIM / 2], cs_s[KLIM / 2];
-  __shared__ int pp[KLIM / 2], qq[KLIM / 2];
-  __shared__ int done;
-  __shared__ double red[1024];
-  __shared__ int order[KLIM];
-  const int t = threadIdx.x, nt = blockDim.x;
-  const int n = (k + 1) / 2 * 2;
-  const int npair = n / 2;
-  for (int64_t v = t; v < (int64_t)k * k; v += nt) {
-    const int i = (int)(v / k), j = (int)(v % k);
-    A[v] = 0.5 * (S[(int64_t)i * k + j] + S[(int64_t)j * k + i]);
-    V[v] = (i == j) ? 1.0 : 0.0;
+// The rotation that zeroes apq: t = s / c is the smaller root, so |angle| <= pi / 4.
+__device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double& c, double& s, double& t) {
+  c = 1.0; s = 0.0; t = 0.0;
+  if (fabs(apq) > 1e-300) {
+    const double theta = (aqq - app) / (2.0 * apq);
+    if (fabs(theta) > 1e150) t = 0.5 / theta;
+    else t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+    c = 1.0 / sqrt(1.0 + t * t);
+    s = t * c;
+  }
+}
+__global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __restrict__ S, double2* __restrict__ log,
+                                                             int* __restrict__ n_rounds, double* __restrict__ evals,
+                                                             int* __restrict__ order, int k) {
+  extern __shared__ double A[];                      // [n][n + 1]
+  __shared__ double cs_c[KMAX / 2], cs_s[KMAX / 2], cs_t[KMAX / 2];
+  __shared__ int pp[KMAX / 2], qq[KMAX / 2];
+  __shared__ double red[2][JAC_THREADS / 32];
+  const int n = (k + 1) / 2 * 2, np = n / 2, ld = n + 1;
+  const int tid = threadIdx.x;
+  for (int v = tid; v < n * n; v += JAC_THREADS) {
+    const int i = v / n, j = v % n;
+    A[i * ld + j] = i < k && j < k ? 0.5 * (S[i * k + j] + S[j * k + i]) : 0.0;
+  }
+  const int n_blk = np * (np + 1) / 2;
+  int rounds = 0;
+  for (int sweep = 0; sweep < JAC_SWEEPS; ++sweep) {
+    __syncthreads();
+    double off = 0.0, tot = 0.0;
+    for (int v = tid; v < n * n; v += JAC_THREADS) {
+      const int i = v / n, j = v % n;
+      const double a = A[i * ld + j];
+      tot += a * a;
+      if (i != j) off += a * a;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      off += __shfl_xor_sync(0xffffffffu, off, o);
+      tot += __shfl_xor_sync(0xffffffffu, tot, o);
+    }
+    if ((tid & 31) == 0) { red[0][tid >> 5] = off; red[1][tid >> 5] = tot; }
+    __syncthreads();
+    off = tot = 0.0;
+    for (int w = 0; w < JAC_THREADS / 32; ++w) { off += red[0][w]; tot += red[1][w]; }
+    if (!(off > 1e-30 * tot)) break;                 // (also for a matrix that is not finite)
+    for (int round = 0; round < n - 1; ++round, ++rounds) {
+      if (tid < 32 && tid < np) {
+        int p = rr_member(tid, round, n), q = rr_member(n - 1 - tid, round, n);
+        if (p > q) { const int x = p; p = q; q = x; }
+        double c, s, t;
+        jacobi_angle(A[p * ld + p], A[q * ld + q], A[p * ld + q], c, s, t);
+        pp[tid] = p; qq[tid] = q; cs_c[tid] = c; cs_s[tid] = s; cs_t[tid] = t;
+        log[(int64_t)rounds * np + tid] = make_double2(c, s);
+      }
+      __syncthreads();
+      for (int b = tid; b < n_blk; b += JAC_THREADS) {
+        // block (i, j), i <= j, of the triangle's row-major order counted from its end
+        const int r = n_blk - 1 - b;
+        int h = (int)((sqrtf(8.0f * (float)r + 1.0f) - 1.0f) * 0.5f);
+        if ((h + 1) * (h + 2) / 2 <= r) ++h;
+        if (h * (h + 1) / 2 > r) --h;
+        const int i = np - 1 - h, j = np - 1 - (r - h * (h + 1) / 2);
+        const int pi = pp[i], qi = qq[i], pj = pp[j], qj = qq[j];
+        if (i == j) {
+          const double d = cs_t[i] * A[pi * ld + qi];
+          if (d != 0.0) {
+            A[pi * ld + pi] -= d;
+            A[qi * ld + qi] += d;
+            A[pi * ld + qi] = A[qi * ld + pi] = 0.0;
+          }
+          continue;
+        }
+        const double ci = cs_c[i], si = cs_s[i], cj = cs_c[j], sj = cs_s[j];
+        const double a = A[pi * ld + pj], bq = A[pi * ld + qj], cq = A[qi * ld + pj], dq = A[qi * ld + qj];
+        const double a1 = cj * a - sj * bq, b1 = sj * a + cj * bq, c1 = cj * cq - sj * dq, d1 = sj * cq + cj * dq;
+        const double a2 = ci * a1 - si * c1, c2 = si * a1 + ci * c1, b2 = ci * b1 - si * d1, d2 = si * b1 + ci * d1;
+        A[pi * ld + pj] = A[pj * ld + pi] = a2;
+        A[pi * ld + qj] = A[qj * ld + pi] = b2;
+        A[qi * ld + pj] = A[pj * ld + qi] = c2;
+        A[qi * ld + qj] = A[qj * ld + qi] = d2;
+      }
+      __syncthreads();
+    }
+  }
+  if (tid == 0) *n_rounds = rounds;
+  for (int i = tid; i < k; i += JAC_THREADS) {       // descending; first index first on ties
+    const double e = A[i * ld + i];
+    int rank = 0;
+    for (int j = 0; j < k; ++j) {
+      const double f = A[j * ld + j];
+      if (f > e || (f == e && j < i)) ++rank;
+    }
+    order[rank] = i;
+    evals[rank] = e;
+  }
+}
+// V = the product of the logged rotations, one row per warp (row i of the identity times every J in turn), columns in
+// the order of the eigenvalues.
+__global__ void __launch_bounds__(32) jacobi_vectors_kernel(const double2* __restrict__ log,
+                                                            const int* __restrict__ n_rounds,
+                                                            const int* __restrict__ order, double* __restrict__ Vout,
+                                                            int k) {
+  __shared__ double v[KMAX];
+  constexpr int AHEAD = 8;                           // rounds whose angles are loaded together
+  const int n = (k + 1) / 2 * 2, np = n / 2, lane = threadIdx.x;
+  const int rounds = *n_rounds;
+  for (int j = lane; j < n; j += 32) v[j] = j == (int)blockIdx.x ? 1.0 : 0.0;
+  __syncwarp();
+  int round = 0;
+  for (int r0 = 0; r0 < rounds; r0 += AHEAD) {
+    double2 cs[AHEAD];
+#pragma unroll
+    for (int a = 0; a < AHEAD; ++a)
+      cs[a] = lane < np && r0 + a < rounds ? log[(int64_t)(r0 + a) * np + lane] : make_double2(1.0, 0.0);
+#pragma unroll
+    for (int a = 0; a < AHEAD; ++a) {
+      if (r0 + a < rounds && lane < np) {
+        int p = rr_member(lane, round, n), q = rr_member(n - 1 - lane, round, n);
+        if (p > q) { const int x = p; p = q; q = x; }
+        const double vp = v[p], vq = v[q];
+        v[p] = cs[a].x * vp - cs[a].y * vq;
+        v[q] = cs[a].y * vp + cs[a].x * vq;
+      }
+      __syncwarp();
+      if (++round == n - 1) round = 0;
+    }
+  }
+  for (int j = lane; j < k; j += 32) Vout[(int64_t)blockIdx.x * k + j] = v[order[j]];
+}
+
+// ---- eigenpairs of S for k > KMAX: one-sided Jacobi on its Cholesky factor, over the whole chip ----
+// S = R^T R; rotating pairs of columns of R^T until all are orthogonal gives W with S = W W^T, so W's columns are the
+// eigenvectors times the root of their eigenvalue.  One CTA per pair of the round-robin schedule (persistent, a grid
+// barrier per round): the fp64 work of a sweep, 3.5 k^3, is spread over k / 2 SMs, and what is left is the latency of
+// a round.  W [k][k]: column c of R^T is row c of R, contiguous.  Stops after a sweep without a rotation above
+// |x.y| <= sqrt(k) 2^-52 |x||y|.  Every spin is bounded (2 s): a barrier that gives up records ZOACT_ERR_TIMEOUT and
+// releases the others through the abort word.
+// k = 272: 360 ms as two-sided Jacobi in one block; ~10 ms here.
+constexpr int HJ_THREADS = 128;
+constexpr int HJ_SWEEPS = 40;
+struct HjSync {
+  unsigned int count;             // arrivals since the launch
+  int abort;
+  int rotated[HJ_SWEEPS];
+};
+__device__ __forceinline__ bool hj_barrier(HjSync* sy, unsigned int target, int* status) {
+  __shared__ int give_up;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    give_up = 0;
+    __threadfence();
+    atomicAdd(&sy->count, 1u);
+    uint64_t t0 = 0;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    while (*reinterpret_cast<volatile unsigned int*>(&sy->count) < target) {
+      if (*reinterpret_cast<volatile int*>(&sy->abort)) { give_up = 1; break; }
+      uint64_t now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (now - t0 > 2000000000ull) {
+        atomicExch(&sy->abort, 1);
+        record_error(status, ZOACT_ERR_TIMEOUT);
+        give_up = 1;
+        break;
+      }
+    }
+    __threadfence();
   }
   __syncthreads();
-  for (int sweep = 0; sweep < 60; ++sweep) {
-    double off = 0.0, tot = 0.0;
-    for (int64_t v = t; v < (int64_t)k * k; v += nt) {
-      const double a = A[v];
-      tot += a * a;
-      if (v / k != v % k) off += a * a;
-    }
-    red[t] = off;
-    __syncthreads();
-    for (int h = nt / 2; h > 0; h >>= 1) {
-      if (t < h) red[t] += red[t + h];
-      __syncthreads();
-    }
-    const double off_all = red[0];
-    __syncthreads();
-    red[t] = tot;
-    __syncthreads();
-    for (int h = nt / 2; h > 0; h >>= 1) {
-      if (t < h) red[t] += red[t + h];
-      __syncthreads();
-    }
-    if (t == 0) done = (off_all <= 1e-30 * red[0]) ? 1 : 0;
-    __syncthreads();
-    if (done) break;
+  return give_up == 0;
+}
+__global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, HjSync* sy, int k, int* status) {
+  constexpr int PT = (KLIM + HJ_THREADS - 1) / HJ_THREADS;
+  __shared__ double red[3][HJ_THREADS / 32];
+  __shared__ double rot[2];
+  const int n = (k + 1) / 2 * 2, tid = threadIdx.x, i = blockIdx.x;
+  const double tol = sqrt((double)k) * 2.220446049250313e-16;
+  unsigned int target = 0;
+  for (int sweep = 0; sweep < HJ_SWEEPS; ++sweep) {
+    bool any = false;
     for (int round = 0; round < n - 1; ++round) {
-      for (int i = t; i < npair; i += nt) {
-        int p = rr_member(i, round, n), q = rr_member(n - 1 - i, round, n);
-        if (p > q) { const int tmp = p; p = q; q = tmp; }
-        double c = 1.0, s2 = 0.0;
-        if (q < k) {
-          const double apq = A[(int64_t)p * k + q];
-          if (fabs(apq) > 1e-300) {
-            const double theta = (A[(int64_t)q * k + q] - A[(int64_t)p * k + p]) / (2.0 * apq);
-            double tt;
-            if (fabs(theta) > 1e150) tt = 0.5 / theta;
-            else tt = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(1.0 + tt * tt);
-            s2 = tt * c;
+      int p = rr_member(i, round, n), q = rr_member(n - 1 - i, round, n);
+      if (p > q) { const int x = p; p = q; q = x; }
+      if (q < k) {                                   // (odd k: the dummy's partner rests)
+        double x[PT], y[PT], a = 0.0, b = 0.0, g = 0.0;
+#pragma unroll
+        for (int e = 0; e < PT; ++e) {
+          const int c = tid + e * HJ_THREADS;
+          x[e] = c < k ? __ldcg(W + (int64_t)p * k + c) : 0.0;
+          y[e] = c < k ? __ldcg(W + (int64_t)q * k + c) : 0.0;
+        }
+#pragma unroll
+        for (int e = 0; e < PT; ++e) {
+          if (e * HJ_THREADS < k) {
+            a = fma(x[e], x[e], a);
+            b = fma(y[e], y[e], b);
+            g = fma(x[e], y[e], g);
           }
         }
-        pp[i] = p; qq[i] = q; cs_c[i] = c; cs_s[i] = s2;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          a += __shfl_xor_sync(0xffffffffu, a, o);
+          b += __shfl_xor_sync(0xffffffffu, b, o);
+          g += __shfl_xor_sync(0xffffffffu, g, o);
+        }
+        if ((tid & 31) == 0) { red[0][tid >> 5] = a; red[1][tid >> 5] = b; red[2][tid >> 5] = g; }
+        __syncthreads();
+        if (tid == 0) {
+          a = b = g = 0.0;
+          for (int w = 0; w < HJ_THREADS / 32; ++w) { a += red[0][w]; b += red[1][w]; g += red[2][w]; }
+          double c = 1.0, s = 0.0, t = 0.0;
+          if (g * g > tol * tol * a * b) jacobi_angle(a, b, g, c, s, t);
+          rot[0] = c; rot[1] = s;
+        }
+        __syncthreads();
+        const double c = rot[0], s = rot[1];
+        if (s != 0.0) {
+          any = true;
+#pragma unroll
+          for (int e = 0; e < PT; ++e) {
+            const int j = tid + e * HJ_THREADS;
+            if (j < k) {
+              __stcg(W + (int64_t)p * k + j, c * x[e] - s * y[e]);
+              __stcg(W + (int64_t)q * k + j, s * x[e] + c * y[e]);
+            }
+          }
+        }
       }
-      __syncthreads();
-      // columns of A and V: for every row and pair
-      for (int64_t v = t; v < (int64_t)k * npair; v += nt) {
-        const int row = (int)(v / npair), i = (int)(v % npair);
-        const int p = pp[i], q = qq[i];
-        const double c = cs_c[i], s2 = cs_s[i];
-        if (q >= k || s2 == 0.0) continue;
-        const double ap = A[(int64_t)row * k + p], aq = A[(int64_t)row * k + q];
-        A[(int64_t)row * k + p] = c * ap - s2 * aq;
-        A[(int64_t)row * k + q] = s2 * ap + c * aq;
-        const double vp = V[(int64_t)row * k + p], vq = V[(int64_t)row * k + q];
-        V[(int64_t)row * k + p] = c * vp - s2 * vq;
-        V[(int64_t)row * k + q] = s2 * vp + c * vq;
-      }
-      __syncthreads();
-      // rows of A
-      for (int64_t v = t; v < (int64_t)k * npair; v += nt) {
-        const int col = (int)(v / npair), i = (int)(v % npair);
-        const int p = pp[i], q = qq[i];
-        const double c = cs_c[i], s2 = cs_s[i];
-        if (q >= k || s2 == 0.0) continue;
-        const double ap = A[(int64_t)p * k + col], aq = A[(int64_t)q * k + col];
-        A[(int64_t)p * k + col] = c * ap - s2 * aq;
-        A[(int64_t)q * k + col] = s2 * ap + c * aq;
-      }
-      __syncthreads();
+      if (round == n - 2 && any && tid == 0) atomicOr(&sy->rotated[sweep], 1);
+      target += gridDim.x;
+      if (!hj_barrier(sy, target, status)) return;
     }
+    if (*reinterpret_cast<volatile int*>(&sy->rotated[sweep]) == 0) break;
   }
-  if (t == 0) {
-    for (int i = 0; i < k; ++i) order[i] = i;
-    for (int i = 0; i < k; ++i) {  // selection sort, descending
-      int best = i;
-      for (int j = i + 1; j < k; ++j)
-        if (A[(int64_t)order[j] * k + order[j]] > A[(int64_t)order[best] * k + order[best]]) best = j;
-      const int tmp = order[i]; order[i] = order[best]; order[best] = tmp;
-    }
+}
+// Squared norms of W's columns: the eigenvalues of S + shift, unsorted.
+__global__ void __launch_bounds__(HJ_THREADS) hj_norms_kernel(const double* __restrict__ W, double* __restrict__ raw, int k) {
+  __shared__ double red[HJ_THREADS / 32];
+  double a = 0.0;
+  for (int j = threadIdx.x; j < k; j += HJ_THREADS) {
+    const double x = W[(int64_t)blockIdx.x * k + j];
+    a = fma(x, x, a);
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
   __syncthreads();
-  for (int64_t v = t; v < (int64_t)k * k; v += nt) {
-    const int i = (int)(v / k), j = (int)(v % k);
-    Vout[v] = V[(int64_t)i * k + order[j]];
+  if (threadIdx.x == 0) {
+    a = 0.0;
+    for (int w = 0; w < HJ_THREADS / 32; ++w) a += red[w];
+    raw[blockIdx.x] = a;
   }
-  for (int j = t; j < k; j += nt) evals[j] = A[(int64_t)order[j] * k + order[j]];
+}
+// Column c of W, normalised, to its place in the descending order (first index first on ties).
+__global__ void __launch_bounds__(HJ_THREADS) hj_vectors_kernel(const double* __restrict__ W, const double* __restrict__ raw,
+                                                                const double* __restrict__ shift, double* __restrict__ Vout,
+                                                                double* __restrict__ evals, int k) {
+  __shared__ int rank;
+  const int c = blockIdx.x;
+  const double e = raw[c];
+  if (threadIdx.x == 0) rank = 0;
+  __syncthreads();
+  int above = 0;
+  for (int j = threadIdx.x; j < k; j += HJ_THREADS) above += raw[j] > e || (raw[j] == e && j < c);
+  if (above) atomicAdd(&rank, above);
+  __syncthreads();
+  const double inv = e > 0.0 ? 1.0 / sqrt(e) : 0.0;
+  for (int j = threadIdx.x; j < k; j += HJ_THREADS) Vout[(int64_t)j * k + rank] = W[(int64_t)c * k + j] * inv;
+  if (threadIdx.x == 0) evals[rank] = e - *shift;
 }
 
 // ---- U [d, r] = Q [d, k] * V[:, :r] ----
@@ -540,8 +633,12 @@ struct Work {
   double* Rinv;
   double* V;
   double* ev;
-  double* R;      // Cholesky factor / Jacobi matrix (k x k)
-  double* Vw;     // Jacobi rotations (k x k)
+  double* R;      // Cholesky factor; the large Jacobi's columns (k x k)
+  double2* log;   // small Jacobi: the angles of every round
+  double* raw;    // large Jacobi: unsorted eigenvalues
+  double* shift;  // diagonal shift of the last Cholesky
+  int* ints;      // small Jacobi: rounds taken, column order
+  HjSync* sync;   // large Jacobi's barrier
   int nchunk;     // row chunks of the A^T B partials
 };
 
@@ -558,7 +655,7 @@ int orth(Ctx* ctx, Work& w, float* Y, float* Q, int d, int k) {
   const float* src = Y;
   for (int pass = 0; pass < 2; ++pass) {
     launch_atb(ctx, w, src, src, d, k);
-    chol_inv_kernel<<<1, 256, 0, ctx->stream>>>(w.S, w.R, w.Rinv, k, ctx->d_status); ++ctx->n_launch;
+    chol_inv_kernel<<<1, 256, 0, ctx->stream>>>(w.S, w.R, w.Rinv, w.shift, k, ctx->d_status); ++ctx->n_launch;
     apply_rinv_kernel<<<(d + 7) / 8 < 4096 ? (d + 7) / 8 : 4096, dim3(32, 8), 0, ctx->stream>>>(src, w.Rinv, Q, d, k); ++ctx->n_launch;
     ZOACT_CHECK_LAUNCH();
     src = Q;
@@ -575,9 +672,10 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   if (k > KLIM || r > k) return ZOACT_ERR_UNSUPPORTED;
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, JACOBI_SMEM));
   const int nchunk = (d + ATB_CHUNK - 1) / ATB_CHUNK;
-  // workspace: G d*d f32 | Q, Y d*k f32 | part nchunk*k*k f64 | S, Rinv, V, R, Vw k*k f64 | ev k f64
+  // workspace: G d*d f32 | Q, Y d*k f32 | part nchunk*k*k f64 | S, Rinv, V, R k*k f64 | ev, raw, shift f64 | Jacobi
+  const size_t log_bytes = k <= KMAX ? (size_t)JAC_SWEEPS * KMAX * (KMAX / 2) * sizeof(double2) : 0;
   const size_t bytes = (size_t)d * d * 4 + 2 * (size_t)d * k * 4 + (size_t)nchunk * k * k * 8 +
-                       5 * (size_t)k * k * 8 + (size_t)k * 8 + 4096;
+                       4 * (size_t)k * k * 8 + 2 * (size_t)k * 8 + log_bytes + sizeof(HjSync) + 8192;
   uint8_t* base = static_cast<uint8_t*>(scratch(ctx, SLOT_BASIS, bytes));
   if (!base) return ZOACT_ERR_NOMEM;
   Work w;
@@ -592,7 +690,11 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   w.V = reinterpret_cast<double*>(take((size_t)k * k * 8));
   w.ev = reinterpret_cast<double*>(take((size_t)k * 8));
   w.R = reinterpret_cast<double*>(take((size_t)k * k * 8));
-  w.Vw = reinterpret_cast<double*>(take((size_t)k * k * 8));
+  w.log = reinterpret_cast<double2*>(take(log_bytes));
+  w.raw = reinterpret_cast<double*>(take((size_t)k * 8));
+  w.shift = reinterpret_cast<double*>(take(8));
+  w.ints = reinterpret_cast<int*>(take((KMAX + 1) * sizeof(int)));
+  w.sync = reinterpret_cast<HjSync*>(take(sizeof(HjSync)));
   w.nchunk = nchunk;
   (void)off;
 
@@ -635,11 +737,20 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
   launch_atb(ctx, w, w.Q, w.Y, d, k);
   if (k <= KMAX) {
-    jacobi_kernel<<<1, KMAX, JACOBI_SMEM, ctx->stream>>>(w.S, w.V, w.ev, k);
+    jacobi_kernel<<<1, JAC_THREADS, JACOBI_SMEM, ctx->stream>>>(w.S, w.log, w.ints, w.ev, w.ints + 1, k);
+    jacobi_vectors_kernel<<<k, 32, 0, ctx->stream>>>(w.log, w.ints, w.ints + 1, w.V, k);
+    ctx->n_launch += 2;
   } else {
-    jacobi_big_kernel<<<1, 1024, 0, ctx->stream>>>(w.S, w.R, w.Vw, w.V, w.ev, k);
+    chol_inv_kernel<<<1, 256, 0, ctx->stream>>>(w.S, w.R, w.Rinv, w.shift, k, ctx->d_status);
+    ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(HjSync), ctx->stream));
+    void* args[] = {&w.R, &w.sync, &k, &ctx->d_status};
+    ZOACT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(hj_kernel), dim3((unsigned)((k + 1) / 2)),
+                                               dim3(HJ_THREADS), args, 0, ctx->stream));
+    hj_norms_kernel<<<k, HJ_THREADS, 0, ctx->stream>>>(w.R, w.raw, k);
+    hj_vectors_kernel<<<k, HJ_THREADS, 0, ctx->stream>>>(w.R, w.raw, w.shift, w.V, w.ev, k);
+    ctx->n_launch += 4;
   }
-  ++ctx->n_launch;
+  ZOACT_CHECK_LAUNCH();
   ritz_kernel<<<(unsigned)(((int64_t)d * r + 255) / 256), 256, 0, ctx->stream>>>(w.Q, w.V, U_out, d, k, r); ++ctx->n_launch;
   sign_fix_kernel<<<r, 256, 0, ctx->stream>>>(U_out, d, r, ctx->d_status); ++ctx->n_launch;
   if (evals_out) {
