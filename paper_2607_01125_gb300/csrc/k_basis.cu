@@ -8,8 +8,8 @@
 //   2. Omega [d, k] from the Z generator (seed, layer 0, query 0), k = r + oversample.
 //   3. Q = orth(Omega); n_iter times Q = orth(G Q).  orth() is CholeskyQR2:
 //      S = Y^T Y (64 x 64 output tiles; fp32 over 32-row slabs, fp64 across
-//      slabs and row chunks), Cholesky S = R^T R and R^-1 in one block (fp64,
-//      in global memory), Q = Y R^-1; done twice for orthogonality.
+//      slabs and row chunks), R^-1 of the Cholesky factor S = R^T R (fp64),
+//      Q = Y R^-1; done twice for orthogonality.
 //   4. Rayleigh-Ritz: S = Q^T G Q (fp64), Jacobi (fp64): two-sided in one block's
 //      shared memory for k <= 64, one-sided on the Cholesky factor over the whole
 //      chip above; eigenpairs sorted by value, U = Q V[:, :r], each column flipped so
@@ -21,7 +21,7 @@
 namespace zoact {
 namespace {
 
-constexpr int KMAX = 64;        // k handled by the shared-memory Jacobi and R^-1 application
+constexpr int KMAX = 64;        // k handled by the shared-memory Cholesky and Jacobi; column tile of the rest
 constexpr int KLIM = 512;       // largest k
 
 // ---- X [n, d] (16-bit) -> Xt [d, n_pad], zero in columns n .. n_pad-1 ----
@@ -131,17 +131,22 @@ __global__ void __launch_bounds__(256) gemm_gq_kernel(const float* __restrict__ 
   }
 }
 
-// ---- partial S = A^T B over a chunk of rows, A, B [d, k]: 64 x 64 output tiles per block (grid x, y),
-// row chunks on grid z; fp32 products over 32-row slabs, added into fp64 per slab ----
-constexpr int ATB_CHUNK = 2048;
+// ---- partial S = A^T B over a chunk of rows, A, B [rows, k]: 64 x 64 output tiles per block (grid x, y), row chunks on
+// grid z; fp32 products over 32-row slabs, added into fp64 per slab.  sym (A = B): tiles below the diagonal are left out.
+// The fp64 adds (2 lanes a cycle and SM) weigh as much as a slab's FMAs, and a slab is a round trip to L2, so the rows
+// are cut into as many chunks as give every SM two tiles: 7 blocks of 64 slabs took 296 us for 14336 x 32, 14 here (and 8 for the sum of the chunks).
 __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restrict__ A, const float* __restrict__ B,
-                                                          double* __restrict__ part, int d, int k) {
+                                                          double* __restrict__ part, int64_t rows, int k, int chunk,
+                                                          int sym) {
   __shared__ float As[32][KMAX + 4];
   __shared__ float Bs[32][KMAX + 4];
   const int p0 = blockIdx.y * KMAX, q0 = blockIdx.x * KMAX;
+  if (sym && q0 < p0) return;
+  const bool one = sym && q0 == p0;                  // one tile serves both sides
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int64_t r_begin = (int64_t)blockIdx.z * ATB_CHUNK;
-  const int64_t r_end = r_begin + ATB_CHUNK < d ? r_begin + ATB_CHUNK : d;
+  const int64_t r_begin = (int64_t)blockIdx.z * chunk;
+  const int64_t r_end = r_begin + chunk < rows ? r_begin + chunk : rows;
+  const bool live = p0 + ty * 4 < k && q0 + tx * 4 < k;
   double acc[4][4] = {};
   for (int64_t s0 = r_begin; s0 < r_end; s0 += 32) {
     __syncthreads();
@@ -149,25 +154,29 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
       const int rr = v / KMAX, c = v % KMAX;
       const int64_t row = s0 + rr;
       As[rr][c] = (row < r_end && p0 + c < k) ? A[row * k + p0 + c] : 0.f;
-      Bs[rr][c] = (row < r_end && q0 + c < k) ? B[row * k + q0 + c] : 0.f;
+      if (!one) Bs[rr][c] = (row < r_end && q0 + c < k) ? B[row * k + q0 + c] : 0.f;
     }
     __syncthreads();
-    float a32[4][4] = {};
+    if (live) {
+      float (*Bt)[KMAX + 4] = one ? As : Bs;
+      float a32[4][4] = {};
 #pragma unroll 8
-    for (int rr = 0; rr < 32; ++rr) {
-      float a[4], b[4];
+      for (int rr = 0; rr < 32; ++rr) {
+        const float4 a = *reinterpret_cast<const float4*>(&As[rr][ty * 4]);
+        const float4 b = *reinterpret_cast<const float4*>(&Bt[rr][tx * 4]);
+        const float av[4] = {a.x, a.y, a.z, a.w}, bv[4] = {b.x, b.y, b.z, b.w};
 #pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = As[rr][ty * 4 + i]; b[i] = Bs[rr][tx * 4 + i]; }
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) a32[i][j] = fmaf(av[i], bv[j], a32[i][j]);
+      }
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) a32[i][j] = fmaf(a[i], b[j], a32[i][j]);
+        for (int j = 0; j < 4; ++j) acc[i][j] += (double)a32[i][j];
     }
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) acc[i][j] += (double)a32[i][j];
   }
+  if (!live) return;
   double* out = part + (int64_t)blockIdx.z * k * k;
   for (int i = 0; i < 4; ++i)
     for (int j = 0; j < 4; ++j) {
@@ -176,110 +185,347 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
     }
 }
 
-__global__ void sum_partials_kernel(const double* __restrict__ part, double* __restrict__ S, int nblk, int kk) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kk; i += gridDim.x * blockDim.x) {
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += part[(int64_t)b * kk + i];
-    S[i] = s;
-  }
+// S = the chunks' partials, eight strided slices of them per output added last; sym: the upper triangle, mirrored.
+__global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ part, double* __restrict__ S,
+                                                           int nchunk, int k, int sym) {
+  __shared__ double red[8][32];
+  const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+  const int o = blockIdx.x * 32 + lane, kk = k * k;
+  const int i = o / k, j = o - i * k;
+  const bool live = o < kk && !(sym && i > j);
+  double s = 0.0;
+  if (live)
+#pragma unroll 4
+    for (int b = slice; b < nchunk; b += 8) s += part[(int64_t)b * kk + o];
+  red[slice][lane] = s;
+  __syncthreads();
+  if (slice != 0 || !live) return;
+#pragma unroll
+  for (int w = 1; w < 8; ++w) s += red[w][lane];
+  S[o] = s;
+  if (sym) S[j * k + i] = s;
 }
 
-// ---- Cholesky S = R^T R (R upper) and Rinv, one block, R in global memory (k x k fp64); shift on breakdown ----
-__global__ void __launch_bounds__(256) chol_inv_kernel(const double* __restrict__ S, double* __restrict__ R,
-                                                       double* __restrict__ Rinv, double* __restrict__ shift_out,
-                                                       int k, int* status) {
-  __shared__ int bad;
-  __shared__ double shift, rjj_s;
-  __shared__ double red[256];
-  const int t = threadIdx.x;
-  if (t == 0) { shift = 0.0; bad = 0; }
+// ---- LDL^T of an n x n block in shared memory (n <= KMAX), with its inverse factor ----
+// A: the upper triangle in; row j of the eliminated matrix out (its diagonal D).  M: L^-1 out (unit lower triangle).
+// One block-wide barrier a column: while the other warps apply column j, warp 0 finishes row j + 1 and forms its
+// multipliers.  Returns false (to every thread) when a pivot is not positive.  f: 2 x KMAX doubles, bad: two ints.
+__device__ bool ldl_shared(double* A, double* M, int ld, int n, double* f, int* bad) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  auto prepare = [&](int j) {                        // warp 0: the multipliers of row j, whose elimination is done
+    const double d = A[j * ld + j];
+    const double inv = 1.0 / d;
+    for (int p = j + 1 + lane; p < n; p += 32) f[(j & 1) * KMAX + p] = A[j * ld + p] * inv;
+    if (lane == 0) bad[j & 1] = !(d > 0.0);
+  };
+  for (int v = threadIdx.x; v < n * n; v += blockDim.x) M[(v / n) * ld + v % n] = v / n == v % n ? 1.0 : 0.0;
   __syncthreads();
-  for (int attempt = 0; attempt < 4; ++attempt) {
-    for (int v = t; v < k * k; v += blockDim.x) {
-      const int i = v / k, j = v % k;
-      R[v] = (j >= i) ? S[v] + (i == j ? shift : 0.0) : 0.0;
-    }
-    if (t == 0) bad = 0;
-    __syncthreads();
-    for (int j = 0; j < k; ++j) {
-      // r_jj = sqrt(R[j][j] - sum_{p<j} R[p][j]^2)
-      double part = 0.0;
-      for (int p = t; p < j; p += blockDim.x) part += R[(int64_t)p * k + j] * R[(int64_t)p * k + j];
-      red[t] = part;
-      __syncthreads();
-      for (int h = blockDim.x / 2; h > 0; h >>= 1) {
-        if (t < h) red[t] += red[t + h];
-        __syncthreads();
+  if (warp == 0) prepare(0);
+  __syncthreads();
+  for (int j = 0; j < n; ++j) {
+    if (bad[j & 1]) return false;
+    const double* fj = f + (j & 1) * KMAX;
+    if (warp == 0) {
+      if (j + 1 < n) {
+        const int p = j + 1;
+        const double m = fj[p];
+        for (int q = p + lane; q < n; q += 32) A[p * ld + q] -= m * A[j * ld + q];
+        for (int c = lane; c <= j; c += 32) M[p * ld + c] -= m * M[j * ld + c];
+        __syncwarp();
+        prepare(p);
       }
-      if (t == 0) {
-        const double djj = R[(int64_t)j * k + j] - red[0];
-        if (!(djj > 0.0)) {
-          bad = 1;
-        } else {
-          rjj_s = sqrt(djj);
-          R[(int64_t)j * k + j] = rjj_s;
-        }
+    } else {
+      for (int p = j + 1 + warp; p < n; p += warps - 1) {
+        const double m = fj[p];
+        for (int q = p + lane; q < n; q += 32) A[p * ld + q] -= m * A[j * ld + q];
+        for (int c = lane; c <= j; c += 32) M[p * ld + c] -= m * M[j * ld + c];
       }
-      __syncthreads();
-      if (bad) break;
-      // R[j][q] = (R[j][q] - sum_{p<j} R[p][j] R[p][q]) / r_jj for q > j
-      for (int q = j + 1 + t; q < k; q += blockDim.x) {
-        double s2 = R[(int64_t)j * k + q];
-        for (int p = 0; p < j; ++p) s2 -= R[(int64_t)p * k + j] * R[(int64_t)p * k + q];
-        R[(int64_t)j * k + q] = s2 / rjj_s;
-      }
-      __syncthreads();
-    }
-    if (!bad) break;
-    if (t == 0) {
-      double tr = 0.0;
-      for (int i = 0; i < k; ++i) tr += S[(int64_t)i * k + i];
-      shift = (shift == 0.0) ? 1e-12 * tr : shift * 1e3;
     }
     __syncthreads();
   }
-  if (bad) {
-    if (t == 0) record_error(status, ZOACT_ERR_NONFINITE);
+  return true;
+}
+
+// The diagonal shift of attempt 0, 1, 2, ...: none, then 1e-12 of the trace, a thousand times more each time.
+__device__ __forceinline__ double chol_shift(int attempt, double trace) {
+  double s = attempt == 0 ? 0.0 : 1e-12 * trace;
+  for (int i = 1; i < attempt; ++i) s *= 1e3;
+  return s;
+}
+constexpr int CHOL_ATTEMPTS = 4;
+
+// ---- R^-1 of the Cholesky factor S = R^T R (R upper), k <= KMAX: one block, everything in shared memory ----
+// R^-1 = L^-T D^-1/2.  Bound by a column's chain (a row's update, a division, a barrier) and the fp64 pipe; k = 48:
+// 228 us with the factor in global memory and a serial inverse per column, 46 here.
+constexpr int CHOL_THREADS = 512;
+constexpr int CHOL_SMEM = 2 * KMAX * (KMAX + 1) * 8;
+__global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(const double* __restrict__ S, double* __restrict__ Rinv,
+                                                                int k, int* status) {
+  extern __shared__ double sm[];
+  __shared__ double f[2 * KMAX], rs[KMAX], trace;
+  __shared__ int bad[2];
+  const int ld = k + 1;
+  double* A = sm;
+  double* M = sm + k * ld;
+  bool ok = false;
+  for (int attempt = 0; attempt < CHOL_ATTEMPTS && !ok; ++attempt) {
+    __syncthreads();
+    if (threadIdx.x == 0 && attempt == 1) {
+      trace = 0.0;
+      for (int i = 0; i < k; ++i) trace += S[i * k + i];
+    }
+    __syncthreads();
+    const double shift = chol_shift(attempt, attempt ? trace : 0.0);
+    for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
+      const int i = v / k, j = v % k;
+      A[i * ld + j] = S[v] + (i == j ? shift : 0.0);
+    }
+    __syncthreads();
+    ok = ldl_shared(A, M, ld, k, f, bad);
+  }
+  if (!ok) {
+    if (threadIdx.x == 0) record_error(status, ZOACT_ERR_NONFINITE);
     return;
   }
-  if (t == 0) *shift_out = shift;
-  // Rinv: solve R * Ri = I column by column (column c per thread)
-  for (int c = t; c < k; c += blockDim.x) {
-    for (int i = k - 1; i >= 0; --i) {
-      double s2 = (i == c) ? 1.0 : 0.0;
-      for (int p = i + 1; p <= c; ++p) s2 -= R[(int64_t)i * k + p] * Rinv[(int64_t)p * k + c];
-      Rinv[(int64_t)i * k + c] = i > c ? 0.0 : s2 / R[(int64_t)i * k + i];
+  for (int i = threadIdx.x; i < k; i += CHOL_THREADS) rs[i] = 1.0 / sqrt(A[i * ld + i]);
+  __syncthreads();
+  for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
+    const int i = v / k, c = v % k;
+    Rinv[v] = i <= c ? M[c * ld + i] * rs[c] : 0.0;
+  }
+}
+
+// ---- grid barrier of a cooperative launch: bounded (2 s); a barrier that gives up records ZOACT_ERR_TIMEOUT and
+// releases the others through the abort word ----
+constexpr int HJ_SWEEPS = 40;
+struct GridSync {
+  unsigned int count;             // arrivals since the launch
+  int abort;
+  int rotated[HJ_SWEEPS];         // large Jacobi: a sweep rotated something
+};
+__device__ __forceinline__ bool grid_barrier(GridSync* sy, unsigned int target, int* status) {
+  __shared__ int give_up;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    give_up = 0;
+    __threadfence();
+    atomicAdd(&sy->count, 1u);
+    uint64_t t0 = 0;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+    while (*reinterpret_cast<volatile unsigned int*>(&sy->count) < target) {
+      if (*reinterpret_cast<volatile int*>(&sy->abort)) { give_up = 1; break; }
+      uint64_t now;
+      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+      if (now - t0 > 2000000000ull) {
+        atomicExch(&sy->abort, 1);
+        record_error(status, ZOACT_ERR_TIMEOUT);
+        give_up = 1;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  return give_up == 0;
+}
+
+// ---- R and R^-1 for k > KMAX: blocked LDL^T over the chip (cooperative) ----
+// Panels of CB columns.  Every block factors the panel's diagonal block by itself (no barrier), the panel's rows of A
+// and of M = L^-1 are multiplied by its inverse factor in 8-column strips, and after a barrier the rows below get their
+// rank-CB update in 16 x 16 tiles.  Two barriers a panel; the columns' chain (as above) is most of the time.  k = 272:
+// 5.6 ms in one block, 0.34 here.
+constexpr int CB = 32;
+constexpr int CHOLB_THREADS = 256;
+constexpr int CHOLB_BLOCKS = 96;
+struct CholBig {
+  const double* S;
+  double* A;          // S eliminated, then R
+  double* M;          // L^-1
+  double* Rinv;
+  double* D;          // pivots
+  double* shift;      // the shift taken
+  GridSync* sync;
+  int k;
+  int* status;
+};
+__global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
+  __shared__ double sA[CB * (CB + 1)], sM[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], trace_s;
+  __shared__ int bad[2];
+  __shared__ double sx[CB][17], sf[CB][17], inv_d[CB];
+  const int k = w.k, tid = threadIdx.x;
+  const int64_t gtid = blockIdx.x * (int64_t)CHOLB_THREADS + tid, gthreads = (int64_t)gridDim.x * CHOLB_THREADS;
+  unsigned int target = 0;
+  auto sync = [&]() { target += gridDim.x; return grid_barrier(w.sync, target, w.status); };
+  // the trace, the same sum in every block
+  double tr = 0.0;
+  for (int i = tid; i < k; i += CHOLB_THREADS) tr += w.S[(int64_t)i * k + i];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
+  if ((tid & 31) == 0) red[tid >> 5] = tr;
+  __syncthreads();
+  if (tid == 0) {
+    trace_s = 0.0;
+    for (int i = 0; i < CHOLB_THREADS / 32; ++i) trace_s += red[i];
+  }
+  __syncthreads();
+  bool ok = false;
+  double shift = 0.0;
+  for (int attempt = 0; attempt < CHOL_ATTEMPTS && !ok; ++attempt) {
+    shift = chol_shift(attempt, trace_s);
+    if (attempt > 0 && !sync()) return;              // every block has seen the failed pivot before A is rewritten
+    for (int64_t v = gtid; v < (int64_t)k * k; v += gthreads) {
+      const int i = (int)(v / k), j = (int)(v % k);
+      __stcg(w.A + v, j >= i ? w.S[v] + (i == j ? shift : 0.0) : 0.0);
+      __stcg(w.M + v, i == j ? 1.0 : 0.0);
+    }
+    if (!sync()) return;
+    ok = true;
+    for (int p0 = 0; p0 < k; p0 += CB) {
+      const int nb = min(CB, k - p0), p1 = p0 + nb;
+      for (int v = tid; v < nb * nb; v += CHOLB_THREADS)
+        sA[(v / nb) * (CB + 1) + v % nb] = __ldcg(w.A + (int64_t)(p0 + v / nb) * k + p0 + v % nb);
+      __syncthreads();
+      if (!ldl_shared(sA, sM, CB + 1, nb, f, bad)) { ok = false; break; }     // the same answer in every block
+      if (tid < nb) inv_d[tid] = 1.0 / sA[tid * (CB + 1) + tid];
+      // strips: columns p1 .. k of A, then 0 .. p0 of M, eight at a time
+      const int na = k - p1, cols = na + p0;
+      for (int g = blockIdx.x; g * 8 < cols; g += gridDim.x) {
+        const int i = tid >> 3, c = g * 8 + (tid & 7);
+        double* base = c < na ? w.A + (int64_t)p0 * k + p1 + c : w.M + (int64_t)p0 * k + (c - na);
+        if (i < nb && c < cols) sx[i][tid & 7] = __ldcg(base + (int64_t)i * k);
+        __syncthreads();
+        double x = 0.0;
+        if (i < nb && c < cols)
+          for (int l = 0; l <= i; ++l) x = fma(sM[i * (CB + 1) + l], sx[l][tid & 7], x);
+        if (i < nb && c < cols) __stcg(base + (int64_t)i * k, x);
+        __syncthreads();
+      }
+      if (blockIdx.x == gridDim.x - 1) {             // the diagonal block itself
+        for (int v = tid; v < nb * nb; v += CHOLB_THREADS) {
+          const int i = v / nb, j = v % nb;
+          if (j <= i) __stcg(w.M + (int64_t)(p0 + i) * k + p0 + j, sM[i * (CB + 1) + j]);
+          if (j >= i) __stcg(w.D + (int64_t)(p0 + i) * k + p0 + j, sA[i * (CB + 1) + j]);
+        }
+      }
+      if (!sync()) return;
+      if (p1 >= k) break;
+      // rows below: A[q][c] (c >= q) and M[q][c] (c < p1) lose sum_l (X[l][q] / D_l) X[l][c]
+      const int nq = (k - p1 + 15) / 16, nm = (p1 + 15) / 16;
+      const int ta = nq * (nq + 1) / 2, total = ta + nq * nm;
+      for (int t = blockIdx.x; t < total; t += gridDim.x) {
+        int qb, cb;
+        const bool in_a = t < ta;
+        if (in_a) {
+          qb = 0;
+          int rest = t;
+          while (rest >= nq - qb) { rest -= nq - qb; ++qb; }
+          cb = qb + rest;
+        } else {
+          qb = (t - ta) / nm;
+          cb = (t - ta) - qb * nm;
+        }
+        const int q0 = p1 + 16 * qb, c0 = in_a ? p1 + 16 * cb : 16 * cb;
+        const int c_end = in_a ? k : p1;
+        __syncthreads();
+        for (int v = tid; v < nb * 16; v += CHOLB_THREADS) {
+          const int l = v >> 4, e = v & 15;
+          const int64_t row = (int64_t)(p0 + l) * k;
+          sf[l][e] = q0 + e < k ? __ldcg(w.A + row + q0 + e) * inv_d[l] : 0.0;
+          double x = 0.0;
+          if (c0 + e < c_end)
+            x = in_a ? __ldcg(w.A + row + c0 + e) : c0 + e < p0 ? __ldcg(w.M + row + c0 + e)
+                                                                : (c0 + e - p0 <= l ? sM[l * (CB + 1) + c0 + e - p0] : 0.0);
+          sx[l][e] = x;
+        }
+        __syncthreads();
+        const int q = q0 + (tid >> 4), c = c0 + (tid & 15);
+        if (q < k && c < c_end && (!in_a || c >= q)) {
+          double* dst = (in_a ? w.A : w.M) + (int64_t)q * k + c;
+          double x = __ldcg(dst);
+          for (int l = 0; l < nb; ++l) x = fma(-sf[l][tid >> 4], sx[l][tid & 15], x);
+          __stcg(dst, x);
+        }
+      }
+      if (!sync()) return;
+    }
+  }
+  if (!ok) {
+    if (gtid == 0) record_error(w.status, ZOACT_ERR_NONFINITE);
+    return;
+  }
+  if (gtid == 0) *w.shift = shift;
+  // R[j][q] = X[j][q] / sqrt(D_j); R^-1 = L^-T D^-1/2 (the diagonal blocks' rows came to D's place)
+  for (int64_t v = gtid; v < (int64_t)k * k; v += gthreads) {
+    const int i = (int)(v / k), j = (int)(v % k);
+    const double di = __ldcg(w.D + (int64_t)i * k + i), dj = __ldcg(w.D + (int64_t)j * k + j);
+    if (j >= i) {
+      const double x = j / CB == i / CB ? __ldcg(w.D + v) : __ldcg(w.A + v);
+      w.Rinv[v] = __ldcg(w.M + (int64_t)j * k + i) / sqrt(dj);
+      __stcg(w.A + v, x / sqrt(di));
+    } else {
+      w.Rinv[v] = 0.0;
+      __stcg(w.A + v, 0.0);
     }
   }
 }
 
-// ---- Q [d, k] = Y [d, k] * Rinv [k, k] (fp64 accumulate, fp32 out); Q may alias Y ----
-// One warp per row: every lane reads the row before any lane writes it.
-// R^-1 is read from shared memory for k <= KMAX, else from global memory (L2).
-__global__ void apply_rinv_kernel(const float* Y, const double* __restrict__ Rinv, float* Q, int d, int k) {
-  __shared__ double Rs[KMAX * KMAX];
-  const bool in_smem = k <= KMAX;
-  if (in_smem)
-    for (int v = threadIdx.y * blockDim.x + threadIdx.x; v < k * k; v += blockDim.x * blockDim.y) Rs[v] = Rinv[v];
-  __syncthreads();
-  const double* Rm = in_smem ? Rs : Rinv;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.y + threadIdx.y; i < d; i += (int64_t)gridDim.x * blockDim.y) {
-    float out[KLIM / 32];
-#pragma unroll
-    for (int h = 0; h < KLIM / 32; ++h) {
-      const int c = threadIdx.x + 32 * h;
-      double s = 0.0;
-      if (c < k)
-        for (int p = 0; p <= c; ++p) s += (double)Y[i * k + p] * Rm[(int64_t)p * k + c];
-      out[h] = (float)s;
+// ---- out [rows, c] = A [rows, k] (fp32) M [k, ldm] (fp64, first c columns): 64 x 64 tiles ----
+// Every product is exact (an fp32 entry times a two-float split of M's, 48 bits) and added with its rounding error
+// carried along (two-sum), so a sum holds ~46 bits: eleven fp32 instructions a term, against one fp64 FMA at a
+// sixty-fourth of their rate.  tri: M is upper triangular.  5120 x 48 x 48: 73 us in fp64, 26 here; 4096 x 272 x 272: 836 and 181.
+__global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A, const double* __restrict__ M,
+                                                    float* __restrict__ out, int64_t rows, int k, int ldm, int c,
+                                                    int tri) {
+  __shared__ float As[32][KMAX + 4];                 // [p][row]
+  __shared__ float Mh[32][KMAX], Ml[32][KMAX];       // [p][column]
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  const int64_t r0 = (int64_t)blockIdx.x * 64;
+  const int c0 = blockIdx.y * 64;
+  const bool live = c0 + tx * 4 < c;
+  float s[4][4] = {}, lo[4][4] = {};
+  const int p_end = tri ? min(k, c0 + 64) : k;
+  for (int p0 = 0; p0 < p_end; p0 += 32) {
+    __syncthreads();
+    for (int v = threadIdx.x; v < 64 * 32; v += 256) {
+      const int rr = v / 32, p = v % 32;
+      As[p][rr] = r0 + rr < rows && p0 + p < k ? A[(r0 + rr) * k + p0 + p] : 0.f;
     }
-    __syncwarp();
-#pragma unroll
-    for (int h = 0; h < KLIM / 32; ++h) {
-      const int c = threadIdx.x + 32 * h;
-      if (c < k) Q[i * k + c] = out[h];
+    for (int v = threadIdx.x; v < 32 * 64; v += 256) {
+      const int p = v / 64, cc = v % 64;
+      const double m = p0 + p < k && c0 + cc < c ? M[(int64_t)(p0 + p) * ldm + c0 + cc] : 0.0;
+      const float h = (float)m;
+      Mh[p][cc] = h;
+      Ml[p][cc] = (float)(m - (double)h);
     }
-    __syncwarp();
+    __syncthreads();
+    if (live) {
+#pragma unroll 4
+      for (int p = 0; p < 32; ++p) {
+        const float4 a4 = *reinterpret_cast<const float4*>(&As[p][ty * 4]);
+        const float4 h4 = *reinterpret_cast<const float4*>(&Mh[p][tx * 4]);
+        const float4 l4 = *reinterpret_cast<const float4*>(&Ml[p][tx * 4]);
+        const float av[4] = {a4.x, a4.y, a4.z, a4.w}, hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float pr = __fmul_rn(av[i], hv[j]);
+            const float e = __fmaf_rn(av[i], lv[j], __fmaf_rn(av[i], hv[j], -pr));
+            const float t = __fadd_rn(s[i][j], pr);
+            const float b = __fsub_rn(t, s[i][j]);
+            const float err = __fadd_rn(__fsub_rn(s[i][j], __fsub_rn(t, b)), __fsub_rn(pr, b));
+            s[i][j] = t;
+            lo[i][j] = __fadd_rn(lo[i][j], __fadd_rn(err, e));
+          }
+      }
+    }
+  }
+  if (!live) return;
+  for (int i = 0; i < 4; ++i) {
+    const int64_t row = r0 + ty * 4 + i;
+    if (row >= rows) continue;
+    for (int j = 0; j < 4; ++j)
+      if (c0 + tx * 4 + j < c) out[row * c + c0 + tx * 4 + j] = s[i][j] + lo[i][j];
   }
 }
 
@@ -434,42 +680,10 @@ __global__ void __launch_bounds__(32) jacobi_vectors_kernel(const double2* __res
 // eigenvectors times the root of their eigenvalue.  One CTA per pair of the round-robin schedule (persistent, a grid
 // barrier per round): the fp64 work of a sweep, 3.5 k^3, is spread over k / 2 SMs, and what is left is the latency of
 // a round.  W [k][k]: column c of R^T is row c of R, contiguous.  Stops after a sweep without a rotation above
-// |x.y| <= sqrt(k) 2^-52 |x||y|.  Every spin is bounded (2 s): a barrier that gives up records ZOACT_ERR_TIMEOUT and
-// releases the others through the abort word.
+// |x.y| <= sqrt(k) 2^-52 |x||y|.
 // k = 272: 360 ms as two-sided Jacobi in one block; ~10 ms here.
 constexpr int HJ_THREADS = 128;
-constexpr int HJ_SWEEPS = 40;
-struct HjSync {
-  unsigned int count;             // arrivals since the launch
-  int abort;
-  int rotated[HJ_SWEEPS];
-};
-__device__ __forceinline__ bool hj_barrier(HjSync* sy, unsigned int target, int* status) {
-  __shared__ int give_up;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    give_up = 0;
-    __threadfence();
-    atomicAdd(&sy->count, 1u);
-    uint64_t t0 = 0;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    while (*reinterpret_cast<volatile unsigned int*>(&sy->count) < target) {
-      if (*reinterpret_cast<volatile int*>(&sy->abort)) { give_up = 1; break; }
-      uint64_t now;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-      if (now - t0 > 2000000000ull) {
-        atomicExch(&sy->abort, 1);
-        record_error(status, ZOACT_ERR_TIMEOUT);
-        give_up = 1;
-        break;
-      }
-    }
-    __threadfence();
-  }
-  __syncthreads();
-  return give_up == 0;
-}
-__global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, HjSync* sy, int k, int* status) {
+__global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, GridSync* sy, int k, int* status) {
   constexpr int PT = (KLIM + HJ_THREADS - 1) / HJ_THREADS;
   __shared__ double red[3][HJ_THREADS / 32];
   __shared__ double rot[2];
@@ -528,7 +742,7 @@ __global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, 
       }
       if (round == n - 2 && any && tid == 0) atomicOr(&sy->rotated[sweep], 1);
       target += gridDim.x;
-      if (!hj_barrier(sy, target, status)) return;
+      if (!grid_barrier(sy, target, status)) return;
     }
     if (*reinterpret_cast<volatile int*>(&sy->rotated[sweep]) == 0) break;
   }
@@ -567,19 +781,6 @@ __global__ void __launch_bounds__(HJ_THREADS) hj_vectors_kernel(const double* __
   const double inv = e > 0.0 ? 1.0 / sqrt(e) : 0.0;
   for (int j = threadIdx.x; j < k; j += HJ_THREADS) Vout[(int64_t)j * k + rank] = W[(int64_t)c * k + j] * inv;
   if (threadIdx.x == 0) evals[rank] = e - *shift;
-}
-
-// ---- U [d, r] = Q [d, k] * V[:, :r] ----
-__global__ void ritz_kernel(const float* __restrict__ Q, const double* __restrict__ V, float* __restrict__ U, int d,
-                            int k, int r) {
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < (int64_t)d * r;
-       v += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = v / r;
-    const int j = (int)(v % r);
-    double s = 0.0;
-    for (int p = 0; p < k; ++p) s += (double)Q[i * k + p] * V[p * k + j];
-    U[v] = (float)s;
-  }
 }
 
 // ---- flip column j so its largest-|.| entry (first index on ties) is positive ----
@@ -633,32 +834,75 @@ struct Work {
   double* Rinv;
   double* V;
   double* ev;
-  double* R;      // Cholesky factor; the large Jacobi's columns (k x k)
+  double* R;      // k > KMAX: Cholesky factor; the large Jacobi's columns (k x k)
+  double* M;      // k > KMAX: its inverse factor L^-1
+  double* D;      // k > KMAX: its diagonal blocks
   double2* log;   // small Jacobi: the angles of every round
   double* raw;    // large Jacobi: unsorted eigenvalues
   double* shift;  // diagonal shift of the last Cholesky
   int* ints;      // small Jacobi: rounds taken, column order
-  HjSync* sync;   // large Jacobi's barrier
-  int nchunk;     // row chunks of the A^T B partials
+  GridSync* sync; // barrier of the cooperative launches
 };
 
-void launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int d, int k) {
-  const unsigned tiles = (unsigned)((k + KMAX - 1) / KMAX);
-  atb_partial_kernel<<<dim3(tiles, tiles, (unsigned)w.nchunk), 256, 0, ctx->stream>>>(A, B, w.part, d, k);
-  ++ctx->n_launch;
-  sum_partials_kernel<<<(k * k + 255) / 256, 256, 0, ctx->stream>>>(w.part, w.S, w.nchunk, k * k);
-  ++ctx->n_launch;
+// Row chunks of an A^T B over `rows` rows: two blocks per SM over all tiles, 32-row slabs.
+int atb_chunks(const Ctx* ctx, int64_t rows, int k, int& chunk) {
+  const int64_t t = (k + KMAX - 1) / KMAX, tiles = t * (t + 1) / 2, slabs = (rows + 31) / 32;
+  int64_t n = (2 * ctx->sm_count + tiles - 1) / tiles;
+  if (n > slabs) n = slabs;
+  const int64_t per = (slabs + n - 1) / n;
+  chunk = (int)(per * 32);
+  return (int)((slabs + per - 1) / per);
 }
 
-int orth(Ctx* ctx, Work& w, float* Y, float* Q, int d, int k) {
-  // CholeskyQR2: Q = Y R^-1 twice
-  const float* src = Y;
+// S = A^T B of A, B [rows, k] (A = B: the symmetric form)
+int launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int64_t rows, int k) {
+  const unsigned tiles = (unsigned)((k + KMAX - 1) / KMAX);
+  const int sym = A == B;
+  int chunk;
+  const int nchunk = atb_chunks(ctx, rows, k, chunk);
+  atb_partial_kernel<<<dim3(tiles, tiles, (unsigned)nchunk), 256, 0, ctx->stream>>>(A, B, w.part, rows, k, chunk, sym);
+  sum_partials_kernel<<<(k * k + 31) / 32, 256, 0, ctx->stream>>>(w.part, w.S, nchunk, k, sym);
+  ctx->n_launch += 2;
+  ZOACT_CHECK_LAUNCH();
+  return ZOACT_OK;
+}
+
+// R^-1 (k > KMAX: and R, the shift) of S
+int launch_chol(Ctx* ctx, const Work& w, int k) {
+  if (k <= KMAX) {
+    chol_inv_kernel<<<1, CHOL_THREADS, CHOL_SMEM, ctx->stream>>>(w.S, w.Rinv, k, ctx->d_status);
+  } else {
+    ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
+    CholBig c{w.S, w.R, w.M, w.Rinv, w.D, w.shift, w.sync, k, ctx->d_status};
+    void* args[] = {&c};
+    const int blocks = CHOLB_BLOCKS < ctx->sm_count ? CHOLB_BLOCKS : ctx->sm_count;
+    ZOACT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(chol_big_kernel), dim3((unsigned)blocks),
+                                               dim3(CHOLB_THREADS), args, 0, ctx->stream));
+  }
+  ++ctx->n_launch;
+  ZOACT_CHECK_LAUNCH();
+  return ZOACT_OK;
+}
+
+int launch_apply(Ctx* ctx, const float* A, const double* M, float* out, int64_t rows, int k, int ldm, int c, int tri) {
+  apply_kernel<<<dim3((unsigned)((rows + 63) / 64), (unsigned)((c + 63) / 64)), 256, 0, ctx->stream>>>(A, M, out, rows, k,
+                                                                                                  ldm, c, tri);
+  ++ctx->n_launch;
+  ZOACT_CHECK_LAUNCH();
+  return ZOACT_OK;
+}
+
+// CholeskyQR2 of Y [d, k], which holds Q afterwards; tmp: another [d, k].
+int orth(Ctx* ctx, const Work& w, float* Y, float* tmp, int d, int k) {
+  float* src = Y;
+  float* dst = tmp;
   for (int pass = 0; pass < 2; ++pass) {
-    launch_atb(ctx, w, src, src, d, k);
-    chol_inv_kernel<<<1, 256, 0, ctx->stream>>>(w.S, w.R, w.Rinv, w.shift, k, ctx->d_status); ++ctx->n_launch;
-    apply_rinv_kernel<<<(d + 7) / 8 < 4096 ? (d + 7) / 8 : 4096, dim3(32, 8), 0, ctx->stream>>>(src, w.Rinv, Q, d, k); ++ctx->n_launch;
-    ZOACT_CHECK_LAUNCH();
-    src = Q;
+    int st = launch_atb(ctx, w, src, src, d, k);
+    if (!st) st = launch_chol(ctx, w, k);
+    if (!st) st = launch_apply(ctx, src, w.Rinv, dst, d, k, k, k, 1);
+    if (st) return st;
+    src = tmp;
+    dst = Y;
   }
   return ZOACT_OK;
 }
@@ -671,32 +915,36 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   if (k > d) k = d;
   if (k > KLIM || r > k) return ZOACT_ERR_UNSUPPORTED;
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, JACOBI_SMEM));
-  const int nchunk = (d + ATB_CHUNK - 1) / ATB_CHUNK;
-  // workspace: G d*d f32 | Q, Y d*k f32 | part nchunk*k*k f64 | S, Rinv, V, R k*k f64 | ev, raw, shift f64 | Jacobi
+  ZOACT_CUDA_TRY(cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_SMEM));
+  int chunk;
+  const size_t nchunk = (size_t)atb_chunks(ctx, d, k, chunk);
+  const size_t kk = (size_t)k * k * 8, dk = (size_t)d * k * 4, big = k > KMAX ? kk : 0;
   const size_t log_bytes = k <= KMAX ? (size_t)JAC_SWEEPS * KMAX * (KMAX / 2) * sizeof(double2) : 0;
-  const size_t bytes = (size_t)d * d * 4 + 2 * (size_t)d * k * 4 + (size_t)nchunk * k * k * 8 +
-                       4 * (size_t)k * k * 8 + 2 * (size_t)k * 8 + log_bytes + sizeof(HjSync) + 8192;
+  // workspace (every piece padded to 256 bytes)
+  const size_t bytes = (size_t)d * d * 4 + 2 * dk + nchunk * kk + 3 * kk + 3 * big + log_bytes + 2 * (size_t)k * 8 +
+                       sizeof(GridSync) + 16 * 256 + 4096;
   uint8_t* base = static_cast<uint8_t*>(scratch(ctx, SLOT_BASIS, bytes));
   if (!base) return ZOACT_ERR_NOMEM;
   Work w;
   size_t off = 0;
   auto take = [&](size_t b) { uint8_t* p = base + off; off += (b + 255) / 256 * 256; return p; };
   w.G = reinterpret_cast<float*>(take((size_t)d * d * 4));
-  w.Q = reinterpret_cast<float*>(take((size_t)d * k * 4));
-  w.Y = reinterpret_cast<float*>(take((size_t)d * k * 4));
-  w.part = reinterpret_cast<double*>(take((size_t)nchunk * k * k * 8));
-  w.S = reinterpret_cast<double*>(take((size_t)k * k * 8));
-  w.Rinv = reinterpret_cast<double*>(take((size_t)k * k * 8));
-  w.V = reinterpret_cast<double*>(take((size_t)k * k * 8));
+  w.Q = reinterpret_cast<float*>(take(dk));
+  w.Y = reinterpret_cast<float*>(take(dk));
+  w.part = reinterpret_cast<double*>(take(nchunk * kk));
+  w.S = reinterpret_cast<double*>(take(kk));
+  w.Rinv = reinterpret_cast<double*>(take(kk));
+  w.V = reinterpret_cast<double*>(take(kk));
+  w.R = reinterpret_cast<double*>(take(big));
+  w.M = reinterpret_cast<double*>(take(big));
+  w.D = reinterpret_cast<double*>(take(big));
   w.ev = reinterpret_cast<double*>(take((size_t)k * 8));
-  w.R = reinterpret_cast<double*>(take((size_t)k * k * 8));
   w.log = reinterpret_cast<double2*>(take(log_bytes));
   w.raw = reinterpret_cast<double*>(take((size_t)k * 8));
   w.shift = reinterpret_cast<double*>(take(8));
   w.ints = reinterpret_cast<int*>(take((KMAX + 1) * sizeof(int)));
-  w.sync = reinterpret_cast<HjSync*>(take(sizeof(HjSync)));
-  w.nchunk = nchunk;
-  (void)off;
+  w.sync = reinterpret_cast<GridSync*>(take(sizeof(GridSync)));
+  if (off > bytes) return ZOACT_ERR_NOMEM;
 
   // 1. Gram
   if (xdtype == ZOACT_DT_FP32) {
@@ -720,11 +968,11 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
     const int st = launch_gemm_tc_f32out(ctx, Xt, Xt, xdtype, d, d, (int)n_pad, w.G);
     if (st) return st;
   }
-  // 2-3. sketch and subspace iteration
+  // 2-3. sketch and subspace iteration: Q stays in w.Q
   const int64_t nq = (int64_t)d * k;
-  omega_kernel<<<(unsigned)((nq / 4 + 255) / 256 + 1), 256, 0, ctx->stream>>>(w.Y, nq, seed); ++ctx->n_launch;
+  omega_kernel<<<(unsigned)((nq / 4 + 255) / 256 + 1), 256, 0, ctx->stream>>>(w.Q, nq, seed); ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
-  int st = orth(ctx, w, w.Y, w.Q, d, k);
+  int st = orth(ctx, w, w.Q, w.Y, d, k);
   if (st) return st;
   const dim3 gq_blocks((unsigned)((d + 63) / 64), (unsigned)((k + KMAX - 1) / KMAX));
   for (int it = 0; it < n_iter; ++it) {
@@ -732,26 +980,31 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
     ZOACT_CHECK_LAUNCH();
     st = orth(ctx, w, w.Y, w.Q, d, k);
     if (st) return st;
+    float* t = w.Q; w.Q = w.Y; w.Y = t;
   }
   // 4. Rayleigh-Ritz
   gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
-  launch_atb(ctx, w, w.Q, w.Y, d, k);
+  ZOACT_CHECK_LAUNCH();
+  st = launch_atb(ctx, w, w.Q, w.Y, d, k);
+  if (st) return st;
   if (k <= KMAX) {
     jacobi_kernel<<<1, JAC_THREADS, JACOBI_SMEM, ctx->stream>>>(w.S, w.log, w.ints, w.ev, w.ints + 1, k);
     jacobi_vectors_kernel<<<k, 32, 0, ctx->stream>>>(w.log, w.ints, w.ints + 1, w.V, k);
     ctx->n_launch += 2;
   } else {
-    chol_inv_kernel<<<1, 256, 0, ctx->stream>>>(w.S, w.R, w.Rinv, w.shift, k, ctx->d_status);
-    ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(HjSync), ctx->stream));
+    st = launch_chol(ctx, w, k);
+    if (st) return st;
+    ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
     void* args[] = {&w.R, &w.sync, &k, &ctx->d_status};
     ZOACT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(hj_kernel), dim3((unsigned)((k + 1) / 2)),
                                                dim3(HJ_THREADS), args, 0, ctx->stream));
     hj_norms_kernel<<<k, HJ_THREADS, 0, ctx->stream>>>(w.R, w.raw, k);
     hj_vectors_kernel<<<k, HJ_THREADS, 0, ctx->stream>>>(w.R, w.raw, w.shift, w.V, w.ev, k);
-    ctx->n_launch += 4;
+    ctx->n_launch += 3;
   }
   ZOACT_CHECK_LAUNCH();
-  ritz_kernel<<<(unsigned)(((int64_t)d * r + 255) / 256), 256, 0, ctx->stream>>>(w.Q, w.V, U_out, d, k, r); ++ctx->n_launch;
+  st = launch_apply(ctx, w.Q, w.V, U_out, d, k, k, r, 0);
+  if (st) return st;
   sign_fix_kernel<<<r, 256, 0, ctx->stream>>>(U_out, d, r, ctx->d_status); ++ctx->n_launch;
   if (evals_out) {
     f64_to_f32_kernel<<<1, 256, 0, ctx->stream>>>(w.ev, evals_out, k);
