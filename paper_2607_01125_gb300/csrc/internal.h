@@ -159,6 +159,15 @@ int launch_lowrank_proj_tc(Ctx* ctx, const void* X, int xdtype, int64_t rows, in
 // The basis in the tensor-core projection's operand form: [basis_tc_rows(r), d_in] 16-bit (xdtype),
 // rows [0, RT) / [RT, 2RT) / [2RT, 3RT) the three 16-bit terms of U^T (RT = r rounded up to 4, 8, 16, 32).
 int basis_tc_rows(int r);
+int proj_rank_tile(int r);       // RT
+int proj_operand_rows(int r);    // operand rows per group of RT ranks
+// A projection left as partials [group][split][rows][RT], every group of ranks in one launch.
+struct ProjPlan {
+  int rt, groups, splits, kbps, num_kb;
+};
+ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits);
+int launch_proj_parts(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d_in, const void* Ut, const ProjPlan& p,
+                      float* part);
 int launch_basis_prepare(Ctx* ctx, const float* U, int d_in, int r, int xdtype, void* Ut);
 int launch_lowrank_proj_tc_prepared(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d_in, const void* Ut,
                                     int r, float* P);

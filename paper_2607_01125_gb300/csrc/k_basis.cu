@@ -2,9 +2,10 @@
 // calibration activations X, i.e. the top-r eigenvectors of G = X^T X).
 //
 // Device pipeline (no host round trip, every step a kernel):
-//   1. G = X^T X in fp32: for 16-bit X, X is transposed into a zero-padded
-//      [d, n_pad] copy and multiplied with itself on the tcgen05 GEMM;
-//      for fp32 X a CUDA-core kernel forms X^T X directly.
+//   1. For 16-bit X, X is transposed into a zero-padded [d, n_pad] copy, and every
+//      product G Q is X^T (X Q) on the tensor cores, in three 16-bit terms of the
+//      fp32 factor.  Only with many more tokens than columns, and for fp32 X, is
+//      G = X^T X formed (fp32; tcgen05 GEMM, or CUDA cores for fp32 X).
 //   2. Omega [d, k] from the Z generator (seed, layer 0, query 0), k = r + oversample.
 //   3. Q = orth(Omega); n_iter times Q = orth(G Q).  orth() is CholeskyQR2:
 //      S = Y^T Y (64 x 64 output tiles; fp32 over 32-row slabs, fp64 across
@@ -24,16 +25,24 @@ namespace {
 constexpr int KMAX = 64;        // k handled by the shared-memory Cholesky and Jacobi; column tile of the rest
 constexpr int KLIM = 512;       // largest k
 
-// ---- X [n, d] (16-bit) -> Xt [d, n_pad], zero in columns n .. n_pad-1 ----
+// ---- X [n, d] (16-bit) -> Xt [d, n_pad], zero in columns n .. n_pad-1; *absmax (zero before) = max |X| ----
 template <typename T>
-__global__ void transpose_pad_kernel(const T* __restrict__ X, T* __restrict__ Xt, int64_t n, int d, int64_t n_pad) {
+__global__ void transpose_pad_kernel(const T* __restrict__ X, T* __restrict__ Xt, int64_t n, int d, int64_t n_pad,
+                                     int* __restrict__ absmax) {
   __shared__ T tile[32][33];
   const int64_t t0 = (int64_t)blockIdx.x * 32;
   const int i0 = blockIdx.y * 32;
+  int top = 0;
   for (int y = threadIdx.y; y < 32; y += 8) {
     const int64_t t = t0 + y;
     const int i = i0 + threadIdx.x;
-    tile[y][threadIdx.x] = (t < n && i < d) ? X[t * d + i] : from_f32<T>(0.f);
+    const T x = (t < n && i < d) ? X[t * d + i] : from_f32<T>(0.f);
+    tile[y][threadIdx.x] = x;
+    top = max(top, __float_as_int(fabsf(to_f32<T>(x))));    // non-negative floats order as integers
+  }
+  if (absmax) {
+    top = __reduce_max_sync(0xffffffffu, top);
+    if (threadIdx.x == 0) atomicMax(absmax, top);
   }
   __syncthreads();
   for (int y = threadIdx.y; y < 32; y += 8) {
@@ -469,13 +478,100 @@ __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
   }
 }
 
+// ---- products with X on the tensor cores ----
+// With 16-bit X and no more than GRAM_TOKENS d tokens the Gram matrix is never formed: G Q = X^T (X Q), two products of
+// the projection kernel (k_proj_tc.cu: X exact in 16 bits, the fp32 factor split into three 16-bit terms), the second
+// on the transposed copy of X.  A step then reads X twice instead of the d x d matrix (14336 wide, 512 tokens: 29 MB
+// against 822 MB) and does 4 n d k operations instead of 2 d^2 k.
+// The factors' operand form: rows [g NB + term RT + j] of a [groups NB, ld] 16-bit matrix, rank g RT + j, rows of the
+// factor as columns.  fp16 cannot hold the small parts of small entries, so its factors are scaled by powers of two:
+// Q, whose entries are at most 1, by 2^13, and P = X Q, bounded by max|X| sqrt(d), to at most 2^14.
+struct Operand {
+  void* op;
+  int64_t ld;
+  int rt, nb;
+};
+constexpr int GRAM_TOKENS = 8;
+constexpr float Q_SCALE_FP16 = 8192.f;
+
+template <typename T16> __device__ __forceinline__ float q_scale() { return 1.f; }
+template <> __device__ __forceinline__ float q_scale<__half>() { return Q_SCALE_FP16; }
+// The power of two that brings max|X| sqrt(d) to [2^13, 2^14).
+template <typename T16> __device__ __forceinline__ float p_scale(const int*, int) { return 1.f; }
+template <> __device__ __forceinline__ float p_scale<__half>(const int* absmax, int d) {
+  const float bound = __int_as_float(*absmax) * sqrtf((float)d);
+  if (!(bound > 0.f) || !isfinite(bound)) return 1.f;
+  return ldexpf(1.f, 13 - ilogbf(bound));
+}
+
+// Eight consecutive rows' values of one rank, scaled, as three 16-bit terms (each the rounding of what is left).
+template <typename T16>
+__device__ __forceinline__ void write_operand(const Operand& o, int rank, int64_t col, const float* v, float scale) {
+  const int g = rank / o.rt, j = rank - g * o.rt;
+  T16* row = static_cast<T16*>(o.op) + ((int64_t)g * o.nb + j) * o.ld + col;
+  float rest[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) rest[i] = v[i] * scale;
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    union { uint4 w; T16 e[8]; } u;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      u.e[i] = from_f32<T16>(rest[i]);
+      rest[i] -= to_f32<T16>(u.e[i]);
+    }
+    *reinterpret_cast<uint4*>(row + (int64_t)t * o.rt * o.ld) = u.w;
+  }
+}
+
+// The K-splits' partials [group][split][rows][rt] of a product, added in split order, to out [rows, k] (or null) and,
+// TO_OP, to the operand form of the next product (zero in its padding columns).  The scales of the product's own
+// operand (Q's: mode 0, P's: mode 1) are taken out.
+constexpr int RED_ROWS = 16;
+template <typename T16, bool TO_OP>
+__global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restrict__ part, int64_t rows, int k, int splits,
+                                                           int rt, float* __restrict__ out, Operand op, int mode,
+                                                           const int* __restrict__ absmax, int d) {
+  __shared__ float tile[64][RED_ROWS + 1];
+  const int g = blockIdx.y;
+  const int64_t r0 = (int64_t)blockIdx.x * RED_ROWS;
+  const float* src = part + (int64_t)g * splits * rows * rt;
+  const float ps = p_scale<T16>(absmax, d);
+  const float un = 1.f / (mode == 0 ? q_scale<T16>() : ps);
+  for (int v = threadIdx.x; v < RED_ROWS * rt; v += 256) {
+    const int rr = v / rt, j = v - rr * rt;
+    const int64_t row = r0 + rr;
+    float s = 0.f;
+    if (row < rows) {
+      const float* p = src + row * rt + j;
+#pragma unroll 8
+      for (int sp = 0; sp < splits; ++sp) s += __ldg(p + (int64_t)sp * rows * rt);
+      s *= un;
+      if (out && g * rt + j < k) out[row * k + g * rt + j] = s;
+    }
+    if (TO_OP) tile[j][rr] = s;
+  }
+  if (!TO_OP) return;
+  __syncthreads();
+  for (int v = threadIdx.x; v < rt * (RED_ROWS / 8); v += 256) {
+    const int j = v / (RED_ROWS / 8), e = (v % (RED_ROWS / 8)) * 8;
+    if (g * rt + j < k && r0 + e < op.ld) {
+      float x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) x[i] = tile[j][e + i];
+      write_operand<T16>(op, g * rt + j, r0 + e, x, ps);
+    }
+  }
+}
+
 // ---- out [rows, c] = A [rows, k] (fp32) M [k, ldm] (fp64, first c columns): 64 x 64 tiles ----
 // Every product is exact (an fp32 entry times a two-float split of M's, 48 bits) and added with its rounding error
 // carried along (two-sum), so a sum holds ~46 bits: eleven fp32 instructions a term, against one fp64 FMA at a
-// sixty-fourth of their rate.  tri: M is upper triangular.  5120 x 48 x 48: 73 us in fp64, 26 here; 4096 x 272 x 272: 836 and 181.
+// sixty-fourth of their rate.  tri: M is upper triangular.  With a 16-bit T16 the result's operand form is written too.  5120 x 48 x 48: 73 us in fp64, 26 here; 4096 x 272 x 272: 836 and 181.
+template <typename T16>
 __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A, const double* __restrict__ M,
                                                     float* __restrict__ out, int64_t rows, int k, int ldm, int c,
-                                                    int tri) {
+                                                    int tri, Operand op) {
   __shared__ float As[32][KMAX + 4];                 // [p][row]
   __shared__ float Mh[32][KMAX], Ml[32][KMAX];       // [p][column]
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
@@ -520,12 +616,35 @@ __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A,
       }
     }
   }
-  if (!live) return;
+#pragma unroll
   for (int i = 0; i < 4; ++i) {
     const int64_t row = r0 + ty * 4 + i;
-    if (row >= rows) continue;
-    for (int j = 0; j < 4; ++j)
-      if (c0 + tx * 4 + j < c) out[row * c + c0 + tx * 4 + j] = s[i][j] + lo[i][j];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      s[i][j] += lo[i][j];
+      if (row < rows && c0 + tx * 4 + j < c) out[row * c + c0 + tx * 4 + j] = s[i][j];
+    }
+  }
+  if constexpr (sizeof(T16) == 2) {
+    // the tile by columns, 32 of its rows at a time (As is free again)
+    float (*tile)[KMAX + 4] = As;                    // [row of the half][column]
+    for (int h = 0; h < 2; ++h) {
+      __syncthreads();
+      if (ty / 8 == h)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) tile[(ty % 8) * 4 + i][tx * 4 + j] = s[i][j];
+      __syncthreads();
+      const int cc = threadIdx.x % 64, e = threadIdx.x / 64 * 8;
+      const int64_t row = r0 + 32 * h + e;
+      if (c0 + cc < c && row < rows) {               // rows is a multiple of 8 here
+        float x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = tile[e + i][cc];
+        write_operand<T16>(op, c0 + cc, row, x, q_scale<T16>());
+      }
+    }
   }
 }
 
@@ -842,7 +961,11 @@ struct Work {
   double* shift;  // diagonal shift of the last Cholesky
   int* ints;      // small Jacobi: rounds taken, column order
   GridSync* sync; // barrier of the cooperative launches
+  int* absmax;    // max |X| (bits)
+  float* P;       // X Q [n_tok, k] (no Gram matrix)
+  Operand qop, pop;   // operand forms of Q and of P
 };
+constexpr int PROJ_MAX_SPLITS = 32;
 
 // Row chunks of an A^T B over `rows` rows: two blocks per SM over all tiles, 32-row slabs.
 int atb_chunks(const Ctx* ctx, int64_t rows, int k, int& chunk) {
@@ -884,26 +1007,51 @@ int launch_chol(Ctx* ctx, const Work& w, int k) {
   return ZOACT_OK;
 }
 
-int launch_apply(Ctx* ctx, const float* A, const double* M, float* out, int64_t rows, int k, int ldm, int c, int tri) {
-  apply_kernel<<<dim3((unsigned)((rows + 63) / 64), (unsigned)((c + 63) / 64)), 256, 0, ctx->stream>>>(A, M, out, rows, k,
-                                                                                                  ldm, c, tri);
+// op (with its 16-bit type): write the result's operand form too.
+int launch_apply(Ctx* ctx, const float* A, const double* M, float* out, int64_t rows, int k, int ldm, int c, int tri,
+                 const Operand* op = nullptr, int dtype = ZOACT_DT_FP32) {
+  const dim3 grid((unsigned)((rows + 63) / 64), (unsigned)((c + 63) / 64));
+  auto kern = !op ? apply_kernel<float> : dtype == ZOACT_DT_BF16 ? apply_kernel<__nv_bfloat16> : apply_kernel<__half>;
+  kern<<<grid, 256, 0, ctx->stream>>>(A, M, out, rows, k, ldm, c, tri, op ? *op : Operand{});
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
 }
 
-// CholeskyQR2 of Y [d, k], which holds Q afterwards; tmp: another [d, k].
-int orth(Ctx* ctx, const Work& w, float* Y, float* tmp, int d, int k) {
+// CholeskyQR2 of Y [d, k], which holds Q afterwards; tmp: another [d, k]; op: Q's operand form too.
+int orth(Ctx* ctx, const Work& w, float* Y, float* tmp, int d, int k, const Operand* op, int dtype) {
   float* src = Y;
   float* dst = tmp;
   for (int pass = 0; pass < 2; ++pass) {
     int st = launch_atb(ctx, w, src, src, d, k);
     if (!st) st = launch_chol(ctx, w, k);
-    if (!st) st = launch_apply(ctx, src, w.Rinv, dst, d, k, k, k, 1);
+    if (!st) st = launch_apply(ctx, src, w.Rinv, dst, d, k, k, k, 1, pass ? op : nullptr, dtype);
     if (st) return st;
     src = tmp;
     dst = Y;
   }
+  return ZOACT_OK;
+}
+
+// dst [rows, k] (or null) = X F for 16-bit X [rows, kd] and F's operand form; to_op: dst's operand form too.
+int launch_product(Ctx* ctx, const Work& w, const void* X, int dtype, int64_t rows, int64_t kd, const Operand& f, int mode,
+                   int k, float* dst, const Operand* to_op, int d) {
+  const ProjPlan plan = proj_plan(ctx, rows, (int)kd, k, PROJ_MAX_SPLITS);
+  float* part = static_cast<float*>(
+      scratch(ctx, SLOT_SPLITK, (size_t)plan.groups * plan.splits * rows * plan.rt * sizeof(float)));
+  if (!part) return ZOACT_ERR_NOMEM;
+  const int st = launch_proj_parts(ctx, X, dtype, rows, (int)kd, f.op, plan, part);
+  if (st) return st;
+  // the operand's padding columns are written (as zeros) too
+  const int64_t cover = to_op ? to_op->ld : rows;
+  const dim3 grid((unsigned)((cover + RED_ROWS - 1) / RED_ROWS), (unsigned)plan.groups);
+  const bool bf = dtype == ZOACT_DT_BF16;
+  auto kern = to_op ? (bf ? reduce_parts_kernel<__nv_bfloat16, true> : reduce_parts_kernel<__half, true>)
+                    : (bf ? reduce_parts_kernel<__nv_bfloat16, false> : reduce_parts_kernel<__half, false>);
+  kern<<<grid, 256, 0, ctx->stream>>>(part, rows, k, plan.splits, plan.rt, dst, to_op ? *to_op : Operand{}, mode, w.absmax,
+                                      d);
+  ++ctx->n_launch;
+  ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
 }
 
@@ -916,19 +1064,32 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   if (k > KLIM || r > k) return ZOACT_ERR_UNSUPPORTED;
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, JACOBI_SMEM));
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CHOL_SMEM));
+  const int64_t n_pad = (n_tok + 7) / 8 * 8;
+  // no Gram matrix (see reduce_parts_kernel): 16-bit X, unless there are so many more tokens than columns that reading
+  // X twice a step costs more than the d x d matrix and its one-off product
+  const bool direct = xdtype != ZOACT_DT_FP32 && n_tok <= (int64_t)GRAM_TOKENS * d;
   int chunk;
-  const size_t nchunk = (size_t)atb_chunks(ctx, d, k, chunk);
+  size_t nchunk = (size_t)atb_chunks(ctx, d, k, chunk);
+  if (direct) {
+    const size_t np = (size_t)atb_chunks(ctx, n_tok, k, chunk);
+    if (np > nchunk) nchunk = np;
+  }
+  const size_t g_bytes = direct ? (size_t)n_tok * k * 4 : (size_t)d * d * 4;
+  const size_t q_op = direct ? (size_t)basis_tc_rows(k) * d * 2 : 0, p_op = direct ? (size_t)basis_tc_rows(k) * n_pad * 2 : 0;
   const size_t kk = (size_t)k * k * 8, dk = (size_t)d * k * 4, big = k > KMAX ? kk : 0;
   const size_t log_bytes = k <= KMAX ? (size_t)JAC_SWEEPS * KMAX * (KMAX / 2) * sizeof(double2) : 0;
   // workspace (every piece padded to 256 bytes)
-  const size_t bytes = (size_t)d * d * 4 + 2 * dk + nchunk * kk + 3 * kk + 3 * big + log_bytes + 2 * (size_t)k * 8 +
-                       sizeof(GridSync) + 16 * 256 + 4096;
+  const size_t bytes = g_bytes + q_op + p_op + 2 * dk + nchunk * kk + 3 * kk + 3 * big + log_bytes + 2 * (size_t)k * 8 +
+                       sizeof(GridSync) + 20 * 256 + 4096;
   uint8_t* base = static_cast<uint8_t*>(scratch(ctx, SLOT_BASIS, bytes));
   if (!base) return ZOACT_ERR_NOMEM;
   Work w;
   size_t off = 0;
   auto take = [&](size_t b) { uint8_t* p = base + off; off += (b + 255) / 256 * 256; return p; };
-  w.G = reinterpret_cast<float*>(take((size_t)d * d * 4));
+  w.G = w.P = reinterpret_cast<float*>(take(g_bytes));
+  uint8_t* ops = take(q_op + p_op);                  // (q_op is a multiple of 16 bytes: d is one of 8)
+  w.qop = Operand{ops, d, proj_rank_tile(k), proj_operand_rows(k)};
+  w.pop = Operand{ops + q_op, n_pad, w.qop.rt, w.qop.nb};
   w.Q = reinterpret_cast<float*>(take(dk));
   w.Y = reinterpret_cast<float*>(take(dk));
   w.part = reinterpret_cast<double*>(take(nchunk * kk));
@@ -944,48 +1105,68 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   w.shift = reinterpret_cast<double*>(take(8));
   w.ints = reinterpret_cast<int*>(take((KMAX + 1) * sizeof(int)));
   w.sync = reinterpret_cast<GridSync*>(take(sizeof(GridSync)));
+  w.absmax = reinterpret_cast<int*>(take(sizeof(int)));
   if (off > bytes) return ZOACT_ERR_NOMEM;
 
-  // 1. Gram
+  // 1. X^T and, where it is used, the Gram matrix
+  void* Xt = nullptr;
   if (xdtype == ZOACT_DT_FP32) {
     dim3 grid((d + 63) / 64, (d + 63) / 64);
     gram_f32_kernel<<<grid, 256, 0, ctx->stream>>>(static_cast<const float*>(X), w.G, n_tok, d); ++ctx->n_launch;
     ZOACT_CHECK_LAUNCH();
   } else {
-    const int64_t n_pad = (n_tok + 7) / 8 * 8;
-    void* Xt = scratch(ctx, SLOT_BASIS_X, (size_t)d * n_pad * 2);
+    Xt = scratch(ctx, SLOT_BASIS_X, (size_t)d * n_pad * 2);
     if (!Xt) return ZOACT_ERR_NOMEM;
+    if (direct) {
+      ZOACT_CUDA_TRY(cudaMemsetAsync(w.absmax, 0, sizeof(int), ctx->stream));
+      ZOACT_CUDA_TRY(cudaMemsetAsync(ops, 0, q_op + p_op, ctx->stream));   // ranks past k stay zero
+    }
     dim3 grid((unsigned)((n_pad + 31) / 32), (unsigned)((d + 31) / 32));
+    int* top = xdtype == ZOACT_DT_FP16 && direct ? w.absmax : nullptr;
     if (xdtype == ZOACT_DT_BF16) {
       transpose_pad_kernel<__nv_bfloat16><<<grid, dim3(32, 8), 0, ctx->stream>>>(
-          static_cast<const __nv_bfloat16*>(X), static_cast<__nv_bfloat16*>(Xt), n_tok, d, n_pad);
+          static_cast<const __nv_bfloat16*>(X), static_cast<__nv_bfloat16*>(Xt), n_tok, d, n_pad, top);
     } else {
       transpose_pad_kernel<__half><<<grid, dim3(32, 8), 0, ctx->stream>>>(static_cast<const __half*>(X),
-                                                                          static_cast<__half*>(Xt), n_tok, d, n_pad);
+                                                                          static_cast<__half*>(Xt), n_tok, d, n_pad, top);
     }
     ++ctx->n_launch;
     ZOACT_CHECK_LAUNCH();
-    const int st = launch_gemm_tc_f32out(ctx, Xt, Xt, xdtype, d, d, (int)n_pad, w.G);
-    if (st) return st;
+    if (!direct) {
+      const int st = launch_gemm_tc_f32out(ctx, Xt, Xt, xdtype, d, d, (int)n_pad, w.G);
+      if (st) return st;
+    }
   }
   // 2-3. sketch and subspace iteration: Q stays in w.Q
   const int64_t nq = (int64_t)d * k;
   omega_kernel<<<(unsigned)((nq / 4 + 255) / 256 + 1), 256, 0, ctx->stream>>>(w.Q, nq, seed); ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
-  int st = orth(ctx, w, w.Q, w.Y, d, k);
+  const Operand* qop = direct ? &w.qop : nullptr;
+  int st = orth(ctx, w, w.Q, w.Y, d, k, qop, xdtype);
   if (st) return st;
   const dim3 gq_blocks((unsigned)((d + 63) / 64), (unsigned)((k + KMAX - 1) / KMAX));
   for (int it = 0; it < n_iter; ++it) {
-    gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
-    ZOACT_CHECK_LAUNCH();
-    st = orth(ctx, w, w.Y, w.Q, d, k);
+    if (direct) {
+      st = launch_product(ctx, w, X, xdtype, n_tok, d, w.qop, 0, k, nullptr, &w.pop, d);
+      if (!st) st = launch_product(ctx, w, Xt, xdtype, d, n_pad, w.pop, 1, k, w.Y, nullptr, d);
+      if (st) return st;
+    } else {
+      gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
+      ZOACT_CHECK_LAUNCH();
+    }
+    st = orth(ctx, w, w.Y, w.Q, d, k, qop, xdtype);
     if (st) return st;
     float* t = w.Q; w.Q = w.Y; w.Y = t;
   }
-  // 4. Rayleigh-Ritz
-  gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
-  ZOACT_CHECK_LAUNCH();
-  st = launch_atb(ctx, w, w.Q, w.Y, d, k);
+  // 4. Rayleigh-Ritz: S = Q^T G Q, of P = X Q as P^T P
+  if (direct) {
+    st = launch_product(ctx, w, X, xdtype, n_tok, d, w.qop, 0, k, w.P, nullptr, d);
+    if (!st) st = launch_atb(ctx, w, w.P, w.P, n_tok, k);
+  } else {
+    gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
+    ZOACT_CHECK_LAUNCH();
+    st = launch_atb(ctx, w, w.Q, w.Y, d, k);
+  }
   if (st) return st;
   if (k <= KMAX) {
     jacobi_kernel<<<1, JAC_THREADS, JACOBI_SMEM, ctx->stream>>>(w.S, w.log, w.ints, w.ev, w.ints + 1, k);

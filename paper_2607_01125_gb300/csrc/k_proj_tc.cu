@@ -10,7 +10,8 @@
 // single tcgen05.mma 128 x NB x 16 per K-step produces all three partial
 // products into TMEM; the epilogue adds them.
 //
-// Grid: (row blocks of 128, K-splits).  Per CTA: warp 0 streams X tiles
+// Grid: (row blocks of 128, K-splits, groups of ranks whose outputs lie group_stride
+// floats apart).  Per CTA: warp 0 streams X tiles
 // (128 x 64) and Ut tiles (NB x 64) through a 4-stage TMA ring (two CTAs per
 // SM; the grid is one wave of them), warp 1 issues
 // the MMAs, then all four warps read the accumulator (one row per thread) and
@@ -65,7 +66,7 @@ __global__ void split_u_kernel(const float* __restrict__ U, T16* __restrict__ Ut
 template <int NB, int RT, int AB_BF16>
 __global__ void __launch_bounds__(128, 1)
 proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmU, float* __restrict__ out,
-               int64_t rows, int r, int ld_out, int kb_per_split, int num_kb, int* status) {
+               int64_t rows, int r, int ld_out, int kb_per_split, int num_kb, int64_t group_stride, int* status) {
   constexpr int STAGE = p_stage_bytes<NB>();
   constexpr uint32_t TCOLS = NB <= 32 ? 32 : (NB <= 64 ? 64 : (NB <= 128 ? 128 : 256));
   extern __shared__ uint8_t smem_raw[];
@@ -110,7 +111,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
       tc::mbar_arrive_expect_tx(full, STAGE);
       const uint32_t sa = tc::smem_u32(smem + stage * STAGE);
       tc::tma_load_2d(sa, &tmX, kb * PBK, m0, full);
-      tc::tma_load_2d(sa + P_A_BYTES, &tmU, kb * PBK, 0, full);
+      tc::tma_load_2d(sa + P_A_BYTES, &tmU, kb * PBK, (int)blockIdx.z * NB, full);
       issued_mask |= 1u << stage;
       issued_parity = (issued_parity & ~(1u << stage)) | (phase << stage);
       if (++stage == PSTAGES) { stage = 0; phase ^= 1u; }
@@ -154,7 +155,7 @@ proj_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ 
   const bool ok = *reinterpret_cast<volatile int*>(&ss->ok) != 0 && kb1 > kb0;
   const int64_t m = m0 + threadIdx.x;
   // r valid ranks of this launch; split partials are [splits][rows][r], direct output rows have stride ld_out
-  float* dst = out + (int64_t)blockIdx.y * rows * ld_out + m * ld_out;
+  float* dst = out + blockIdx.z * group_stride + (int64_t)blockIdx.y * rows * ld_out + m * ld_out;
   const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
   if constexpr (RT <= 8) {
     float acc[NB];
@@ -214,11 +215,11 @@ __global__ void splitk_sum_kernel(const float* __restrict__ part, float* __restr
 
 template <int NB, int RT, int AB>
 int launch_one(Ctx* ctx, const CUtensorMap& mx, const CUtensorMap& mu, float* out, int64_t rows, int r, int ld_out,
-               int kbps, int num_kb, dim3 grid) {
+               int kbps, int num_kb, int64_t group_stride, dim3 grid) {
   auto kern = proj_tc_kernel<NB, RT, AB>;
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, p_smem_bytes<NB>()));
   ZOACT_CUDA_TRY(launch_pdl(ctx, kern, grid, dim3(128), p_smem_bytes<NB>(), mx, mu, out, rows, r, ld_out, kbps,
-                            num_kb, ctx->d_status));
+                            num_kb, group_stride, ctx->d_status));
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
@@ -226,13 +227,13 @@ int launch_one(Ctx* ctx, const CUtensorMap& mx, const CUtensorMap& mu, float* ou
 
 template <int AB>
 int dispatch(Ctx* ctx, int rt, const CUtensorMap& mx, const CUtensorMap& mu, float* out, int64_t rows, int r,
-             int ld_out, int kbps, int num_kb, dim3 grid) {
+             int ld_out, int kbps, int num_kb, int64_t group_stride, dim3 grid) {
   switch (rt) {
-    case 4: return launch_one<16, 4, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, grid);
-    case 8: return launch_one<32, 8, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, grid);
-    case 16: return launch_one<48, 16, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, grid);
-    case 32: return launch_one<96, 32, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, grid);
-    default: return launch_one<192, 64, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, grid);
+    case 4: return launch_one<16, 4, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, group_stride, grid);
+    case 8: return launch_one<32, 8, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, group_stride, grid);
+    case 16: return launch_one<48, 16, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, group_stride, grid);
+    case 32: return launch_one<96, 32, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, group_stride, grid);
+    default: return launch_one<192, 64, AB>(ctx, mx, mu, out, rows, r, ld_out, kbps, num_kb, group_stride, grid);
   }
 }
 
@@ -245,6 +246,38 @@ int proj_nb(int rt) { return rt == 4 ? 16 : rt == 8 ? 32 : rt == 16 ? 48 : rt ==
 int basis_tc_rows(int r) {
   const int rt = proj_rt(r);
   return proj_nb(rt) * ((r + rt - 1) / rt);
+}
+
+int proj_rank_tile(int r) { return proj_rt(r); }
+int proj_operand_rows(int r) { return proj_nb(proj_rt(r)); }
+
+ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits) {
+  ProjPlan p;
+  p.rt = proj_rt(r);
+  p.groups = (r + p.rt - 1) / p.rt;
+  p.num_kb = (d_in + PBK - 1) / PBK;
+  // one wave of two CTAs per SM over all groups, at least 2 K-blocks per split
+  const int64_t blocks = (rows + PBM - 1) / PBM * p.groups;
+  int64_t splits = 2LL * ctx->sm_count / blocks;
+  if (splits > p.num_kb / 2) splits = p.num_kb / 2;
+  if (splits > max_splits) splits = max_splits;
+  if (splits < 1) splits = 1;
+  p.kbps = (int)((p.num_kb + splits - 1) / splits);
+  p.splits = (p.num_kb + p.kbps - 1) / p.kbps;
+  return p;
+}
+
+int launch_proj_parts(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d_in, const void* Ut, const ProjPlan& p,
+                      float* part) {
+  const int nb = proj_nb(p.rt);
+  CUtensorMap mx, mu;
+  int st = encode_tmap_2d_16bit(&mx, X, xdtype, rows, d_in, PBM);
+  if (!st) st = encode_tmap_2d_16bit(&mu, Ut, xdtype, (int64_t)p.groups * nb, d_in, nb);
+  if (st) return st;
+  const int64_t stride = (int64_t)p.splits * rows * p.rt;
+  const dim3 grid((unsigned)((rows + PBM - 1) / PBM), (unsigned)p.splits, (unsigned)p.groups);
+  return xdtype == ZOACT_DT_BF16 ? dispatch<1>(ctx, p.rt, mx, mu, part, rows, p.rt, p.rt, p.kbps, p.num_kb, stride, grid)
+                                 : dispatch<0>(ctx, p.rt, mx, mu, part, rows, p.rt, p.rt, p.kbps, p.num_kb, stride, grid);
 }
 
 int launch_basis_prepare(Ctx* ctx, const float* U, int d_in, int r, int xdtype, void* Ut) {
@@ -307,8 +340,8 @@ int launch_lowrank_proj_tc_prepared(Ctx* ctx, const void* X, int xdtype, int64_t
       ld_out = rg;
     }
     const dim3 grid((unsigned)row_blocks, (unsigned)splits);
-    st = xdtype == ZOACT_DT_BF16 ? dispatch<1>(ctx, rt, mx, mu, out, rows, rg, ld_out, kbps, num_kb, grid)
-                                 : dispatch<0>(ctx, rt, mx, mu, out, rows, rg, ld_out, kbps, num_kb, grid);
+    st = xdtype == ZOACT_DT_BF16 ? dispatch<1>(ctx, rt, mx, mu, out, rows, rg, ld_out, kbps, num_kb, 0, grid)
+                                 : dispatch<0>(ctx, rt, mx, mu, out, rows, rg, ld_out, kbps, num_kb, 0, grid);
     if (st) return st;
     if (splits > 1) {
       const int64_t n = rows * rg;
