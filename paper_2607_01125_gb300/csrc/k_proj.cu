@@ -136,6 +136,64 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ part, float* __re
   }
 }
 
+// Short rows (fp32 X of at most PROJ_ROW_MAX columns, the 256-wide toy graph): a warp owns R rows and eight basis
+// columns; its lanes take every 32nd k, with all of a row's loads in flight, and a butterfly adds them.  The blocks above
+// walk such a row in 32-wide chunks, a round trip to L2 each: 64 x 256, r = 8 took 41 us on one 64-thread block (ncu),
+// 7.3 here (cold caches; a launch alone is ~3).
+constexpr int PROJ_ROW_MAX = 1024;
+template <int R>
+__global__ void __launch_bounds__(128)
+proj_rows_kernel(const float* __restrict__ X, const float* __restrict__ U, float* __restrict__ P, int64_t rows, int d_in,
+                 int r, int vec) {
+  pdl_wait();                              // X written by the previous kernel
+  pdl_trigger();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t m0 = ((int64_t)blockIdx.x * 4 + warp) * R;
+  const int j0 = blockIdx.y * 8;
+  float acc[R][8] = {};
+#pragma unroll 4
+  for (int k = lane; k < d_in; k += 32) {
+    float u[8], x[R];
+    const float* src = U + (int64_t)k * r + j0;
+    if (vec) {                             // r a multiple of 8, U 16-byte aligned
+      const float4 a = *reinterpret_cast<const float4*>(src), b = *reinterpret_cast<const float4*>(src + 4);
+      u[0] = a.x; u[1] = a.y; u[2] = a.z; u[3] = a.w; u[4] = b.x; u[5] = b.y; u[6] = b.z; u[7] = b.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 8; ++j) u[j] = j0 + j < r ? src[j] : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < R; ++i) x[i] = m0 + i < rows ? X[(m0 + i) * d_in + k] : 0.f;
+#pragma unroll
+    for (int i = 0; i < R; ++i)
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(x[i], u[j], acc[i][j]);
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[i][j] += __shfl_xor_sync(0xffffffffu, acc[i][j], o);
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+      if (lane == j && m0 + i < rows && j0 + j < r) P[(m0 + i) * r + j0 + j] = acc[i][j];
+}
+
+int launch_proj_rows(Ctx* ctx, const float* X, int64_t rows, int d_in, const float* U, int r, float* P) {
+  // one row a warp until the rows alone give every SM 16 warps
+  const int R = rows >= 16LL * ctx->sm_count ? 4 : 1;
+  const dim3 grid((unsigned)((rows + 4 * R - 1) / (4 * R)), (unsigned)((r + 7) / 8));
+  const int vec = r % 8 == 0 && ((uintptr_t)U & 15u) == 0;
+  ZOACT_CUDA_TRY(launch_pdl(ctx, R == 4 ? proj_rows_kernel<4> : proj_rows_kernel<1>, grid, dim3(128), 0, X, U, P, rows,
+                            d_in, r, vec));
+  ++ctx->n_launch;
+  ZOACT_CHECK_LAUNCH();
+  return ZOACT_OK;
+}
+
 template <typename TX>
 int proj_dispatch(Ctx* ctx, const TX* X, int64_t rows, int d_in, const float* U, int r, float* P) {
   const int64_t row_blocks = (rows + PROJ_RB - 1) / PROJ_RB;
@@ -186,7 +244,9 @@ int launch_lowrank_proj(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d
                         float* P) {
   if (rows <= 0) return ZOACT_OK;
   switch (xdtype) {
-    case ZOACT_DT_FP32: return proj_dispatch(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
+    case ZOACT_DT_FP32:
+      if (d_in <= PROJ_ROW_MAX) return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
+      return proj_dispatch(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
     case ZOACT_DT_BF16:
     case ZOACT_DT_FP16: return launch_lowrank_proj_tc(ctx, X, xdtype, rows, d_in, U, r, P);
     default: return ZOACT_ERR_INVALID_ARG;
@@ -239,6 +299,7 @@ int launch_lowrank_proj_into(Ctx* ctx, const void* X, int xdtype, int64_t rows, 
   if (rows <= 0) return ZOACT_OK;
   switch (xdtype) {
     case ZOACT_DT_FP32:
+      if (d_in <= PROJ_ROW_MAX) return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
       return proj_dispatch_into(ctx, static_cast<const float*>(X), rows, d_in, U, r, P, part, part_floats);
     case ZOACT_DT_BF16:
       return proj_dispatch_into(ctx, static_cast<const __nv_bfloat16*>(X), rows, d_in, U, r, P, part, part_floats);
