@@ -62,14 +62,51 @@ __device__ __forceinline__ uint2 split_quad(float4 v, bool want_lo) {
   return make_uint2(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]));
 }
 
-// One thread per 16-byte chunk (8 K columns) of an output row: rows [0, nA)
-// of A_aug, then the nB rows of B_aug (block b, column n), then those of
-// B_aug2.  Each column k of a row maps to (slot, half, part, rank j); the chunk
-// is built from the source values it needs (P or P2 for A rows, T = C + c_b Z_b
-// for B rows; source rows are re-read from L1/L2 by the row's chunks).  With
-// QUAD (r a multiple of 4 and 16-byte aligned sources) every 4 columns are one
-// part of one slot: one float4 load and one Philox call per 4 columns.
-template <bool QUAD>
+// Transposed Z tables: Zt[q][j][n] for each distinct query (gate, then up); one thread per (matrix, query, group of 4
+// ranks, column n), columns fastest so that the stores coalesce.
+__device__ __forceinline__ void write_z_tables(const AugBlocks& blk, int d_out, int r, uint64_t seed, uint32_t lid,
+                                               uint32_t lid2, float* __restrict__ Zt, float* __restrict__ Zt2) {
+  if (Zt && blk.nzq > 0) {
+    const int groups = (r + 3) / 4;
+    const int n_mat = Zt2 ? 2 : 1;
+    const int64_t items = (int64_t)n_mat * blk.nzq * groups * d_out;
+    for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
+         it += (int64_t)gridDim.x * blockDim.x) {
+      const int n = (int)(it % d_out);
+      int64_t rest = it / d_out;
+      const int jg = (int)(rest % groups);
+      rest /= groups;
+      const int qi = (int)(rest % blk.nzq);
+      const int mat = (int)(rest / blk.nzq);
+      float* dst = (mat ? Zt2 : Zt) + (int64_t)qi * r * d_out;
+      const uint32_t layer = mat ? lid2 : lid;
+      if ((r & 3) == 0) {
+        // the four ranks are one Philox group
+        const float4 z = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(((int64_t)n * r + 4 * jg) >> 2));
+        dst[(int64_t)(4 * jg) * d_out + n] = z.x;
+        dst[(int64_t)(4 * jg + 1) * d_out + n] = z.y;
+        dst[(int64_t)(4 * jg + 2) * d_out + n] = z.z;
+        dst[(int64_t)(4 * jg + 3) * d_out + n] = z.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int j = 4 * jg + i;
+          if (j < r) {
+            const int64_t e = (int64_t)n * r + j;
+            dst[(int64_t)j * d_out + n] =
+                z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2)), (int)(e & 3));
+          }
+        }
+      }
+    }
+  }
+}
+
+// Any rank (the quad kernel below serves ranks that are multiples of 4 with 16-byte aligned sources): one thread per
+// 16-byte chunk (8 K columns) of an output row: rows [0, nA) of A_aug, then the nB rows of B_aug (block b, column n),
+// then those of B_aug2.  Each column k of a row maps to (slot, half, part, rank j); the chunk is built from the source
+// values it needs (P or P2 for A rows, T = C + c_b Z_b for B rows; source rows are re-read from L1/L2 by the row's
+// chunks).
 __global__ void __launch_bounds__(256)
 aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const float* __restrict__ C,
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
@@ -122,34 +159,7 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
     uint32_t w[4];
 #pragma unroll
     for (int h4 = 0; h4 < 2; ++h4) {
-      if (QUAD) {
-        const int k0 = 8 * c + 4 * h4;
-        const int slot = k0 / ka_row;
-        const int kk = k0 - slot * ka_row;
-        const int half = kk >= ka ? 1 : 0, kq = kk - half * ka;
-        const int part = kq / r, j0 = kq - part * r;
-        // A: [hi | hi | lo], B: [hi | lo | hi]; distinct gated A: [gate parts | up parts];
-        // distinct gated B: gate rows fill the first half, up rows the second
-        const bool live = part < 3 && slot == my_slot && (is_a || !distinct || half == (up ? 1 : 0));
-        uint2 o = make_uint2(0u, 0u);
-        if (live) {
-          float4 v;
-          if (is_a) {
-            v = *reinterpret_cast<const float4*>((distinct && half ? P2 : P) + orow * r + j0);
-          } else {
-            const int64_t e = (int64_t)n * r + j0;
-            v = *reinterpret_cast<const float4*>(Cs + e);
-            if (cb != 0.f) {
-              const float4 z = z_normals4(seed, layer, q, (uint64_t)(e >> 2));
-              v.x = fmaf(cb, z.x, v.x); v.y = fmaf(cb, z.y, v.y);
-              v.z = fmaf(cb, z.z, v.z); v.w = fmaf(cb, z.w, v.w);
-            }
-          }
-          o = split_quad(v, is_a ? part == 2 : part == 1);
-        }
-        w[2 * h4] = o.x;
-        w[2 * h4 + 1] = o.y;
-      } else {
+      {
         __nv_bfloat16 e4[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
@@ -181,42 +191,91 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
     const int64_t row_w = 8 * (int64_t)(is_a ? cA : cB);
     *reinterpret_cast<uint4*>(dst + orow * row_w + 8 * c) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  // transposed Z tables: Zt[q][j][n] for each distinct query (gate, then up); one thread per
-  // (matrix, query, group of 4 ranks, column n), columns fastest so that the stores coalesce
-  if (Zt && blk.nzq > 0) {
-    const int groups = (r + 3) / 4;
-    const int n_mat = Zt2 ? 2 : 1;
-    const int64_t items = (int64_t)n_mat * blk.nzq * groups * d_out;
-    for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-         it += (int64_t)gridDim.x * blockDim.x) {
-      const int n = (int)(it % d_out);
-      int64_t rest = it / d_out;
-      const int jg = (int)(rest % groups);
-      rest /= groups;
-      const int qi = (int)(rest % blk.nzq);
-      const int mat = (int)(rest / blk.nzq);
-      float* dst = (mat ? Zt2 : Zt) + (int64_t)qi * r * d_out;
-      const uint32_t layer = mat ? lid2 : lid;
-      if ((r & 3) == 0) {
-        // the four ranks are one Philox group
-        const float4 z = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(((int64_t)n * r + 4 * jg) >> 2));
-        dst[(int64_t)(4 * jg) * d_out + n] = z.x;
-        dst[(int64_t)(4 * jg + 1) * d_out + n] = z.y;
-        dst[(int64_t)(4 * jg + 2) * d_out + n] = z.z;
-        dst[(int64_t)(4 * jg + 3) * d_out + n] = z.w;
-      } else {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int j = 4 * jg + i;
-          if (j < r) {
-            const int64_t e = (int64_t)n * r + j;
-            dst[(int64_t)j * d_out + n] =
-                z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2)), (int)(e & 3));
-          }
+  write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+}
+
+// The same tables for ranks that are multiples of 4 with aligned sources: one thread per four ranks of a row, which
+// forms their values once -- a Philox call serves the three parts and, where two evaluation blocks share a query (the
+// two signs), both of them -- and writes 8 bytes to each part and its share of the row's zeros.  A chunk per thread drew
+// every Z three times: 20480 x 32, two signs, 666 rows 20.3 us there, 6.0 here; gated 14336 x 16, two signs, 8192
+// rows 15.6 and 5.6.  I: 32-bit item indexes where they fit.
+template <typename I>
+__global__ void __launch_bounds__(256)
+aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const float* __restrict__ C,
+                const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
+                __nv_bfloat16* __restrict__ B2, int64_t rows, int d_out, int r, int ka, int distinct, int full,
+                int nb, const __grid_constant__ AugBlocks blk, uint64_t seed, uint32_t lid, uint32_t lid2,
+                float* __restrict__ Zt, float* __restrict__ Zt2, int slots, int64_t T) {
+  pdl_wait();                                         // P and C written by the previous kernels
+  pdl_trigger();
+  const int rq = r / 4, kq = ka / 4, halves = distinct ? 2 : 1;
+  const int row_q = halves * kq;                      // quads of one slot (= B_aug row)
+  const int nbB = full ? nb : 1, pairs = (nbB + 1) / 2;
+  const I itA = (I)rows * (I)(halves * rq);
+  const I itB = (I)pairs * (I)d_out * (I)rq;
+  const I items = itA + itB * (B2 ? 2 : 1);
+  const uint2 zero = make_uint2(0u, 0u);
+  // one half of one slot: this quad's three parts (live), and its share of the zeros
+  auto put = [&](uint2* half_q, int g, float4 v, bool is_a, bool live) {
+    if (live) {
+      const uint2 hi = split_quad(v, false), lo = split_quad(v, true);
+      half_q[g] = hi;
+      half_q[rq + g] = is_a ? hi : lo;
+      half_q[2 * rq + g] = is_a ? lo : hi;
+    }
+    for (int z = (live ? 3 * rq : 0) + g; z < kq; z += rq) half_q[z] = zero;
+  };
+  const I stride = (I)gridDim.x * blockDim.x;
+  for (I it = (I)blockIdx.x * blockDim.x + threadIdx.x; it < items; it += stride) {
+    if (it < itA) {
+      const I rh = it / (I)rq;
+      const int g = (int)(it - rh * (I)rq);
+      const int h = distinct ? (int)(rh & 1) : 0;
+      const int64_t row = distinct ? (int64_t)(rh >> 1) : (int64_t)rh;
+      const float4 v = *reinterpret_cast<const float4*>((h ? P2 : P) + row * r + 4 * g);
+      const int mine = slots > 1 ? (int)((row / T) % slots) : 0;
+      uint2* q = reinterpret_cast<uint2*>(A) + row * ((int64_t)slots * row_q) + h * kq;
+      for (int s = 0; s < slots; ++s) put(q + s * row_q, g, v, true, s == mine);
+    } else {
+      I ib = it - itA;
+      const bool up = ib >= itB;
+      if (up) ib -= itB;
+      const I bn = ib / (I)rq;
+      const int g = (int)(ib - bn * (I)rq);
+      const int bp = (int)(bn / (I)d_out);
+      const int n_all = (int)(bn - (I)bp * (I)d_out);
+      int n = n_all;
+      uint32_t layer = up ? lid2 : lid;
+      const float* Cs = up ? C2 : C;                  // the coefficients row n indexes (a grouped layer's own)
+      if (blk.nseg > 1) {
+        int sg = 0;
+        while (sg + 1 < blk.nseg && n >= blk.seg_off[sg + 1]) ++sg;
+        n -= blk.seg_off[sg];
+        Cs = blk.seg_C[sg];
+        layer = blk.seg_lid[sg];
+      }
+      const int64_t e = (int64_t)n * r + 4 * g;
+      const float4 c = *reinterpret_cast<const float4*>(Cs + e);
+      float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      uint64_t drawn = 0;
+      bool have = false;
+      for (int b = 2 * bp; b < min(2 * bp + 2, nbB); ++b) {
+        float4 v = c;
+        const float cb = full ? blk.coef[b] : 0.f;
+        if (cb != 0.f) {
+          if (!have || blk.qry[b] != drawn) z = z_normals4(seed, layer, blk.qry[b], (uint64_t)(e >> 2));
+          have = true;
+          drawn = blk.qry[b];
+          v.x = fmaf(cb, z.x, v.x); v.y = fmaf(cb, z.y, v.y);
+          v.z = fmaf(cb, z.z, v.z); v.w = fmaf(cb, z.w, v.w);
         }
+        uint2* q = reinterpret_cast<uint2*>(up ? B2 : B) + ((int64_t)b * d_out + n_all) * row_q;
+        // distinct: gate rows fill the first half, up rows the second
+        for (int h = 0; h < halves; ++h) put(q + h * kq, g, v, false, !distinct || h == (up ? 1 : 0));
       }
     }
   }
+  write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -252,7 +311,17 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   bool quad = a.r % 4 == 0 && aligned16_or_null(a.P) && aligned16_or_null(distinct ? a.P2 : nullptr) &&
               aligned16_or_null(a.C) && aligned16_or_null(a.C2);
   for (int g = 0; g < blk.nseg; ++g) quad = quad && aligned16_or_null(a.seg_C[g]);
-  auto kern = quad ? aug_prep_kernel<true> : aug_prep_kernel<false>;
+  auto kern = aug_prep_kernel;
+  if (quad) {
+    const int64_t q_items = a.rows * ((distinct ? 2 : 1) * (a.r / 4)) +
+                            (B_aug2 ? 2 : 1) * ((nbB + 1) / 2) * a.d_out * (int64_t)(a.r / 4);
+    const int64_t q_work = q_items > z_items ? q_items : z_items;
+    grid = (q_work + 255) / 256;
+    if (grid > cap) grid = cap;
+    if (grid < 1) grid = 1;
+    // (a grid-stride step past the last item must fit too)
+    kern = q_items + grid * 256 < ((int64_t)1 << 31) ? aug_quad_kernel<uint32_t> : aug_quad_kernel<int64_t>;
+  }
   ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)grid), dim3(256), 0, a.P, distinct ? a.P2 : nullptr, a.C,
                             a.C2, static_cast<__nv_bfloat16*>(A_aug), static_cast<__nv_bfloat16*>(B_aug),
                             static_cast<__nv_bfloat16*>(B_aug2), a.rows, a.d_out, a.r, ka, distinct, full, a.nb, blk,
