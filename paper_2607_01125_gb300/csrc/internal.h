@@ -165,7 +165,7 @@ int proj_operand_rows(int r);    // operand rows per group of RT ranks
 struct ProjPlan {
   int rt, groups, splits, kbps, num_kb;
 };
-ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits);
+ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits, int most_kb);
 int launch_proj_parts(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d_in, const void* Ut, const ProjPlan& p,
                       float* part);
 int launch_basis_prepare(Ctx* ctx, const float* U, int d_in, int r, int xdtype, void* Ut);

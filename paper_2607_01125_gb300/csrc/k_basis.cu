@@ -25,30 +25,44 @@ namespace {
 constexpr int KMAX = 64;        // k handled by the shared-memory Cholesky and Jacobi; column tile of the rest
 constexpr int KLIM = 512;       // largest k
 
-// ---- X [n, d] (16-bit) -> Xt [d, n_pad], zero in columns n .. n_pad-1; *absmax (zero before) = max |X| ----
+// ---- X [n, d] (16-bit, d a multiple of 8, 16-byte aligned) -> Xt [d, n_pad], zero in columns n .. n_pad-1 ----
+// 64 x 64 tiles, 16-byte loads and stores.  absmax (or null; zero before): max |X|, one atomic per block that raises it.
+// 4096 x 5120 fp16: 111 us as 32 x 32 tiles of single elements with an atomic per warp (45 without), 22 here.
 template <typename T>
-__global__ void transpose_pad_kernel(const T* __restrict__ X, T* __restrict__ Xt, int64_t n, int d, int64_t n_pad,
-                                     int* __restrict__ absmax) {
-  __shared__ T tile[32][33];
-  const int64_t t0 = (int64_t)blockIdx.x * 32;
-  const int i0 = blockIdx.y * 32;
+__global__ void __launch_bounds__(256) transpose_pad_kernel(const T* __restrict__ X, T* __restrict__ Xt, int64_t n, int d,
+                                                            int64_t n_pad, int* __restrict__ absmax) {
+  __shared__ T tile[64][66];                         // [token][column]
+  __shared__ int top_s;
+  const int64_t t0 = (int64_t)blockIdx.x * 64;
+  const int i0 = blockIdx.y * 64;
+  if (threadIdx.x == 0) top_s = 0;
+  __syncthreads();
   int top = 0;
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int64_t t = t0 + y;
-    const int i = i0 + threadIdx.x;
-    const T x = (t < n && i < d) ? X[t * d + i] : from_f32<T>(0.f);
-    tile[y][threadIdx.x] = x;
-    top = max(top, __float_as_int(fabsf(to_f32<T>(x))));    // non-negative floats order as integers
+  for (int v = threadIdx.x; v < 64 * 8; v += 256) {
+    const int y = v >> 3, c = (v & 7) * 8;
+    union { uint4 w; T e[8]; } u;
+    u.w = make_uint4(0u, 0u, 0u, 0u);
+    if (t0 + y < n && i0 + c < d) u.w = *reinterpret_cast<const uint4*>(X + (t0 + y) * d + i0 + c);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      tile[y][c + e] = u.e[e];
+      top = max(top, __float_as_int(fabsf(to_f32<T>(u.e[e]))));    // non-negative floats order as integers
+    }
   }
   if (absmax) {
     top = __reduce_max_sync(0xffffffffu, top);
-    if (threadIdx.x == 0) atomicMax(absmax, top);
+    if ((threadIdx.x & 31) == 0) atomicMax(&top_s, top);
   }
   __syncthreads();
-  for (int y = threadIdx.y; y < 32; y += 8) {
-    const int i = i0 + y;
-    const int64_t t = t0 + threadIdx.x;
-    if (i < d && t < n_pad) Xt[(int64_t)i * n_pad + t] = tile[threadIdx.x][y];
+  if (absmax && threadIdx.x == 0 && top_s > *reinterpret_cast<volatile int*>(absmax)) atomicMax(absmax, top_s);
+  for (int v = threadIdx.x; v < 64 * 8; v += 256) {
+    const int i = v & 63, y = (v >> 6) * 8;
+    if (i0 + i < d && t0 + y < n_pad) {              // (n_pad is a multiple of 8)
+      union { uint4 w; T e[8]; } u;
+#pragma unroll
+      for (int e = 0; e < 8; ++e) u.e[e] = tile[y + e][i];
+      *reinterpret_cast<uint4*>(Xt + (int64_t)(i0 + i) * n_pad + t0 + y) = u.w;
+    }
   }
 }
 
@@ -89,6 +103,8 @@ __global__ void __launch_bounds__(256) gram_f32_kernel(const float* __restrict__
 
 // ---- Omega [d, k]: element i*k + j of the (seed, 0, 0) stream ----
 __global__ void omega_kernel(float* __restrict__ Om, int64_t n, uint64_t seed) {
+  pdl_wait();
+  pdl_trigger();
   for (int64_t g = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; 4 * g < n; g += (int64_t)gridDim.x * blockDim.x) {
     const float4 z = z_normals4(seed, 0u, 0ull, (uint64_t)g);
 #pragma unroll
@@ -141,14 +157,19 @@ __global__ void __launch_bounds__(256) gemm_gq_kernel(const float* __restrict__ 
 }
 
 // ---- partial S = A^T B over a chunk of rows, A, B [rows, k]: 64 x 64 output tiles per block (grid x, y), row chunks on
-// grid z; fp32 products over 32-row slabs, added into fp64 per slab.  sym (A = B): tiles below the diagonal are left out.
-// The fp64 adds (2 lanes a cycle and SM) weigh as much as a slab's FMAs, and a slab is a round trip to L2, so the rows
-// are cut into as many chunks as give every SM two tiles: 7 blocks of 64 slabs took 296 us for 14336 x 32, 14 here (and 8 for the sum of the chunks).
+// grid z; fp32 products over 32-row slabs, added into fp64 per slab -- where there are several tiles (TILES), and the fp64
+// adds of their many slabs would weigh twice their FMAs, into two floats that carry the rounding errors along (~46 bits;
+// k = 272: 67 us a call with fp64 adds, 47 so; one tile, bound by latency: 9.4 with fp64, 11.8).  sym (A = B): tiles below the diagonal are left out.  A slab is a round
+// trip to L2, so the rows are cut into as many chunks as give every SM two tiles: 7 blocks of 64 slabs took 296 us for
+// 14336 x 32, 13 here (and 7 for the sum of the chunks).
+template <bool TILES>
 __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restrict__ A, const float* __restrict__ B,
                                                           double* __restrict__ part, int64_t rows, int k, int chunk,
                                                           int sym) {
   __shared__ float As[32][KMAX + 4];
   __shared__ float Bs[32][KMAX + 4];
+  pdl_wait();
+  pdl_trigger();
   const int p0 = blockIdx.y * KMAX, q0 = blockIdx.x * KMAX;
   if (sym && q0 < p0) return;
   const bool one = sym && q0 == p0;                  // one tile serves both sides
@@ -156,7 +177,8 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
   const int64_t r_begin = (int64_t)blockIdx.z * chunk;
   const int64_t r_end = r_begin + chunk < rows ? r_begin + chunk : rows;
   const bool live = p0 + ty * 4 < k && q0 + tx * 4 < k;
-  double acc[4][4] = {};
+  float acc[4][4] = {}, low[4][4] = {};
+  double acc64[4][4] = {};
   for (int64_t s0 = r_begin; s0 < r_end; s0 += 32) {
     __syncthreads();
     for (int v = threadIdx.x; v < 32 * KMAX; v += 256) {
@@ -182,7 +204,15 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += (double)a32[i][j];
+        for (int j = 0; j < 4; ++j) {
+          if (!TILES) {
+            acc64[i][j] += (double)a32[i][j];
+            continue;
+          }
+          const float x = a32[i][j], t = __fadd_rn(acc[i][j], x), y = __fsub_rn(t, acc[i][j]);
+          low[i][j] = __fadd_rn(low[i][j], __fadd_rn(__fsub_rn(acc[i][j], __fsub_rn(t, y)), __fsub_rn(x, y)));
+          acc[i][j] = t;
+        }
     }
   }
   if (!live) return;
@@ -190,7 +220,7 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
   for (int i = 0; i < 4; ++i)
     for (int j = 0; j < 4; ++j) {
       const int p = p0 + ty * 4 + i, q = q0 + tx * 4 + j;
-      if (p < k && q < k) out[(int64_t)p * k + q] = acc[i][j];
+      if (p < k && q < k) out[(int64_t)p * k + q] = TILES ? (double)acc[i][j] + (double)low[i][j] : acc64[i][j];
     }
 }
 
@@ -198,6 +228,8 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ part, double* __restrict__ S,
                                                            int nchunk, int k, int sym) {
   __shared__ double red[8][32];
+  pdl_wait();
+  pdl_trigger();
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int o = blockIdx.x * 32 + lane, kk = k * k;
   const int i = o / k, j = o - i * k;
@@ -216,39 +248,51 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 }
 
 // ---- LDL^T of an n x n block in shared memory (n <= KMAX), with its inverse factor ----
-// A: the upper triangle in; row j of the eliminated matrix out (its diagonal D).  M: L^-1 out (unit lower triangle).
-// One block-wide barrier a column: while the other warps apply column j, warp 0 finishes row j + 1 and forms its
-// multipliers.  Returns false (to every thread) when a pivot is not positive.  f: 2 x KMAX doubles, bad: two ints.
-__device__ bool ldl_shared(double* A, double* M, int ld, int n, double* f, int* bad) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
-  auto prepare = [&](int j) {                        // warp 0: the multipliers of row j, whose elimination is done
-    const double d = A[j * ld + j];
+// N: the upper triangle in, zeros below; out: row j of the eliminated matrix in the upper triangle (its diagonal D) and
+// L^-1 (unit lower triangle) strictly below.  One block-wide barrier a column: while the other warps apply column j to
+// the rows below, warp 0 finishes row j + 1, which it keeps in registers (two columns a lane) for its multipliers and
+// for the step after; that chain -- a load, a multiply-add, the pivot's reciprocal, a product -- is a step's length.
+// Returns false (to every thread) when a pivot is not positive.  f: 2 x KMAX doubles, bad: two ints.
+__device__ bool ldl_shared(double* N, int ld, int n, double* f, int* bad) {
+  const int lane = threadIdx.x & 31;
+  const bool wide = n > 32;
+  double x0 = 0.0, x1 = 0.0, f0 = 0.0, f1 = 0.0;     // warp 0: row j (1 in column j) and its multipliers
+  auto pivot = [&](int p, double a0, double a1) {    // warp 0: row p is eliminated: its multipliers
+    const double d = __shfl_sync(0xffffffffu, p < 32 ? a0 : a1, p & 31);
     const double inv = 1.0 / d;
-    for (int p = j + 1 + lane; p < n; p += 32) f[(j & 1) * KMAX + p] = A[j * ld + p] * inv;
-    if (lane == 0) bad[j & 1] = !(d > 0.0);
+    f0 = a0 * inv;
+    f1 = a1 * inv;
+    double* fp = f + (p & 1) * KMAX;
+    fp[lane] = f0;
+    if (wide) fp[lane + 32] = f1;
+    if (lane == 0) bad[p & 1] = !(d > 0.0);
+    x0 = lane == p ? 1.0 : a0;
+    x1 = lane + 32 == p ? 1.0 : a1;
   };
-  for (int v = threadIdx.x; v < n * n; v += blockDim.x) M[(v / n) * ld + v % n] = v / n == v % n ? 1.0 : 0.0;
+  if (threadIdx.x < 32) pivot(0, lane < n ? N[lane] : 0.0, lane + 32 < n ? N[lane + 32] : 0.0);
   __syncthreads();
-  if (warp == 0) prepare(0);
-  __syncthreads();
+  const int t = (int)threadIdx.x - 32, shift = wide ? 6 : 5;
+  const int c = t & ((1 << shift) - 1), rows = ((int)blockDim.x - 32) >> shift, first = t >> shift;
   for (int j = 0; j < n; ++j) {
     if (bad[j & 1]) return false;
-    const double* fj = f + (j & 1) * KMAX;
-    if (warp == 0) {
-      if (j + 1 < n) {
-        const int p = j + 1;
-        const double m = fj[p];
-        for (int q = p + lane; q < n; q += 32) A[p * ld + q] -= m * A[j * ld + q];
-        for (int c = lane; c <= j; c += 32) M[p * ld + c] -= m * M[j * ld + c];
-        __syncwarp();
-        prepare(p);
+    if (threadIdx.x < 32) {
+      const int p = j + 1;
+      if (p < n) {
+        double* row = N + p * ld;
+        double a0 = lane < n ? row[lane] : 0.0, a1 = lane + 32 < n ? row[lane + 32] : 0.0;
+        const double m = __shfl_sync(0xffffffffu, p < 32 ? f0 : f1, p & 31);
+        a0 = fma(-m, x0, a0);                        // (columns 0 .. j and p .. n: all of them)
+        a1 = fma(-m, x1, a1);
+        if (lane < n) row[lane] = a0;
+        if (lane + 32 < n) row[lane + 32] = a1;
+        pivot(p, a0, a1);
       }
-    } else {
-      for (int p = j + 1 + warp; p < n; p += warps - 1) {
-        const double m = fj[p];
-        for (int q = p + lane; q < n; q += 32) A[p * ld + q] -= m * A[j * ld + q];
-        for (int c = lane; c <= j; c += 32) M[p * ld + c] -= m * M[j * ld + c];
-      }
+    } else if (c < n && first < rows) {
+      const double x = c == j ? 1.0 : N[j * ld + c];
+      const double* fj = f + (j & 1) * KMAX;
+#pragma unroll 4
+      for (int p = j + 2 + first; p < n; p += rows)
+        if (c <= j || c >= p) N[p * ld + c] = fma(-fj[p], x, N[p * ld + c]);
     }
     __syncthreads();
   }
@@ -265,17 +309,17 @@ constexpr int CHOL_ATTEMPTS = 4;
 
 // ---- R^-1 of the Cholesky factor S = R^T R (R upper), k <= KMAX: one block, everything in shared memory ----
 // R^-1 = L^-T D^-1/2.  Bound by a column's chain (a row's update, a division, a barrier) and the fp64 pipe; k = 48:
-// 228 us with the factor in global memory and a serial inverse per column, 46 here.
+// 228 us with the factor in global memory and a serial inverse per column, 44 here.
 constexpr int CHOL_THREADS = 512;
-constexpr int CHOL_SMEM = 2 * KMAX * (KMAX + 1) * 8;
+constexpr int CHOL_SMEM = KMAX * (KMAX + 1) * 8;
 __global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(const double* __restrict__ S, double* __restrict__ Rinv,
                                                                 int k, int* status) {
   extern __shared__ double sm[];
   __shared__ double f[2 * KMAX], rs[KMAX], trace;
   __shared__ int bad[2];
+  pdl_wait();
+  pdl_trigger();
   const int ld = k + 1;
-  double* A = sm;
-  double* M = sm + k * ld;
   bool ok = false;
   for (int attempt = 0; attempt < CHOL_ATTEMPTS && !ok; ++attempt) {
     __syncthreads();
@@ -287,20 +331,20 @@ __global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(const double* __
     const double shift = chol_shift(attempt, attempt ? trace : 0.0);
     for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
       const int i = v / k, j = v % k;
-      A[i * ld + j] = S[v] + (i == j ? shift : 0.0);
+      sm[i * ld + j] = j < i ? 0.0 : S[v] + (i == j ? shift : 0.0);
     }
     __syncthreads();
-    ok = ldl_shared(A, M, ld, k, f, bad);
+    ok = ldl_shared(sm, ld, k, f, bad);
   }
   if (!ok) {
     if (threadIdx.x == 0) record_error(status, ZOACT_ERR_NONFINITE);
     return;
   }
-  for (int i = threadIdx.x; i < k; i += CHOL_THREADS) rs[i] = 1.0 / sqrt(A[i * ld + i]);
+  for (int i = threadIdx.x; i < k; i += CHOL_THREADS) rs[i] = 1.0 / sqrt(sm[i * ld + i]);
   __syncthreads();
   for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
     const int i = v / k, c = v % k;
-    Rinv[v] = i <= c ? M[c * ld + i] * rs[c] : 0.0;
+    Rinv[v] = i > c ? 0.0 : (i == c ? 1.0 : sm[c * ld + i]) * rs[c];
   }
 }
 
@@ -317,22 +361,26 @@ __device__ __forceinline__ bool grid_barrier(GridSync* sy, unsigned int target, 
   __syncthreads();
   if (threadIdx.x == 0) {
     give_up = 0;
-    __threadfence();
-    atomicAdd(&sy->count, 1u);
+    // the block's writes, ordered before this thread by the barrier above, are released with the arrival
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&sy->count) : "memory");
+    unsigned int seen;
     uint64_t t0 = 0;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    while (*reinterpret_cast<volatile unsigned int*>(&sy->count) < target) {
-      if (*reinterpret_cast<volatile int*>(&sy->abort)) { give_up = 1; break; }
-      uint64_t now;
-      asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-      if (now - t0 > 2000000000ull) {
-        atomicExch(&sy->abort, 1);
-        record_error(status, ZOACT_ERR_TIMEOUT);
-        give_up = 1;
-        break;
+    for (unsigned int it = 0;; ++it) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(&sy->count) : "memory");
+      if (seen >= target) break;
+      if ((it & 63u) == 63u) {
+        uint64_t now;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
+        if (t0 == 0) t0 = now;
+        if (*reinterpret_cast<volatile int*>(&sy->abort)) { give_up = 1; break; }
+        if (now - t0 > 2000000000ull) {
+          atomicExch(&sy->abort, 1);
+          record_error(status, ZOACT_ERR_TIMEOUT);
+          give_up = 1;
+          break;
+        }
       }
     }
-    __threadfence();
   }
   __syncthreads();
   return give_up == 0;
@@ -342,7 +390,7 @@ __device__ __forceinline__ bool grid_barrier(GridSync* sy, unsigned int target, 
 // Panels of CB columns.  Every block factors the panel's diagonal block by itself (no barrier), the panel's rows of A
 // and of M = L^-1 are multiplied by its inverse factor in 8-column strips, and after a barrier the rows below get their
 // rank-CB update in 16 x 16 tiles.  Two barriers a panel; the columns' chain (as above) is most of the time.  k = 272:
-// 5.6 ms in one block, 0.34 here.
+// 5.6 ms in one block, 0.27 here.
 constexpr int CB = 32;
 constexpr int CHOLB_THREADS = 256;
 constexpr int CHOLB_BLOCKS = 96;
@@ -358,7 +406,7 @@ struct CholBig {
   int* status;
 };
 __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
-  __shared__ double sA[CB * (CB + 1)], sM[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], trace_s;
+  __shared__ double sN[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], trace_s;
   __shared__ int bad[2];
   __shared__ double sx[CB][17], sf[CB][17], inv_d[CB];
   const int k = w.k, tid = threadIdx.x;
@@ -392,10 +440,10 @@ __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
     for (int p0 = 0; p0 < k; p0 += CB) {
       const int nb = min(CB, k - p0), p1 = p0 + nb;
       for (int v = tid; v < nb * nb; v += CHOLB_THREADS)
-        sA[(v / nb) * (CB + 1) + v % nb] = __ldcg(w.A + (int64_t)(p0 + v / nb) * k + p0 + v % nb);
+        sN[(v / nb) * (CB + 1) + v % nb] = v % nb < v / nb ? 0.0 : __ldcg(w.A + (int64_t)(p0 + v / nb) * k + p0 + v % nb);
       __syncthreads();
-      if (!ldl_shared(sA, sM, CB + 1, nb, f, bad)) { ok = false; break; }     // the same answer in every block
-      if (tid < nb) inv_d[tid] = 1.0 / sA[tid * (CB + 1) + tid];
+      if (!ldl_shared(sN, CB + 1, nb, f, bad)) { ok = false; break; }     // the same answer in every block
+      if (tid < nb) inv_d[tid] = 1.0 / sN[tid * (CB + 1) + tid];
       // strips: columns p1 .. k of A, then 0 .. p0 of M, eight at a time
       const int na = k - p1, cols = na + p0;
       for (int g = blockIdx.x; g * 8 < cols; g += gridDim.x) {
@@ -404,16 +452,18 @@ __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
         if (i < nb && c < cols) sx[i][tid & 7] = __ldcg(base + (int64_t)i * k);
         __syncthreads();
         double x = 0.0;
-        if (i < nb && c < cols)
-          for (int l = 0; l <= i; ++l) x = fma(sM[i * (CB + 1) + l], sx[l][tid & 7], x);
+        if (i < nb && c < cols) {
+          x = sx[i][tid & 7];
+          for (int l = 0; l < i; ++l) x = fma(sN[i * (CB + 1) + l], sx[l][tid & 7], x);
+        }
         if (i < nb && c < cols) __stcg(base + (int64_t)i * k, x);
         __syncthreads();
       }
       if (blockIdx.x == gridDim.x - 1) {             // the diagonal block itself
         for (int v = tid; v < nb * nb; v += CHOLB_THREADS) {
           const int i = v / nb, j = v % nb;
-          if (j <= i) __stcg(w.M + (int64_t)(p0 + i) * k + p0 + j, sM[i * (CB + 1) + j]);
-          if (j >= i) __stcg(w.D + (int64_t)(p0 + i) * k + p0 + j, sA[i * (CB + 1) + j]);
+          if (j <= i) __stcg(w.M + (int64_t)(p0 + i) * k + p0 + j, i == j ? 1.0 : sN[i * (CB + 1) + j]);
+          if (j >= i) __stcg(w.D + (int64_t)(p0 + i) * k + p0 + j, sN[i * (CB + 1) + j]);
         }
       }
       if (!sync()) return;
@@ -443,7 +493,7 @@ __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
           double x = 0.0;
           if (c0 + e < c_end)
             x = in_a ? __ldcg(w.A + row + c0 + e) : c0 + e < p0 ? __ldcg(w.M + row + c0 + e)
-                                                                : (c0 + e - p0 <= l ? sM[l * (CB + 1) + c0 + e - p0] : 0.0);
+                : c0 + e - p0 < l ? sN[l * (CB + 1) + c0 + e - p0] : c0 + e - p0 == l ? 1.0 : 0.0;
           sx[l][e] = x;
         }
         __syncthreads();
@@ -527,12 +577,14 @@ __device__ __forceinline__ void write_operand(const Operand& o, int rank, int64_
 // The K-splits' partials [group][split][rows][rt] of a product, added in split order, to out [rows, k] (or null) and,
 // TO_OP, to the operand form of the next product (zero in its padding columns).  The scales of the product's own
 // operand (Q's: mode 0, P's: mode 1) are taken out.
-constexpr int RED_ROWS = 16;
+constexpr int RED_ROWS = 8;
 template <typename T16, bool TO_OP>
 __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restrict__ part, int64_t rows, int k, int splits,
                                                            int rt, float* __restrict__ out, Operand op, int mode,
                                                            const int* __restrict__ absmax, int d) {
   __shared__ float tile[64][RED_ROWS + 1];
+  pdl_wait();
+  pdl_trigger();
   const int g = blockIdx.y;
   const int64_t r0 = (int64_t)blockIdx.x * RED_ROWS;
   const float* src = part + (int64_t)g * splits * rows * rt;
@@ -542,12 +594,12 @@ __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restri
     const int rr = v / rt, j = v - rr * rt;
     const int64_t row = r0 + rr;
     float s = 0.f;
-    if (row < rows) {
+    if (row < rows && g * rt + j < k) {
       const float* p = src + row * rt + j;
 #pragma unroll 8
       for (int sp = 0; sp < splits; ++sp) s += __ldg(p + (int64_t)sp * rows * rt);
       s *= un;
-      if (out && g * rt + j < k) out[row * k + g * rt + j] = s;
+      if (out) out[row * k + g * rt + j] = s;
     }
     if (TO_OP) tile[j][rr] = s;
   }
@@ -564,30 +616,38 @@ __global__ void __launch_bounds__(256) reduce_parts_kernel(const float* __restri
   }
 }
 
-// ---- out [rows, c] = A [rows, k] (fp32) M [k, ldm] (fp64, first c columns): 64 x 64 tiles ----
+// ---- out [rows, c] = A [rows, k] (fp32) M [k, ldm] (fp64, first c columns) ----
 // Every product is exact (an fp32 entry times a two-float split of M's, 48 bits) and added with its rounding error
 // carried along (two-sum), so a sum holds ~46 bits: eleven fp32 instructions a term, against one fp64 FMA at a
-// sixty-fourth of their rate.  tri: M is upper triangular.  With a 16-bit T16 the result's operand form is written too.  5120 x 48 x 48: 73 us in fp64, 26 here; 4096 x 272 x 272: 836 and 181.
-template <typename T16>
+// sixty-fourth of their rate.  tri: M is upper triangular.  With a 16-bit T16 the result's operand form is written too.
+// 5120 x 48 x 48: 73 us in fp64, 28 here; 4096 x 272 x 272: 836 and 121.
+// CT columns by 4096 / CT rows a block (32 columns where k <= 32 or the triangle leaves more out); the widest columns,
+// whose sums are longest, come first.
+template <typename T16, int CT>
 __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A, const double* __restrict__ M,
                                                     float* __restrict__ out, int64_t rows, int k, int ldm, int c,
                                                     int tri, Operand op) {
-  __shared__ float As[32][KMAX + 4];                 // [p][row]
-  __shared__ float Mh[32][KMAX], Ml[32][KMAX];       // [p][column]
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  const int64_t r0 = (int64_t)blockIdx.x * 64;
-  const int c0 = blockIdx.y * 64;
+  constexpr int RT = 4096 / CT, TX = CT / 4;         // rows of the tile; threads along its columns
+  constexpr int AP = RT + 4, HB = 2048 / CT, TP = CT + 4;
+  __shared__ __align__(16) float As[32 * AP];        // [p][row]; the epilogue's [row of half a tile][column]
+  __shared__ __align__(16) float Mh[32][CT], Ml[32][CT];   // [p][column]
+  static_assert(HB * TP <= 32 * AP, "the epilogue's tile exceeds the operand's room");
+  pdl_wait();
+  pdl_trigger();
+  const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
+  const int64_t r0 = (int64_t)blockIdx.x * RT;
+  const int c0 = (int)(gridDim.y - 1 - blockIdx.y) * CT;
   const bool live = c0 + tx * 4 < c;
   float s[4][4] = {}, lo[4][4] = {};
-  const int p_end = tri ? min(k, c0 + 64) : k;
+  const int p_end = tri ? min(k, c0 + CT) : k;
   for (int p0 = 0; p0 < p_end; p0 += 32) {
     __syncthreads();
-    for (int v = threadIdx.x; v < 64 * 32; v += 256) {
+    for (int v = threadIdx.x; v < RT * 32; v += 256) {
       const int rr = v / 32, p = v % 32;
-      As[p][rr] = r0 + rr < rows && p0 + p < k ? A[(r0 + rr) * k + p0 + p] : 0.f;
+      As[p * AP + rr] = r0 + rr < rows && p0 + p < k ? A[(r0 + rr) * k + p0 + p] : 0.f;
     }
-    for (int v = threadIdx.x; v < 32 * 64; v += 256) {
-      const int p = v / 64, cc = v % 64;
+    for (int v = threadIdx.x; v < 32 * CT; v += 256) {
+      const int p = v / CT, cc = v % CT;
       const double m = p0 + p < k && c0 + cc < c ? M[(int64_t)(p0 + p) * ldm + c0 + cc] : 0.0;
       const float h = (float)m;
       Mh[p][cc] = h;
@@ -597,7 +657,7 @@ __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A,
     if (live) {
 #pragma unroll 4
       for (int p = 0; p < 32; ++p) {
-        const float4 a4 = *reinterpret_cast<const float4*>(&As[p][ty * 4]);
+        const float4 a4 = *reinterpret_cast<const float4*>(&As[p * AP + ty * 4]);
         const float4 h4 = *reinterpret_cast<const float4*>(&Mh[p][tx * 4]);
         const float4 l4 = *reinterpret_cast<const float4*>(&Ml[p][tx * 4]);
         const float av[4] = {a4.x, a4.y, a4.z, a4.w}, hv[4] = {h4.x, h4.y, h4.z, h4.w}, lv[4] = {l4.x, l4.y, l4.z, l4.w};
@@ -626,22 +686,21 @@ __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A,
     }
   }
   if constexpr (sizeof(T16) == 2) {
-    // the tile by columns, 32 of its rows at a time (As is free again)
-    float (*tile)[KMAX + 4] = As;                    // [row of the half][column]
+    // the tile by columns, half of its rows at a time
     for (int h = 0; h < 2; ++h) {
       __syncthreads();
-      if (ty / 8 == h)
+      if (ty * 4 / HB == h)
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) tile[(ty % 8) * 4 + i][tx * 4 + j] = s[i][j];
+          for (int j = 0; j < 4; ++j) As[(ty * 4 % HB + i) * TP + tx * 4 + j] = s[i][j];
       __syncthreads();
-      const int cc = threadIdx.x % 64, e = threadIdx.x / 64 * 8;
-      const int64_t row = r0 + 32 * h + e;
+      const int cc = threadIdx.x % CT, e = threadIdx.x / CT * 8;
+      const int64_t row = r0 + HB * h + e;
       if (c0 + cc < c && row < rows) {               // rows is a multiple of 8 here
         float x[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = tile[e + i][cc];
+        for (int i = 0; i < 8; ++i) x[i] = As[(e + i) * TP + cc];
         write_operand<T16>(op, c0 + cc, row, x, q_scale<T16>());
       }
     }
@@ -654,7 +713,7 @@ __global__ void __launch_bounds__(256) apply_kernel(const float* __restrict__ A,
 // shared memory, half of them (i <= j).  Bound by the fp64 pipe (2 lanes a cycle and SM), so the eigenvectors are left
 // out: the angles are logged and jacobi_vectors_kernel applies them to every row of V on its own SM.  The matrix is
 // padded to n with a zero row, whose rotations are trivial.  Stops when off(A)^2 <= 1e-30 |A|_F^2.
-// k = 48: 17.2 ms as rotations taken one by one with the vectors beside them; 0.92 ms here (its vectors 0.07).
+// k = 48: 17.2 ms as rotations taken one by one with the vectors beside them; 0.60 ms here (its vectors 0.07).
 constexpr int JAC_THREADS = 512;
 constexpr int JAC_SWEEPS = 60;
 constexpr int JACOBI_SMEM = KMAX * (KMAX + 1) * 8;
@@ -664,24 +723,39 @@ __device__ __forceinline__ int rr_member(int slot, int round, int n) {
   if (m >= n - 1) m -= n - 1;
   return slot == 0 ? 0 : 1 + m;
 }
-// The rotation that zeroes apq: t = s / c is the smaller root, so |angle| <= pi / 4.
-__device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double& c, double& s, double& t) {
-  c = 1.0; s = 0.0; t = 0.0;
-  if (fabs(apq) > 1e-300) {
-    const double theta = (aqq - app) / (2.0 * apq);
-    if (fabs(theta) > 1e150) t = 0.5 / theta;
-    else t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-    c = 1.0 / sqrt(1.0 + t * t);
-    s = t * c;
-  }
+// The float nearest below |x| 2^(1023 - e), signed: an fp64 value's leading 23 bits, by integer instructions alone.
+__device__ __forceinline__ float scaled_float(double x, int e) {
+  const int hi = __double2hiint(x), ex = ((hi >> 20) & 0x7ff) - e + 127;
+  const uint32_t mant = (((uint32_t)hi & 0xfffffu) << 3) | ((uint32_t)__double2loint(x) >> 29);
+  return ex <= 0 ? 0.f : __uint_as_float(((uint32_t)hi & 0x80000000u) | ((uint32_t)ex << 23) | mant);
+}
+// A rotation (c, s) that zeroes apq to about 2^-20 of itself: its tangent (the smaller root, so |angle| <= pi / 4) is
+// formed in fp32, c and s are orthonormal to fp64 for that tangent (rsqrtf and a third-order step).  In fp64 throughout
+// the divisions and roots were most of a round: a dependent fp64 instruction takes ~70 cycles.  d = aqq - app.
+__device__ __forceinline__ void jacobi_angle(double d, double apq, double& c, double& s) {
+  c = 1.0; s = 0.0;
+  const int ed = (__double2hiint(d) >> 20) & 0x7ff, eg = ((__double2hiint(apq) >> 20) & 0x7ff) + 1;
+  const int e = max(ed, eg);
+  if (eg < 3 || e > 2044) return;                    // (a matrix at the ends of fp64's range is left as it is)
+  const float fg = 2.f * scaled_float(apq, e);
+  if (fg == 0.f) return;                             // below 2^-126 of d
+  const float theta = __fdividef(scaled_float(d, e), fg);
+  const float t = copysignf(__fdividef(1.f, fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f))), theta);
+  if (!(fabsf(t) > 0.f)) return;
+  const double td = (double)t, x = fma(td, td, 1.0), y = (double)rsqrtf((float)x);
+  const double rr = fma(-x, y * y, 1.0);             // |rr| < 2^-21: y (1 + rr / 2 + 3 rr^2 / 8) is off by 2^-64
+  c = fma(y, rr * fma(0.375, rr, 0.5), y);
+  s = td * c;
 }
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __restrict__ S, double2* __restrict__ log,
                                                              int* __restrict__ n_rounds, double* __restrict__ evals,
                                                              int* __restrict__ order, int k) {
   extern __shared__ double A[];                      // [n][n + 1]
-  __shared__ double cs_c[KMAX / 2], cs_s[KMAX / 2], cs_t[KMAX / 2];
+  __shared__ double cs_c[KMAX / 2], cs_s[KMAX / 2];
   __shared__ int pp[KMAX / 2], qq[KMAX / 2];
   __shared__ double red[2][JAC_THREADS / 32];
+  pdl_wait();
+  pdl_trigger();
   const int n = (k + 1) / 2 * 2, np = n / 2, ld = n + 1;
   const int tid = threadIdx.x;
   for (int v = tid; v < n * n; v += JAC_THREADS) {
@@ -709,13 +783,16 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __res
     off = tot = 0.0;
     for (int w = 0; w < JAC_THREADS / 32; ++w) { off += red[0][w]; tot += red[1][w]; }
     if (!(off > 1e-30 * tot)) break;                 // (also for a matrix that is not finite)
+    // elements that could all stay and still meet that bound are not rotated
+    const double skip = 1e-30 * tot / ((double)n * (double)n);
     for (int round = 0; round < n - 1; ++round, ++rounds) {
       if (tid < 32 && tid < np) {
         int p = rr_member(tid, round, n), q = rr_member(n - 1 - tid, round, n);
         if (p > q) { const int x = p; p = q; q = x; }
-        double c, s, t;
-        jacobi_angle(A[p * ld + p], A[q * ld + q], A[p * ld + q], c, s, t);
-        pp[tid] = p; qq[tid] = q; cs_c[tid] = c; cs_s[tid] = s; cs_t[tid] = t;
+        double c = 1.0, s = 0.0;
+        const double apq = A[p * ld + q];
+        if (apq * apq > skip) jacobi_angle(A[q * ld + q] - A[p * ld + p], apq, c, s);
+        pp[tid] = p; qq[tid] = q; cs_c[tid] = c; cs_s[tid] = s;
         log[(int64_t)rounds * np + tid] = make_double2(c, s);
       }
       __syncthreads();
@@ -727,23 +804,15 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __res
         if (h * (h + 1) / 2 > r) --h;
         const int i = np - 1 - h, j = np - 1 - (r - h * (h + 1) / 2);
         const int pi = pp[i], qi = qq[i], pj = pp[j], qj = qq[j];
-        if (i == j) {
-          const double d = cs_t[i] * A[pi * ld + qi];
-          if (d != 0.0) {
-            A[pi * ld + pi] -= d;
-            A[qi * ld + qi] += d;
-            A[pi * ld + qi] = A[qi * ld + pi] = 0.0;
-          }
-          continue;
-        }
         const double ci = cs_c[i], si = cs_s[i], cj = cs_c[j], sj = cs_s[j];
+        if (si == 0.0 && sj == 0.0) continue;
         const double a = A[pi * ld + pj], bq = A[pi * ld + qj], cq = A[qi * ld + pj], dq = A[qi * ld + qj];
         const double a1 = cj * a - sj * bq, b1 = sj * a + cj * bq, c1 = cj * cq - sj * dq, d1 = sj * cq + cj * dq;
         const double a2 = ci * a1 - si * c1, c2 = si * a1 + ci * c1, b2 = ci * b1 - si * d1, d2 = si * b1 + ci * d1;
         A[pi * ld + pj] = A[pj * ld + pi] = a2;
-        A[pi * ld + qj] = A[qj * ld + pi] = b2;
-        A[qi * ld + pj] = A[pj * ld + qi] = c2;
         A[qi * ld + qj] = A[qj * ld + qi] = d2;
+        A[pi * ld + qj] = A[qj * ld + pi] = b2;
+        if (i != j) A[qi * ld + pj] = A[pj * ld + qi] = c2;      // (i = j: the same element)
       }
       __syncthreads();
     }
@@ -768,6 +837,8 @@ __global__ void __launch_bounds__(32) jacobi_vectors_kernel(const double2* __res
                                                             int k) {
   __shared__ double v[KMAX];
   constexpr int AHEAD = 8;                           // rounds whose angles are loaded together
+  pdl_wait();
+  pdl_trigger();
   const int n = (k + 1) / 2 * 2, np = n / 2, lane = threadIdx.x;
   const int rounds = *n_rounds;
   for (int j = lane; j < n; j += 32) v[j] = j == (int)blockIdx.x ? 1.0 : 0.0;
@@ -783,9 +854,11 @@ __global__ void __launch_bounds__(32) jacobi_vectors_kernel(const double2* __res
       if (r0 + a < rounds && lane < np) {
         int p = rr_member(lane, round, n), q = rr_member(n - 1 - lane, round, n);
         if (p > q) { const int x = p; p = q; q = x; }
-        const double vp = v[p], vq = v[q];
-        v[p] = cs[a].x * vp - cs[a].y * vq;
-        v[q] = cs[a].y * vp + cs[a].x * vq;
+        if (cs[a].y != 0.0) {
+          const double vp = v[p], vq = v[q];
+          v[p] = cs[a].x * vp - cs[a].y * vq;
+          v[q] = cs[a].y * vp + cs[a].x * vq;
+        }
       }
       __syncwarp();
       if (++round == n - 1) round = 0;
@@ -800,53 +873,69 @@ __global__ void __launch_bounds__(32) jacobi_vectors_kernel(const double2* __res
 // barrier per round): the fp64 work of a sweep, 3.5 k^3, is spread over k / 2 SMs, and what is left is the latency of
 // a round.  W [k][k]: column c of R^T is row c of R, contiguous.  Stops after a sweep without a rotation above
 // |x.y| <= sqrt(k) 2^-52 |x||y|.
-// k = 272: 360 ms as two-sided Jacobi in one block; ~10 ms here.
+// k = 272: 360 ms as two-sided Jacobi in one block; 7.5 ms here.
 constexpr int HJ_THREADS = 128;
-__global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, GridSync* sy, int k, int* status) {
+// Squared norms are formed in a sweep's first round and carried through its rotations (they only steer the angles).
+__global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, double* __restrict__ norms, GridSync* sy,
+                                                        int k, int* status) {
   constexpr int PT = (KLIM + HJ_THREADS - 1) / HJ_THREADS;
-  __shared__ double red[3][HJ_THREADS / 32];
-  __shared__ double rot[2];
-  const int n = (k + 1) / 2 * 2, tid = threadIdx.x, i = blockIdx.x;
-  const double tol = sqrt((double)k) * 2.220446049250313e-16;
+  __shared__ double red[3][HJ_THREADS];
+  __shared__ double sums[3], rot[5];
+  const int n = (k + 1) / 2 * 2, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, i = blockIdx.x;
+  const double tol2 = (double)k * 4.930380657631324e-32;            // k 2^-104
   unsigned int target = 0;
   for (int sweep = 0; sweep < HJ_SWEEPS; ++sweep) {
     bool any = false;
     for (int round = 0; round < n - 1; ++round) {
       int p = rr_member(i, round, n), q = rr_member(n - 1 - i, round, n);
       if (p > q) { const int x = p; p = q; q = x; }
-      if (q < k) {                                   // (odd k: the dummy's partner rests)
-        double x[PT], y[PT], a = 0.0, b = 0.0, g = 0.0;
+      if (q < k) {                                   // (odd k: the dummy's partner rests, its norm formed all the same)
+        double x[PT], y[PT], g = 0.0;
 #pragma unroll
         for (int e = 0; e < PT; ++e) {
           const int c = tid + e * HJ_THREADS;
           x[e] = c < k ? __ldcg(W + (int64_t)p * k + c) : 0.0;
           y[e] = c < k ? __ldcg(W + (int64_t)q * k + c) : 0.0;
         }
+        const int vals = round == 0 ? 3 : 1;
+        double a = 0.0, b = 0.0;
+        if (tid == 0 && round > 0) { a = __ldcg(norms + p); b = __ldcg(norms + q); }
 #pragma unroll
-        for (int e = 0; e < PT; ++e) {
-          if (e * HJ_THREADS < k) {
-            a = fma(x[e], x[e], a);
-            b = fma(y[e], y[e], b);
-            g = fma(x[e], y[e], g);
-          }
-        }
+        for (int e = 0; e < PT; ++e)
+          if (warp * 32 + e * HJ_THREADS < k) g = fma(x[e], y[e], g);
+        red[0][tid] = g;
+        if (round == 0) {
+          double nx = 0.0, ny = 0.0;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          a += __shfl_xor_sync(0xffffffffu, a, o);
-          b += __shfl_xor_sync(0xffffffffu, b, o);
-          g += __shfl_xor_sync(0xffffffffu, g, o);
+          for (int e = 0; e < PT; ++e)
+            if (warp * 32 + e * HJ_THREADS < k) { nx = fma(x[e], x[e], nx); ny = fma(y[e], y[e], ny); }
+          red[1][tid] = nx;
+          red[2][tid] = ny;
         }
-        if ((tid & 31) == 0) { red[0][tid >> 5] = a; red[1][tid >> 5] = b; red[2][tid >> 5] = g; }
         __syncthreads();
+        if (warp < vals) {
+          double v = red[warp][lane];
+#pragma unroll
+          for (int w = 1; w < HJ_THREADS / 32; ++w) v += red[warp][lane + 32 * w];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) sums[warp] = v;
+        }
+        if (vals == 3) __syncthreads();
         if (tid == 0) {
-          a = b = g = 0.0;
-          for (int w = 0; w < HJ_THREADS / 32; ++w) { a += red[0][w]; b += red[1][w]; g += red[2][w]; }
-          double c = 1.0, s = 0.0, t = 0.0;
-          if (g * g > tol * tol * a * b) jacobi_angle(a, b, g, c, s, t);
-          rot[0] = c; rot[1] = s;
+          g = sums[0];
+          if (round == 0) { a = sums[1]; b = sums[2]; }
+          double c = 1.0, s = 0.0;
+          if (g * g > tol2 * a * b) jacobi_angle(b - a, g, c, s);
+          rot[0] = c; rot[1] = s; rot[2] = a; rot[3] = b; rot[4] = g;
         }
         __syncthreads();
         const double c = rot[0], s = rot[1];
+        if (tid == HJ_THREADS - 1 && (s != 0.0 || round == 0)) {     // (the last warp has the fewest elements)
+          const double cg = c * rot[4], sg = s * rot[4];
+          __stcg(norms + p, c * (c * rot[2] - sg) - s * (cg - s * rot[3]));
+          __stcg(norms + q, s * (s * rot[2] + cg) + c * (sg + c * rot[3]));
+        }
         if (s != 0.0) {
           any = true;
 #pragma unroll
@@ -857,6 +946,22 @@ __global__ void __launch_bounds__(HJ_THREADS) hj_kernel(double* __restrict__ W, 
               __stcg(W + (int64_t)q * k + j, s * x[e] + c * y[e]);
             }
           }
+        }
+      } else if (round == 0) {
+        double nx = 0.0;
+        for (int c = tid; c < k; c += HJ_THREADS) {
+          const double v = __ldcg(W + (int64_t)p * k + c);
+          nx = fma(v, v, nx);
+        }
+        red[0][tid] = nx;
+        __syncthreads();
+        if (warp == 0) {
+          double v = red[0][lane];
+#pragma unroll
+          for (int w = 1; w < HJ_THREADS / 32; ++w) v += red[0][lane + 32 * w];
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+          if (lane == 0) __stcg(norms + p, v);
         }
       }
       if (round == n - 2 && any && tid == 0) atomicOr(&sy->rotated[sweep], 1);
@@ -905,12 +1010,16 @@ __global__ void __launch_bounds__(HJ_THREADS) hj_vectors_kernel(const double* __
 // ---- flip column j so its largest-|.| entry (first index on ties) is positive ----
 // A column without a finite entry (non-finite calibration data) is left as it is and
 // the status word records ZOACT_ERR_NONFINITE.
-__global__ void sign_fix_kernel(float* __restrict__ U, int d, int r, int* __restrict__ status) {
+constexpr int SIGN_THREADS = 1024;      // 14336 rows: 48 us with 256 threads, 24 here
+__global__ void __launch_bounds__(SIGN_THREADS) sign_fix_kernel(float* __restrict__ U, int d, int r, int* __restrict__ status) {
+  pdl_wait();
+  pdl_trigger();
   const int j = blockIdx.x;
-  __shared__ float bv[256];
-  __shared__ int bi[256];
+  __shared__ float bv[SIGN_THREADS];
+  __shared__ int bi[SIGN_THREADS];
   float best = -1.f;
   int idx = 0x7fffffff;
+#pragma unroll 8
   for (int i = threadIdx.x; i < d; i += blockDim.x) {
     const float a = fabsf(U[(int64_t)i * r + j]);
     if (a > best || (a == best && i < idx)) { best = a; idx = i; }
@@ -983,8 +1092,10 @@ int launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int64_t 
   const int sym = A == B;
   int chunk;
   const int nchunk = atb_chunks(ctx, rows, k, chunk);
-  atb_partial_kernel<<<dim3(tiles, tiles, (unsigned)nchunk), 256, 0, ctx->stream>>>(A, B, w.part, rows, k, chunk, sym);
-  sum_partials_kernel<<<(k * k + 31) / 32, 256, 0, ctx->stream>>>(w.part, w.S, nchunk, k, sym);
+  ZOACT_CUDA_TRY(launch_pdl(ctx, tiles > 1 ? atb_partial_kernel<true> : atb_partial_kernel<false>, dim3(tiles, tiles, (unsigned)nchunk), dim3(256), 0, A, B, w.part, rows,
+                            k, chunk, sym));
+  ZOACT_CUDA_TRY(launch_pdl(ctx, sum_partials_kernel, dim3((unsigned)((k * k + 31) / 32)), dim3(256), 0, w.part, w.S,
+                            nchunk, k, sym));
   ctx->n_launch += 2;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
@@ -993,7 +1104,7 @@ int launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int64_t 
 // R^-1 (k > KMAX: and R, the shift) of S
 int launch_chol(Ctx* ctx, const Work& w, int k) {
   if (k <= KMAX) {
-    chol_inv_kernel<<<1, CHOL_THREADS, CHOL_SMEM, ctx->stream>>>(w.S, w.Rinv, k, ctx->d_status);
+    ZOACT_CUDA_TRY(launch_pdl(ctx, chol_inv_kernel, dim3(1), dim3(CHOL_THREADS), CHOL_SMEM, w.S, w.Rinv, k, ctx->d_status));
   } else {
     ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
     CholBig c{w.S, w.R, w.M, w.Rinv, w.D, w.shift, w.sync, k, ctx->d_status};
@@ -1010,9 +1121,14 @@ int launch_chol(Ctx* ctx, const Work& w, int k) {
 // op (with its 16-bit type): write the result's operand form too.
 int launch_apply(Ctx* ctx, const float* A, const double* M, float* out, int64_t rows, int k, int ldm, int c, int tri,
                  const Operand* op = nullptr, int dtype = ZOACT_DT_FP32) {
-  const dim3 grid((unsigned)((rows + 63) / 64), (unsigned)((c + 63) / 64));
-  auto kern = !op ? apply_kernel<float> : dtype == ZOACT_DT_BF16 ? apply_kernel<__nv_bfloat16> : apply_kernel<__half>;
-  kern<<<grid, 256, 0, ctx->stream>>>(A, M, out, rows, k, ldm, c, tri, op ? *op : Operand{});
+  const int ct = c <= 32 || (tri && c > KMAX) ? 32 : 64;
+  const int rt = 4096 / ct;
+  const dim3 grid((unsigned)((rows + rt - 1) / rt), (unsigned)((c + ct - 1) / ct));
+  auto kern = ct == 32 ? (!op ? apply_kernel<float, 32> : dtype == ZOACT_DT_BF16 ? apply_kernel<__nv_bfloat16, 32>
+                                                                                : apply_kernel<__half, 32>)
+                       : (!op ? apply_kernel<float, 64> : dtype == ZOACT_DT_BF16 ? apply_kernel<__nv_bfloat16, 64>
+                                                                                : apply_kernel<__half, 64>);
+  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, grid, dim3(256), 0, A, M, out, rows, k, ldm, c, tri, op ? *op : Operand{}));
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
@@ -1033,10 +1149,11 @@ int orth(Ctx* ctx, const Work& w, float* Y, float* tmp, int d, int k, const Oper
   return ZOACT_OK;
 }
 
-// dst [rows, k] (or null) = X F for 16-bit X [rows, kd] and F's operand form; to_op: dst's operand form too.
+// dst [rows, k] (or null) = X F for 16-bit X [rows, kd] and F's operand form; to_op: dst's operand form too.  most_kb:
+// K-blocks accumulated by one MMA chain at most (0: as the chip is filled).
 int launch_product(Ctx* ctx, const Work& w, const void* X, int dtype, int64_t rows, int64_t kd, const Operand& f, int mode,
-                   int k, float* dst, const Operand* to_op, int d) {
-  const ProjPlan plan = proj_plan(ctx, rows, (int)kd, k, PROJ_MAX_SPLITS);
+                   int k, float* dst, const Operand* to_op, int d, int most_kb = 0) {
+  const ProjPlan plan = proj_plan(ctx, rows, (int)kd, k, PROJ_MAX_SPLITS, most_kb);
   float* part = static_cast<float*>(
       scratch(ctx, SLOT_SPLITK, (size_t)plan.groups * plan.splits * rows * plan.rt * sizeof(float)));
   if (!part) return ZOACT_ERR_NOMEM;
@@ -1048,8 +1165,8 @@ int launch_product(Ctx* ctx, const Work& w, const void* X, int dtype, int64_t ro
   const bool bf = dtype == ZOACT_DT_BF16;
   auto kern = to_op ? (bf ? reduce_parts_kernel<__nv_bfloat16, true> : reduce_parts_kernel<__half, true>)
                     : (bf ? reduce_parts_kernel<__nv_bfloat16, false> : reduce_parts_kernel<__half, false>);
-  kern<<<grid, 256, 0, ctx->stream>>>(part, rows, k, plan.splits, plan.rt, dst, to_op ? *to_op : Operand{}, mode, w.absmax,
-                                      d);
+  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, grid, dim3(256), 0, part, rows, k, plan.splits, plan.rt, dst,
+                            to_op ? *to_op : Operand{}, mode, w.absmax, d));
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
@@ -1121,13 +1238,13 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
       ZOACT_CUDA_TRY(cudaMemsetAsync(w.absmax, 0, sizeof(int), ctx->stream));
       ZOACT_CUDA_TRY(cudaMemsetAsync(ops, 0, q_op + p_op, ctx->stream));   // ranks past k stay zero
     }
-    dim3 grid((unsigned)((n_pad + 31) / 32), (unsigned)((d + 31) / 32));
+    const dim3 grid((unsigned)((n_pad + 63) / 64), (unsigned)((d + 63) / 64));
     int* top = xdtype == ZOACT_DT_FP16 && direct ? w.absmax : nullptr;
     if (xdtype == ZOACT_DT_BF16) {
-      transpose_pad_kernel<__nv_bfloat16><<<grid, dim3(32, 8), 0, ctx->stream>>>(
+      transpose_pad_kernel<__nv_bfloat16><<<grid, 256, 0, ctx->stream>>>(
           static_cast<const __nv_bfloat16*>(X), static_cast<__nv_bfloat16*>(Xt), n_tok, d, n_pad, top);
     } else {
-      transpose_pad_kernel<__half><<<grid, dim3(32, 8), 0, ctx->stream>>>(static_cast<const __half*>(X),
+      transpose_pad_kernel<__half><<<grid, 256, 0, ctx->stream>>>(static_cast<const __half*>(X),
                                                                           static_cast<__half*>(Xt), n_tok, d, n_pad, top);
     }
     ++ctx->n_launch;
@@ -1139,7 +1256,8 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   }
   // 2-3. sketch and subspace iteration: Q stays in w.Q
   const int64_t nq = (int64_t)d * k;
-  omega_kernel<<<(unsigned)((nq / 4 + 255) / 256 + 1), 256, 0, ctx->stream>>>(w.Q, nq, seed); ++ctx->n_launch;
+  ZOACT_CUDA_TRY(launch_pdl(ctx, omega_kernel, dim3((unsigned)((nq / 4 + 255) / 256 + 1)), dim3(256), 0, w.Q, nq, seed));
+  ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   const Operand* qop = direct ? &w.qop : nullptr;
   int st = orth(ctx, w, w.Q, w.Y, d, k, qop, xdtype);
@@ -1160,7 +1278,11 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   }
   // 4. Rayleigh-Ritz: S = Q^T G Q, of P = X Q as P^T P
   if (direct) {
-    st = launch_product(ctx, w, X, xdtype, n_tok, d, w.qop, 0, k, w.P, nullptr, d);
+    // The Ritz values are squares of P's sums, whose terms mostly share a sign, and the tensor core truncates every
+    // 16-wide step of its fp32 accumulator: chains of n_tok / 256 K-blocks keep that bias at half of what a Gram matrix
+    // summed over the tokens had (14336 wide, 512 tokens: 1.0e-6 of the values in chains of 7 K-blocks, 3.0e-7 in 2).
+    const int most_kb = n_tok < 256 ? 1 : (int)(n_tok / 256);
+    st = launch_product(ctx, w, X, xdtype, n_tok, d, w.qop, 0, k, w.P, nullptr, d, most_kb);
     if (!st) st = launch_atb(ctx, w, w.P, w.P, n_tok, k);
   } else {
     gemm_gq_kernel<<<gq_blocks, 256, 0, ctx->stream>>>(w.G, w.Q, w.Y, d, k); ++ctx->n_launch;
@@ -1169,14 +1291,15 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   }
   if (st) return st;
   if (k <= KMAX) {
-    jacobi_kernel<<<1, JAC_THREADS, JACOBI_SMEM, ctx->stream>>>(w.S, w.log, w.ints, w.ev, w.ints + 1, k);
-    jacobi_vectors_kernel<<<k, 32, 0, ctx->stream>>>(w.log, w.ints, w.ints + 1, w.V, k);
+    ZOACT_CUDA_TRY(launch_pdl(ctx, jacobi_kernel, dim3(1), dim3(JAC_THREADS), JACOBI_SMEM, w.S, w.log, w.ints, w.ev,
+                              w.ints + 1, k));
+    ZOACT_CUDA_TRY(launch_pdl(ctx, jacobi_vectors_kernel, dim3((unsigned)k), dim3(32), 0, w.log, w.ints, w.ints + 1, w.V, k));
     ctx->n_launch += 2;
   } else {
     st = launch_chol(ctx, w, k);
     if (st) return st;
     ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
-    void* args[] = {&w.R, &w.sync, &k, &ctx->d_status};
+    void* args[] = {&w.R, &w.raw, &w.sync, &k, &ctx->d_status};
     ZOACT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(hj_kernel), dim3((unsigned)((k + 1) / 2)),
                                                dim3(HJ_THREADS), args, 0, ctx->stream));
     hj_norms_kernel<<<k, HJ_THREADS, 0, ctx->stream>>>(w.R, w.raw, k);
@@ -1186,7 +1309,8 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
   ZOACT_CHECK_LAUNCH();
   st = launch_apply(ctx, w.Q, w.V, U_out, d, k, k, r, 0);
   if (st) return st;
-  sign_fix_kernel<<<r, 256, 0, ctx->stream>>>(U_out, d, r, ctx->d_status); ++ctx->n_launch;
+  ZOACT_CUDA_TRY(launch_pdl(ctx, sign_fix_kernel, dim3((unsigned)r), dim3(SIGN_THREADS), 0, U_out, d, r, ctx->d_status));
+  ++ctx->n_launch;
   if (evals_out) {
     f64_to_f32_kernel<<<1, 256, 0, ctx->stream>>>(w.ev, evals_out, k);
     ++ctx->n_launch;

@@ -276,7 +276,7 @@ int basis_tc_rows(int r) {
 int proj_rank_tile(int r) { return proj_rt(r); }
 int proj_operand_rows(int r) { return proj_nb(proj_rt(r)); }
 
-ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits) {
+ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits, int most_kb) {
   ProjPlan p;
   p.rt = proj_rt(r);
   p.groups = (r + p.rt - 1) / p.rt;
@@ -288,6 +288,7 @@ ProjPlan proj_plan(const Ctx* ctx, int64_t rows, int d_in, int r, int max_splits
   if (splits > max_splits) splits = max_splits;
   if (splits < 1) splits = 1;
   p.kbps = (int)((p.num_kb + splits - 1) / splits);
+  if (most_kb > 0 && p.kbps > most_kb) p.kbps = most_kb;
   p.splits = (p.num_kb + p.kbps - 1) / p.kbps;
   return p;
 }
