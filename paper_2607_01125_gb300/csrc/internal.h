@@ -142,6 +142,15 @@ __device__ __forceinline__ float apply_act(float y, int act) {
   return y;
 }
 
+// The next bf16 part of x and of y (y's in the upper half), taken off them: three parts hold 24 bits.
+__device__ __forceinline__ uint32_t next_part_bf16x2(float& x, float& y) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  const uint32_t w = *reinterpret_cast<const uint32_t*>(&h);
+  x -= __uint_as_float(w << 16);
+  y -= __uint_as_float(w & 0xffff0000u);
+  return w;
+}
+
 __device__ __forceinline__ float silu_f(float x) { return x / (1.0f + expf(-x)); }
 
 inline size_t dtype_size(int dt) {
@@ -250,12 +259,19 @@ enum LowrankMode { LOWRANK_EPILOGUE = 0, LOWRANK_C_ON_TC = 1, LOWRANK_ALL_ON_TC 
 // Extra K columns per layer for rank r: the three 16-bit products P_hi T_hi, P_hi T_lo, P_lo T_hi
 // padded to whole 64-column K-blocks.
 inline int aug_cols(int r) { return (3 * r + 63) / 64 * 64; }
+// Z as B operands of a warp's m16n8k16 MMA (rank tile rt <= 32, zero past r and d_out): per 16 columns and bf16 part of
+// three, what lane l reads lies together -- columns l / 4 and 8 + l / 4, of each group of eight ranks the pair
+// 2 (l % 4), + 1 -- except that four groups take two reads, 8 columns each.
+__host__ __device__ constexpr int z_groups(int rt) { return rt <= 8 ? 1 : rt / 8; }
+__host__ __device__ constexpr int z_chunk_words(int rt) { return 3 * 32 * 2 * z_groups(rt); }
+inline size_t z_table_words(int rt, int64_t d_out) { return (size_t)((d_out + 63) / 64 * 4 * z_chunk_words(rt)); }
 // Writes A_aug [rows, ka_tot] and B_aug / B_aug2 [nbB * d_out, ka_tot] (bf16) for one pair forward.
 // distinct: gate and up have their own projections (A_aug holds both, B_aug zero-pads the other half).
-// Zt / Zt2 (optional): Z of the nzq queries zq, transposed, [nzq][r][d_out] fp32 each.
+// Zt / Zt2 (optional): Z of the nzq queries zq, transposed, [nzq][r][d_out] fp32 each; with z_rt, operand tables of that
+// rank tile (z_table_words each).
 // slots (LOWRANK_ALL_ON_TC): S > 1 puts row t's parts in K slot block(t) mod S of an A_aug row of S ka columns.
 int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct, int slots, void* A_aug,
-                    void* B_aug, void* B_aug2, float* Zt, float* Zt2, const uint64_t* zq, int nzq);
+                    void* B_aug, void* B_aug2, float* Zt, float* Zt2, const uint64_t* zq, int nzq, int z_rt);
 int launch_gemm_tc_f32out(Ctx* ctx, const void* A, const void* B, int dtype, int M, int N, int K,
                           float* D);
 

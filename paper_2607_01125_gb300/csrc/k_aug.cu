@@ -18,8 +18,10 @@
 // has S K slots and row t fills slot block(t) mod S, so each slot meets the
 // table of the tile's block congruent to it), and the single table T = C otherwise.  With C
 // on the tensor cores the epilogue still adds c_b Z_b p: for it this kernel
-// also writes Z of every distinct query transposed, Zt[q][j][n] (fp32), so the
-// pair kernel copies its tile's columns instead of regenerating them per tile.
+// also writes Z of every distinct query, so the pair kernel copies its tile's
+// columns instead of regenerating them per tile: transposed, Zt[q][j][n] (fp32),
+// or, where several blocks' terms go on the epilogue's matrix instruction, in its
+// operand order and three bf16 parts.
 // Purely memory-bound and small (rows x r and d_out x r inputs).
 #include "internal.h"
 #include "philox.cuh"
@@ -30,7 +32,7 @@ namespace {
 struct AugBlocks {
   float coef[ZOACT_MAX_EVAL_BLOCKS];
   uint64_t qry[ZOACT_MAX_EVAL_BLOCKS];
-  uint64_t zq[ZOACT_MAX_EVAL_BLOCKS];   // distinct queries whose Z is written transposed
+  uint64_t zq[ZOACT_MAX_EVAL_BLOCKS];   // distinct queries whose Z is written
   int nzq;
   // layers run as one (B rows only): row n of the table belongs to layer s with seg_off[s] <= n <
   // seg_off[s + 1]; its T = C_s + c_b Z_b takes C_s and Z from that layer's own rows and Philox stream
@@ -66,40 +68,108 @@ __device__ __forceinline__ uint2 split_quad(float4 v, bool want_lo) {
 // ranks, column n), columns fastest so that the stores coalesce.
 __device__ __forceinline__ void write_z_tables(const AugBlocks& blk, int d_out, int r, uint64_t seed, uint32_t lid,
                                                uint32_t lid2, float* __restrict__ Zt, float* __restrict__ Zt2) {
-  if (Zt && blk.nzq > 0) {
-    const int groups = (r + 3) / 4;
-    const int n_mat = Zt2 ? 2 : 1;
-    const int64_t items = (int64_t)n_mat * blk.nzq * groups * d_out;
-    for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
-         it += (int64_t)gridDim.x * blockDim.x) {
-      const int n = (int)(it % d_out);
-      int64_t rest = it / d_out;
-      const int jg = (int)(rest % groups);
-      rest /= groups;
-      const int qi = (int)(rest % blk.nzq);
-      const int mat = (int)(rest / blk.nzq);
-      float* dst = (mat ? Zt2 : Zt) + (int64_t)qi * r * d_out;
-      const uint32_t layer = mat ? lid2 : lid;
-      if ((r & 3) == 0) {
-        // the four ranks are one Philox group
-        const float4 z = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(((int64_t)n * r + 4 * jg) >> 2));
-        dst[(int64_t)(4 * jg) * d_out + n] = z.x;
-        dst[(int64_t)(4 * jg + 1) * d_out + n] = z.y;
-        dst[(int64_t)(4 * jg + 2) * d_out + n] = z.z;
-        dst[(int64_t)(4 * jg + 3) * d_out + n] = z.w;
-      } else {
+  const int groups = (r + 3) / 4;
+  const int n_mat = Zt2 ? 2 : 1;
+  const int64_t items = (int64_t)n_mat * blk.nzq * groups * d_out;
+  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
+       it += (int64_t)gridDim.x * blockDim.x) {
+    const int n = (int)(it % d_out);
+    int64_t rest = it / d_out;
+    const int jg = (int)(rest % groups);
+    rest /= groups;
+    const int qi = (int)(rest % blk.nzq);
+    const int mat = (int)(rest / blk.nzq);
+    float* dst = (mat ? Zt2 : Zt) + (int64_t)qi * r * d_out;
+    const uint32_t layer = mat ? lid2 : lid;
+    if ((r & 3) == 0) {
+      // the four ranks are one Philox group
+      const float4 z = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(((int64_t)n * r + 4 * jg) >> 2));
+      dst[(int64_t)(4 * jg) * d_out + n] = z.x;
+      dst[(int64_t)(4 * jg + 1) * d_out + n] = z.y;
+      dst[(int64_t)(4 * jg + 2) * d_out + n] = z.z;
+      dst[(int64_t)(4 * jg + 3) * d_out + n] = z.w;
+    } else {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int j = 4 * jg + i;
-          if (j < r) {
-            const int64_t e = (int64_t)n * r + j;
-            dst[(int64_t)j * d_out + n] =
-                z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2)), (int)(e & 3));
-          }
+      for (int i = 0; i < 4; ++i) {
+        const int j = 4 * jg + i;
+        if (j < r) {
+          const int64_t e = (int64_t)n * r + j;
+          dst[(int64_t)j * d_out + n] =
+              z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2)), (int)(e & 3));
         }
       }
     }
   }
+}
+
+// The Z tables in operand order (see z_chunk_words): one thread per (matrix, query, 16 columns, lanes l and l + 1 with l
+// even): its two columns and, of each group of eight, four ranks -- one Philox group where the rank is a multiple of
+// four -- of which it writes 32 H bytes a part.
+template <int H>
+__device__ __forceinline__ void write_z_operands(const AugBlocks& blk, int d_out, int r, uint64_t seed, uint32_t lid,
+                                                 uint32_t lid2, uint32_t* __restrict__ Zt, uint32_t* __restrict__ Zt2) {
+  constexpr int CHUNK = 3 * 32 * 2 * H, G = H > 2 ? 4 : 2 * H;
+  const int chunks = (d_out + 63) / 64 * 4;
+  const int64_t items = (int64_t)(Zt2 ? 2 : 1) * blk.nzq * chunks * 16;
+  for (int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; it < items;
+       it += (int64_t)gridDim.x * blockDim.x) {
+    const int l = 2 * (int)(it & 15);
+    int64_t rest = it >> 4;
+    const int ch = (int)(rest % chunks);
+    rest /= chunks;
+    const int qi = (int)(rest % blk.nzq), mat = (int)(rest / blk.nzq);
+    const uint32_t layer = mat ? lid2 : lid;
+    float z[2][H][4];                                 // [8 columns][group][rank]
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      const int n = ch * 16 + nt * 8 + l / 4;
+#pragma unroll
+      for (int h = 0; h < H; ++h) {
+        const int j0 = 8 * h + 4 * ((l >> 1) & 1);
+        const int64_t e = (int64_t)n * r + j0;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (n < d_out && j0 < r && (r & 3) == 0) v = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2));
+        z[nt][h][0] = v.x; z[nt][h][1] = v.y; z[nt][h][2] = v.z; z[nt][h][3] = v.w;
+        if (n < d_out && (r & 3) != 0)
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (j0 + i < r)
+              z[nt][h][i] = z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)((e + i) >> 2)), (int)((e + i) & 3));
+      }
+    }
+    uint32_t* dst = (mat ? Zt2 : Zt) + ((int64_t)qi * chunks + ch) * CHUNK;
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {
+      uint32_t w[2][2 * H];                           // [lane][8 columns, group]
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          w[0][nt * H + h] = next_part_bf16x2(z[nt][h][0], z[nt][h][1]);
+          w[1][nt * H + h] = next_part_bf16x2(z[nt][h][2], z[nt][h][3]);
+        }
+#pragma unroll
+      for (int g = 0; g < 2 * H / G; ++g) {
+        uint32_t* d = dst + part * (CHUNK / 3) + g * 32 * G + l * G;
+#pragma unroll
+        for (int i = 0; i < 2 * G; i += 4)
+          *reinterpret_cast<uint4*>(d + i) = make_uint4(w[i / G][g * G + i % G], w[(i + 1) / G][g * G + (i + 1) % G],
+                                                        w[(i + 2) / G][g * G + (i + 2) % G],
+                                                        w[(i + 3) / G][g * G + (i + 3) % G]);
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void write_z(int z_rt, const AugBlocks& blk, int d_out, int r, uint64_t seed, uint32_t lid,
+                                        uint32_t lid2, float* __restrict__ Zt, float* __restrict__ Zt2) {
+  if (!Zt || blk.nzq == 0) return;
+  uint32_t* z1 = reinterpret_cast<uint32_t*>(Zt);
+  uint32_t* z2 = reinterpret_cast<uint32_t*>(Zt2);
+  if (z_rt == 0) write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  else if (z_rt <= 8) write_z_operands<1>(blk, d_out, r, seed, lid, lid2, z1, z2);
+  else if (z_rt == 16) write_z_operands<2>(blk, d_out, r, seed, lid, lid2, z1, z2);
+  else write_z_operands<4>(blk, d_out, r, seed, lid, lid2, z1, z2);
 }
 
 // Any rank (the quad kernel below serves ranks that are multiples of 4 with 16-byte aligned sources): one thread per
@@ -112,7 +182,7 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
                 __nv_bfloat16* __restrict__ B2, int64_t rows, int d_out, int r, int ka, int distinct, int full,
                 int nb, const __grid_constant__ AugBlocks blk, uint64_t seed, uint32_t lid, uint32_t lid2,
-                float* __restrict__ Zt, float* __restrict__ Zt2, int slots, int64_t T) {
+                float* __restrict__ Zt, float* __restrict__ Zt2, int z_rt, int slots, int64_t T) {
   pdl_wait();                                         // P and C written by the previous kernels
   pdl_trigger();
   const int ka_row = distinct ? 2 * ka : ka;          // columns of one slot (= B_aug row width)
@@ -191,7 +261,7 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
     const int64_t row_w = 8 * (int64_t)(is_a ? cA : cB);
     *reinterpret_cast<uint4*>(dst + orow * row_w + 8 * c) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  write_z(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 // The same tables for ranks that are multiples of 4 with aligned sources: one thread per four ranks of a row, which
@@ -205,7 +275,7 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
                 __nv_bfloat16* __restrict__ B2, int64_t rows, int d_out, int r, int ka, int distinct, int full,
                 int nb, const __grid_constant__ AugBlocks blk, uint64_t seed, uint32_t lid, uint32_t lid2,
-                float* __restrict__ Zt, float* __restrict__ Zt2, int slots, int64_t T) {
+                float* __restrict__ Zt, float* __restrict__ Zt2, int z_rt, int slots, int64_t T) {
   pdl_wait();                                         // P and C written by the previous kernels
   pdl_trigger();
   const int rq = r / 4, kq = ka / 4, halves = distinct ? 2 : 1;
@@ -275,7 +345,7 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
       }
     }
   }
-  write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  write_z(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -283,7 +353,7 @@ bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 }  // namespace
 
 int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct, int slots, void* A_aug,
-                    void* B_aug, void* B_aug2, float* Zt, float* Zt2, const uint64_t* zq, int nzq) {
+                    void* B_aug, void* B_aug2, float* Zt, float* Zt2, const uint64_t* zq, int nzq, int z_rt) {
   AugBlocks blk{};
   for (int b = 0; b < a.nb; ++b) { blk.coef[b] = a.coef[b]; blk.qry[b] = a.qry[b]; }
   blk.nseg = a.nseg > 1 ? a.nseg : 0;
@@ -301,7 +371,8 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   const int ka_row = distinct ? 2 * ka : ka;
   const int64_t nbB = full ? a.nb : 1;
   const int64_t items = a.rows * (slots * ka_row / 8) + (B_aug2 ? 2 : 1) * nbB * a.d_out * (ka_row / 8);
-  const int64_t z_items = Zt ? (int64_t)(Zt2 ? 2 : 1) * blk.nzq * ((a.r + 3) / 4) * a.d_out : 0;
+  const int64_t z_each = z_rt ? (int64_t)(a.d_out + 63) / 64 * 64 : (int64_t)((a.r + 3) / 4) * a.d_out;
+  const int64_t z_items = Zt ? (Zt2 ? 2 : 1) * blk.nzq * z_each : 0;
   const int64_t work = items > z_items ? items : z_items;
   int64_t grid = (work + 255) / 256;
   const int64_t cap = (int64_t)ctx->sm_count * 32;
@@ -325,7 +396,7 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)grid), dim3(256), 0, a.P, distinct ? a.P2 : nullptr, a.C,
                             a.C2, static_cast<__nv_bfloat16*>(A_aug), static_cast<__nv_bfloat16*>(B_aug),
                             static_cast<__nv_bfloat16*>(B_aug2), a.rows, a.d_out, a.r, ka, distinct, full, a.nb, blk,
-                            a.seed, a.layer_id, a.layer_id2, Zt, Zt2, slots, a.T));
+                            a.seed, a.layer_id, a.layer_id2, Zt, Zt2, z_rt, slots, a.T));
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;

@@ -302,8 +302,14 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
       zq_of[b] = nzq++;
     }
   }
+  // 16-bit outputs of several evaluation blocks on a shared input, on CTA pairs: the two signs of one query, or others
+  const bool one_p = !gated || a.P2 == a.P;
+  const bool blocks16 = two && lmode == LOWRANK_C_ON_TC && a.shared && a.nb >= 2 && dtype_size(a.ydtype) == 2;
+  const bool mirror = blocks16 && a.nb == 2 && a.qry[0] == a.qry[1] && a.coef[1] == -a.coef[0] && a.coef[0] != 0.f;
+  const bool multi = blocks16 && !mirror && one_p;
   float* zt = nullptr;
   float* zt2 = nullptr;
+  const size_t z_words = multi ? z_table_words(rt, a.d_out) : (size_t)a.r * a.d_out;   // of one query
   if (lmode != LOWRANK_EPILOGUE) {
     const int64_t nbB = lmode == LOWRANK_ALL_ON_TC ? a.nb : 1;
     const size_t a_bytes = (size_t)a.rows * slots * ka_tot * 2;
@@ -313,12 +319,12 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
     if (!abuf || !bbuf) return ZOACT_ERR_NOMEM;
     uint8_t* bbuf2 = gated ? bbuf + b_bytes : nullptr;
     if (nzq > 0) {
-      const size_t z_floats = (size_t)nzq * a.r * a.d_out;
-      zt = static_cast<float*>(scratch(ctx, SLOT_AUG_Z, (gated ? 2 : 1) * z_floats * sizeof(float)));
+      zt = static_cast<float*>(scratch(ctx, SLOT_AUG_Z, (gated ? 2 : 1) * nzq * z_words * sizeof(float)));
       if (!zt) return ZOACT_ERR_NOMEM;
-      zt2 = gated ? zt + z_floats : nullptr;
+      zt2 = gated ? zt + nzq * z_words : nullptr;
     }
-    st = launch_aug_prep(ctx, a, lmode, ka, distinct ? 1 : 0, slots, abuf, bbuf, bbuf2, zt, zt2, zq_list, nzq);
+    st = launch_aug_prep(ctx, a, lmode, ka, distinct ? 1 : 0, slots, abuf, bbuf, bbuf2, zt, zt2, zq_list, nzq,
+                         multi ? rt : 0);
     if (st) return st;
     st = encode_tmap_2d_16bit(&tm.aa, abuf, ZOACT_DT_BF16, a.rows, (int64_t)slots * ka_tot, BM);
     if (st) return st;
@@ -387,19 +393,17 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
     st = encode_tmap_store(&tm.y16, a.Y, a.ydtype, a.rows, a.d_out, 16, BM, false);
     if (st) return st;
     p.y_staged = STAGE_ALL;
-  } else if (two && lmode == LOWRANK_C_ON_TC && a.shared && a.nb == 2 && es == 2 && a.qry[0] == a.qry[1] &&
-             a.coef[1] == -a.coef[0] && a.coef[0] != 0.f) {
+  } else if (mirror) {
     uint8_t* y0 = static_cast<uint8_t*>(a.Y);
     st = encode_tmap_store(&tm.y, y0, a.ydtype, a.T, a.d_out, 16, BM, false);
     if (st) return st;
     st = encode_tmap_store(&tm.y16, y0 + (size_t)a.T * a.d_out * es, a.ydtype, a.T, a.d_out, 16, BM, false);
     if (st) return st;
     // four rows per thread where the projections fit in registers (rank tile <= 16, one P for gate and up)
-    p.y_staged = (rt <= 16 && (!gated || a.P2 == a.P)) ? STAGE_MIRROR4 : STAGE_MIRROR;
-  } else if (two && lmode == LOWRANK_C_ON_TC && a.shared && a.nb >= 2 && es == 2 && rt <= 16 &&
-             (!gated || a.P2 == a.P)) {
+    p.y_staged = (rt <= 16 && one_p) ? STAGE_MIRROR4 : STAGE_MIRROR;
+  } else if (multi) {
     // other evaluation blocks on a shared input (the one-sided q-query estimator): one 3-D store map
-    st = encode_tmap_store3(&tm.y, a.Y, a.ydtype, a.nb, a.T, a.d_out, 16, BM);
+    st = encode_tmap_store3(&tm.y, a.Y, a.ydtype, a.nb, a.T, a.d_out, 16, MULTI4_ROWS);
     if (st) return st;
     tm.y16 = tm.y;
     p.y_staged = STAGE_MULTI4;
@@ -414,7 +418,7 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   p.aug_block_rows = aug_block_rows;
   p.Zt = zt;
   p.Zt2 = zt2;
-  p.zt_qstride = (int64_t)a.r * a.d_out;
+  p.zt_qstride = (int64_t)z_words;
   for (int b = 0; b < ZOACT_MAX_EVAL_BLOCKS; ++b) p.zq[b] = b < a.nb ? zq_of[b] : -1;
   // (al16: 16-byte alignment, defined above)
   p.vec_ok = al16(a.C) && al16(a.C2) && al16(a.P) && al16(a.P2);

@@ -28,12 +28,13 @@ static int by_rank_two(Ctx* ctx, int mode, int rt, const TmaSet& tm, const Param
       return mode == MODE_PAIR && rt == 4 ? launch_two<TO, 4, MODE_PAIR, STAGE_LOSS>(ctx, tm, p) : ZOACT_ERR_UNSUPPORTED;
     if (p.y_staged == STAGE_MULTI4) {
       switch (rt) {
-        case 4: return mode == MODE_GATED ? launch_two<TO, 4, MODE_GATED, STAGE_MULTI4>(ctx, tm, p)
-                                          : launch_two<TO, 4, MODE_PAIR, STAGE_MULTI4>(ctx, tm, p);
+        case 4:
         case 8: return mode == MODE_GATED ? launch_two<TO, 8, MODE_GATED, STAGE_MULTI4>(ctx, tm, p)
                                           : launch_two<TO, 8, MODE_PAIR, STAGE_MULTI4>(ctx, tm, p);
         case 16: return mode == MODE_GATED ? launch_two<TO, 16, MODE_GATED, STAGE_MULTI4>(ctx, tm, p)
                                            : launch_two<TO, 16, MODE_PAIR, STAGE_MULTI4>(ctx, tm, p);
+        case 32: return mode == MODE_GATED ? launch_two<TO, 32, MODE_GATED, STAGE_MULTI4>(ctx, tm, p)
+                                           : launch_two<TO, 32, MODE_PAIR, STAGE_MULTI4>(ctx, tm, p);
         default: return ZOACT_ERR_UNSUPPORTED;
       }
     }

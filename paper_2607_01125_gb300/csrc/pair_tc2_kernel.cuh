@@ -66,7 +66,7 @@ struct SharedState2 {
   uint64_t tmem_full[2];
   uint64_t tmem_empty[2];
   uint64_t drain;
-  uint64_t tload[2];      // fused loss: target chunk landed in a warpgroup's staging buffer
+  uint64_t tload[2];      // fused loss: target chunk landed in a warpgroup's staging buffer; q queries: Z tables in buffer i
   uint32_t tmem_base;
   int abort_flag;
   int epi_ok;
@@ -532,126 +532,193 @@ __device__ __forceinline__ bool epi_mirror4_staged(const Params& prm, const TmaS
   return true;
 }
 
-// Column width of one table pass of the staged q-query epilogue: four permuted tables
-// (two blocks x gate, up) of RT x (MULTI4_SLOTS + TPAD) floats below the staging buffers.
-constexpr int MULTI4_SLOTS = 64;
+// D += A B for 16 rows x 8 columns x 16 ranks by one warp (rows lane / 4 and + 8, columns 2 (lane % 4), + 1).
+__device__ __forceinline__ void mma_16x8x16(float* d, const uint32_t* a_lo, const uint32_t* a_hi, uint32_t b_lo,
+                                            uint32_t b_hi) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a_lo[0]), "r"(a_lo[1]), "r"(a_hi[0]), "r"(a_hi[1]), "r"(b_lo), "r"(b_hi));
+}
+
+// Staging offset of the staged q-query epilogue: two buffers of Z tables (gate, up) lie below it, a warp's 32 rows x 32
+// bytes above.
+constexpr int MULTI4_STG_OFF = 24576;
+static_assert(MULTI4_STG_OFF % 1024 == 0 && MULTI4_STG_OFF + EPI_WARPS * MULTI4_ROWS * 32 <= TBL_FLOATS * 4,
+              "q-query staging exceeds the table region");
 
 // The staged epilogue of several evaluation blocks on a shared input (C p in the
 // accumulator; the one-sided q-query estimator, or any blocks that are not the two
-// signs of one query), four rows per thread as in epi_mirror4_staged.  Blocks go in
-// pairs: per column pass the permuted tables c_b Z_b of both (gate at tbl + t TSZ,
-// up at tbl + (2 + t) TSZ; none for c_b = 0) are built, then each warpgroup forms
-// acc + c_b Z_b p for 16 columns of its 128 rows, one block after the other, stages
-// both blocks' outputs and one thread stores them through tm.y, a 3-D map over
-// the blocks' [T, d_out] slabs that drops rows past T and columns past d_out.
+// signs of one query), four rows per thread as in epi_mirror4_staged.  A pass is one
+// block of SLOTS columns: its Z tables (none for c_b = 0), which the operand kernel
+// wrote in the order the lanes read them, come by bulk copies, two passes ahead, into
+// two buffers; one barrier ends a pass.  Each warp forms acc + c_b Z_b p for 16 columns
+// of its 32 rows at a time and stores them by itself through tm.y, a 3-D map over the
+// blocks' [T, d_out] slabs that drops rows past T and columns past d_out.
+// The term is added from registers in the layout of the accumulator read, so it goes
+// on the warp's own matrix instruction: p and Z as sums of three bf16 values each, the
+// six products that reach 2^-24, summed in fp32 apart from the accumulator (rank 16,
+// against 64 bits: a chain of fp32 FMAs errs by 3.1 rms, this by 1.4 to 2.3).  Nine
+// blocks of 512 x 14336 gated, rank 16: 248 us with fp32 FMAs, passes of two blocks whose
+// tables were fetched between two barriers, and two barriers more per 16 columns
+// around a warpgroup's store (28% of the issue slots used); 197 with passes as here and
+// stores by warp; 166 with the matrix instruction (an FMA of two columns took 5 cycles);
+// 159 with the tables split once for all tiles.  Left: the main loop 76, and a chunk's chain of reads, MMAs and stores.
 template <typename TO, int RT, int MODE>
 __device__ __forceinline__ bool epi_multi4_staged(const Params& prm, const TmaSet& tm, SharedState2* ss, float* tbl,
                                                   int etid, int half, int quad, int lane, int64_t row0, int n_blk,
                                                   int bn, int buf, uint32_t acc_phase, uint32_t t_q,
-                                                  volatile int* abort_flag, bool& pending) {
+                                                  volatile int* abort_flag, bool& pending, uint32_t& tphase) {
   constexpr bool GATED = MODE == MODE_GATED;
-  constexpr int SLOTS = MULTI4_SLOTS;
-  constexpr int STRIDE = SLOTS + TPAD;
-  constexpr int TSZ = RT * STRIDE;
-  static_assert(RT <= 16, "four rows of projections per thread");
-  static_assert((GATED ? 4 : 2) * TSZ * 4 <= MIRROR_STG_OFF, "q-query tables overlap the staging buffers");
+  constexpr int H = z_groups(RT);                           // groups of eight ranks
+  constexpr int SLOTS = H > 2 ? 32 : 64;                    // columns of a pass
+  constexpr int CHUNK = z_chunk_words(RT);                  // words of 16 columns of a table
+  constexpr int TSZ = SLOTS / 16 * CHUNK;
+  constexpr int BSZ = (GATED ? 2 : 1) * TSZ;                // one buffer
+  constexpr int G = H > 2 ? 4 : 2 * H;                      // words of one read
+  static_assert(2 * BSZ * 4 <= MULTI4_STG_OFF, "q-query tables overlap the staging buffers");
   static_assert(sizeof(TO) == 2, "staged q-query output is 16-bit");
   const int r = prm.r;
   const int q = lane & 3, rq = lane >> 2;
-  const bool vec = prm.vec_ok != 0;
-  float p[4][RT];
+  // P of rows rq + 8k, ranks 8h + 2q and + 1, in three parts: [part][group][row pair][row]
+  uint32_t pa[3][H][2][2];
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const int64_t m = row0 + quad * 32 + rq + 8 * k;
-    load_p<RT>(p[k], prm.P, m, r, m < prm.rows, vec);
+#pragma unroll
+    for (int h = 0; h < H; ++h) {
+      const int j = 8 * h + 2 * q;
+      float x = m < prm.rows && j < r ? prm.P[m * r + j] : 0.f;
+      float y = m < prm.rows && j + 1 < r ? prm.P[m * r + j + 1] : 0.f;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) pa[i][h][k >> 1][k & 1] = next_part_bf16x2(x, y);
+    }
   }
   const int ncol_tile = GATED ? BN / 2 : bn;
-  const bool issuer = (etid & 127) == 0;
-  const uint32_t sp = tc::smem_u32(tbl) + MIRROR_STG_OFF + half * MIRROR_STG_BYTES;   // block slot t at +4096 t
-  bool waited = false;
-  for (int s0 = 0; s0 < ncol_tile; s0 += SLOTS) {
+  const int row_w = (int)row0 + quad * 32;                  // the warp's first row
+  const bool live = row0 + quad * 32 < prm.rows;
+  const uint32_t sp = tc::smem_u32(tbl) + MULTI4_STG_OFF + (uint32_t)(etid >> 5) * (MULTI4_ROWS * 32);
+  const uint32_t* const tw = reinterpret_cast<const uint32_t*>(tbl);
+  const int ncol = min(ncol_tile, prm.d_out - n_blk * ncol_tile);   // (the tables end with the 64 columns d_out lies in)
+  const int passes = (ncol + SLOTS - 1) / SLOTS * prm.nb;
+  auto load = [&](int pass, int bufi) {                     // one thread: pass's tables into a buffer
+    if (pass >= passes) return;
+    const int s = pass / prm.nb, b = pass - s * prm.nb;
+    if (prm.coef[b] == 0.f) return;
+    const int64_t at = prm.zq[b] * prm.zt_qstride + (int64_t)((n_blk * ncol_tile + s * SLOTS) / 16) * CHUNK;
+    const uint32_t bar = tc::smem_u32(&ss->tload[bufi]), dst = tc::smem_u32(tbl + bufi * BSZ);
+    tc::mbar_arrive_expect_tx(bar, BSZ * 4);
+    tc::bulk_load(dst, prm.Zt + at, TSZ * 4, bar);
+    if (GATED) tc::bulk_load(dst + TSZ * 4, prm.Zt2 + at, TSZ * 4, bar);
+  };
+  if (etid == 0) {                                          // (the previous tile's last barrier freed both buffers)
+    load(0, 0);
+    load(1, 1);
+  }
+  bool ok = epi_wait_full(ss, buf, acc_phase, abort_flag, prm.status, etid);
+  if (!ok) {                                                // the loads in flight land before the block gives up
+    if (etid == 0) tc::pause_ns(2000000ull);
+    return false;
+  }
+  int cur = 0, pass = 0;
+  for (int s0 = 0; s0 < ncol; s0 += SLOTS) {
     const int cwid = min(SLOTS, ncol_tile - s0);            // a multiple of 32
-    const int col0 = n_blk * ncol_tile + s0;
-    for (int bp = 0; bp < prm.nb; bp += 2) {
-      const int nblk = min(2, prm.nb - bp);
-      tc::named_bar_sync(1, EPI_THREADS);                   // previous pass's readers are done
-      for (int t = 0; t < nblk; ++t) {
-        const int b = bp + t;
-        if (prm.coef[b] == 0.f) continue;                   // its term is already in the accumulator
-        build_tables_z16<RT>(tbl + t * TSZ, STRIDE, prm.Zt + prm.zq[b] * prm.zt_qstride, prm.coef[b], col0, cwid,
-                             prm.d_out, r, etid);
-        if (GATED)
-          build_tables_z16<RT>(tbl + (2 + t) * TSZ, STRIDE, prm.Zt2 + prm.zq[b] * prm.zt_qstride, prm.coef[b], col0,
-                               cwid, prm.d_out, r, etid);
+    for (int b = 0; b < prm.nb; ++b, ++pass) {
+      const float c = prm.coef[b];
+      if (c != 0.f) {
+        // a wait that gives up ends the tile's loads but not its passes: every thread meets the barriers
+        ok = tc::mbar_wait(tc::smem_u32(&ss->tload[cur]), (tphase >> cur) & 1u, abort_flag, prm.status) && ok;
+        tphase ^= 1u << cur;
       }
-      tc::named_bar_sync(1, EPI_THREADS);
-      if (!waited) {
-        if (!epi_wait_full(ss, buf, acc_phase, abort_flag, prm.status, etid)) return false;
-        waited = true;
-      }
-      const int cbeg = s0 + half * (cwid / 2);
-      for (int c0 = cbeg; c0 < cbeg + cwid / 2; c0 += 16) {
-        const int n = n_blk * ncol_tile + c0;
-        if (n >= prm.d_out) break;                          // uniform over the warpgroup
-        float g[16], u[16];
-        tc::tmem_ld_rows4(t_q + (uint32_t)c0, g);
-        if (GATED) tc::tmem_ld_rows4(t_q + (uint32_t)(BN / 2 + c0), u);
-        if (issuer && pending) tc::bulk_wait_read0();       // the buffers' previous stores have read them
-        tc::named_bar_sync(4 + half, 128);
+      const int cbeg = half * (cwid / 2);
 #pragma unroll 1
-        for (int t = 0; t < nblk; ++t) {
-          float2 zg[4][2], zu[4][2];
+      for (int c0 = cbeg; c0 < cbeg + cwid / 2; c0 += 16) {
+        const int n = n_blk * ncol_tile + s0 + c0;
+        if (n >= prm.d_out || !live) break;                 // uniform over the warp
+        uint32_t acc[2][16];
+        tc::tmem_ld_rows4_issue(t_q + (uint32_t)(s0 + c0), acc[0]);
+        if (GATED) tc::tmem_ld_rows4_issue(t_q + (uint32_t)(BN / 2 + s0 + c0), acc[1]);
+        float z[2][2][2][4] = {};                           // [gate, up][row pair][8 columns][row, column]
+        if (c != 0.f) {
+          uint32_t zb[2][3][2 * H];                         // [gate, up][part][8 columns, group]
 #pragma unroll
-          for (int k = 0; k < 4; ++k) zg[k][0] = zg[k][1] = zu[k][0] = zu[k][1] = make_float2(0.f, 0.f);
-          if (prm.coef[bp + t] != 0.f) {
-            const float* tg = tbl + t * TSZ + (c0 - s0) + 4 * q;
-            const float* tu = tbl + (2 + t) * TSZ + (c0 - s0) + 4 * q;
+          for (int t = 0; t < (GATED ? 2 : 1); ++t)
 #pragma unroll
-            for (int j = 0; j < RT; ++j) {
-              const float4 a = *reinterpret_cast<const float4*>(tg + j * STRIDE);
-              float4 bv = a;
-              if (GATED) bv = *reinterpret_cast<const float4*>(tu + j * STRIDE);
+            for (int i = 0; i < 3; ++i) {
+              const uint32_t* src = tw + cur * BSZ + t * TSZ + (c0 >> 4) * CHUNK + i * (CHUNK / 3) + lane * G;
 #pragma unroll
-              for (int k = 0; k < 4; ++k) {
-                const float2 pj = make_float2(p[k][j], p[k][j]);
-                zg[k][0] = ffma2(make_float2(a.x, a.y), pj, zg[k][0]);
-                zg[k][1] = ffma2(make_float2(a.z, a.w), pj, zg[k][1]);
-                if (GATED) {
-                  zu[k][0] = ffma2(make_float2(bv.x, bv.y), pj, zu[k][0]);
-                  zu[k][1] = ffma2(make_float2(bv.z, bv.w), pj, zu[k][1]);
+              for (int w = 0; w < 2 * H; w += G) {
+                if (G == 4) {
+                  const uint4 v = *reinterpret_cast<const uint4*>(src + w * 32);
+                  zb[t][i][w] = v.x; zb[t][i][w + 1] = v.y; zb[t][i][w + G - 2] = v.z; zb[t][i][w + G - 1] = v.w;
+                } else {
+                  const uint2 v = *reinterpret_cast<const uint2*>(src + w * 32);
+                  zb[t][i][w] = v.x; zb[t][i][w + 1] = v.y;
                 }
               }
             }
-          }
-          const uint32_t sb = sp + 4096u * (uint32_t)t;
+          // products (part of p, part of Z) of 8 ranks, two an instruction: two groups of one product, or two products
+          constexpr int PP[6] = {2, 1, 0, 1, 0, 0}, PZ[6] = {0, 1, 2, 0, 1, 0};
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const float zgk[4] = {zg[k][0].x, zg[k][0].y, zg[k][1].x, zg[k][1].y};
-            const float zuk[4] = {zu[k][0].x, zu[k][0].y, zu[k][1].x, zu[k][1].y};
-            float h[4];
+          for (int s = 0; s < 6 * H; s += 2) {
+            const int p0 = s / H, p1 = (s + 1) / H, h0 = s % H, h1 = (s + 1) % H;
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              if (GATED)
-                h[i] = silu_fast(g[4 * k + i] + zgk[i]) * (u[4 * k + i] + zuk[i]);
-              else
-                h[i] = apply_act(g[4 * k + i] + zgk[i], prm.act);
-            }
-            const uint32_t ro = (uint32_t)((quad * 32 + rq + 8 * k) * 32 + 4 * q);
-            tc::st_shared_b32(sb + ro, pack2(h[0], h[1], (TO*)nullptr));
-            tc::st_shared_b32(sb + ro + 16u, pack2(h[2], h[3], (TO*)nullptr));
+            for (int t = 0; t < (GATED ? 2 : 1); ++t)
+#pragma unroll
+              for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+                for (int nt = 0; nt < 2; ++nt)
+                  mma_16x8x16(z[t][mt][nt], pa[PP[p0]][h0][mt], pa[PP[p1]][h1][mt], zb[t][PZ[p0]][nt * H + h0],
+                              zb[t][PZ[p1]][nt * H + h1]);
           }
         }
+        float g[16], u[16];
+        tc::tmem_ld_rows4_wait(acc[0], g);
+        if (GATED) tc::tmem_ld_rows4_wait(acc[1], u);
+        uint32_t out[4][2];                                 // [row][column pair]
+        const float2 c2 = make_float2(c, c);
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float* zg = z[0][k >> 1][i] + 2 * (k & 1);
+            const float* zu = z[1][k >> 1][i] + 2 * (k & 1);
+            float2 y = ffma2(c2, make_float2(zg[0], zg[1]), make_float2(g[4 * k + 2 * i], g[4 * k + 2 * i + 1]));
+            if (GATED) {                                    // silu_fast(y) u, two columns an instruction
+              const float2 uz =
+                  ffma2(c2, make_float2(zu[0], zu[1]), make_float2(u[4 * k + 2 * i], u[4 * k + 2 * i + 1]));
+              const float2 t = fmul2(y, make_float2(-1.44269504f, -1.44269504f));
+              const float2 d = fadd2(make_float2(exp2_sfu(t.x), exp2_sfu(t.y)), make_float2(1.f, 1.f));
+              y = fmul2(fmul2(y, make_float2(rcp_sfu(d.x), rcp_sfu(d.y))), uz);
+            } else {
+              y = make_float2(apply_act(y.x, prm.act), apply_act(y.y, prm.act));
+            }
+            out[k][i] = pack2(y.x, y.y, (TO*)nullptr);
+          }
+        if (lane == 0 && pending) tc::bulk_wait_read0();    // the buffer's previous store has read it
+        __syncwarp();
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t ro = (uint32_t)((rq + 8 * k) * 32 + 4 * q);
+          tc::st_shared_b32(sp + ro, out[k][0]);
+          tc::st_shared_b32(sp + ro + 16u, out[k][1]);
+        }
         tc::fence_proxy_async_smem();
-        tc::named_bar_sync(4 + half, 128);
-        if (issuer) {
-          for (int t = 0; t < nblk; ++t) tc::tma_store_3d(&tm.y, n, (int)row0, bp + t, sp + 4096u * (uint32_t)t);
+        __syncwarp();
+        if (lane == 0) {
+          tc::tma_store_3d(&tm.y, n, row_w, b, sp);
           tc::bulk_commit();
           pending = true;
         }
       }
+      if (pass + 1 < passes) {
+        tc::named_bar_sync(1, EPI_THREADS);                 // this pass's buffer is free
+        if (etid == 0 && ok) load(pass + 2, cur);
+        cur ^= 1;
+      }
     }
   }
-  return true;
+  if (!ok && etid == 0) tc::pause_ns(2000000ull);
+  return ok;
 }
 
 // Compensated fp32 sum of squares: d^2 = p + e exactly (p = fp32(d d), e = fma(d, d, -p));
@@ -1197,7 +1264,7 @@ pair_tc2_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
     const uint32_t tmem_empty_leader1 = tc2::map_to(tc::smem_u32(&ss->tmem_empty[1]), 0);
     int local = 0;
     bool pending = false;                   // staged output: this thread has bulk stores in flight
-    uint32_t tphase = 0;                    // fused loss: parity of this warpgroup's next target load
+    uint32_t tphase = 0;                    // fused loss: parity of this warpgroup's next target load; q queries: of buffer i's tables in bit i
     CompSum lacc[2];                        // fused loss: running sums of the + and - rows
     bool aborted = false;
     WorkUnit u;
@@ -1234,7 +1301,7 @@ pair_tc2_kernel(const __grid_constant__ TmaSet tm, const Params prm) {
                                               acc_phase, t_row, abort_flag, pending);
       else if constexpr (SMODE == STAGE_MULTI4)
         ok = epi_multi4_staged<TO, RT, MODE>(prm, tm, ss, tbl, etid, half, quad, lane, row0, n_blk, bn, buf,
-                                             acc_phase, t_row, abort_flag, pending);
+                                             acc_phase, t_row, abort_flag, pending, tphase);
       else if constexpr (SMODE == STAGE_LOSS)
         ok = epi_loss_staged<TO>(prm, tm, ss, reinterpret_cast<uint8_t*>(tbl), etid, half, row_in_tile, row0, n_blk,
                                  bn, buf, acc_phase, t_row, abort_flag, tphase, lacc);

@@ -81,6 +81,7 @@ enum Mode { MODE_PAIR = 0, MODE_GATED = 1, MODE_PLAIN = 2 };
 // all: the loss pair of the rounded outputs, fused (zoact_pair_forward_loss).
 enum StageMode { STAGE_NONE = 0, STAGE_ALL = 1, STAGE_MIRROR = 2, STAGE_MIRROR4 = 3, STAGE_MULTI4 = 4,
                  STAGE_LOSS = 5 };
+constexpr int MULTI4_ROWS = 32;   // rows of a bulk store of STAGE_MULTI4: a warp's
 
 struct TmaSet {
   CUtensorMap a, b, b2, aa, ba, ba2;
@@ -113,10 +114,11 @@ struct Params {
   int aug_kb_slot;   // K-blocks of one slot (B_aug row width / 64)
   int aug_slots;     // LOWRANK_ALL_ON_TC: 1, or S when a tile spans up to S evaluation blocks (slot = block mod S)
   int64_t aug_block_rows;   // rows of one block's table in B_aug (LOWRANK_ALL_ON_TC)
-  // LOWRANK_C_ON_TC: Z of each distinct query, transposed [q][r][d_out] (gate / up), and the table of each block
+  // LOWRANK_C_ON_TC: Z of each distinct query (gate / up), transposed [q][r][d_out] or, with STAGE_MULTI4, in operand
+  // order (z_chunk_words), and the table of each block
   const float* Zt;
   const float* Zt2;
-  int64_t zt_qstride;       // floats per query table (r * d_out)
+  int64_t zt_qstride;       // words per query table
   int zq[ZOACT_MAX_EVAL_BLOCKS];   // block b's table in Zt (-1: coefficient 0)
   int64_t ldy;       // plain mode: row stride of D
   int vec_ok;        // C, C2, P, P2 and ldy allow 16-byte vector access
@@ -292,6 +294,28 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
   return d;
 }
+__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\t"
+      "mov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\t"
+      "mov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 fmul2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\t"
+      "mov.b64 rb, {%4, %5};\n\t"
+      "mul.rn.f32x2 rd, ra, rb;\n\t"
+      "mov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 
 // Low-rank sums of CW consecutive table columns for one token row:
 //   s[i] = sum_j tb[j * stride + c + i] p[j]     (j ascending).
@@ -316,7 +340,19 @@ __device__ __forceinline__ void lowrank_t(const float* tb, int stride, int c, co
   for (int i = 0; i < CW / 2; ++i) { s[2 * i] = acc[i].x; s[2 * i + 1] = acc[i].y; }
 }
 
-__device__ __forceinline__ float silu_fast(float x) { return __fdividef(x, 1.0f + __expf(-x)); }
+// x / (1 + 2^(-x log2 e)) by the special-function unit's 2^t and 1/t.  Both flush subnormals, which are lost in 1 + e
+// and below any 16-bit output; without the flush their range scaling doubles the instructions.
+__device__ __forceinline__ float exp2_sfu(float t) {
+  float e;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
+  return e;
+}
+__device__ __forceinline__ float rcp_sfu(float t) {
+  float e;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(t));
+  return e;
+}
+__device__ __forceinline__ float silu_fast(float x) { return x * rcp_sfu(1.0f + exp2_sfu(x * -1.44269504f)); }
 
 __device__ __forceinline__ uint32_t pack2(float a, float b, __nv_bfloat16*) {
   __nv_bfloat162 h = __floats2bfloat162_rn(a, b);

@@ -24,6 +24,12 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
+__device__ __forceinline__ void pause_ns(uint64_t ns) {
+  const uint64_t t0 = global_timer_ns();
+  while (global_timer_ns() - t0 < ns) {
+  }
+}
+
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -209,29 +215,39 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 // Four rows x four columns per thread from 32 TMEM lanes (two 16x256b.x2 loads at lanes +0
 // and +16 of taddr, one wait): thread t holds rows t/4 + 8k (k = 0..3) and columns
 // (2(t%4), 2(t%4)+1, 8+2(t%4), 9+2(t%4)) of the 16 at taddr, as v[4k + i].
-__device__ __forceinline__ void tmem_ld_rows4(uint32_t taddr, float* v) {
-  uint32_t a[8], b[8];
+__device__ __forceinline__ void tmem_ld_rows4_issue(uint32_t taddr, uint32_t* a) {
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7])
                : "r"(taddr)
                : "memory");
   asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
+               : "=r"(a[8]), "=r"(a[9]), "=r"(a[10]), "=r"(a[11]), "=r"(a[12]), "=r"(a[13]), "=r"(a[14]), "=r"(a[15])
                : "r"(taddr + (16u << 16))
                : "memory");
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+// The values of tmem_ld_rows4_issue, which pass through the wait so that nothing reads them before it.
+__device__ __forceinline__ void tmem_ld_rows4_wait(uint32_t* a, float* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(a[0]), "+r"(a[1]), "+r"(a[2]), "+r"(a[3]), "+r"(a[4]), "+r"(a[5]), "+r"(a[6]), "+r"(a[7]),
+                 "+r"(a[8]), "+r"(a[9]), "+r"(a[10]), "+r"(a[11]), "+r"(a[12]), "+r"(a[13]), "+r"(a[14]), "+r"(a[15])
+               :
+               : "memory");
   // registers of one load: {0,1,4,5} = first row's columns, {2,3,6,7} = the row 8 lanes down
-  const uint32_t* src[2] = {a, b};
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-      v[8 * h + 4 * k + 0] = __uint_as_float(src[h][2 * k + 0]);
-      v[8 * h + 4 * k + 1] = __uint_as_float(src[h][2 * k + 1]);
-      v[8 * h + 4 * k + 2] = __uint_as_float(src[h][2 * k + 4]);
-      v[8 * h + 4 * k + 3] = __uint_as_float(src[h][2 * k + 5]);
+      v[8 * h + 4 * k + 0] = __uint_as_float(a[8 * h + 2 * k + 0]);
+      v[8 * h + 4 * k + 1] = __uint_as_float(a[8 * h + 2 * k + 1]);
+      v[8 * h + 4 * k + 2] = __uint_as_float(a[8 * h + 2 * k + 4]);
+      v[8 * h + 4 * k + 3] = __uint_as_float(a[8 * h + 2 * k + 5]);
     }
   }
+}
+__device__ __forceinline__ void tmem_ld_rows4(uint32_t taddr, float* v) {
+  uint32_t a[16];
+  tmem_ld_rows4_issue(taddr, a);
+  tmem_ld_rows4_wait(a, v);
 }
 
 __device__ __forceinline__ void st_shared_b32(uint32_t addr, uint32_t v) {
@@ -289,6 +305,12 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int32_t x, 
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap* map, int32_t x, int32_t y, int32_t z, uint32_t src) {
   asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%1, %2, %3}], [%4];" ::"l"(map), "r"(x),
                "r"(y), "r"(z), "r"(src)
+               : "memory");
+}
+// Contiguous bytes (16-byte aligned, a multiple of 16) into this CTA's shared memory, counted on `bar`.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar)
                : "memory");
 }
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
