@@ -245,133 +245,107 @@ int loss_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, float eps
 // Losses of a multi-point evaluation (Algorithm 2, one-sided, q queries):
 //   L_b = mean((y_b - t)^2) for every block b,
 //   D_j = mean((y_j - y_0)(y_j + y_0 - 2t)) (= L_j - L_0),  a_j = D_j / mu.
-// blockIdx.y is the block b; each CTA reads y_b, y_0 and t over its share of
-// the elements (y_0 and t are re-read once per block, from L2 when they fit).
-// Partials [nb][gridDim.x][2] are added in a fixed order by the last CTA.
+// Bound by HBM and the latency of its loads.  One CTA per SM; a thread keeps its vector of y_0 and t in registers and
+// goes over the blocks, eight at a time with all their loads issued first; a block's compensated sums {s, c, s, c} lie in the thread's own slot
+// [b][thread] of shared memory.  At the end each warp adds whole sums over the threads, compensated and then in fp64,
+// and in the last CTA over the CTAs' partials [sum][CTA], both in a fixed order.  Nine blocks of 512 x 4096 bf16 with a target (42 MB): 41 us
+// with the blocks on a grid axis, y_0 and t read once for each, and a tree of barriers per block at the end;
+// 24 here (both with cold caches, as in a profile).
+constexpr int MULTI_THREADS = 512;
 template <typename TY>
-__global__ void __launch_bounds__(LOSS_THREADS, 4)
+__global__ void __launch_bounds__(MULTI_THREADS, 1)
 loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t count, int vec_ok, int nb, float mu,
                   double* __restrict__ out, double* __restrict__ partials, unsigned int* __restrict__ ticket,
                   int* __restrict__ status) {
+  extern __shared__ float4 slots[];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int b = 0; b < nb; ++b) slots[b * MULTI_THREADS + tid] = make_float4(0.f, 0.f, 0.f, 0.f);
   pdl_wait();
   pdl_trigger();
-  const int b = blockIdx.y;
-  const TY* yb = Y + (int64_t)b * count;
-  const TY* y0 = Y;
-  CSum as, ad;
+  auto add = [&](int b, float ss, float sd) {
+    float4 w = slots[b * MULTI_THREADS + tid];
+    CSum s, d;
+    s.s = w.x; s.c = w.y; d.s = w.z; d.c = w.w;
+    s.add(ss);
+    d.add(sd);
+    slots[b * MULTI_THREADS + tid] = make_float4(s.s, s.c, d.s, d.c);
+  };
   const int64_t n_vec = vec_ok ? count / 8 : 0;
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t first = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  // rounds of two vectors, all loads issued first; one compensated add per accumulator per round
-  int64_t v = first;
-  constexpr int R = sizeof(TY) == 4 ? 1 : 2;   // vectors per round (fp32 words take twice the registers)
-  for (; v + (R - 1) * stride < n_vec; v += R * stride) {
-    Raw8<TY> ry[R], rz[R], rt[R];
+  const int64_t stride = (int64_t)gridDim.x * MULTI_THREADS;
+  const int64_t first = blockIdx.x * (int64_t)MULTI_THREADS + tid;
+  constexpr int AHEAD = sizeof(TY) == 4 ? 4 : 8;     // blocks of a round, their loads issued first
+  for (int64_t v = first; v < n_vec; v += stride) {
+    const Raw8<TY> rz = ld8<TY>(Y + 8 * v);
+    const Raw8<TY> rt = tgt ? ld8<TY>(tgt + 8 * v) : Raw8<TY>{};
+    auto one = [&](int b, const Raw8<TY>& ry) {
+      float y[8], z[8], t[8], ss = 0.f, sd = 0.f;
+      unpack8<TY>(ry, y);
+      unpack8<TY>(rz, z);
+      unpack8<TY>(rt, t);
 #pragma unroll
-    for (int u = 0; u < R; ++u) {
-      ry[u] = ld8<TY>(yb + 8 * (v + u * stride));
-      if (b > 0) rz[u] = ld8<TY>(y0 + 8 * (v + u * stride));
-      if (tgt) rt[u] = ld8<TY>(tgt + 8 * (v + u * stride));
-    }
-    float ss = 0.f, sd = 0.f;
-#pragma unroll
-    for (int u = 0; u < R; ++u) {
-      float y[8], z[8], t[8];
-      unpack8<TY>(ry[u], y);
-      if (b > 0) unpack8<TY>(rz[u], z);
-      if (tgt) {
-        unpack8<TY>(rt[u], t);
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) t[i] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float dy = y[i] - t[i];
+      for (int e = 0; e < 8; ++e) {
+        const float dy = y[e] - t[e];
         ss = fmaf(dy, dy, ss);
-        if (b > 0) sd = fmaf(y[i] - z[i], dy + (z[i] - t[i]), sd);
+        sd = fmaf(y[e] - z[e], dy + (z[e] - t[e]), sd);
       }
-    }
-    as.add(ss); ad.add(sd);
-  }
-  for (; v < n_vec; v += stride) {
-    float y[8], z[8], t[8];
-    load8<TY>(yb + 8 * v, y);
-    if (b > 0) load8<TY>(y0 + 8 * v, z);
-    if (tgt) {
-      load8<TY>(tgt + 8 * v, t);
-    } else {
+      add(b, ss, sd);
+    };
+    for (int b0 = 1; b0 < nb; b0 += AHEAD) {
+      Raw8<TY> ry[AHEAD];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) t[i] = 0.f;
-    }
-    float ss = 0.f, sd = 0.f;
+      for (int i = 0; i < AHEAD; ++i)
+        if (b0 + i < nb) ry[i] = ld8<TY>(Y + (b0 + i) * count + 8 * v);
+      if (b0 == 1) one(0, rz);
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float dy = y[i] - t[i];
-      ss = fmaf(dy, dy, ss);
-      if (b > 0) sd = fmaf(y[i] - z[i], dy + (z[i] - t[i]), sd);
+      for (int i = 0; i < AHEAD; ++i)
+        if (b0 + i < nb) one(b0 + i, ry[i]);
     }
-    as.add(ss); ad.add(sd);
   }
   for (int64_t i = 8 * n_vec + first; i < count; i += stride) {
-    const float tv = tgt ? to_f32<TY>(tgt[i]) : 0.f;
-    const float yv = to_f32<TY>(yb[i]);
-    const float dy = yv - tv;
-    as.add(dy * dy);
-    if (b > 0) {
-      const float zv = to_f32<TY>(y0[i]);
-      ad.add((yv - zv) * (dy + (zv - tv)));
+    const float tv = tgt ? to_f32<TY>(tgt[i]) : 0.f, zv = to_f32<TY>(Y[i]);
+    for (int b = 0; b < nb; ++b) {
+      const float yv = to_f32<TY>(Y[b * count + i]), dy = yv - tv;
+      add(b, dy * dy, (yv - zv) * (dy + (zv - tv)));
     }
   }
-  __shared__ double red[2][LOSS_THREADS];
   __shared__ bool is_last;
-  double bs[2];
-  block_sum<2>({as.value(), ad.value()}, bs, red);
-  if (threadIdx.x == 0) {
-    const double s0 = bs[0], s1 = bs[1];
-    double* pb = partials + 2 * ((int64_t)b * gridDim.x + blockIdx.x);
-    pb[0] = s0;
-    pb[1] = s1;
-    __threadfence();
-    const unsigned int prev = atomicAdd(ticket, 1u);
-    is_last = (prev == gridDim.x * gridDim.y - 1);
+  __shared__ int bad;
+  __syncthreads();
+  for (int i = warp; i < 2 * nb; i += MULTI_THREADS / 32) {   // sum i: block i / 2, squares or differences
+    CSum w;                                    // (fp64 adds of every thread's two floats took 10 us here)
+    for (int t = lane; t < MULTI_THREADS; t += 32) {
+      const float4 x = slots[(i >> 1) * MULTI_THREADS + t];
+      w.add((i & 1) ? x.z : x.x);
+      w.c += (i & 1) ? x.w : x.y;
+    }
+    const double a = warp_sum(w.value());
+    if (lane == 0) {
+      partials[(int64_t)i * gridDim.x + blockIdx.x] = a;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    is_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    bad = 0;
   }
   __syncthreads();
   if (!is_last) return;
   __threadfence();
-  __shared__ double tree[2][LOSS_THREADS];
   const double inv = 1.0 / (double)count;
-  bool finite = true;
-  for (int bb = 0; bb < nb; ++bb) {
-    double s0 = 0.0, s1 = 0.0;
-    for (unsigned int x = threadIdx.x; x < gridDim.x; x += LOSS_THREADS) {
-      const double* pb = partials + 2 * ((int64_t)bb * gridDim.x + x);
-      s0 += __ldcg(pb);
-      s1 += __ldcg(pb + 1);
+  for (int i = warp; i < 2 * nb; i += MULTI_THREADS / 32) {
+    double a = 0.0;
+    for (unsigned int x = lane; x < gridDim.x; x += 32) a += __ldcg(partials + (int64_t)i * gridDim.x + x);
+    a = warp_sum(a) * inv;
+    if (lane == 0 && i != 1) {
+      const double o = (i & 1) ? a / (double)mu : a;
+      out[(i & 1) ? nb + (i >> 1) - 1 : i >> 1] = o;
+      if (!isfinite(o)) bad = 1;
     }
-    tree[0][threadIdx.x] = s0; tree[1][threadIdx.x] = s1;
-    __syncthreads();
-    for (int h = LOSS_THREADS / 2; h > 0; h >>= 1) {
-      if (threadIdx.x < h) {
-        tree[0][threadIdx.x] += tree[0][threadIdx.x + h];
-        tree[1][threadIdx.x] += tree[1][threadIdx.x + h];
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      const double L = tree[0][0] * inv;
-      out[bb] = L;
-      finite = finite && isfinite(L);
-      if (bb > 0) {
-        const double a = tree[1][0] * inv / (double)mu;
-        out[nb + bb - 1] = a;
-        finite = finite && isfinite(a);
-      }
-    }
-    __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    if (!finite) record_error(status, ZOACT_ERR_NONFINITE);
+  __syncthreads();
+  if (tid == 0) {
+    if (bad) record_error(status, ZOACT_ERR_NONFINITE);
     *ticket = 0u;
   }
 }
@@ -380,14 +354,15 @@ template <typename TY>
 int loss_multi_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, int nb, float mu, double* out,
                         double* partials, int max_blocks, unsigned int* ticket) {
   const int vec_ok = (count % 8 == 0) && ((uintptr_t)Y % 16 == 0) && ((uintptr_t)tgt % 16 == 0);
-  int64_t bx = ((vec_ok ? count / 8 : count) + LOSS_THREADS - 1) / LOSS_THREADS;
+  int64_t bx = ((vec_ok ? count / 8 : count) + MULTI_THREADS - 1) / MULTI_THREADS;
   if (bx < 1) bx = 1;
-  int64_t cap = max_blocks / nb;
-  if (cap < 1) cap = 1;
-  if (bx > cap) bx = cap;
-  dim3 grid((unsigned)bx, (unsigned)nb);
-  ZOACT_CUDA_TRY(launch_pdl(ctx, loss_multi_kernel<TY>, grid, dim3(LOSS_THREADS), 0, Y, tgt, count, vec_ok, nb, mu,
-                            out, partials, ticket, ctx->d_status));
+  if (bx > ctx->sm_count) bx = ctx->sm_count;
+  if (bx > max_blocks) bx = max_blocks;
+  const int smem = nb * MULTI_THREADS * (int)sizeof(float4);
+  ZOACT_CUDA_TRY(cudaFuncSetAttribute(loss_multi_kernel<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      ZOACT_MAX_EVAL_BLOCKS * MULTI_THREADS * (int)sizeof(float4)));
+  ZOACT_CUDA_TRY(launch_pdl(ctx, loss_multi_kernel<TY>, dim3((unsigned)bx), dim3(MULTI_THREADS), smem, Y, tgt, count,
+                            vec_ok, nb, mu, out, partials, ticket, ctx->d_status));
   ++ctx->n_launch;
   return ZOACT_OK;
 }

@@ -1,13 +1,13 @@
 """Several evaluation blocks on a shared input with 16-bit outputs on CTA pairs: the low-rank term of each block goes on
 the epilogue warps' matrix instruction from Z tables in operand order.  Sizes at the edges of the layout: ranks around
 the groups of eight (and ones that split a Philox group), columns that end inside a pass, rows that end inside a warp's
-32 and a CTA without rows, zero and repeated evaluation points."""
+32 and a CTA without rows, zero and repeated evaluation points.  And the losses of several blocks."""
 import numpy as np
 import pytest
 import torch
 
 import paper_2607_01125_gb300 as zo
-from oracle import layers
+from oracle import layers, loss as oloss
 from test_gpu_multi import DEV, _oracle, ctx, normal, np64  # noqa: F401  (ctx: fixture)
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +47,27 @@ def test_query_blocks_edges(ctx, gated, T, d_out, r, dt):  # noqa: F811
     # equal points give equal bits
     b = Y[:n].view(len(pts), T, d_out)
     assert torch.equal(b[0], b[3])
+
+
+@pytest.mark.parametrize("T,n,nb,dt,with_target", [(640, 1000, 7, torch.float32, False), (640, 1000, 6, torch.float32, True),
+                                                   (641, 1000, 10, torch.bfloat16, True), (1, 8, 2, torch.float16, True),
+                                                   (1, 1, 17, torch.float32, True), (997, 643, 9, torch.float16, False)])
+def test_loss_blocks_edges(ctx, T, n, nb, dt, with_target):  # noqa: F811
+    # a vector more than the grid's threads, blocks past a round's eight (four in fp32), the scalar path, one element
+    y0 = normal((T, n), 61, DEV)
+    Y = torch.cat([y0] + [y0 + 1e-2 * normal((T, n), 62 + j, DEV) for j in range(nb - 1)]).to(dt)
+    tgt = normal((T, n), 80, DEV, dtype=dt) if with_target else None
+    out = torch.full((2 * nb,), 7.0, dtype=torch.float64, device=DEV)
+    mu = 1e-3
+    for _ in range(2):                       # the ticket is back at zero
+        zo.zoact_loss_multi(ctx, Y, T, nb, mu, out, target=tgt)
+    torch.cuda.synchronize()
+    o, Yn = out.cpu().numpy(), np64(Y)
+    L, a = oloss.loss_queries(Yn, T, nb, None if tgt is None else np64(tgt), mu)
+    # fp32 differences, squares and sums of 8 a vector (10 roundings), then compensated sums
+    np.testing.assert_allclose(o[:nb], L, rtol=16 * 2.0 ** -24)
+    t = 0.0 if tgt is None else np64(tgt)
+    for j in range(1, nb):
+        scale = np.mean(np.abs((Yn[j * T:(j + 1) * T] - Yn[:T]) * (Yn[j * T:(j + 1) * T] + Yn[:T] - 2 * t))) / mu
+        assert abs(o[nb + j - 1] - a[j - 1]) <= 16 * 2.0 ** -24 * scale + 2.0 ** -50 * abs(a[j - 1])
+    assert o[-1] == 7.0
