@@ -250,53 +250,97 @@ __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restr
 // ---- LDL^T of an n x n block in shared memory (n <= KMAX), with its inverse factor ----
 // N: the upper triangle in, zeros below; out: row j of the eliminated matrix in the upper triangle (its diagonal D) and
 // L^-1 (unit lower triangle) strictly below.  One block-wide barrier a column: while the other warps apply column j to
-// the rows below, warp 0 finishes row j + 1, which it keeps in registers (two columns a lane) for its multipliers and
-// for the step after; that chain -- a load, a multiply-add, the pivot's reciprocal, a product -- is a step's length.
-// Returns false (to every thread) when a pivot is not positive.  f: 2 x KMAX doubles, bad: two ints.
+// the rows below, which they keep in registers until the row is the next but one, warp 0 finishes row j + 1 for its
+// multipliers and for the step after (one or two columns a lane).
+// A scheduler takes a warp's fp64 instruction in 68 cycles (whatever its active lanes), so a column's time is warp 0's
+// chain, 710 to 810 cycles (nine such, five in the reciprocal; warps 4, 8, ... leave it the scheduler), or the other
+// warps' row updates, 68 for each of the rows below over three schedulers, more beyond 32 columns.  With the rows in
+// shared memory (three reads and a write an element), a comparison in the chain and a check of it every column: a factor
+// of 32 columns with its inverse 23.6 us, 48 columns 43.6; 18.4 and 38.7 here.
+// Returns false (to every thread) when a pivot is not positive.  f: 2 x KMAX doubles, bad: an int.
+constexpr int LDL_ROWS = 6;                          // rows a warp may own: 64 over 12 warps, 32 over 6
 __device__ bool ldl_shared(double* N, int ld, int n, double* f, int* bad) {
-  const int lane = threadIdx.x & 31;
-  const bool wide = n > 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const bool wide = n > 32, in0 = lane < n, in1 = lane + 32 < n;
+  const int workers = warps - (warps + 3) / 4, mine = warp - 1 - warp / 4;
+  const bool worker = (warp & 3) != 0;
   double x0 = 0.0, x1 = 0.0, f0 = 0.0, f1 = 0.0;     // warp 0: row j (1 in column j) and its multipliers
+  bool fail = false;
   auto pivot = [&](int p, double a0, double a1) {    // warp 0: row p is eliminated: its multipliers
     const double d = __shfl_sync(0xffffffffu, p < 32 ? a0 : a1, p & 31);
     const double inv = 1.0 / d;
-    f0 = a0 * inv;
-    f1 = a1 * inv;
     double* fp = f + (p & 1) * KMAX;
+    f0 = a0 * inv;
     fp[lane] = f0;
-    if (wide) fp[lane + 32] = f1;
-    if (lane == 0) bad[p & 1] = !(d > 0.0);
+    if (wide) {
+      f1 = a1 * inv;
+      fp[lane + 32] = f1;
+    }
+    const long long bits = __double_as_longlong(d);  // (an fp64 comparison would be one more in the chain)
+    fail = fail || bits <= 0 || bits > 0x7ff0000000000000ll;
     x0 = lane == p ? 1.0 : a0;
     x1 = lane + 32 == p ? 1.0 : a1;
   };
-  if (threadIdx.x < 32) pivot(0, lane < n ? N[lane] : 0.0, lane + 32 < n ? N[lane + 32] : 0.0);
+  // the other warps: columns 0 .. 31 of rows mine + s workers (r0), and from 32 on (r1) as many, or where they are at most
+  // 16 those of two rows, one per half warp
+  const bool two = n <= 48;
+  const int c1 = 32 + (two ? lane & 15 : lane);
+  auto row1 = [&](int s) { return mine + (two ? 2 * s + (lane >> 4) : s) * workers; };
+  double r0[LDL_ROWS], r1[LDL_ROWS];
+#pragma unroll
+  for (int s = 0; s < LDL_ROWS; ++s) {
+    const int p = mine + s * workers, q = row1(s);
+    r0[s] = worker && p < n && in0 ? N[p * ld + lane] : 0.0;
+    r1[s] = worker && q < n && c1 < n ? N[q * ld + c1] : 0.0;
+  }
+  if (warp == 0) pivot(0, in0 ? N[lane] : 0.0, in1 ? N[lane + 32] : 0.0);
   __syncthreads();
-  const int t = (int)threadIdx.x - 32, shift = wide ? 6 : 5;
-  const int c = t & ((1 << shift) - 1), rows = ((int)blockDim.x - 32) >> shift, first = t >> shift;
-  for (int j = 0; j < n; ++j) {
-    if (bad[j & 1]) return false;
-    if (threadIdx.x < 32) {
+  for (int j = 0; j < n - 1; ++j) {
+    if (warp == 0) {
       const int p = j + 1;
-      if (p < n) {
-        double* row = N + p * ld;
-        double a0 = lane < n ? row[lane] : 0.0, a1 = lane + 32 < n ? row[lane + 32] : 0.0;
-        const double m = __shfl_sync(0xffffffffu, p < 32 ? f0 : f1, p & 31);
-        a0 = fma(-m, x0, a0);                        // (columns 0 .. j and p .. n: all of them)
+      double* row = N + p * ld;
+      double a0 = in0 ? row[lane] : 0.0, a1 = in1 ? row[lane + 32] : 0.0;
+      const double m = __shfl_sync(0xffffffffu, p < 32 ? f0 : f1, p & 31);
+      a0 = fma(-m, x0, a0);                          // (columns 0 .. j and p .. n: all of them)
+      if (in0) row[lane] = a0;
+      if (wide) {
         a1 = fma(-m, x1, a1);
-        if (lane < n) row[lane] = a0;
-        if (lane + 32 < n) row[lane + 32] = a1;
-        pivot(p, a0, a1);
+        if (in1) row[lane + 32] = a1;
       }
-    } else if (c < n && first < rows) {
-      const double x = c == j ? 1.0 : N[j * ld + c];
+      pivot(p, a0, a1);
+    } else if (worker) {
       const double* fj = f + (j & 1) * KMAX;
-#pragma unroll 4
-      for (int p = j + 2 + first; p < n; p += rows)
-        if (c <= j || c >= p) N[p * ld + c] = fma(-fj[p], x, N[p * ld + c]);
+      double m[LDL_ROWS];
+#pragma unroll
+      for (int s = 0; s < LDL_ROWS; ++s) m[s] = fj[min(mine + s * workers, KMAX - 1)];
+      const double y0 = lane == j ? 1.0 : in0 ? N[j * ld + lane] : 0.0;
+#pragma unroll
+      for (int s = 0; s < LDL_ROWS; ++s) {
+        const int p = mine + s * workers;
+        if (p > j + 1 && p < n) {                    // columns 0 .. j and from p on
+          if (lane <= j || lane >= p) r0[s] = fma(-m[s], y0, r0[s]);
+          if (p == j + 2 && in0) N[p * ld + lane] = r0[s];
+        }
+      }
+      if (wide) {
+#pragma unroll
+        for (int s = 0; s < LDL_ROWS; ++s) m[s] = fj[min(row1(s), KMAX - 1)];
+        const double y1 = c1 == j ? 1.0 : c1 < n ? N[j * ld + c1] : 0.0;
+#pragma unroll
+        for (int s = 0; s < LDL_ROWS; ++s) {
+          const int p = row1(s);
+          if (__any_sync(0xffffffffu, p > j + 1 && p < n)) {
+            if (p > j + 1 && p < n && (c1 <= j || c1 >= p)) r1[s] = fma(-m[s], y1, r1[s]);
+            if (p == j + 2 && c1 < n) N[p * ld + c1] = r1[s];
+          }
+        }
+      }
     }
     __syncthreads();
   }
-  return true;
+  if (threadIdx.x == 0) *bad = fail;
+  __syncthreads();
+  return *bad == 0;
 }
 
 // The diagonal shift of attempt 0, 1, 2, ...: none, then 1e-12 of the trace, a thousand times more each time.
@@ -309,14 +353,14 @@ constexpr int CHOL_ATTEMPTS = 4;
 
 // ---- R^-1 of the Cholesky factor S = R^T R (R upper), k <= KMAX: one block, everything in shared memory ----
 // R^-1 = L^-T D^-1/2.  Bound by a column's chain (a row's update, a division, a barrier) and the fp64 pipe; k = 48:
-// 228 us with the factor in global memory and a serial inverse per column, 44 here.
-constexpr int CHOL_THREADS = 512;
+// 228 us with the factor in global memory and a serial inverse per column, 39 here.
+constexpr int CHOL_THREADS = 512;       // (half of it to 32 columns: as many rows a warp, fewer warps at the barrier)
 constexpr int CHOL_SMEM = KMAX * (KMAX + 1) * 8;
 __global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(const double* __restrict__ S, double* __restrict__ Rinv,
                                                                 int k, int* status) {
   extern __shared__ double sm[];
   __shared__ double f[2 * KMAX], rs[KMAX], trace;
-  __shared__ int bad[2];
+  __shared__ int bad;
   pdl_wait();
   pdl_trigger();
   const int ld = k + 1;
@@ -329,20 +373,20 @@ __global__ void __launch_bounds__(CHOL_THREADS) chol_inv_kernel(const double* __
     }
     __syncthreads();
     const double shift = chol_shift(attempt, attempt ? trace : 0.0);
-    for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
+    for (int v = threadIdx.x; v < k * k; v += blockDim.x) {
       const int i = v / k, j = v % k;
       sm[i * ld + j] = j < i ? 0.0 : S[v] + (i == j ? shift : 0.0);
     }
     __syncthreads();
-    ok = ldl_shared(sm, ld, k, f, bad);
+    ok = ldl_shared(sm, ld, k, f, &bad);
   }
   if (!ok) {
     if (threadIdx.x == 0) record_error(status, ZOACT_ERR_NONFINITE);
     return;
   }
-  for (int i = threadIdx.x; i < k; i += CHOL_THREADS) rs[i] = 1.0 / sqrt(sm[i * ld + i]);
+  for (int i = threadIdx.x; i < k; i += blockDim.x) rs[i] = 1.0 / sqrt(sm[i * ld + i]);
   __syncthreads();
-  for (int v = threadIdx.x; v < k * k; v += CHOL_THREADS) {
+  for (int v = threadIdx.x; v < k * k; v += blockDim.x) {
     const int i = v / k, c = v % k;
     Rinv[v] = i > c ? 0.0 : (i == c ? 1.0 : sm[c * ld + i]) * rs[c];
   }
@@ -390,7 +434,7 @@ __device__ __forceinline__ bool grid_barrier(GridSync* sy, unsigned int target, 
 // Panels of CB columns.  Every block factors the panel's diagonal block by itself (no barrier), the panel's rows of A
 // and of M = L^-1 are multiplied by its inverse factor in 8-column strips, and after a barrier the rows below get their
 // rank-CB update in 16 x 16 tiles.  Two barriers a panel; the columns' chain (as above) is most of the time.  k = 272:
-// 5.6 ms in one block, 0.27 here.
+// 5.6 ms in one block, 0.21 here.
 constexpr int CB = 32;
 constexpr int CHOLB_THREADS = 256;
 constexpr int CHOLB_BLOCKS = 96;
@@ -407,7 +451,7 @@ struct CholBig {
 };
 __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
   __shared__ double sN[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], trace_s;
-  __shared__ int bad[2];
+  __shared__ int bad;
   __shared__ double sx[CB][17], sf[CB][17], inv_d[CB];
   const int k = w.k, tid = threadIdx.x;
   const int64_t gtid = blockIdx.x * (int64_t)CHOLB_THREADS + tid, gthreads = (int64_t)gridDim.x * CHOLB_THREADS;
@@ -442,7 +486,7 @@ __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
       for (int v = tid; v < nb * nb; v += CHOLB_THREADS)
         sN[(v / nb) * (CB + 1) + v % nb] = v % nb < v / nb ? 0.0 : __ldcg(w.A + (int64_t)(p0 + v / nb) * k + p0 + v % nb);
       __syncthreads();
-      if (!ldl_shared(sN, CB + 1, nb, f, bad)) { ok = false; break; }     // the same answer in every block
+      if (!ldl_shared(sN, CB + 1, nb, f, &bad)) { ok = false; break; }     // the same answer in every block
       if (tid < nb) inv_d[tid] = 1.0 / sN[tid * (CB + 1) + tid];
       // strips: columns p1 .. k of A, then 0 .. p0 of M, eight at a time
       const int na = k - p1, cols = na + p0;
@@ -1104,7 +1148,7 @@ int launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int64_t 
 // R^-1 (k > KMAX: and R, the shift) of S
 int launch_chol(Ctx* ctx, const Work& w, int k) {
   if (k <= KMAX) {
-    ZOACT_CUDA_TRY(launch_pdl(ctx, chol_inv_kernel, dim3(1), dim3(CHOL_THREADS), CHOL_SMEM, w.S, w.Rinv, k, ctx->d_status));
+    ZOACT_CUDA_TRY(launch_pdl(ctx, chol_inv_kernel, dim3(1), dim3(k <= 32 ? CHOL_THREADS / 2 : CHOL_THREADS), CHOL_SMEM, w.S, w.Rinv, k, ctx->d_status));
   } else {
     ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
     CholBig c{w.S, w.R, w.M, w.Rinv, w.D, w.shift, w.sync, k, ctx->d_status};
