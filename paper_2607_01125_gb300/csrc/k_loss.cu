@@ -245,17 +245,19 @@ int loss_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, float eps
 // Losses of a multi-point evaluation (Algorithm 2, one-sided, q queries):
 //   L_b = mean((y_b - t)^2) for every block b,
 //   D_j = mean((y_j - y_0)(y_j + y_0 - 2t)) (= L_j - L_0),  a_j = D_j / mu.
-// Bound by HBM and the latency of its loads.  One CTA per SM; a thread keeps its vector of y_0 and t in registers and
-// goes over the blocks, eight at a time with all their loads issued first; a block's compensated sums {s, c, s, c} lie in the thread's own slot
-// [b][thread] of shared memory.  At the end each warp adds whole sums over the threads, compensated and then in fp64,
-// and in the last CTA over the CTAs' partials [sum][CTA], both in a fixed order.  Nine blocks of 512 x 4096 bf16 with a target (42 MB): 41 us
-// with the blocks on a grid axis, y_0 and t read once for each, and a tree of barriers per block at the end;
-// 24 here (both with cold caches, as in a profile).
+// Bound by HBM and the latency of its loads.  One CTA per SM; a thread keeps its group of two vectors of y_0 and t in
+// registers and goes over the blocks, four at a time with all their loads issued first.  A group's sixteen terms are
+// added in fp32 (vectors v and v + apart), everything above in compensated sums: its rounding is a_j's, and Adam
+// amplifies a_j's last bits where v is near zero, so the groups do not depend on this kernel's grid.  A block's
+// compensated sums {s, c, s, c} lie in the thread's own slot [b][thread] of shared memory.  At the end each warp adds
+// whole sums over the threads, compensated and then in fp64, and in the last CTA over the CTAs' partials [sum][CTA], both
+// in a fixed order.  Nine blocks of 512 x 4096 bf16 (42 MB): 41 us with the blocks on a grid axis, y_0 and t read once for
+// each, and a tree of barriers per block at the end; 24 here (both with cold caches, as in a profile).
 constexpr int MULTI_THREADS = 512;
 template <typename TY>
 __global__ void __launch_bounds__(MULTI_THREADS, 1)
-loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t count, int vec_ok, int nb, float mu,
-                  double* __restrict__ out, double* __restrict__ partials, unsigned int* __restrict__ ticket,
+loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t count, int vec_ok, int64_t apart, int nb,
+                  float mu, double* __restrict__ out, double* __restrict__ partials, unsigned int* __restrict__ ticket,
                   int* __restrict__ status) {
   extern __shared__ float4 slots[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -273,28 +275,47 @@ loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t 
   const int64_t n_vec = vec_ok ? count / 8 : 0;
   const int64_t stride = (int64_t)gridDim.x * MULTI_THREADS;
   const int64_t first = blockIdx.x * (int64_t)MULTI_THREADS + tid;
-  constexpr int AHEAD = sizeof(TY) == 4 ? 4 : 8;     // blocks of a round, their loads issued first
-  for (int64_t v = first; v < n_vec; v += stride) {
-    const Raw8<TY> rz = ld8<TY>(Y + 8 * v);
-    const Raw8<TY> rt = tgt ? ld8<TY>(tgt + 8 * v) : Raw8<TY>{};
-    auto one = [&](int b, const Raw8<TY>& ry) {
-      float y[8], z[8], t[8], ss = 0.f, sd = 0.f;
-      unpack8<TY>(ry, y);
-      unpack8<TY>(rz, z);
-      unpack8<TY>(rt, t);
+  constexpr int R = sizeof(TY) == 4 ? 1 : 2;         // vectors of a group (fp32 words take twice the registers)
+  constexpr int AHEAD = 4;                           // blocks of a round, their loads issued first
+  for (int64_t g = first;; g += stride) {
+    const int64_t v = R == 1 ? g : g + g / apart * apart;
+    if (v >= n_vec) break;
+    const bool two = R == 2 && v + apart < n_vec;
+    Raw8<TY> rz[R], rt[R];
 #pragma unroll
-      for (int e = 0; e < 8; ++e) {
-        const float dy = y[e] - t[e];
-        ss = fmaf(dy, dy, ss);
-        sd = fmaf(y[e] - z[e], dy + (z[e] - t[e]), sd);
+    for (int u = 0; u < R; ++u) {
+      rz[u] = rt[u] = Raw8<TY>{};
+      if (u == 0 || two) {
+        rz[u] = ld8<TY>(Y + 8 * (v + u * apart));
+        if (tgt) rt[u] = ld8<TY>(tgt + 8 * (v + u * apart));
+      }
+    }
+    auto one = [&](int b, const Raw8<TY> (&ry)[R]) {
+      float ss = 0.f, sd = 0.f;
+#pragma unroll
+      for (int u = 0; u < R; ++u) {                  // (a missing second vector adds zeros)
+        float y[8], z[8], t[8];
+        unpack8<TY>(ry[u], y);
+        unpack8<TY>(rz[u], z);
+        unpack8<TY>(rt[u], t);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const float dy = y[e] - t[e];
+          ss = fmaf(dy, dy, ss);
+          sd = fmaf(y[e] - z[e], dy + (z[e] - t[e]), sd);
+        }
       }
       add(b, ss, sd);
     };
     for (int b0 = 1; b0 < nb; b0 += AHEAD) {
-      Raw8<TY> ry[AHEAD];
+      Raw8<TY> ry[AHEAD][R];
 #pragma unroll
       for (int i = 0; i < AHEAD; ++i)
-        if (b0 + i < nb) ry[i] = ld8<TY>(Y + (b0 + i) * count + 8 * v);
+#pragma unroll
+        for (int u = 0; u < R; ++u) {
+          ry[i][u] = Raw8<TY>{};
+          if (b0 + i < nb && (u == 0 || two)) ry[i][u] = ld8<TY>(Y + (b0 + i) * count + 8 * (v + u * apart));
+        }
       if (b0 == 1) one(0, rz);
 #pragma unroll
       for (int i = 0; i < AHEAD; ++i)
@@ -358,11 +379,15 @@ int loss_multi_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, int
   if (bx < 1) bx = 1;
   if (bx > ctx->sm_count) bx = ctx->sm_count;
   if (bx > max_blocks) bx = max_blocks;
+  // (the stride of two 256-thread blocks per SM shared by the nb blocks, at most one vector a thread)
+  int64_t strides = ((vec_ok ? count / 8 : count) + 255) / 256;
+  if (strides > max_blocks / nb) strides = max_blocks / nb;
+  const int64_t apart = 256 * (strides < 1 ? 1 : strides);
   const int smem = nb * MULTI_THREADS * (int)sizeof(float4);
   ZOACT_CUDA_TRY(cudaFuncSetAttribute(loss_multi_kernel<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       ZOACT_MAX_EVAL_BLOCKS * MULTI_THREADS * (int)sizeof(float4)));
   ZOACT_CUDA_TRY(launch_pdl(ctx, loss_multi_kernel<TY>, dim3((unsigned)bx), dim3(MULTI_THREADS), smem, Y, tgt, count,
-                            vec_ok, nb, mu, out, partials, ticket, ctx->d_status));
+                            vec_ok, apart, nb, mu, out, partials, ticket, ctx->d_status));
   ++ctx->n_launch;
   return ZOACT_OK;
 }
