@@ -8,8 +8,8 @@
 //      G = X^T X formed (fp32; tcgen05 GEMM, or CUDA cores for fp32 X).
 //   2. Omega [d, k] from the Z generator (seed, layer 0, query 0), k = r + oversample.
 //   3. Q = orth(Omega); n_iter times Q = orth(G Q).  orth() is CholeskyQR2:
-//      S = Y^T Y (64 x 64 output tiles; fp32 over 32-row slabs, fp64 across
-//      slabs and row chunks), R^-1 of the Cholesky factor S = R^T R (fp64),
+//      S = Y^T Y (64 x 64 output tiles; fp32 over 32-row slabs, fp64 or two floats
+//      across slabs, fp64 across row chunks), R^-1 of the Cholesky factor S = R^T R (fp64),
 //      Q = Y R^-1; done twice for orthogonality.
 //   4. Rayleigh-Ritz: S = Q^T G Q (fp64), Jacobi (fp64): two-sided in one block's
 //      shared memory for k <= 64, one-sided on the Cholesky factor over the whole
