@@ -1,5 +1,6 @@
 // Host side of the few-row pair forward: which calls it serves, its split of the
 // work and its tensor maps.
+#include <atomic>
 #include <cstdlib>
 #include <cstring>
 
@@ -11,15 +12,35 @@ namespace pairfr {
 int dispatch_fr_bf16(Ctx* ctx, bool gated, const TmaSet& tm, const Params& p, const FrArgs& fr, int smem);
 int dispatch_fr_fp16(Ctx* ctx, bool gated, const TmaSet& tm, const Params& p, const FrArgs& fr, int smem);
 int dispatch_fr_w4(Ctx* ctx, bool gated, const TmaSet& tm, const Params& p, const FrArgs& fr, int smem);
+int fr_max_clusters(int size, int smem);
 }  // namespace pairfr
 
 namespace {
 
 constexpr int SM_SMEM = 228 * 1024;            // shared memory of an SM, 1 KB of it reserved per CTA
-constexpr int CTA_SMEM = 232448;               // most that one CTA may use
+using pairfr::CTA_SMEM;
 constexpr int FR_TOK = 256;                    // most accumulator columns (the MMA's N)
 
 int64_t round16(int64_t v) { return (v + 15) / 16 * 16; }
+
+// Clusters of `size` CTAs that the device runs at once, per_sm (1 or 2) CTAs on an SM: what it answers for one CTA per SM
+// (asked once per device); two per SM fit twice as many, or a cluster takes half its SMs.
+int64_t clusters_at_once(const Ctx* ctx, int size, int per_sm) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[DEVICES][pairfr::MAX_SPLITS + 1];
+  auto one = [&](int n) {
+    const bool keep = ctx->device >= 0 && ctx->device < DEVICES;
+    int v = keep ? known[ctx->device][n].load(std::memory_order_relaxed) : 0;
+    if (v == 0) {
+      v = pairfr::fr_max_clusters(n, SM_SMEM / 2 + 1024);
+      if (keep) known[ctx->device][n].store(v, std::memory_order_relaxed);
+    }
+    return (int64_t)v;
+  };
+  if (per_sm == 1) return one(size);
+  const int64_t twice = 2 * one(size), half = one((size + 1) / 2);
+  return twice > half ? twice : half;
+}
 
 }  // namespace
 
@@ -112,9 +133,14 @@ int launch_pair_fr(Ctx* ctx, const PairArgs& a) {
   // K ranges: as many as fill the chip's CTA slots once, each at least four K-blocks, at most a portable cluster.  More
   // would add waves, whose prologues and epilogues nothing hides (4096 -> 14336 gated, 128 rows: 59 us a call with one
   // range per tile, 81 with two, 93 with four; 14336 -> 4096, 32 rows: 50 with two, 34 with four, 33 with eight).
+  // A cluster lies within a GPC, so fewer than slots / S clusters of S run at once, and those left over are a second
+  // wave: fp16 5120 -> 5120, 64 rows (40 tiles) takes 30.2 us with 7 ranges, 20.8 with 6; INT4 4096 -> 5120, 48 rows
+  // 34.0 and 24.3; gated 4096 -> 2560, 80 rows (20 tiles) 33.7 and 21.0.
   int64_t splits = (int64_t)per_sm * ctx->sm_count / tiles;
   if (splits > p.num_k / 4) splits = p.num_k / 4;
-  fr.splits = (int)(splits < 1 ? 1 : splits > MAX_SPLITS ? MAX_SPLITS : splits);
+  if (splits > MAX_SPLITS) splits = MAX_SPLITS;
+  while (splits > 1 && tiles > clusters_at_once(ctx, (int)splits, per_sm)) --splits;
+  fr.splits = (int)(splits < 1 ? 1 : splits);
 
   st = timing_begin(ctx);
   if (st) return st;

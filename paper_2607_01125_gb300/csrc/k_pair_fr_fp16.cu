@@ -7,7 +7,8 @@ namespace pairfr {
 template <bool GATED>
 static int launch_one(Ctx* ctx, const TmaSet& tm, const Params& p, const FrArgs& fr, int smem) {
   auto kern = pair_fr_kernel<__half, GATED, false>;
-  ZOACT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  // (the most a plan may take: another thread's call never lowers it between this and the launch)
+  ZOACT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, CTA_SMEM));
   const unsigned tiles = (unsigned)((p.d_out + WR - 1) / WR);
   ZOACT_CUDA_TRY(launch_pdl_cluster(ctx, kern, dim3(tiles * fr.splits), dim3(fr_threads(false)), (size_t)smem,
                                     (unsigned)fr.splits, tm, p, fr));

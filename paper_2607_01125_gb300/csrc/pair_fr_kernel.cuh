@@ -60,6 +60,7 @@ constexpr int FR_BARS = 512;                   // shared-memory bytes kept for F
 constexpr int LR_RANKS = 8;                    // ranks per low-rank K-block (six products each: 48 of 64 columns)
 constexpr int LR_AT = 4;                       // K-blocks of W that a CTA takes ahead of its low-rank ones
 constexpr int MAX_SPLITS = 8;                  // a portable cluster
+constexpr int CTA_SMEM = 232448;               // most shared memory that one CTA may use
 __host__ __device__ constexpr int fr_threads(bool w4) { return 64 + WORK_THREADS + (w4 ? 32 : 0); }
 
 struct FrArgs {

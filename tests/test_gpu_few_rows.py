@@ -60,6 +60,7 @@ def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4):
     ("bf16", 64, 8, 1, 1, False, 2, False),         # one K-block, two rows, eight outputs
     ("bf16", 1000, 520, 37, 5, False, 2, False),    # ragged K and N tiles, rank 5
     ("bf16", 4096, 1024, 16, 16, False, 2, False),  # eight K ranges; 32 rows
+    ("fp16", 1792, 5120, 33, 16, False, 2, False),  # six: seven would fill the CTA slots, but not as clusters at once
     ("fp16", 2048, 136, 127, 32, False, 2, False),  # 254 rows
     ("bf16", 8200, 256, 17, 16, True, 2, False),    # shared input, K ending inside a block
     ("fp16", 512, 264, 255, 8, True, 2, False),     # the most rows
