@@ -161,15 +161,20 @@ __device__ __forceinline__ void write_z_operands(const AugBlocks& blk, int d_out
   }
 }
 
+// Z's tables, transposed or (OPS; a kernel of its own, the others need fewer registers) in operand order.
+template <bool OPS>
 __device__ __forceinline__ void write_z(int z_rt, const AugBlocks& blk, int d_out, int r, uint64_t seed, uint32_t lid,
                                         uint32_t lid2, float* __restrict__ Zt, float* __restrict__ Zt2) {
   if (!Zt || blk.nzq == 0) return;
-  uint32_t* z1 = reinterpret_cast<uint32_t*>(Zt);
-  uint32_t* z2 = reinterpret_cast<uint32_t*>(Zt2);
-  if (z_rt == 0) write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
-  else if (z_rt <= 8) write_z_operands<1>(blk, d_out, r, seed, lid, lid2, z1, z2);
-  else if (z_rt == 16) write_z_operands<2>(blk, d_out, r, seed, lid, lid2, z1, z2);
-  else write_z_operands<4>(blk, d_out, r, seed, lid, lid2, z1, z2);
+  if constexpr (OPS) {
+    uint32_t* z1 = reinterpret_cast<uint32_t*>(Zt);
+    uint32_t* z2 = reinterpret_cast<uint32_t*>(Zt2);
+    if (z_rt <= 8) write_z_operands<1>(blk, d_out, r, seed, lid, lid2, z1, z2);
+    else if (z_rt == 16) write_z_operands<2>(blk, d_out, r, seed, lid, lid2, z1, z2);
+    else write_z_operands<4>(blk, d_out, r, seed, lid, lid2, z1, z2);
+  } else {
+    write_z_tables(blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  }
 }
 
 // Any rank (the quad kernel below serves ranks that are multiples of 4 with 16-byte aligned sources): one thread per
@@ -177,6 +182,7 @@ __device__ __forceinline__ void write_z(int z_rt, const AugBlocks& blk, int d_ou
 // then those of B_aug2.  Each column k of a row maps to (slot, half, part, rank j); the chunk is built from the source
 // values it needs (P or P2 for A rows, T = C + c_b Z_b for B rows; source rows are re-read from L1/L2 by the row's
 // chunks).
+template <bool OPS>
 __global__ void __launch_bounds__(256)
 aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const float* __restrict__ C,
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
@@ -261,7 +267,7 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
     const int64_t row_w = 8 * (int64_t)(is_a ? cA : cB);
     *reinterpret_cast<uint4*>(dst + orow * row_w + 8 * c) = make_uint4(w[0], w[1], w[2], w[3]);
   }
-  write_z(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  write_z<OPS>(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 // The same tables for ranks that are multiples of 4 with aligned sources: one thread per four ranks of a row, which
@@ -269,7 +275,7 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
 // two signs), both of them -- and writes 8 bytes to each part and its share of the row's zeros.  A chunk per thread drew
 // every Z three times: 20480 x 32, two signs, 666 rows 20.3 us there, 6.0 here; gated 14336 x 16, two signs, 8192
 // rows 15.6 and 5.6.  I: 32-bit item indexes where they fit.
-template <typename I>
+template <typename I, bool OPS>
 __global__ void __launch_bounds__(256)
 aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const float* __restrict__ C,
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
@@ -345,7 +351,7 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
       }
     }
   }
-  write_z(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
+  write_z<OPS>(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
@@ -382,7 +388,7 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   bool quad = a.r % 4 == 0 && aligned16_or_null(a.P) && aligned16_or_null(distinct ? a.P2 : nullptr) &&
               aligned16_or_null(a.C) && aligned16_or_null(a.C2);
   for (int g = 0; g < blk.nseg; ++g) quad = quad && aligned16_or_null(a.seg_C[g]);
-  auto kern = aug_prep_kernel;
+  auto kern = z_rt ? aug_prep_kernel<true> : aug_prep_kernel<false>;
   if (quad) {
     const int64_t q_items = a.rows * ((distinct ? 2 : 1) * (a.r / 4)) +
                             (B_aug2 ? 2 : 1) * ((nbB + 1) / 2) * a.d_out * (int64_t)(a.r / 4);
@@ -391,7 +397,9 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     // (a grid-stride step past the last item must fit too)
-    kern = q_items + grid * 256 < ((int64_t)1 << 31) ? aug_quad_kernel<uint32_t> : aug_quad_kernel<int64_t>;
+    const bool narrow = q_items + grid * 256 < ((int64_t)1 << 31);
+    kern = z_rt ? (narrow ? aug_quad_kernel<uint32_t, true> : aug_quad_kernel<int64_t, true>)
+                : (narrow ? aug_quad_kernel<uint32_t, false> : aug_quad_kernel<int64_t, false>);
   }
   ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)grid), dim3(256), 0, a.P, distinct ? a.P2 : nullptr, a.C,
                             a.C2, static_cast<__nv_bfloat16*>(A_aug), static_cast<__nv_bfloat16*>(B_aug),
