@@ -791,6 +791,13 @@ __device__ __forceinline__ void jacobi_angle(double d, double apq, double& c, do
   c = fma(y, rr * fma(0.375, rr, 0.5), y);
   s = td * c;
 }
+// Integers in the order of fp64 values: -0 equals 0, a NaN comes below all others.  With ties broken by index, ranks by
+// these keys are a permutation whatever the values (comparisons of a NaN would give several columns one rank).
+__device__ __forceinline__ long long order_key(double x) {
+  const long long b = __double_as_longlong(x), mag = b & 0x7fffffffffffffffll;
+  if (mag > 0x7ff0000000000000ll) return -0x7fffffffffffffffll - 1;
+  return b < 0 ? -mag : mag;
+}
 __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __restrict__ S, double2* __restrict__ log,
                                                              int* __restrict__ n_rounds, double* __restrict__ evals,
                                                              int* __restrict__ order, int k) {
@@ -864,10 +871,11 @@ __global__ void __launch_bounds__(JAC_THREADS) jacobi_kernel(const double* __res
   if (tid == 0) *n_rounds = rounds;
   for (int i = tid; i < k; i += JAC_THREADS) {       // descending; first index first on ties
     const double e = A[i * ld + i];
+    const long long key = order_key(e);
     int rank = 0;
     for (int j = 0; j < k; ++j) {
-      const double f = A[j * ld + j];
-      if (f > e || (f == e && j < i)) ++rank;
+      const long long f = order_key(A[j * ld + j]);
+      if (f > key || (f == key && j < i)) ++rank;
     }
     order[rank] = i;
     evals[rank] = e;
@@ -1043,7 +1051,11 @@ __global__ void __launch_bounds__(HJ_THREADS) hj_vectors_kernel(const double* __
   if (threadIdx.x == 0) rank = 0;
   __syncthreads();
   int above = 0;
-  for (int j = threadIdx.x; j < k; j += HJ_THREADS) above += raw[j] > e || (raw[j] == e && j < c);
+  const long long key = order_key(e);
+  for (int j = threadIdx.x; j < k; j += HJ_THREADS) {
+    const long long f = order_key(raw[j]);
+    above += f > key || (f == key && j < c);
+  }
   if (above) atomicAdd(&rank, above);
   __syncthreads();
   const double inv = e > 0.0 ? 1.0 / sqrt(e) : 0.0;

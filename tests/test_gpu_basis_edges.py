@@ -70,3 +70,25 @@ def test_basis_fp16_scales(ctx, scale):
     assert ctx.device_status() == 0 and bool(torch.isfinite(X).all())
     ref, _ = basis.subspace_iteration(basis.gram(X.double().cpu().numpy()), 8, 16, 8, 2)
     np.testing.assert_allclose(U.double().cpu().numpy(), ref, atol=1e-4)
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16, torch.float16])
+@pytest.mark.parametrize("n,d,r,over", [(300, 256, 8, 16),       # k = 24
+                                        (300, 256, 1, 0),        # k = 1
+                                        (300, 256, 64, 15),      # k = 79: chip-wide
+                                        (2100, 256, 8, 33)])     # a Gram matrix in every type, k = 41
+def test_basis_nonfinite_tokens(ctx, n, d, r, over, dtype, bad):
+    # one bad element: no finite entry in any column, the status says so, and the context stays usable
+    X = _tokens(n, d, 128, dtype, 5)
+    X[7, 11] = bad
+    U = torch.zeros(d, r, device=DEV)
+    ev = torch.zeros(r + over, device=DEV)
+    zo.zoact_basis_init(ctx, X, r, U, oversample=over, n_iter=2, seed=3, evals_out=ev)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == -4
+    assert not bool(torch.isfinite(U).any())
+    X[7, 11] = 0.0
+    zo.zoact_basis_init(ctx, X, r, U, oversample=over, n_iter=2, seed=3, evals_out=ev)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0 and bool(torch.isfinite(U).all()) and bool(torch.isfinite(ev).all())
