@@ -600,23 +600,30 @@ __device__ __forceinline__ bool epi_multi4_staged(const Params& prm, const TmaSe
   const uint32_t* const tw = reinterpret_cast<const uint32_t*>(tbl);
   const int ncol = min(ncol_tile, prm.d_out - n_blk * ncol_tile);   // (the tables end with the 64 columns d_out lies in)
   const int passes = (ncol + SLOTS - 1) / SLOTS * prm.nb;
+  uint32_t sent = 0, sent_phase = 0;                        // the loading thread's buffers, and the parity of their last load
   auto load = [&](int pass, int bufi) {                     // one thread: pass's tables into a buffer
     if (pass >= passes) return;
     const int s = pass / prm.nb, b = pass - s * prm.nb;
     if (prm.coef[b] == 0.f) return;
     const int64_t at = prm.zq[b] * prm.zt_qstride + (int64_t)((n_blk * ncol_tile + s * SLOTS) / 16) * CHUNK;
     const uint32_t bar = tc::smem_u32(&ss->tload[bufi]), dst = tc::smem_u32(tbl + bufi * BSZ);
+    sent |= 1u << bufi;
+    sent_phase = (sent_phase & ~(1u << bufi)) | (tphase & (1u << bufi));
     tc::mbar_arrive_expect_tx(bar, BSZ * 4);
     tc::bulk_load(dst, prm.Zt + at, TSZ * 4, bar);
     if (GATED) tc::bulk_load(dst + TSZ * 4, prm.Zt2 + at, TSZ * 4, bar);
+  };
+  auto drain = [&] {                                        // the loads in flight land before the block gives up
+    for (int i = 0; i < 2; ++i)
+      if (sent >> i & 1u) tc::mbar_wait_drain(tc::smem_u32(&ss->tload[i]), (sent_phase >> i) & 1u, 100000000ull);
   };
   if (etid == 0) {                                          // (the previous tile's last barrier freed both buffers)
     load(0, 0);
     load(1, 1);
   }
   bool ok = epi_wait_full(ss, buf, acc_phase, abort_flag, prm.status, etid);
-  if (!ok) {                                                // the loads in flight land before the block gives up
-    if (etid == 0) tc::pause_ns(2000000ull);
+  if (!ok) {
+    if (etid == 0) drain();
     return false;
   }
   int cur = 0, pass = 0;
@@ -717,7 +724,9 @@ __device__ __forceinline__ bool epi_multi4_staged(const Params& prm, const TmaSe
       }
     }
   }
-  if (!ok && etid == 0) tc::pause_ns(2000000ull);
+  // one answer for all threads, each of which waited for the tables by itself: the caller's barriers are met by all or none
+  ok = tc::named_bar_and(1, EPI_THREADS, ok);
+  if (!ok && etid == 0) drain();
   return ok;
 }
 

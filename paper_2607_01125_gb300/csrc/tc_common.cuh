@@ -24,12 +24,6 @@ __device__ __forceinline__ uint64_t global_timer_ns() {
   return t;
 }
 
-__device__ __forceinline__ void pause_ns(uint64_t ns) {
-  const uint64_t t0 = global_timer_ns();
-  while (global_timer_ns() - t0 < ns) {
-  }
-}
-
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
@@ -291,6 +285,21 @@ __host__ __device__ constexpr uint32_t idesc_f16(int M, int N, int ab_bf16) {
 
 __device__ __forceinline__ void named_bar_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
+}
+
+// named_bar_sync whose `count` threads all learn whether v held for every one of them.
+__device__ __forceinline__ bool named_bar_and(int id, int count, bool v) {
+  uint32_t all;
+  __syncwarp();
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %3, 0;\n\t"
+      "bar.red.and.pred p, %1, %2, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(all)
+      : "r"(id), "r"(count), "r"((uint32_t)v)
+      : "memory");
+  return all != 0;
 }
 
 // ---- bulk stores from shared memory (output staging) ----
