@@ -224,27 +224,40 @@ __global__ void __launch_bounds__(256) atb_partial_kernel(const float* __restric
     }
 }
 
-// S = the chunks' partials, eight strided slices of them per output added last; sym: the upper triangle, mirrored.
+// S = the chunks' partials, eight strided slices of them per output added last; SYM: the upper triangle, mirrored; else
+// (S + S^T) / 2, which the two roundings of Q^T (G Q) leave a little apart.
+template <bool SYM>
 __global__ void __launch_bounds__(256) sum_partials_kernel(const double* __restrict__ part, double* __restrict__ S,
-                                                           int nchunk, int k, int sym) {
-  __shared__ double red[8][32];
+                                                           int nchunk, int k) {
+  __shared__ double red[SYM ? 1 : 2][8][32];
   pdl_wait();
   pdl_trigger();
   const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
   const int o = blockIdx.x * 32 + lane, kk = k * k;
   const int i = o / k, j = o - i * k;
-  const bool live = o < kk && !(sym && i > j);
-  double s = 0.0;
+  const bool live = o < kk && !(SYM && i > j);
+  double s = 0.0, t = 0.0;
   if (live)
 #pragma unroll 4
     for (int b = slice; b < nchunk; b += 8) s += part[(int64_t)b * kk + o];
-  red[slice][lane] = s;
+  red[0][slice][lane] = s;
+  if constexpr (!SYM) {
+    if (live)
+#pragma unroll 4
+      for (int b = slice; b < nchunk; b += 8) t += part[(int64_t)b * kk + j * k + i];
+    red[1][slice][lane] = t;
+  }
   __syncthreads();
   if (slice != 0 || !live) return;
 #pragma unroll
-  for (int w = 1; w < 8; ++w) s += red[w][lane];
-  S[o] = s;
-  if (sym) S[j * k + i] = s;
+  for (int w = 1; w < 8; ++w) s += red[0][w][lane];
+  if constexpr (SYM) {
+    S[o] = S[j * k + i] = s;
+  } else {
+#pragma unroll
+    for (int w = 1; w < 8; ++w) t += red[1][w][lane];
+    S[o] = 0.5 * (s + t);
+  }
 }
 
 // ---- LDL^T of an n x n block in shared memory (n <= KMAX), with its inverse factor ----
@@ -447,32 +460,45 @@ struct CholBig {
   double* shift;      // the shift taken
   GridSync* sync;
   int k;
+  int any;            // S need not be positive: where those shifts fail, one that no symmetric matrix outweighs
   int* status;
 };
 __global__ void __launch_bounds__(CHOLB_THREADS) chol_big_kernel(CholBig w) {
-  __shared__ double sN[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], trace_s;
+  __shared__ double sN[CB * (CB + 1)], f[2 * KMAX], red[CHOLB_THREADS / 32], sum_s;
   __shared__ int bad;
   __shared__ double sx[CB][17], sf[CB][17], inv_d[CB];
   const int k = w.k, tid = threadIdx.x;
   const int64_t gtid = blockIdx.x * (int64_t)CHOLB_THREADS + tid, gthreads = (int64_t)gridDim.x * CHOLB_THREADS;
   unsigned int target = 0;
   auto sync = [&]() { target += gridDim.x; return grid_barrier(w.sync, target, w.status); };
-  // the trace, the same sum in every block
+  // the sum of the threads' values, the same in every block
+  auto block_sum = [&](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((tid & 31) == 0) red[tid >> 5] = v;
+    __syncthreads();
+    if (tid == 0) {
+      sum_s = 0.0;
+      for (int i = 0; i < CHOLB_THREADS / 32; ++i) sum_s += red[i];
+    }
+    __syncthreads();
+    return sum_s;
+  };
   double tr = 0.0;
   for (int i = tid; i < k; i += CHOLB_THREADS) tr += w.S[(int64_t)i * k + i];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
-  if ((tid & 31) == 0) red[tid >> 5] = tr;
-  __syncthreads();
-  if (tid == 0) {
-    trace_s = 0.0;
-    for (int i = 0; i < CHOLB_THREADS / 32; ++i) trace_s += red[i];
-  }
-  __syncthreads();
+  const double trace = block_sum(tr);
   bool ok = false;
   double shift = 0.0;
-  for (int attempt = 0; attempt < CHOL_ATTEMPTS && !ok; ++attempt) {
-    shift = chol_shift(attempt, trace_s);
+  for (int attempt = 0; attempt < CHOL_ATTEMPTS + w.any && !ok; ++attempt) {
+    shift = chol_shift(attempt, trace);
+    if (attempt == CHOL_ATTEMPTS) {
+      // eigenvalues of at least |S|_F, at most three times that: as exact, relative to |S|_F, as without a shift
+      double sq = 0.0;
+      for (int64_t v = tid; v < (int64_t)k * k; v += CHOLB_THREADS) sq = fma(w.S[v], w.S[v], sq);
+      shift = 2.0 * sqrt(block_sum(sq));
+      if (shift == 0.0) shift = 1.0;
+    }
     if (attempt > 0 && !sync()) return;              // every block has seen the failed pivot before A is rewritten
     for (int64_t v = gtid; v < (int64_t)k * k; v += gthreads) {
       const int i = (int)(v / k), j = (int)(v % k);
@@ -1150,20 +1176,20 @@ int launch_atb(Ctx* ctx, const Work& w, const float* A, const float* B, int64_t 
   const int nchunk = atb_chunks(ctx, rows, k, chunk);
   ZOACT_CUDA_TRY(launch_pdl(ctx, tiles > 1 ? atb_partial_kernel<true> : atb_partial_kernel<false>, dim3(tiles, tiles, (unsigned)nchunk), dim3(256), 0, A, B, w.part, rows,
                             k, chunk, sym));
-  ZOACT_CUDA_TRY(launch_pdl(ctx, sum_partials_kernel, dim3((unsigned)((k * k + 31) / 32)), dim3(256), 0, w.part, w.S,
-                            nchunk, k, sym));
+  ZOACT_CUDA_TRY(launch_pdl(ctx, sym ? sum_partials_kernel<true> : sum_partials_kernel<false>,
+                            dim3((unsigned)((k * k + 31) / 32)), dim3(256), 0, w.part, w.S, nchunk, k));
   ctx->n_launch += 2;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
 }
 
-// R^-1 (k > KMAX: and R, the shift) of S
-int launch_chol(Ctx* ctx, const Work& w, int k) {
+// R^-1 (k > KMAX: and R, the shift; any: of any symmetric S) of S
+int launch_chol(Ctx* ctx, const Work& w, int k, int any = 0) {
   if (k <= KMAX) {
     ZOACT_CUDA_TRY(launch_pdl(ctx, chol_inv_kernel, dim3(1), dim3(k <= 32 ? CHOL_THREADS / 2 : CHOL_THREADS), CHOL_SMEM, w.S, w.Rinv, k, ctx->d_status));
   } else {
     ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
-    CholBig c{w.S, w.R, w.M, w.Rinv, w.D, w.shift, w.sync, k, ctx->d_status};
+    CholBig c{w.S, w.R, w.M, w.Rinv, w.D, w.shift, w.sync, k, any, ctx->d_status};
     void* args[] = {&c};
     const int blocks = CHOLB_BLOCKS < ctx->sm_count ? CHOLB_BLOCKS : ctx->sm_count;
     ZOACT_CUDA_TRY(cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(chol_big_kernel), dim3((unsigned)blocks),
@@ -1352,7 +1378,9 @@ int run_basis_init(Ctx* ctx, const void* X, int xdtype, int64_t n_tok, int d, in
     ZOACT_CUDA_TRY(launch_pdl(ctx, jacobi_vectors_kernel, dim3((unsigned)k), dim3(32), 0, w.log, w.ints, w.ints + 1, w.V, k));
     ctx->n_launch += 2;
   } else {
-    st = launch_chol(ctx, w, k);
+    // Q^T (G Q) of a Gram matrix has eigenvalues down to -1e-7 of its trace for a spectrum that falls quickly, and to
+    // -7e-6 for 400 K tokens of rank one (fp32 chains over the tokens)
+    st = launch_chol(ctx, w, k, 1);
     if (st) return st;
     ZOACT_CUDA_TRY(cudaMemsetAsync(w.sync, 0, sizeof(GridSync), ctx->stream));
     void* args[] = {&w.R, &w.raw, &w.sync, &k, &ctx->d_status};

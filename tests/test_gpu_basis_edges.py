@@ -23,11 +23,11 @@ def ctx():
     c.close()
 
 
-def _tokens(n, d, rank, dtype, seed, scale=1.0):
+def _tokens(n, d, rank, dtype, seed, scale=1.0, decay=0.93):
     g = torch.Generator(device=DEV).manual_seed(seed)
     B = torch.linalg.qr(torch.randn(d, rank, generator=g, device=DEV))[0].T
     A = torch.linalg.qr(torch.randn(max(n, rank), rank, generator=g, device=DEV))[0][:n]
-    s = 0.93 ** torch.arange(rank, device=DEV, dtype=torch.float32)
+    s = decay ** torch.arange(rank, device=DEV, dtype=torch.float32)
     return ((A * s) @ B * scale * (n * d) ** 0.5 / 4).to(dtype)
 
 
@@ -92,3 +92,39 @@ def test_basis_nonfinite_tokens(ctx, n, d, r, over, dtype, bad):
     zo.zoact_basis_init(ctx, X, r, U, oversample=over, n_iter=2, seed=3, evals_out=ev)
     torch.cuda.synchronize()
     assert ctx.device_status() == 0 and bool(torch.isfinite(U).all()) and bool(torch.isfinite(ev).all())
+
+
+def test_basis_fast_falling_fp32(ctx):
+    # k = 78 columns of a spectrum that is spent after ~12: Q^T (G Q) is not positive within fp32's rounding.  Column i errs
+    # by 2^-24 times its eigenvalue's distance: at i = 3, 3e-7 x 1.33 x (sigma_1 / sigma_4)^2 = 64, 3e-5
+    X = _tokens(300, 128, 128, torch.float32, 8, decay=0.5)
+    U, ev = torch.empty(128, 8, device=DEV), torch.empty(78, device=DEV)
+    zo.zoact_basis_init(ctx, X, 8, U, oversample=70, n_iter=8, seed=9, evals_out=ev)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    Un = U.double().cpu().numpy()
+    np.testing.assert_allclose(Un.T @ Un, np.eye(8), atol=1e-5)
+    ref, theta = basis.subspace_iteration(basis.gram(X.double().cpu().numpy()), 8, 70, 8, 9)
+    np.testing.assert_allclose(Un[:, :4], ref[:, :4], atol=1e-4)
+    np.testing.assert_allclose(ev.cpu().numpy()[:4], np.asarray(theta)[:4], rtol=1e-4)
+
+
+def test_basis_indefinite_gram(ctx):
+    # Rank one and many fp32 tokens: the Gram matrix's chains leave eigenvalues down to -7e-6 of its trace (a model of the
+    # chains in numpy), and the Ritz problem of the k = 78 largest in absolute value is indefinite.  An entry of G errs by
+    # sqrt(n) 2^-24 = 4e-5 of itself (a random walk), the eigenvector by 2 / sqrt(d) of that.
+    n, d, r, over = 400_000, 128, 8, 70
+    g = torch.Generator(device=DEV).manual_seed(4)
+    a = torch.rand(d, generator=g, device=DEV) + 0.5
+    X = (torch.rand(n, 1, generator=g, device=DEV) + 0.5) * a
+    U, ev = torch.empty(d, r, device=DEV), torch.empty(r + over, device=DEV)
+    zo.zoact_basis_init(ctx, X, r, U, oversample=over, n_iter=8, seed=9, evals_out=ev)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    ev = ev.double().cpu().numpy()
+    assert np.all(np.diff(ev) <= 0) and ev[-1] < 0
+    np.testing.assert_allclose(ev[0], float((X.double() ** 2).sum()), rtol=1e-3)
+    Un = U.double().cpu().numpy()
+    np.testing.assert_allclose(Un.T @ Un, np.eye(r), atol=1e-5)
+    an = a.double().cpu().numpy()
+    np.testing.assert_allclose(Un[:, 0], an / np.linalg.norm(an), atol=1e-4)
