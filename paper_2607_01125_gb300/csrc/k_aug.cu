@@ -275,13 +275,17 @@ aug_prep_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
 // two signs), both of them -- and writes 8 bytes to each part and its share of the row's zeros.  A chunk per thread drew
 // every Z three times: 20480 x 32, two signs, 666 rows 20.3 us there, 6.0 here; gated 14336 x 16, two signs, 8192
 // rows 15.6 and 5.6.  I: 32-bit item indexes where they fit.
-template <typename I, bool OPS>
-__global__ void __launch_bounds__(256)
+// ZEROS: the zeros of A's rows or of both as items of their own (zeros; see spread_zeros).  A kernel of its own: its
+// branches cost the others 1.5 us at 20480 x 32.
+constexpr int SPREAD_A = 1, SPREAD_B = 2;
+template <typename I, bool OPS, bool ZEROS>
+__global__ void __launch_bounds__(256, ZEROS ? 4 : 0)
 aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const float* __restrict__ C,
                 const float* __restrict__ C2, __nv_bfloat16* __restrict__ A, __nv_bfloat16* __restrict__ B,
                 __nv_bfloat16* __restrict__ B2, int64_t rows, int d_out, int r, int ka, int distinct, int full,
                 int nb, const __grid_constant__ AugBlocks blk, uint64_t seed, uint32_t lid, uint32_t lid2,
-                float* __restrict__ Zt, float* __restrict__ Zt2, int z_rt, int slots, int64_t T) {
+                float* __restrict__ Zt, float* __restrict__ Zt2, int z_rt, int slots, int64_t T, int zeros) {
+  const int spread = ZEROS ? zeros : 0;
   pdl_wait();                                         // P and C written by the previous kernels
   pdl_trigger();
   const int rq = r / 4, kq = ka / 4, halves = distinct ? 2 : 1;
@@ -290,8 +294,12 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
   const I itA = (I)rows * (I)(halves * rq);
   const I itB = (I)pairs * (I)d_out * (I)rq;
   const I items = itA + itB * (B2 ? 2 : 1);
+  // the zeros of A's and of B's rows as items of their own, two quads (16 bytes) each over whole rows
+  const I pa = (I)(slots * row_q / 2), pb = (I)(row_q / 2);
+  const I zA = spread & SPREAD_A ? (I)rows * pa : 0, zB = spread & SPREAD_B ? (I)nbB * (I)d_out * pb : 0;
+  const I total = items + zA + zB * (B2 ? 2 : 1);
   const uint2 zero = make_uint2(0u, 0u);
-  // one half of one slot: this quad's three parts (live), and its share of the zeros
+  // one half of one slot: this quad's three parts (live), and, unless they are spread, its share of the zeros
   auto put = [&](uint2* half_q, int g, float4 v, bool is_a, bool live) {
     if (live) {
       const uint2 hi = split_quad(v, false), lo = split_quad(v, true);
@@ -299,10 +307,11 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
       half_q[rq + g] = is_a ? hi : lo;
       half_q[2 * rq + g] = is_a ? lo : hi;
     }
+    if (spread & (is_a ? SPREAD_A : SPREAD_B)) return;
     for (int z = (live ? 3 * rq : 0) + g; z < kq; z += rq) half_q[z] = zero;
   };
   const I stride = (I)gridDim.x * blockDim.x;
-  for (I it = (I)blockIdx.x * blockDim.x + threadIdx.x; it < items; it += stride) {
+  for (I it = (I)blockIdx.x * blockDim.x + threadIdx.x; it < total; it += stride) {
     if (it < itA) {
       const I rh = it / (I)rq;
       const int g = (int)(it - rh * (I)rq);
@@ -311,8 +320,10 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
       const float4 v = *reinterpret_cast<const float4*>((h ? P2 : P) + row * r + 4 * g);
       const int mine = slots > 1 ? (int)((row / T) % slots) : 0;
       uint2* q = reinterpret_cast<uint2*>(A) + row * ((int64_t)slots * row_q) + h * kq;
-      for (int s = 0; s < slots; ++s) put(q + s * row_q, g, v, true, s == mine);
-    } else {
+      if (spread & SPREAD_A) put(q + mine * row_q, g, v, true, true);
+      else
+        for (int s = 0; s < slots; ++s) put(q + s * row_q, g, v, true, s == mine);
+    } else if (it < items) {
       I ib = it - itA;
       const bool up = ib >= itB;
       if (up) ib -= itB;
@@ -349,12 +360,37 @@ aug_quad_kernel(const float* __restrict__ P, const float* __restrict__ P2, const
         // distinct: gate rows fill the first half, up rows the second
         for (int h = 0; h < halves; ++h) put(q + h * kq, g, v, false, !distinct || h == (up ? 1 : 0));
       }
+    } else {
+      I ib = it - items;
+      const bool is_a = ib < zA;
+      if (!is_a) ib -= zA;
+      const bool up = !is_a && ib >= zB;
+      if (up) ib -= zB;
+      const I row = ib / (is_a ? pa : pb);
+      const int q0 = 2 * (int)(ib - row * (is_a ? pa : pb)), s = q0 / row_q, h = (q0 - s * row_q) / kq;
+      const int z0 = q0 - s * row_q - h * kq;         // quad of the half (kq is even)
+      const bool live = is_a ? slots == 1 || s == (int)(((int64_t)row / T) % slots) : !distinct || h == (up ? 1 : 0);
+      uint2* q = reinterpret_cast<uint2*>(is_a ? A : up ? B2 : B) + 2 * (int64_t)ib;
+      if (!live || z0 >= 3 * rq) *reinterpret_cast<uint4*>(q) = make_uint4(0u, 0u, 0u, 0u);
+      else if (z0 + 1 >= 3 * rq) q[1] = zero;
     }
   }
   write_z<OPS>(z_rt, blk, d_out, r, seed, lid, lid2, Zt, Zt2);
 }
 
 bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
+
+// Whose zeros are items of their own.  A quad's thread writes its share of them beside its three parts while these are
+// few: zero to five stores for ranks from 12 in one or two slots.  Ranks 4 and 8 have one or two threads a row, and rows
+// of several slots many zeros a thread.  Calls on 256 columns, their zeros by the quads' threads, spread, and with a thread
+// per chunk for everything: rank 4, two signs of 2048 rows on 14336 outputs 98.1, 69.4, 69.7 us; rank 8 70.2, 67.0, 69.8;
+// rank 12, 333 rows each on 256 outputs 9.4, 9.2, 9.3; 17 blocks of 14 rows (11 slots), rank 24 25.2, 23.6, 24.4.  The
+// other way: rank 16, 333 rows each on 4096 outputs (two slots) 11.1 and 11.5; B's rows, which the two threads' stores
+// fill whole, gate and up with a projection each, 17 blocks on 14336 outputs, rank 16 68.6 and 96.4.
+int spread_zeros(int slots, int row_q, int rq, int distinct) {
+  if (rq <= 2) return SPREAD_A | SPREAD_B;
+  return slots * row_q / ((distinct ? 2 : 1) * rq) - 3 > 6 ? SPREAD_A : 0;
+}
 
 }  // namespace
 
@@ -388,23 +424,35 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   bool quad = a.r % 4 == 0 && aligned16_or_null(a.P) && aligned16_or_null(distinct ? a.P2 : nullptr) &&
               aligned16_or_null(a.C) && aligned16_or_null(a.C2);
   for (int g = 0; g < blk.nseg; ++g) quad = quad && aligned16_or_null(a.seg_C[g]);
-  auto kern = z_rt ? aug_prep_kernel<true> : aug_prep_kernel<false>;
   if (quad) {
-    const int64_t q_items = a.rows * ((distinct ? 2 : 1) * (a.r / 4)) +
-                            (B_aug2 ? 2 : 1) * ((nbB + 1) / 2) * a.d_out * (int64_t)(a.r / 4);
+    const int rq = a.r / 4, row_q = ka_row / 4;
+    const int64_t itA = a.rows * ((distinct ? 2 : 1) * rq), itB = (B_aug2 ? 2 : 1) * ((nbB + 1) / 2) * a.d_out * (int64_t)rq;
+    const int spread = spread_zeros(slots, row_q, rq, distinct);
+    const int64_t q_items = itA + itB + (spread & SPREAD_A ? a.rows * (slots * row_q / 2) : 0) +
+                            (spread & SPREAD_B ? (B_aug2 ? 2 : 1) * nbB * a.d_out * (int64_t)(row_q / 2) : 0);
     const int64_t q_work = q_items > z_items ? q_items : z_items;
     grid = (q_work + 255) / 256;
     if (grid > cap) grid = cap;
     if (grid < 1) grid = 1;
     // (a grid-stride step past the last item must fit too)
     const bool narrow = q_items + grid * 256 < ((int64_t)1 << 31);
-    kern = z_rt ? (narrow ? aug_quad_kernel<uint32_t, true> : aug_quad_kernel<int64_t, true>)
-                : (narrow ? aug_quad_kernel<uint32_t, false> : aug_quad_kernel<int64_t, false>);
+    auto pick = [&](auto index) {
+      using I = decltype(index);
+      return spread ? (z_rt ? aug_quad_kernel<I, true, true> : aug_quad_kernel<I, false, true>)
+                    : (z_rt ? aug_quad_kernel<I, true, false> : aug_quad_kernel<I, false, false>);
+    };
+    auto quad_kern = narrow ? pick(uint32_t{}) : pick(int64_t{});
+    ZOACT_CUDA_TRY(launch_pdl(ctx, quad_kern, dim3((unsigned)grid), dim3(256), 0, a.P, distinct ? a.P2 : nullptr, a.C,
+                              a.C2, static_cast<__nv_bfloat16*>(A_aug), static_cast<__nv_bfloat16*>(B_aug),
+                              static_cast<__nv_bfloat16*>(B_aug2), a.rows, a.d_out, a.r, ka, distinct, full, a.nb, blk,
+                              a.seed, a.layer_id, a.layer_id2, Zt, Zt2, z_rt, slots, a.T, spread));
+  } else {
+    ZOACT_CUDA_TRY(launch_pdl(ctx, z_rt ? aug_prep_kernel<true> : aug_prep_kernel<false>, dim3((unsigned)grid), dim3(256),
+                              0, a.P, distinct ? a.P2 : nullptr, a.C, a.C2, static_cast<__nv_bfloat16*>(A_aug),
+                              static_cast<__nv_bfloat16*>(B_aug), static_cast<__nv_bfloat16*>(B_aug2), a.rows, a.d_out,
+                              a.r, ka, distinct, full, a.nb, blk, a.seed, a.layer_id, a.layer_id2, Zt, Zt2, z_rt, slots,
+                              a.T));
   }
-  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)grid), dim3(256), 0, a.P, distinct ? a.P2 : nullptr, a.C,
-                            a.C2, static_cast<__nv_bfloat16*>(A_aug), static_cast<__nv_bfloat16*>(B_aug),
-                            static_cast<__nv_bfloat16*>(B_aug2), a.rows, a.d_out, a.r, ka, distinct, full, a.nb, blk,
-                            a.seed, a.layer_id, a.layer_id2, Zt, Zt2, z_rt, slots, a.T));
   ++ctx->n_launch;
   ZOACT_CHECK_LAUNCH();
   return ZOACT_OK;
