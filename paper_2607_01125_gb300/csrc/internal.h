@@ -241,13 +241,14 @@ inline void set_pair_blocks(PairArgs& a, float eps, uint64_t query) {
 int launch_pair_simt(Ctx* ctx, const PairArgs& a);
 // INT4 g128 weight [d_out, d_in/2] + fp16 scales -> bf16 [d_out, d_in].
 int launch_dequant_int4(Ctx* ctx, const void* Wq, const void* Ws, void* Wb, int64_t d_out, int d_in);
-// Fewer rows than this take the few-row kernel (W read once, rows on the MMA's N side; INT4 dequantised in it).
+// Fewer rows than this may take the few-row kernel (W read once, rows on the MMA's N side; INT4 dequantised in it).
 constexpr int64_t FEW_ROWS = 256;
 // Row count from which an INT4 pair forward takes row scales and layer groups (the library's contract).
 constexpr int64_t INT4_ROWSCALE_MIN_ROWS = 1024;
 int launch_pair_tc(Ctx* ctx, const PairArgs& a);
-// The few-row kernel serves fewer than FEW_ROWS rows whose outputs (every block padded to 16 rows) fit one tile.
-bool pair_fr_supported(const PairArgs& a);
+// The few-row kernel can serve fewer than FEW_ROWS rows whose outputs (every block padded to 16 rows) fit one tile; it is
+// chosen where its estimated time is the smaller one.
+bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a);
 int launch_pair_fr(Ctx* ctx, const PairArgs& a);
 // Plain product D[M, N] (fp32) = A[M, K] * B[N, K]^T with 16-bit A, B (K-major), on tcgen05.
 // Low-rank term of the tensor-core pair forward (see k_aug.cu):

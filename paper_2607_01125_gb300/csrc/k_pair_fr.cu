@@ -1,6 +1,7 @@
 // Host side of the few-row pair forward: which calls it serves, its split of the
 // work and its tensor maps.
 #include <atomic>
+#include <cmath>
 #include <cstdlib>
 #include <cstring>
 
@@ -42,32 +43,19 @@ int64_t clusters_at_once(const Ctx* ctx, int size, int per_sm) {
   return twice > half ? twice : half;
 }
 
-}  // namespace
+// Tiles, stages and K ranges of a call.
+struct FrPlan {
+  pairfr::FrArgs fr;
+  int per_sm, smem;
+  int64_t tiles;
+};
 
-// Few rows: fewer than 256, and every block's rows padded to 16 within one MMA's 256 columns.  The 128-row one-CTA kernel
-// takes what is left (17 blocks of 20 rows, say).  A call (projection included) on 32 / 128 / 240 rows, this kernel
-// against that one: bf16 4096 -> 4096 16 / 21 / 32 against 33 / 36 / 37 us, bf16 gated 4096 -> 14336 52 / 59 / 70 against
-// 65 / 68 / 84, fp16 5120 -> 20480 (r = 32) 55 / 67 / 93 against 70 / 76 / 102.  INT4 14336 -> 4096 (r = 32): 41 / 48 / 66
-// against 69 / 80 / 98 with W expanded to bf16 first.
-bool pair_fr_supported(const PairArgs& a) {
-  if (a.rows <= 0 || a.nseg > 1 || a.fuse_loss || a.in_scale || a.out_sumsq) return false;
-  if (a.xdtype != ZOACT_DT_BF16 && a.xdtype != ZOACT_DT_FP16) return false;
-  if (a.T > FR_TOK || a.nb * round16(a.T) > FR_TOK || a.rows >= FEW_ROWS) return false;
-  const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
-  if (sel && std::strcmp(sel, "1cta") == 0) return false;
-  if (a.wtype == ZOACT_DT_INT4_G128) {
-    const char* isel = std::getenv("ZOACT_INT4");
-    return a.xdtype == ZOACT_DT_BF16 && !(isel && std::strcmp(isel, "staged") == 0);
-  }
-  return a.wtype == a.xdtype;
-}
-
-int launch_pair_fr(Ctx* ctx, const PairArgs& a) {
+FrPlan fr_plan(const Ctx* ctx, const PairArgs& a) {
   using namespace pairfr;
   const bool w4 = a.wtype == ZOACT_DT_INT4_G128, gated = a.W2 != nullptr;
-  if (a.ydtype != a.xdtype && a.ydtype != ZOACT_DT_FP32) return ZOACT_ERR_UNSUPPORTED;
   const int nw = gated ? 2 : 1;
-  FrArgs fr{};
+  FrPlan p{};
+  FrArgs& fr = p.fr;
   fr.tpad = (int)round16(a.T);
   fr.tok = a.nb * fr.tpad;
   fr.out32 = a.ydtype == ZOACT_DT_FP32;
@@ -75,6 +63,170 @@ int launch_pair_fr(Ctx* ctx, const PairArgs& a) {
   while (fr.tmem_cols < nw * fr.tok) fr.tmem_cols *= 2;
   fr.lr_mats = gated && a.P2 != a.P ? 2 : 1;
   fr.lr_groups = fr.lr_mats * ((a.r + LR_RANKS - 1) / LR_RANKS);
+  const int num_k = (a.d_in + BKF - 1) / BKF;
+
+  // Two CTAs per SM where their TMEM (256 columns each) and rings fit twice; a CTA that must not share an SM takes
+  // more than half of its shared memory, so that no CTA of this launch ever waits for another one's TMEM.
+  const int stage = nw * W_TILE + fr.tok * BKF * 2, raw = w4 ? nw * RAW_TILE : 0;
+  const int most = w4 ? 4 : MAX_STAGES;                 // INT4: the rest goes to the packed rows in flight
+  auto fit = [&](int budget) {
+    budget -= FR_BARS;
+    fr.stages = (budget - 4 * raw) / stage;
+    if (fr.stages > most) fr.stages = most;
+    fr.raw_slots = w4 ? (budget - fr.stages * stage) / raw / 2 * 2 : 0;   // an even number (see the kernel)
+    if (fr.raw_slots > MAX_RAW) fr.raw_slots = MAX_RAW;
+  };
+  p.per_sm = 2;
+  fit(SM_SMEM / 2 - 1024);
+  // Two stages only where one CTA per SM would leave a second wave of tiles (fp16 5120 -> 20480, 200 rows, 160 tiles:
+  // 99.0 us a call with one CTA per SM and 3 stages, 90.2 with two CTAs and 2).
+  p.tiles = (a.d_out + WR - 1) / WR;
+  const bool second_wave = p.tiles > ctx->sm_count && p.tiles <= 2 * ctx->sm_count;
+  if (fr.tmem_cols > 256 || fr.stages < (second_wave ? 2 : 3)) {
+    p.per_sm = 1;
+    fit(CTA_SMEM);                                      // at least 3 stages of at most 64 KB, and 4 packed slots of 8 KB
+  }
+  const int ring = fr.stages * stage + fr.raw_slots * raw;
+  p.smem = FR_BARS + ring;
+  if (p.per_sm == 1 && p.smem <= SM_SMEM / 2) p.smem = SM_SMEM / 2 + 1024;
+  fr.chunk = ring / (nw * WR * 4) / 16 * 16;
+  if (fr.chunk > fr.tok) fr.chunk = fr.tok;
+  // K ranges: as many as fill the chip's CTA slots once, each at least four K-blocks, at most a portable cluster.  More
+  // would add waves, whose prologues and epilogues nothing hides (4096 -> 14336 gated, 128 rows: 59 us a call with one
+  // range per tile, 81 with two, 93 with four; 14336 -> 4096, 32 rows: 50 with two, 34 with four, 33 with eight).
+  // A cluster lies within a GPC, so fewer than slots / S clusters of S run at once, and those left over are a second
+  // wave: fp16 5120 -> 5120, 64 rows (40 tiles) takes 30.2 us with 7 ranges, 20.8 with 6; INT4 4096 -> 5120, 48 rows
+  // 34.0 and 24.3; gated 4096 -> 2560, 80 rows (20 tiles) 33.7 and 21.0.
+  int64_t splits = (int64_t)p.per_sm * ctx->sm_count / p.tiles;
+  if (splits > num_k / 4) splits = num_k / 4;
+  if (splits > MAX_SPLITS) splits = MAX_SPLITS;
+  while (splits > 1 && p.tiles > clusters_at_once(ctx, (int)splits, p.per_sm)) --splits;
+  fr.splits = (int)(splits < 1 ? 1 : splits);
+  return p;
+}
+
+// Padded rows that fit one tile, and types that the kernel takes.
+bool fr_supported(const PairArgs& a) {
+  if (a.rows <= 0 || a.nseg > 1 || a.fuse_loss || a.in_scale || a.out_sumsq) return false;
+  if (a.xdtype != ZOACT_DT_BF16 && a.xdtype != ZOACT_DT_FP16) return false;
+  if (a.T > FR_TOK || a.nb * round16(a.T) > FR_TOK || a.rows >= FEW_ROWS) return false;
+  return a.wtype == ZOACT_DT_INT4_G128 ? a.xdtype == ZOACT_DT_BF16 : a.wtype == a.xdtype;
+}
+
+// The other route for few rows, one-CTA tiles of 128 rows (INT4: on W expanded to bf16), in what its time depends on.
+struct OneCta {
+  bool stacked;               // the low-rank term as K columns of stacked rows (above rank 32 a shared input is copied)
+  int64_t rows;               // of the stacked X, or of the shared one
+  int slots, ka, nw;
+  int64_t table_rows;         // of B_aug, both matrices
+};
+OneCta one_cta(const PairArgs& a) {
+  OneCta o{};
+  o.nw = a.W2 ? 2 : 1;
+  o.stacked = !a.shared || a.r > 32;
+  o.rows = o.stacked ? a.nb * a.T : a.T;
+  const int64_t span = o.stacked && a.T % 128 != 0 ? 127 / a.T + 2 : 1;
+  o.slots = (int)(span < a.nb ? span : a.nb);
+  o.ka = aug_cols(a.r) * (a.W2 && a.P2 != a.P ? 2 : 1);
+  o.table_rows = (int64_t)o.nw * (o.stacked ? a.nb : 1) * a.d_out;
+  return o;
+}
+
+// Estimates of a call's time (its projection apart) by this kernel and by the other route, in us on a GB300: sums of the
+// main loop or the read of W, whichever is longer (a fourth-power mean), the low-rank K-blocks or table elements, and the
+// epilogue, fitted to 6000 calls drawn over d_in 64 .. 20480, d_out 8 .. 20480, 2 to 17 blocks, ranks 1 .. 256, gated ones
+// (rms 8% for this kernel, 15% for the other), and to 800 without scratch.  This kernel is behind where W is small and the
+// low-rank K-blocks, 1 to 2 us each to write, or the partials of many rows are most of its work: two signs of 127 rows,
+// 512 -> 512, rank 4 25.5 us against 10.7, and nine blocks of 7 rows, 256 -> 1024 gated, rank 256 595 against 154.  It is
+// ahead on wide layers: 32 / 128 / 240 rows, projection included, bf16 4096 -> 4096 16 / 21 / 32 against 33 / 36 / 37 us,
+// gated 4096 -> 14336 52 / 59 / 70 against 65 / 68 / 84, INT4 14336 -> 4096 (r = 32) 41 / 48 / 66 against 69 / 80 / 98.
+// Of 3908 16-bit calls (2092 INT4 ones) the estimates choose a slower kernel by more than 3% in 2%; they take 0.851
+// (0.866) of this kernel's time alone, against 0.846 (0.864) by the better one of each.
+double longer(double a, double b) {
+  a *= a;
+  b *= b;
+  return std::sqrt(std::sqrt(a * a + b * b));
+}
+double fr_us(const Ctx* ctx, const PairArgs& a, const FrPlan& p) {
+  const bool w4 = a.wtype == ZOACT_DT_INT4_G128;
+  const pairfr::FrArgs& fr = p.fr;
+  const int nw = a.W2 ? 2 : 1, S = fr.splits;
+  const int64_t slots = (int64_t)p.per_sm * ctx->sm_count;
+  const double waves = (double)((p.tiles * S + slots - 1) / slots), tok = fr.tok / 64.0;
+  const double nm = ((a.d_in + pairfr::BKF - 1) / pairfr::BKF + S - 1) / S, nl = a.nb * ((fr.lr_groups + S - 1) / S);
+  const double mb = (w4 ? 0.5e-6 : 2e-6) * a.d_out * (double)a.d_in * nw;
+  const double block = w4 ? (p.per_sm == 1 ? 0.24 * nw + 0.11 * tok : 0.37 * nw + 0.16 * tok)
+                          : (p.per_sm == 1 ? 0.13 * nw + 0.093 * tok : 0.18 * nw + 0.17 * tok);
+  const double lr = 1.1 + (nw == 2 && fr.lr_mats == 1 ? 0.54 : 0.0) + 0.2 * ((fr.tpad + 63) / 64) + (a.r % 4 ? 0.15 : 0.0);
+  const double out = S == 1 ? tok * nw : 6.4 * tok * nw / S + 1.8 * ((fr.tok + fr.chunk - 1) / fr.chunk);
+  return (w4 ? 2.8 : 1.2) + longer(waves * nm * block, (w4 ? 0.76 : 0.15) * mb) + waves * (nl * lr + out);
+}
+double one_cta_us(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
+  const int bn = o.nw == 2 ? 128 : 256, num_k = (a.d_in + 63) / 64;
+  const int64_t tiles = (o.rows + 127) / 128 * ((a.d_out + bn - 1) / bn);
+  const double waves = (double)((tiles + ctx->sm_count - 1) / ctx->sm_count);
+  const double cols = a.d_out < bn ? (double)a.d_out / bn : 1.0;
+  const double rt = a.r <= 4 ? 4 : a.r <= 8 ? 8 : a.r <= 16 ? 16 : 32, mb = 2e-6 * a.d_out * (double)a.d_in * o.nw;
+  if (!ctx->may_allocate) return 3.5 + 0.27 * waves * num_k + waves * rt * (0.35 * cols + 0.03) + 0.06 * mb;
+  const double main = (o.nw == 2 ? 0.33 : 0.3) * waves * (num_k + o.slots * (o.ka / 64));
+  double us = 5.6 + 0.9 * waves * cols + longer(main, 0.2 * mb) + (a.r % 4 ? 0.62e-5 : 0.12e-5) * o.table_rows * o.ka +
+              2.4e-5 * o.rows * o.slots * o.ka;
+  if (!o.stacked) us += waves * ((a.nb + 1) / 2) * (1.6 + rt * cols * (o.nw == 2 ? 0.57 : 0.35));
+  if (a.shared && o.stacked) us += 2.7 * a.nb;                     // copies of X and P
+  if (a.wtype == ZOACT_DT_INT4_G128) us += 0.3 * mb + 0.7 * o.nw;
+  return us;
+}
+
+// Whether the other route's scratch is there, or may be had now: a capture cannot allocate.
+bool one_cta_ready(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
+  if (!ctx->may_allocate) return true;
+  auto held = [&](ScratchSlot slot, size_t bytes) { return ctx->slot_bytes[slot] >= bytes; };
+  const int np = a.W2 && a.P2 != a.P ? 2 : 1;
+  const size_t x_bytes = (size_t)a.T * a.d_in * 2 + (size_t)np * a.T * a.r * sizeof(float);
+  int queries = 0;                                                  // distinct ones of the perturbed blocks
+  for (int b = 0; b < a.nb; ++b) {
+    bool seen = a.coef[b] == 0.f;
+    for (int i = 0; i < b; ++i) seen = seen || (a.coef[i] != 0.f && a.qry[i] == a.qry[b]);
+    queries += !seen;
+  }
+  const size_t w_bytes = a.wtype == ZOACT_DT_INT4_G128 ? (size_t)a.d_out * a.d_in * 2 : 0;
+  if (held(SLOT_AUG_A, (size_t)o.rows * o.slots * o.ka * 2) && held(SLOT_AUG_B, (size_t)o.table_rows * o.ka * 2) &&
+      (o.stacked || held(SLOT_AUG_Z, (size_t)o.nw * queries * a.r * a.d_out * sizeof(float))) &&
+      (!(a.shared && o.stacked) || held(SLOT_STACKED_X, a.nb * x_bytes + 1024)) && held(SLOT_WDQ0, w_bytes) &&
+      (!a.W2 || held(SLOT_WDQ1, w_bytes)))
+    return true;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
+
+}  // namespace
+
+// ZOACT_PAIR_KERNEL=few / =1cta: this kernel wherever it can run / never; ZOACT_INT4=staged: not on INT4 weights.
+bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a) {
+  if (!fr_supported(a)) return false;
+  const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
+  if (sel && std::strcmp(sel, "1cta") == 0) return false;
+  if (a.wtype == ZOACT_DT_INT4_G128) {
+    const char* isel = std::getenv("ZOACT_INT4");
+    if (isel && std::strcmp(isel, "staged") == 0) return false;
+  }
+  if (sel && std::strcmp(sel, "few") == 0) return true;
+  const OneCta o = one_cta(a);
+  // (0.9: about as many calls lose by an error of the estimates one way as the other)
+  return one_cta_us(ctx, a, o) >= 0.9 * fr_us(ctx, a, fr_plan(ctx, a)) || !one_cta_ready(ctx, a, o);
+}
+
+int launch_pair_fr(Ctx* ctx, const PairArgs& a) {
+  using namespace pairfr;
+  const bool w4 = a.wtype == ZOACT_DT_INT4_G128, gated = a.W2 != nullptr;
+  if (a.ydtype != a.xdtype && a.ydtype != ZOACT_DT_FP32) return ZOACT_ERR_UNSUPPORTED;
+  const FrPlan plan = fr_plan(ctx, a);
+  const FrArgs& fr = plan.fr;
+  const int smem = plan.smem;
 
   TmaSet tm;
   int st = encode_tmap_2d_16bit(&tm.a, a.X, a.xdtype, a.rows, a.d_in, fr.tpad);
@@ -103,44 +255,6 @@ int launch_pair_fr(Ctx* ctx, const PairArgs& a) {
   p.status = ctx->d_status;
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15u) == 0; };
   p.vec_ok = al16(a.C) && al16(a.C2) && al16(a.P) && al16(a.P2);
-
-  // Two CTAs per SM where their TMEM (256 columns each) and rings fit twice; a CTA that must not share an SM takes
-  // more than half of its shared memory, so that no CTA of this launch ever waits for another one's TMEM.
-  const int stage = nw * W_TILE + fr.tok * BKF * 2, raw = w4 ? nw * RAW_TILE : 0;
-  const int most = w4 ? 4 : MAX_STAGES;                 // INT4: the rest goes to the packed rows in flight
-  auto fit = [&](int budget) {
-    budget -= FR_BARS;
-    fr.stages = (budget - 4 * raw) / stage;
-    if (fr.stages > most) fr.stages = most;
-    fr.raw_slots = w4 ? (budget - fr.stages * stage) / raw / 2 * 2 : 0;   // an even number (see the kernel)
-    if (fr.raw_slots > MAX_RAW) fr.raw_slots = MAX_RAW;
-  };
-  int per_sm = 2;
-  fit(SM_SMEM / 2 - 1024);
-  // Two stages only where one CTA per SM would leave a second wave of tiles (fp16 5120 -> 20480, 200 rows, 160 tiles:
-  // 99.0 us a call with one CTA per SM and 3 stages, 90.2 with two CTAs and 2).
-  const int64_t tiles = (a.d_out + WR - 1) / WR;
-  const bool second_wave = tiles > ctx->sm_count && tiles <= 2 * ctx->sm_count;
-  if (fr.tmem_cols > 256 || fr.stages < (second_wave ? 2 : 3)) {
-    per_sm = 1;
-    fit(CTA_SMEM);                                      // at least 3 stages of at most 64 KB, and 4 packed slots of 8 KB
-  }
-  const int ring = fr.stages * stage + fr.raw_slots * raw;
-  int smem = FR_BARS + ring;
-  if (per_sm == 1 && smem <= SM_SMEM / 2) smem = SM_SMEM / 2 + 1024;
-  fr.chunk = ring / (nw * WR * 4) / 16 * 16;
-  if (fr.chunk > fr.tok) fr.chunk = fr.tok;
-  // K ranges: as many as fill the chip's CTA slots once, each at least four K-blocks, at most a portable cluster.  More
-  // would add waves, whose prologues and epilogues nothing hides (4096 -> 14336 gated, 128 rows: 59 us a call with one
-  // range per tile, 81 with two, 93 with four; 14336 -> 4096, 32 rows: 50 with two, 34 with four, 33 with eight).
-  // A cluster lies within a GPC, so fewer than slots / S clusters of S run at once, and those left over are a second
-  // wave: fp16 5120 -> 5120, 64 rows (40 tiles) takes 30.2 us with 7 ranges, 20.8 with 6; INT4 4096 -> 5120, 48 rows
-  // 34.0 and 24.3; gated 4096 -> 2560, 80 rows (20 tiles) 33.7 and 21.0.
-  int64_t splits = (int64_t)per_sm * ctx->sm_count / tiles;
-  if (splits > p.num_k / 4) splits = p.num_k / 4;
-  if (splits > MAX_SPLITS) splits = MAX_SPLITS;
-  while (splits > 1 && tiles > clusters_at_once(ctx, (int)splits, per_sm)) --splits;
-  fr.splits = (int)(splits < 1 ? 1 : splits);
 
   st = timing_begin(ctx);
   if (st) return st;

@@ -141,9 +141,12 @@ bool pair_rowscale_supported(const Ctx* ctx, int64_t rows, int shared, int xdtyp
   return true;
 }
 
-int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
+namespace {
+
+// few: the few-row kernel may take the call.
+int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
   using namespace pairtc;
-  if (pair_fr_supported(a)) return launch_pair_fr(ctx, a);
+  if (few && pair_fr_chosen(ctx, a)) return launch_pair_fr(ctx, a);
   // ranks above 32 have no epilogue tables: the low-rank term must ride the MMA, which needs stacked rows
   const bool big_r = a.r > 32;
   if (big_r && !ctx->may_allocate) return ZOACT_ERR_UNSUPPORTED;
@@ -170,7 +173,7 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
     b.P2 = a.W2 ? ps2 : nullptr;
     b.shared = 0;
     b.rows = (int64_t)a.nb * a.T;
-    return launch_pair_tc(ctx, b);
+    return pair_tc(ctx, b, false);       // (the copies are for the other route)
   }
   // INT4 weights: the few-row kernel dequantises in the kernel; from FEW_ROWS rows W is expanded to bf16 once
   // per call and the bf16 kernel runs (the default: measured faster, see pair_tc2_kernel.cuh).
@@ -210,7 +213,7 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
       b.W2 = wb2;
       b.w_scales2 = nullptr;
     }
-    st = launch_pair_tc(ctx, b);
+    st = pair_tc(ctx, b, few);
     if (st) return st;
     return timing_end(ctx);
   }
@@ -457,6 +460,10 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
   if (st) return st;
   return timing_end(ctx);
 }
+
+}  // namespace
+
+int launch_pair_tc(Ctx* ctx, const PairArgs& a) { return pair_tc(ctx, a, true); }
 
 int launch_gemm_tc_f32out(Ctx* ctx, const void* A, const void* B, int dtype, int M, int N, int K, float* D) {
   using namespace pairtc;

@@ -1,9 +1,11 @@
-"""The few-row pair forward (fewer than 256 rows of X) at the edges of its tiles, against the fp64 oracle.
+"""The pair forward of fewer than 256 rows of X: the few-row kernel at the edges of its tiles, and the kernel that is
+chosen by the estimated times, against the fp64 oracle.
 
 Tolerances, per element: fp32 accumulation 8 sqrt(d_in) 2^-24 sum |terms| (the K ranges of a cluster are added in a
-fixed order, so the bound of one sum holds), the 16-bit split of the low-rank term above 32 ranks (2^-14 of its
-|terms|), INT4 weights rounded once to bf16 (2^-9 of sum |x w|).  Gated outputs: the same bound on gate and up, through
-|d silu| <= 1.1, plus __expf / __fdividef in SiLU (2^-20 of the product).
+fixed order, so the bound of one sum holds), INT4 weights rounded once to bf16 (2^-9 of sum |x w|); the other route's
+two-part operands of the low-rank term (2^-14 of its |terms|; the few-row kernel has three parts).  Gated outputs: the
+same bound on gate and up, through |d silu| <= 1.1, plus the approximate exponential and reciprocal in SiLU (2^-20 of the
+product).
 """
 import numpy as np
 import pytest
@@ -25,6 +27,13 @@ def ctx():
     c.close()
 
 
+@pytest.fixture(params=["few", "chosen"], autouse=True)
+def route(request, monkeypatch):
+    if request.param == "few":
+        monkeypatch.setenv("ZOACT_PAIR_KERNEL", "few")
+    return request.param
+
+
 def np64(t):
     return t.detach().double().cpu().numpy()
 
@@ -41,7 +50,7 @@ def _layer(d_in, d_out, r, wtype, seed, lid, U=None):
     return zo.make_layer(W, U, C, lid), np64(W), U, C
 
 
-def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4):
+def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4, split):
     """Blocks of outputs and the bound of their error."""
     Xn, Un, Cn = np64(X), np64(U), np64(C).reshape(W.shape[0], r)
     out, bound = [], []
@@ -51,7 +60,7 @@ def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4):
         out.append(x @ W.T + (x @ Un) @ Tb.T)
         base = np.abs(x) @ np.abs(W).T
         lr = np.abs(x @ Un) @ np.abs(Tb).T + (np.abs(x) @ np.abs(Un)) @ np.abs(Tb).T * 2.0 ** -10
-        bound.append(8 * np.sqrt(W.shape[1]) * 2.0 ** -24 * (base + lr) + (2.0 ** -14 * lr if r > 32 else 0.0) +
+        bound.append(8 * np.sqrt(W.shape[1]) * 2.0 ** -24 * (base + lr) + (2.0 ** -14 * lr if split else 0.0) +
                      (2.0 ** -9 * base if int4 else 0.0) + 1e-6)
     return np.concatenate(out), np.concatenate(bound)
 
@@ -77,16 +86,16 @@ def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4):
     ("int4", 1024, 200, 40, 16, False, 2, True),
     ("int4", 1024, 520, 120, 32, True, 3, True),    # gated, rank 32: one CTA per SM
 ])
-def test_few_rows(ctx, wtype, d_in, d_out, T, r, shared, nb, gated):
-    seed, eps = 11, 0.5
+def test_few_rows(ctx, route, wtype, d_in, d_out, T, r, shared, nb, gated):
+    seed, eps, split = 11, 0.5, route != "few"
     pts = [(eps, 7), (-eps, 7)] if nb == 2 else [(0.0, 0)] + [(eps * (1 + j) / nb, j) for j in range(nb - 1)]
     L, W, U, C = _layer(d_in, d_out, r, wtype, 100, 3)
     dt = torch.float16 if wtype == "fp16" else torch.bfloat16
     X = normal(((T if shared else nb * T), d_in), 5, DEV, dtype=dt)
-    ref, bound = _ref(W, U, C, X, T, shared, pts, seed, 3, r, wtype == "int4")
+    ref, bound = _ref(W, U, C, X, T, shared, pts, seed, 3, r, wtype == "int4", split)
     if gated:
         L2, W2, U2, C2 = _layer(d_in, d_out, r, wtype, 200, 4)      # its own basis: a second projection
-        u, ub = _ref(W2, U2, C2, X, T, shared, pts, seed, 4, r, wtype == "int4")
+        u, ub = _ref(W2, U2, C2, X, T, shared, pts, seed, 4, r, wtype == "int4", split)
         g = layers.silu(ref)
         bound = 1.1 * bound * np.abs(u) + np.abs(g) * ub + 1.1 * bound * ub + 2.0 ** -20 * np.abs(g * u)
         ref = g * u
@@ -116,3 +125,89 @@ def test_few_rows_two_signs_equal_at_zero_eps(ctx):
     zo.zoact_pair_forward(ctx, L, torch.cat([x, x]), T, False, 0.0, 1, 2, Y)
     torch.cuda.synchronize()
     assert torch.equal(Y[:T], Y[T:])
+
+
+@pytest.mark.parametrize("wtype,r,T,shared,gated", [("bf16", 1, 5, False, False), ("fp16", 8, 40, True, False),
+                                                    ("bf16", 7, 16, False, True), ("int4", 8, 33, False, False),
+                                                    ("bf16", 21, 100, False, False)])
+def test_lowrank_term_alone(ctx, monkeypatch, wtype, r, T, shared, gated):
+    # W = 0 and fp32 outputs (gate: a constant): the low-rank term in six products of three bf16 parts.  Left out are
+    # mid lo, lo mid and the parts' own remainders, 4 x 2^-27 of |T||P|; the accumulator truncates each of the steps that
+    # hold terms (three a K-block of eight ranks) and aligns its products to about as much: 2^-23 each.  A product that
+    # is missing is 2^-9 (hi mid) or 2^-18 (hi lo, mid mid) of |T||P|, far above that.
+    monkeypatch.setenv("ZOACT_PAIR_KERNEL", "few")
+    d_in, d_out, seed = 128, 264, 3
+    dt = torch.float16 if wtype == "fp16" else torch.bfloat16
+    X = normal(((T if shared else 2 * T), d_in), 1, DEV, dtype=dt)
+    P = normal(((T if shared else 2 * T), r), 2, DEV)
+    U = normal((d_in, r), 3, DEV)
+    C = normal((d_out * r,), 4, DEV)
+
+    def layer(c, lid):
+        if wtype == "int4":
+            return zo.make_layer(torch.zeros(d_out, d_in // 2, dtype=torch.uint8, device=DEV), U, c, lid,
+                                 w_scales=torch.ones(d_out, 1, dtype=torch.float16, device=DEV), wtype=zo.DT_INT4_G128,
+                                 d_in=d_in)
+        return zo.make_layer(torch.zeros(d_out, d_in, dtype=dt, device=DEV), U, c, lid)
+
+    Y = torch.empty(2 * T, d_out, device=DEV)
+    if gated:
+        # the gate's term the constant 20 (one rank of P is 1 there): silu(20) = 20 within 2^-23, the up term under test
+        P[:, 0] = 1.0
+        Cg = torch.zeros(d_out, r, device=DEV)
+        Cg[:, 0] = 20.0
+        zo.zoact_pair_forward_gated(ctx, layer(Cg.reshape(-1), 0), layer(C, 1), X, T, shared, 0.0, seed, 1, Y, P_gate=P,
+                                    P_up=P)
+    else:
+        zo.zoact_pair_forward(ctx, layer(C, 0), X, T, shared, 0.0, seed, 1, Y, P=P)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    Pn, Cn = np64(P), np64(C).reshape(d_out, r)
+    if shared:
+        Pn = np.concatenate([Pn, Pn])
+    scale = 20.0 / (1.0 + np.exp(-20.0)) if gated else 1.0
+    blocks = (r + 7) // 8
+    bound = (4 * 2.0 ** -27 + (6 * blocks) * 2.0 ** -23 + (2.0 ** -21 if gated else 0.0)) * (np.abs(Pn) @ np.abs(Cn).T) * scale
+    err = np.abs(np64(Y) - scale * (Pn @ Cn.T))
+    assert np.all(err <= bound), float((err / bound).max())
+    lost = 2.0 ** -20 * scale * np.abs(Pn) @ np.abs(Cn).T       # what the smallest part is on average
+    assert r > 8 or gated or float(err.max()) < float(lost.max())
+
+
+@pytest.mark.parametrize("wtype,d_in,d_out,T,r,shared,gated", [
+    ("bf16", 64, 64, 100, 64, False, False),        # the other route by its estimate
+    ("bf16", 256, 512, 64, 16, False, True),
+    ("bf16", 256, 512, 100, 64, True, False),       # ... with copies of the shared input
+    ("int4", 128, 64, 100, 64, False, True),        # ... with W expanded
+    ("bf16", 4096, 1024, 16, 16, False, False),     # the few-row kernel
+])
+def test_first_call_captured(route, wtype, d_in, d_out, T, r, shared, gated):
+    # A first call with the projection given, on a context without scratch, in a capture that may not allocate: the
+    # few-row kernel needs no scratch, so it is taken where the other one's is not there.
+    L, W, U, C = _layer(d_in, d_out, r, wtype, 100, 3)
+    L2 = _layer(d_in, d_out, r, wtype, 200, 4, U=U)[0]
+    X = normal(((T if shared else 2 * T), d_in), 5, DEV, dtype=torch.bfloat16)
+    P = X.float() @ U
+    Y = [torch.zeros(2 * T, d_out, dtype=torch.bfloat16, device=DEV) for _ in range(2)]
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        c = zo.Context(0)
+        c.sync_stream()
+
+        def run(y):
+            if gated:
+                zo.zoact_pair_forward_gated(c, L, L2, X, T, shared, 0.5, 1, 2, y, P_gate=P, P_up=P)
+            else:
+                zo.zoact_pair_forward(c, L, X, T, shared, 0.5, 1, 2, y, P=P)
+
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            run(Y[0])
+        g.replay()
+        run(Y[1])
+        torch.cuda.synchronize()
+        assert c.device_status() == 0
+    a, b = np64(Y[0]), np64(Y[1])
+    assert np.linalg.norm(a - b) <= 2.0 ** -8 * np.linalg.norm(b) and np.abs(a).max() > 0
+    c.close()
