@@ -36,6 +36,17 @@ void* scratch(Ctx* ctx, ScratchSlot slot, size_t bytes) {
   return p;
 }
 
+bool scratch_ready(const Ctx* ctx, ScratchSlot slot, size_t bytes) {
+  if (ctx->slot_bytes[slot] >= bytes) return true;
+  if (!ctx->may_allocate) return false;
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return st == cudaStreamCaptureStatusNone;
+}
+
 void* scratch_zeroed(Ctx* ctx, ScratchSlot slot, size_t bytes) {
   const void* before = ctx->slot_ptr[slot];
   const size_t had = ctx->slot_bytes[slot];

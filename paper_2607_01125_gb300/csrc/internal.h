@@ -67,6 +67,8 @@ int timing_end(Ctx* ctx);
 int cuda_fail(cudaError_t e, const char* what);
 // Returns a device pointer of at least `bytes` for the slot, or nullptr on failure.
 void* scratch(Ctx* ctx, ScratchSlot slot, size_t bytes);
+// Whether scratch() would succeed without an allocation, or may allocate (a stream capture may not).
+bool scratch_ready(const Ctx* ctx, ScratchSlot slot, size_t bytes);
 // As scratch(), and a newly allocated buffer is zero-filled (on the context's stream).
 void* scratch_zeroed(Ctx* ctx, ScratchSlot slot, size_t bytes);
 

@@ -177,30 +177,23 @@ double one_cta_us(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
   return us;
 }
 
-// Whether the other route's scratch is there, or may be had now: a capture cannot allocate.
+// Whether the other route's scratch is there, or may be had now.
 bool one_cta_ready(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
-  if (!ctx->may_allocate) return true;
-  auto held = [&](ScratchSlot slot, size_t bytes) { return ctx->slot_bytes[slot] >= bytes; };
-  const int np = a.W2 && a.P2 != a.P ? 2 : 1;
-  const size_t x_bytes = (size_t)a.T * a.d_in * 2 + (size_t)np * a.T * a.r * sizeof(float);
+  if (!ctx->may_allocate) return true;                              // (its form without scratch)
   int queries = 0;                                                  // distinct ones of the perturbed blocks
   for (int b = 0; b < a.nb; ++b) {
     bool seen = a.coef[b] == 0.f;
     for (int i = 0; i < b; ++i) seen = seen || (a.coef[i] != 0.f && a.qry[i] == a.qry[b]);
     queries += !seen;
   }
+  const int np = a.W2 && a.P2 != a.P ? 2 : 1;
+  const size_t copy = (size_t)a.T * a.d_in * 2 + (size_t)np * a.T * a.r * sizeof(float);
   const size_t w_bytes = a.wtype == ZOACT_DT_INT4_G128 ? (size_t)a.d_out * a.d_in * 2 : 0;
-  if (held(SLOT_AUG_A, (size_t)o.rows * o.slots * o.ka * 2) && held(SLOT_AUG_B, (size_t)o.table_rows * o.ka * 2) &&
-      (o.stacked || held(SLOT_AUG_Z, (size_t)o.nw * queries * a.r * a.d_out * sizeof(float))) &&
-      (!(a.shared && o.stacked) || held(SLOT_STACKED_X, a.nb * x_bytes + 1024)) && held(SLOT_WDQ0, w_bytes) &&
-      (!a.W2 || held(SLOT_WDQ1, w_bytes)))
-    return true;
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(ctx->stream, &st) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return st == cudaStreamCaptureStatusNone;
+  return scratch_ready(ctx, SLOT_AUG_A, (size_t)o.rows * o.slots * o.ka * 2) &&
+         scratch_ready(ctx, SLOT_AUG_B, (size_t)o.table_rows * o.ka * 2) &&
+         (o.stacked || scratch_ready(ctx, SLOT_AUG_Z, (size_t)o.nw * queries * a.r * a.d_out * sizeof(float))) &&
+         (!(a.shared && o.stacked) || scratch_ready(ctx, SLOT_STACKED_X, a.nb * copy + 1024)) &&
+         scratch_ready(ctx, SLOT_WDQ0, w_bytes) && (!a.W2 || scratch_ready(ctx, SLOT_WDQ1, w_bytes));
 }
 
 }  // namespace

@@ -139,7 +139,8 @@ __global__ void splitk_reduce_kernel(const float* __restrict__ part, float* __re
 // Short rows (fp32 X of at most PROJ_ROW_MAX columns, the 256-wide toy graph): a warp owns R rows and eight basis
 // columns; its lanes take every 32nd k, with all of a row's loads in flight, and a butterfly adds them.  The blocks above
 // walk such a row in 32-wide chunks, a round trip to L2 each: 64 x 256, r = 8 took 41 us on one 64-thread block (ncu),
-// 7.3 here (cold caches; a launch alone is ~3).
+// 7.3 here (cold caches; a launch alone is ~3).  It reads X once per eight ranks and U once per R rows, so many rows at
+// high ranks stay with the blocks (proj_by_rows).
 constexpr int PROJ_ROW_MAX = 1024;
 template <int R>
 __global__ void __launch_bounds__(128)
@@ -182,9 +183,21 @@ proj_rows_kernel(const float* __restrict__ X, const float* __restrict__ U, float
       if (lane == j && m0 + i < rows && j0 + j < r) P[(m0 + i) * r + j0 + j] = acc[i][j];
 }
 
+// fp32 X of at most PROJ_ROW_MAX columns: whether a warp per row is the faster form, by times in us on a GB300 (straight
+// lines fitted to d_in 16 .. 1024, 1 .. 16384 rows, r = 1 .. 256): the work of the rows, against a chain over a block's
+// K range per 32 ranks, which hardly grows with the rows.  1024 columns, r = 32: 1024 rows 12.8 us by warps, 22.9 by
+// blocks; 16384 rows 139 and 48.6.  64 columns, r = 256: 4096 rows 41 and 49, 16384 rows 156 and 51.
+bool proj_by_rows(int64_t rows, int d_in, int r) {
+  if (d_in > PROJ_ROW_MAX) return false;
+  const double by_rows = 1.5 + (double)rows * ((r + 7) / 8) * (1.7e-6 * d_in + 2.5e-4);
+  const double by_blocks = ((r + 31) / 32) * (2.2 + 0.076 * (d_in < 256 ? d_in : 256) + 1.1e-6 * (double)rows * d_in);
+  return by_rows <= by_blocks;
+}
+
 int launch_proj_rows(Ctx* ctx, const float* X, int64_t rows, int d_in, const float* U, int r, float* P) {
-  // one row a warp until the rows alone give every SM 16 warps
-  const int R = rows >= 16LL * ctx->sm_count ? 4 : 1;
+  // one row a warp until rows and rank groups give every SM 16 warps, 64 where rows are shorter than four K steps (1024
+  // rows, 1024 columns, r = 32: 50 us with one row a warp, 12.8 with four; 64 columns, r = 24: 2.5 and 3.2)
+  const int R = rows * ((r + 7) / 8) >= (d_in >= 128 ? 16LL : 64LL) * ctx->sm_count ? 4 : 1;
   const dim3 grid((unsigned)((rows + 4 * R - 1) / (4 * R)), (unsigned)((r + 7) / 8));
   const int vec = r % 8 == 0 && ((uintptr_t)U & 15u) == 0;
   ZOACT_CUDA_TRY(launch_pdl(ctx, R == 4 ? proj_rows_kernel<4> : proj_rows_kernel<1>, grid, dim3(128), 0, X, U, P, rows,
@@ -194,17 +207,23 @@ int launch_proj_rows(Ctx* ctx, const float* X, int64_t rows, int d_in, const flo
   return ZOACT_OK;
 }
 
-template <typename TX>
-int proj_dispatch(Ctx* ctx, const TX* X, int64_t rows, int d_in, const float* U, int r, float* P) {
+// K-splits of the blocked form: enough to give every SM about two blocks, each split >= 256 wide
+int proj_splits(const Ctx* ctx, int64_t rows, int d_in, int& k_per_split) {
   const int64_t row_blocks = (rows + PROJ_RB - 1) / PROJ_RB;
-  // enough K-splits to give every SM about two blocks, each split >= 256 wide
   int splits = (int)((2LL * ctx->sm_count + row_blocks - 1) / row_blocks);
   const int max_splits = (d_in + 255) / 256;
   if (splits > max_splits) splits = max_splits;
   if (splits < 1) splits = 1;
-  int k_per_split = (d_in + splits - 1) / splits;
+  k_per_split = (d_in + splits - 1) / splits;
   k_per_split = (k_per_split + PROJ_KC - 1) / PROJ_KC * PROJ_KC;
-  splits = (d_in + k_per_split - 1) / k_per_split;
+  return (d_in + k_per_split - 1) / k_per_split;
+}
+
+template <typename TX>
+int proj_dispatch(Ctx* ctx, const TX* X, int64_t rows, int d_in, const float* U, int r, float* P) {
+  const int64_t row_blocks = (rows + PROJ_RB - 1) / PROJ_RB;
+  int k_per_split;
+  const int splits = proj_splits(ctx, rows, d_in, k_per_split);
   dim3 grid((unsigned)row_blocks, (unsigned)splits);
   // groups of up to 32 basis columns, one launch each
   for (int j0 = 0; j0 < r; j0 += 32) {
@@ -244,9 +263,16 @@ int launch_lowrank_proj(Ctx* ctx, const void* X, int xdtype, int64_t rows, int d
                         float* P) {
   if (rows <= 0) return ZOACT_OK;
   switch (xdtype) {
-    case ZOACT_DT_FP32:
-      if (d_in <= PROJ_ROW_MAX) return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
+    case ZOACT_DT_FP32: {
+      // (the warps need no scratch: a capture that cannot get the blocks' takes them)
+      int k_per_split;
+      const int splits = proj_splits(ctx, rows, d_in, k_per_split);
+      if (proj_by_rows(rows, d_in, r) ||
+          (d_in <= PROJ_ROW_MAX && splits > 1 &&
+           !scratch_ready(ctx, SLOT_SPLITK, (size_t)splits * rows * (r < 32 ? r : 32) * sizeof(float))))
+        return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
       return proj_dispatch(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
+    }
     case ZOACT_DT_BF16:
     case ZOACT_DT_FP16: return launch_lowrank_proj_tc(ctx, X, xdtype, rows, d_in, U, r, P);
     default: return ZOACT_ERR_INVALID_ARG;
@@ -299,7 +325,7 @@ int launch_lowrank_proj_into(Ctx* ctx, const void* X, int xdtype, int64_t rows, 
   if (rows <= 0) return ZOACT_OK;
   switch (xdtype) {
     case ZOACT_DT_FP32:
-      if (d_in <= PROJ_ROW_MAX) return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
+      if (proj_by_rows(rows, d_in, r)) return launch_proj_rows(ctx, static_cast<const float*>(X), rows, d_in, U, r, P);
       return proj_dispatch_into(ctx, static_cast<const float*>(X), rows, d_in, U, r, P, part, part_floats);
     case ZOACT_DT_BF16:
       return proj_dispatch_into(ctx, static_cast<const __nv_bfloat16*>(X), rows, d_in, U, r, P, part, part_floats);

@@ -59,3 +59,37 @@ def test_pair_forward_fp32_tiles(ctx, d_in, d_out, T, r, shared, nb):
         lr = np.abs(x) @ np.abs(Un) @ np.abs(Tb).T
         bound = 4 * np.sqrt(d_in) * 2.0 ** -24 * (np.abs(x) @ np.abs(Wn).T + lr) + 1e-6 * lr + 1e-7
         assert np.all(np.abs(n64(Y[b * T:(b + 1) * T]) - ref) <= bound), b
+
+
+def _check_projection(X, U, P):
+    Xn, Un = X.double().cpu().numpy(), U.double().cpu().numpy()
+    bound = 4 * np.sqrt(X.shape[1]) * 2.0 ** -24 * (np.abs(Xn) @ np.abs(Un))
+    assert np.all(np.abs(P.double().cpu().numpy() - Xn @ Un) <= bound)
+
+
+@pytest.mark.parametrize("rows,d_in,r", [(9001, 1024, 40), (16384, 64, 96), (4097, 512, 72),   # blocks: many rows, ranks
+                                         (700, 64, 24), (1000, 1024, 36), (305, 1024, 64)])     # four rows a warp
+def test_projection_fp32_forms(ctx, rows, d_in, r):
+    X, U = normal((rows, d_in), 1, DEV), normal((d_in, r), 2, DEV)
+    P = torch.full((rows, r), float("nan"), device=DEV)
+    zo.zoact_lowrank_proj(ctx, X, U, P)
+    torch.cuda.synchronize()
+    _check_projection(X, U, P)
+
+
+def test_projection_fp32_first_call_captured():
+    # K-splits in scratch that a capture cannot allocate: the form without scratch
+    X, U = normal((4096, 1024), 1, DEV), normal((1024, 64), 2, DEV)
+    P = torch.full((4096, 64), float("nan"), device=DEV)
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        c = zo.Context(0)
+        c.sync_stream()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            zo.zoact_lowrank_proj(c, X, U, P)
+        g.replay()
+        torch.cuda.synchronize()
+    _check_projection(X, U, P)
+    c.close()
