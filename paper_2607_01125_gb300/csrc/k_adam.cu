@@ -95,7 +95,10 @@ zo_update_kernel(float* __restrict__ C, float* __restrict__ m, float* __restrict
       c4[u] = m4[u] = v4[u] = make_float4(0.f, 0.f, 0.f, 0.f);
       left[u] = 0;
       if (g0 + u * 256 < last) {
-        while (b + 1 < tab.n && tab.begin[b + 1] <= e) ++b;
+        if (b + 1 < tab.n && tab.begin[b + 1] <= e) {    // the next layer, or (many short ones) a search
+          ++b;
+          if (b + 1 < tab.n && tab.begin[b + 1] <= e) b = find_block(tab, e);
+        }
         const int64_t rest = tab.end[b] - e;             // <= 0: a gap between blocks
         left[u] = rest >= 4 ? 4 : rest > 0 ? (int)rest : 0;
       }
@@ -183,13 +186,14 @@ int launch_adam(Ctx* ctx, float* C, float* m, float* v, const zoact_coeff_block*
     }
     if (hi <= lo) continue;
     const int64_t g_begin = lo / 4, g_end = (hi + 3) / 4;
-    // a block's range: whole rounds of its threads, as even as eight blocks per SM allow; a round is one group a thread
-    // until the arena gives every SM that many
-    int64_t nb = (g_end - g_begin + 255) / 256;
-    const int64_t cap = (int64_t)ctx->sm_count * 8;
-    if (nb > cap) nb = cap;
-    const int64_t per_block = ((g_end - g_begin + nb - 1) / nb + 255) / 256 * 256;
-    nb = (g_end - g_begin + per_block - 1) / per_block;
+    // a block's range: whole rounds of its threads (one group each), eight blocks per SM.  With several queries the draws
+    // are the time, and few rounds go to rather more blocks, which the SMs take as they come, than to ranges that leave
+    // some SM a round ahead (1310720 elements, 8 queries: 28.2 us in 640 blocks of two rounds, 26.1 in 1280 of one; with
+    // one query, where a thread's two groups in flight count, 7.4 and 7.7).
+    const int64_t groups = g_end - g_begin, cap = (int64_t)ctx->sm_count * 8;
+    int64_t rounds = (groups + 255) / 256 / cap;
+    if (q < 4 || rounds >= 8) rounds = (groups + cap * 256 - 1) / (cap * 256);
+    const int64_t per_block = 256 * (rounds < 1 ? 1 : rounds), nb = (groups + per_block - 1) / per_block;
     ZOACT_CUDA_TRY(launch_pdl(ctx, sgd ? zo_update_kernel<true> : zo_update_kernel<false>, dim3((unsigned)nb),
                               dim3(256), 0, C, m, v, tab, g_begin, g_end, per_block, a, q, qs, lr, b1, b2, adam_eps, step_size,
                               inv_sqrt_bc2, seed, ctx->d_status));
