@@ -59,4 +59,5 @@ def test_layer_walk(ctx, blocks, queries):
         for x, y, z in zip(one, each, arena):
             assert torch.equal(x, y)
             assert torch.equal(x[~inside], z[~inside])
-        assert bool((one[0][inside] != arena[0][inside]).all())
+        # (a change below half an ulp leaves an element as it was)
+        assert float((one[0][inside] != arena[0][inside]).double().mean()) > 0.99
