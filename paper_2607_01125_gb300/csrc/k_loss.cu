@@ -333,13 +333,26 @@ loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t 
   __shared__ int bad;
   __syncthreads();
   for (int i = warp; i < 2 * nb; i += MULTI_THREADS / 32) {   // sum i: block i / 2, squares or differences
-    CSum w;                                    // (fp64 adds of every thread's two floats took 10 us here)
-    for (int t = lane; t < MULTI_THREADS; t += 32) {
+    // (a lane's sixteen compensated, ~46 bits; fp64 adds of every thread's two floats took 10 us here, and are left to sums
+    // that fp32 cannot hold)
+    auto slot = [&](int t) {
       const float4 x = slots[(i >> 1) * MULTI_THREADS + t];
-      w.add((i & 1) ? x.z : x.x);
-      w.c += (i & 1) ? x.w : x.y;
+      return (i & 1) ? make_float2(x.z, x.w) : make_float2(x.x, x.y);
+    };
+    CSum w;
+    float top = 0.f;
+    for (int t = lane; t < MULTI_THREADS; t += 32) {
+      const float2 x = slot(t);
+      w.add(x.x);
+      w.c += x.y;
+      top = fmaxf(top, fabsf(x.x));
     }
-    const double a = warp_sum(w.value());
+    double a = w.value();
+    if (top > 0x1p120f) {
+      a = 0.0;
+      for (int t = lane; t < MULTI_THREADS; t += 32) a += (double)slot(t).x + (double)slot(t).y;
+    }
+    a = warp_sum(a);
     if (lane == 0) {
       partials[(int64_t)i * gridDim.x + blockIdx.x] = a;
       __threadfence();

@@ -53,7 +53,7 @@ def test_query_blocks_edges(ctx, gated, T, d_out, r, dt):  # noqa: F811
                                                    (641, 1000, 10, torch.bfloat16, True), (1, 8, 2, torch.float16, True),
                                                    (1, 1, 17, torch.float32, True), (997, 643, 9, torch.float16, False)])
 def test_loss_blocks_edges(ctx, T, n, nb, dt, with_target):  # noqa: F811
-    # a vector more than the grid's threads, blocks past a round's eight (four in fp32), the scalar path, one element
+    # a vector more than the grid's threads, blocks past a round of four, the scalar path, one element
     y0 = normal((T, n), 61, DEV)
     Y = torch.cat([y0] + [y0 + 1e-2 * normal((T, n), 62 + j, DEV) for j in range(nb - 1)]).to(dt)
     tgt = normal((T, n), 80, DEV, dtype=dt) if with_target else None
@@ -71,3 +71,32 @@ def test_loss_blocks_edges(ctx, T, n, nb, dt, with_target):  # noqa: F811
         scale = np.mean(np.abs((Yn[j * T:(j + 1) * T] - Yn[:T]) * (Yn[j * T:(j + 1) * T] + Yn[:T] - 2 * t))) / mu
         assert abs(o[nb + j - 1] - a[j - 1]) <= 16 * 2.0 ** -24 * scale + 2.0 ** -50 * abs(a[j - 1])
     assert o[-1] == 7.0
+
+
+@pytest.mark.parametrize("T,n,nb,dt,with_target", [
+    (1027, 1000, 5, torch.bfloat16, True),    # one round of four blocks and a last thread group of one vector
+    (1027, 1000, 6, torch.float16, False),    # a block past it
+    (1027, 1000, 9, torch.bfloat16, False),   # two rounds
+    (2055, 1000, 2, torch.bfloat16, True),    # one block beside y0
+    (2055, 1000, 2, torch.float32, False),
+])
+def test_loss_blocks_rounds(ctx, T, n, nb, dt, with_target):  # noqa: F811
+    test_loss_blocks_edges(ctx, T, n, nb, dt, with_target)
+
+
+@pytest.mark.parametrize("dt", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("nb", [2, 3])
+def test_loss_blocks_large_values(ctx, nb, dt):  # noqa: F811
+    # a thread's sum of squares fits fp32 (8 or 16 values of 2e18 a vector group), sixteen threads' do not
+    T, n, mu = 640, 1000, 1.0
+    Y = (2e18 * (1.0 + 0.25 * torch.rand(nb * T, n, device=DEV))).to(dt)
+    out = torch.zeros(2 * nb, dtype=torch.float64, device=DEV)
+    zo.zoact_loss_multi(ctx, Y, T, nb, mu, out)
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    o, Yn = out.cpu().numpy(), np64(Y)
+    L, a = oloss.loss_queries(Yn, T, nb, None, mu)
+    np.testing.assert_allclose(o[:nb], L, rtol=16 * 2.0 ** -24)
+    for j in range(1, nb):
+        scale = np.mean(np.abs((Yn[j * T:(j + 1) * T] - Yn[:T]) * (Yn[j * T:(j + 1) * T] + Yn[:T])))
+        assert abs(o[nb + j - 1] - a[j - 1]) <= 16 * 2.0 ** -24 * scale
