@@ -253,9 +253,11 @@ int loss_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, float eps
 // whole sums over the threads, compensated and then in fp64, and in the last CTA over the CTAs' partials [sum][CTA], both
 // in a fixed order.  Nine blocks of 512 x 4096 bf16 (42 MB): 41 us with the blocks on a grid axis, y_0 and t read once for
 // each, and a tree of barriers per block at the end; 24 here (both with cold caches, as in a profile).
+// AHEAD: the blocks of a round.  Two blocks (one query) have one beside y_0: fewer registers, and two CTAs per SM for the
+// loads in flight (4096 x 4096 bf16 without a target: 23.2 us with one, 20.2 with two; 21.4 with the blocks on a grid axis).
 constexpr int MULTI_THREADS = 512;
-template <typename TY>
-__global__ void __launch_bounds__(MULTI_THREADS, 1)
+template <typename TY, int AHEAD>
+__global__ void __launch_bounds__(MULTI_THREADS, AHEAD == 1 ? 2 : 1)
 loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t count, int vec_ok, int64_t apart, int nb,
                   float mu, double* __restrict__ out, double* __restrict__ partials, unsigned int* __restrict__ ticket,
                   int* __restrict__ status) {
@@ -276,7 +278,6 @@ loss_multi_kernel(const TY* __restrict__ Y, const TY* __restrict__ tgt, int64_t 
   const int64_t stride = (int64_t)gridDim.x * MULTI_THREADS;
   const int64_t first = blockIdx.x * (int64_t)MULTI_THREADS + tid;
   constexpr int R = sizeof(TY) == 4 ? 1 : 2;         // vectors of a group (fp32 words take twice the registers)
-  constexpr int AHEAD = 4;                           // blocks of a round, their loads issued first
   for (int64_t g = first;; g += stride) {
     const int64_t v = R == 1 ? g : g + g / apart * apart;
     if (v >= n_vec) break;
@@ -390,16 +391,19 @@ int loss_multi_dispatch(Ctx* ctx, const TY* Y, const TY* tgt, int64_t count, int
   const int vec_ok = (count % 8 == 0) && ((uintptr_t)Y % 16 == 0) && ((uintptr_t)tgt % 16 == 0);
   int64_t bx = ((vec_ok ? count / 8 : count) + MULTI_THREADS - 1) / MULTI_THREADS;
   if (bx < 1) bx = 1;
-  if (bx > ctx->sm_count) bx = ctx->sm_count;
+  // (from eight vectors of y_0 a thread; 512 x 4096 bf16 8.2 us with one CTA per SM, 8.6 with two)
+  const bool two = nb == 2 && bx >= 8 * (int64_t)ctx->sm_count;
+  if (bx > (two ? 2 : 1) * ctx->sm_count) bx = (two ? 2 : 1) * ctx->sm_count;
   if (bx > max_blocks) bx = max_blocks;
   // (the stride of two 256-thread blocks per SM shared by the nb blocks, at most one vector a thread)
   int64_t strides = ((vec_ok ? count / 8 : count) + 255) / 256;
   if (strides > max_blocks / nb) strides = max_blocks / nb;
   const int64_t apart = 256 * (strides < 1 ? 1 : strides);
   const int smem = nb * MULTI_THREADS * (int)sizeof(float4);
-  ZOACT_CUDA_TRY(cudaFuncSetAttribute(loss_multi_kernel<TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  auto kern = two ? loss_multi_kernel<TY, 1> : loss_multi_kernel<TY, 4>;
+  ZOACT_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       ZOACT_MAX_EVAL_BLOCKS * MULTI_THREADS * (int)sizeof(float4)));
-  ZOACT_CUDA_TRY(launch_pdl(ctx, loss_multi_kernel<TY>, dim3((unsigned)bx), dim3(MULTI_THREADS), smem, Y, tgt, count,
+  ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)bx), dim3(MULTI_THREADS), smem, Y, tgt, count,
                             vec_ok, apart, nb, mu, out, partials, ticket, ctx->d_status));
   ++ctx->n_launch;
   return ZOACT_OK;

@@ -79,6 +79,8 @@ def test_loss_blocks_edges(ctx, T, n, nb, dt, with_target):  # noqa: F811
     (1027, 1000, 9, torch.bfloat16, False),   # two rounds
     (2055, 1000, 2, torch.bfloat16, True),    # one block beside y0
     (2055, 1000, 2, torch.float32, False),
+    (5603, 1000, 2, torch.bfloat16, True),    # ... with two CTAs per SM
+    (5603, 1000, 2, torch.float32, False),
 ])
 def test_loss_blocks_rounds(ctx, T, n, nb, dt, with_target):  # noqa: F811
     test_loss_blocks_edges(ctx, T, n, nb, dt, with_target)
