@@ -130,11 +130,16 @@ __device__ __forceinline__ void write_z_operands(const AugBlocks& blk, int d_out
         float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
         if (n < d_out && j0 < r && (r & 3) == 0) v = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2));
         z[nt][h][0] = v.x; z[nt][h][1] = v.y; z[nt][h][2] = v.z; z[nt][h][3] = v.w;
-        if (n < d_out && (r & 3) != 0)
+        if (n < d_out && j0 < r && (r & 3) != 0) {
+          // four ranks in at most two Philox groups
+          const int at = (int)(e & 3), ranks = min(4, r - j0);
+          const float4 a = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2));
+          float4 b = a;
+          if (at + ranks > 4) b = z_normals4(seed, layer, blk.zq[qi], (uint64_t)(e >> 2) + 1);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            if (j0 + i < r)
-              z[nt][h][i] = z_select(z_normals4(seed, layer, blk.zq[qi], (uint64_t)((e + i) >> 2)), (int)((e + i) & 3));
+            if (i < ranks) z[nt][h][i] = at + i < 4 ? z_select(a, at + i) : z_select(b, at + i - 4);
+        }
       }
     }
     uint32_t* dst = (mat ? Zt2 : Zt) + ((int64_t)qi * chunks + ch) * CHUNK;
