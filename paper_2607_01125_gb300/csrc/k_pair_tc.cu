@@ -143,6 +143,28 @@ bool pair_rowscale_supported(const Ctx* ctx, int64_t rows, int shared, int xdtyp
 
 namespace {
 
+// Any number of rows by the few-row kernel, which needs no scratch: up to 240 rows of one evaluation block at a time.
+int few_row_pieces(Ctx* ctx, const PairArgs& a) {
+  constexpr int64_t PIECE = 240;
+  int st = timing_begin(ctx);
+  for (int b = 0; b < a.nb && !st; ++b)
+    for (int64_t t = 0; t < a.T && !st; t += PIECE) {
+      const int64_t row = (a.shared ? 0 : b * a.T) + t;
+      PairArgs s = a;
+      s.X = static_cast<const uint8_t*>(a.X) + row * a.d_in * dtype_size(a.xdtype);
+      s.P = a.P + row * a.r;
+      if (a.W2) s.P2 = a.P2 + row * a.r;
+      s.Y = static_cast<uint8_t*>(a.Y) + ((int64_t)b * a.T + t) * a.d_out * dtype_size(a.ydtype);
+      s.T = s.rows = a.T - t < PIECE ? a.T - t : PIECE;
+      s.shared = 0;
+      s.nb = 1;
+      s.coef[0] = a.coef[b];
+      s.qry[0] = a.qry[b];
+      st = launch_pair_fr(ctx, s);
+    }
+  return st ? st : timing_end(ctx);
+}
+
 // few: the few-row kernel may take the call.
 int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
   using namespace pairtc;
@@ -193,8 +215,14 @@ int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
                       (a.ydtype == ZOACT_DT_BF16 || a.ydtype == ZOACT_DT_FP32) && !one_cta && !lr_epi &&
                       int4_kernel;
   if (a.wtype == ZOACT_DT_INT4_G128 && !w4_two) {
-    // staged INT4: expand W (and W2) to bf16 in context scratch, then the bf16 kernel (timed together)
+    // staged INT4: expand W (and W2) to bf16 in context scratch, then the bf16 kernel (timed together).  Fewer rows than
+    // 1024 do without where that scratch cannot be had (a capture, memory): the few-row kernel takes them in pieces.
     const size_t bytes = (size_t)a.d_out * a.d_in * 2;
+    const bool pieces = a.rows < INT4_ROWSCALE_MIN_ROWS && !one_cta && !(isel && std::strcmp(isel, "staged") == 0) &&
+                        a.nseg <= 1 && !a.fuse_loss && !a.in_scale && !a.out_sumsq && a.xdtype == ZOACT_DT_BF16;
+    if (pieces && (!scratch_ready(ctx, SLOT_WDQ0, bytes) || (a.W2 && !scratch_ready(ctx, SLOT_WDQ1, bytes)) ||
+                   !scratch(ctx, SLOT_WDQ0, bytes) || (a.W2 && !scratch(ctx, SLOT_WDQ1, bytes))))
+      return few_row_pieces(ctx, a);
     void* wb = scratch(ctx, SLOT_WDQ0, bytes);
     if (!wb) return ZOACT_ERR_NOMEM;
     int st = timing_begin(ctx);

@@ -180,6 +180,9 @@ def test_lowrank_term_alone(ctx, monkeypatch, wtype, r, T, shared, gated):
     ("bf16", 256, 512, 100, 64, True, False),       # ... with copies of the shared input
     ("int4", 128, 64, 100, 64, False, True),        # ... with W expanded
     ("bf16", 4096, 1024, 16, 16, False, False),     # the few-row kernel
+    ("int4", 1024, 264, 245, 16, False, False),     # 490 rows: INT4 in pieces of 240 rows and five, without W expanded
+    ("int4", 512, 136, 500, 7, True, False),
+    ("int4", 512, 264, 130, 32, False, True),
 ])
 def test_first_call_captured(route, wtype, d_in, d_out, T, r, shared, gated):
     # A first call with the projection given, on a context without scratch, in a capture that may not allocate: the
