@@ -321,14 +321,16 @@ def zoact_loss_pair(ctx, Y, T, eps, out, target=None):
                                                       float(eps), _ptr(out)))
 
 
+_BLOCK = struct.Struct("=qiiI4x")     # zoact_coeff_block
+
+
 def _blocks(blocks):
-    """The zoact_coeff_block array of a list of (offset, d_out, r, layer_id): packed in one call (a ctypes structure per
-    block took 130 us of the Llama stack's 224-layer update), or one by one where a value is not a plain integer."""
+    """The zoact_coeff_block array of a list of (offset, d_out, r, layer_id): packed without a ctypes structure per block
+    (which took 130 us of the Llama stack's 224-layer update), or one by one where a value is not a plain integer."""
     n = len(blocks)
     try:
-        raw = struct.pack("=" + "qiiI4x" * n, *itertools.chain.from_iterable(blocks))
         if n > 0:
-            return (zoact_coeff_block * n).from_buffer_copy(raw)
+            return (zoact_coeff_block * n).from_buffer_copy(b"".join(itertools.starmap(_BLOCK.pack, blocks)))
     except struct.error:
         pass
     arr = (zoact_coeff_block * max(1, n))()

@@ -6,6 +6,9 @@ import ctypes
 import os
 import re
 
+import numpy as np
+import pytest
+
 from paper_2607_01125_gb300 import build as zbuild
 from paper_2607_01125_gb300 import _lib
 
@@ -44,3 +47,17 @@ def test_layer_struct_matches_c_layout():
     assert ctypes.sizeof(_lib.zoact_layer) == 56
     assert _lib.zoact_layer.W.offset == 16 and _lib.zoact_layer.layer_id.offset == 48
     assert ctypes.sizeof(_lib.zoact_coeff_block) == 24
+
+
+def test_layer_table_packs_each_layer_by_itself():
+    def rows(arr, n):
+        return [(arr[i].offset, arr[i].d_out, arr[i].r, arr[i].layer_id) for i in range(n)]
+
+    plain = [(0, 4096, 16, 0), (1 << 35, 7, 3, 0xFFFFFFFF)]
+    assert rows(_lib._blocks(plain), 2) == plain
+    assert rows(_lib._blocks([tuple(np.int64(v) for v in b) for b in plain]), 2) == plain
+    assert rows(_lib._blocks([(4.0, 2.0, 1, 5)]), 1) == [(4, 2, 1, 5)]          # converted one by one
+    assert rows(_lib._blocks([(0, 1, 1, -1)]), 1) == [(0, 1, 1, 0xFFFFFFFF)]
+    # entries of the wrong length are refused, also where their lengths add up
+    with pytest.raises((TypeError, ValueError)):
+        _lib._blocks([(0, 1, 2, 3, 4), (5, 6, 7)])
