@@ -600,22 +600,19 @@ __device__ __forceinline__ bool epi_multi4_staged(const Params& prm, const TmaSe
   const uint32_t* const tw = reinterpret_cast<const uint32_t*>(tbl);
   const int ncol = min(ncol_tile, prm.d_out - n_blk * ncol_tile);   // (the tables end with the 64 columns d_out lies in)
   const int passes = (ncol + SLOTS - 1) / SLOTS * prm.nb;
-  uint32_t sent = 0, sent_phase = 0;                        // the loading thread's buffers, and the parity of their last load
   auto load = [&](int pass, int bufi) {                     // one thread: pass's tables into a buffer
     if (pass >= passes) return;
     const int s = pass / prm.nb, b = pass - s * prm.nb;
     if (prm.coef[b] == 0.f) return;
     const int64_t at = prm.zq[b] * prm.zt_qstride + (int64_t)((n_blk * ncol_tile + s * SLOTS) / 16) * CHUNK;
     const uint32_t bar = tc::smem_u32(&ss->tload[bufi]), dst = tc::smem_u32(tbl + bufi * BSZ);
-    sent |= 1u << bufi;
-    sent_phase = (sent_phase & ~(1u << bufi)) | (tphase & (1u << bufi));
     tc::mbar_arrive_expect_tx(bar, BSZ * 4);
     tc::bulk_load(dst, prm.Zt + at, TSZ * 4, bar);
     if (GATED) tc::bulk_load(dst + TSZ * 4, prm.Zt2 + at, TSZ * 4, bar);
   };
-  auto drain = [&] {                                        // the loads in flight land before the block gives up
-    for (int i = 0; i < 2; ++i)
-      if (sent >> i & 1u) tc::mbar_wait_drain(tc::smem_u32(&ss->tload[i]), (sent_phase >> i) & 1u, 100000000ull);
+  // before the block gives up: loads that no one has waited for land (at most this long where there are none)
+  auto drain = [&] {
+    for (int i = 0; i < 2; ++i) tc::mbar_wait_drain(tc::smem_u32(&ss->tload[i]), (tphase >> i) & 1u, 10000000ull);
   };
   if (etid == 0) {                                          // (the previous tile's last barrier freed both buffers)
     load(0, 0);
@@ -633,8 +630,9 @@ __device__ __forceinline__ bool epi_multi4_staged(const Params& prm, const TmaSe
       const float c = prm.coef[b];
       if (c != 0.f) {
         // a wait that gives up ends the tile's loads but not its passes: every thread meets the barriers
-        ok = tc::mbar_wait(tc::smem_u32(&ss->tload[cur]), (tphase >> cur) & 1u, abort_flag, prm.status) && ok;
-        tphase ^= 1u << cur;
+        const bool got = tc::mbar_wait(tc::smem_u32(&ss->tload[cur]), (tphase >> cur) & 1u, abort_flag, prm.status);
+        tphase ^= (uint32_t)got << cur;
+        ok = ok && got;
       }
       const int cbeg = half * (cwid / 2);
 #pragma unroll 1
