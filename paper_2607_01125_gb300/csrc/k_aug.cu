@@ -392,8 +392,10 @@ bool aligned16_or_null(const void* p) { return ((uintptr_t)p & 15u) == 0; }
 // rank 12, 333 rows each on 256 outputs 9.4, 9.2, 9.3; 17 blocks of 14 rows (11 slots), rank 24 25.2, 23.6, 24.4.  The
 // other way: rank 16, 333 rows each on 4096 outputs (two slots) 11.1 and 11.5; B's rows, which the two threads' stores
 // fill whole, gate and up with a projection each, 17 blocks on 14336 outputs, rank 16 68.6 and 96.4.
-int spread_zeros(int slots, int row_q, int rq, int distinct) {
-  if (rq <= 2) return SPREAD_A | SPREAD_B;
+// Rank 8's B rows only while the quads' threads leave SMs idle (eight queries, 512 tokens each through an MLP block: 530
+// us a step with B's zeros spread too, 525 so).
+int spread_zeros(int slots, int row_q, int rq, int distinct, bool few_b) {
+  if (rq <= 2) return SPREAD_A | (rq == 1 || few_b ? SPREAD_B : 0);
   return slots * row_q / ((distinct ? 2 : 1) * rq) - 3 > 6 ? SPREAD_A : 0;
 }
 
@@ -432,7 +434,7 @@ int launch_aug_prep(Ctx* ctx, const PairArgs& a, int mode, int ka, int distinct,
   if (quad) {
     const int rq = a.r / 4, row_q = ka_row / 4;
     const int64_t itA = a.rows * ((distinct ? 2 : 1) * rq), itB = (B_aug2 ? 2 : 1) * ((nbB + 1) / 2) * a.d_out * (int64_t)rq;
-    const int spread = spread_zeros(slots, row_q, rq, distinct);
+    const int spread = spread_zeros(slots, row_q, rq, distinct, itB < 512 * (int64_t)ctx->sm_count);
     const int64_t q_items = itA + itB + (spread & SPREAD_A ? a.rows * (slots * row_q / 2) : 0) +
                             (spread & SPREAD_B ? (B_aug2 ? 2 : 1) * nbB * a.d_out * (int64_t)(row_q / 2) : 0);
     const int64_t q_work = q_items > z_items ? q_items : z_items;
