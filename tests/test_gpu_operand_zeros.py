@@ -24,9 +24,10 @@ def ctx():
 
 @pytest.mark.parametrize("own", [None, False, True])          # one layer; gate and up; each with its own projection
 @pytest.mark.parametrize("r", [4, 8, 12, 16, 24, 64])
-@pytest.mark.parametrize("T,nb", [(256, 2), (130, 2), (100, 3), (16, 17)])   # one slot, two, three, seventeen
-def test_operand_zeros(ctx, T, nb, r, own):
-    d_in, d_out, seed, rows = 128, 136, 3, nb * T
+@pytest.mark.parametrize("T,nb,d_out", [(256, 2, 136), (130, 2, 136), (100, 3, 136), (16, 17, 136),   # 1, 2, 3, 17 slots
+                                        (16, 17, 4408)])         # enough columns for rank 8's own threads
+def test_operand_zeros(ctx, T, nb, d_out, r, own):
+    d_in, seed, rows = 128, 3, nb * T
     pts = [(0.5, 7), (-0.5, 7)] if nb == 2 else [(0.25 * (1 + j) / nb, j) for j in range(nb)]
     X = normal((rows, d_in), 1, DEV, dtype=torch.bfloat16)
     W = [normal((d_out, d_in), 2 + i, DEV, std=d_in ** -0.5, dtype=torch.bfloat16) for i in range(2)]
