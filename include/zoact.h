@@ -189,7 +189,11 @@ int zoact_lowrank_proj_prepared(zoact_ctx* ctx, const void* X, int xdtype, int64
  * Requirements: d_in % 8 == 0 (BF16/FP16), d_in % 128 == 0 (INT4), d_out % 8 == 0,
  * 16-byte aligned X, W, Y.  Ranks above 32 (16-bit X) add the whole low-rank term on
  * the tensor cores, which needs stacked rows: a shared input is first copied once
- * per sign into context scratch.                                                 */
+ * per sign into context scratch (fewer than 256 rows: only where that is faster).
+ * INT4 weights take 2 bytes of context scratch a weight where they are expanded to
+ * BF16: from 256 rows, and below where that is faster.  Up to 1023 rows a call runs
+ * without that scratch (slower) where it cannot be had: in a capture before a first
+ * call of its size, or for lack of memory.                                       */
 int zoact_pair_forward(zoact_ctx* ctx, const zoact_layer* layer, const void* X, int xdtype,
                        int64_t T, int input_shared, const float* P, float eps, uint64_t seed,
                        uint64_t query, int act, void* Y, int ydtype);
@@ -252,7 +256,8 @@ int zoact_multi_forward_gated_rs(zoact_ctx* ctx, const zoact_layer* gate, const 
  * process under a hard memory budget).  It computes the pair forward of
  * zoact_pair_forward with P == NULL, on `stream` (a cudaStream_t), without a
  * context and without calling cudaMalloc, cudaFree or any allocating library
- * routine.  It adds the low-rank term from fp32 epilogue tables, so its
+ * routine.  It adds the low-rank term from fp32 epilogue tables, or (fewer than
+ * 256 rows) in products of three-part operands that keep 24 bits, so its
  * outputs agree with zoact_pair_forward within the pair forward's tolerance
  * (1e-4 of the output scale for fp32 outputs), not bit for bit.  Limits beyond
  * zoact_pair_forward's: r <= 32, and weights of type FP32, BF16 or FP16 (INT4
@@ -438,10 +443,16 @@ int zoact_sgd_step_multi(zoact_ctx* ctx, float* C, int64_t n_total, const zoact_
  * (element i*k + j), Q0 = orth(Omega), Q <- orth(G Q) n_iter times, then
  * Rayleigh-Ritz.  Columns in descending eigenvalue order, each flipped so its
  * largest-magnitude entry is positive.  Optional evals_out [k] fp32 (device)
- * receives the Ritz values.  Requires k <= 512 and k <= d_in; uses d_in^2 * 4
- * bytes of context scratch.  Non-finite calibration data gives a non-finite
- * basis and sets the device status word to ZOACT_ERR_NONFINITE (a column with
- * no finite entry is left unflipped).                                          */
+ * receives the Ritz values.  Requires k <= 512 and k <= d_in.  G Q is formed as
+ * X^T (X Q) for 16-bit X with n_tok <= 8 d_in; context scratch is then X^T (2 bytes
+ * an element), about 4 n_tok k + 6 (n_tok + d_in) k bytes of factors (k rounded up to
+ * the projection's rank tile) and the largest product's K ranges: 4 bytes times k
+ * times the larger of up to 32 max(n_tok, d_in) and n_tok d_in / max(64, n_tok / 4).
+ * Otherwise G is formed: 4 d_in^2 bytes (and X^T for 16-bit X).  Both add 8 d_in k
+ * bytes for Q and Y and k x k fp64 partials of Q^T Y (up to two for each SM).
+ * Non-finite calibration data gives a non-finite basis (n_iter > 0) and sets the
+ * device status word to ZOACT_ERR_NONFINITE (a column with no finite entry is left
+ * unflipped).                                                                   */
 int zoact_basis_init(zoact_ctx* ctx, const void* X_cal, int xdtype, int64_t n_tok, int32_t d_in,
                      int32_t r, int32_t oversample, int32_t n_iter, uint64_t seed, float* U_out,
                      float* evals_out);

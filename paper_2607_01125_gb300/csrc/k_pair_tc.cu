@@ -197,7 +197,7 @@ int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
     b.rows = (int64_t)a.nb * a.T;
     return pair_tc(ctx, b, false);       // (the copies are for the other route)
   }
-  // INT4 weights: the few-row kernel dequantises in the kernel; from FEW_ROWS rows W is expanded to bf16 once
+  // INT4 weights: the few-row kernel dequantises in the kernel; else, and from FEW_ROWS rows, W is expanded to bf16 once
   // per call and the bf16 kernel runs (the default: measured faster, see pair_tc2_kernel.cuh).
   // ZOACT_INT4=kernel runs stacked rows from 256 on the CTA-pair kernel with its own dequantising warps
   // (bf16 or fp32 output, d_in a multiple of 1024); ZOACT_INT4=staged expands W at every row count.

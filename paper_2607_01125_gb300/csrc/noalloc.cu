@@ -13,8 +13,9 @@
 // slot), which every GPU that loads libzoact holds until the process exits.
 // Limits beyond the regular entry point's: ranks up to 32 and 16-bit or fp32
 // weights (INT4 is refused with ZOACT_ERR_UNSUPPORTED); the low-rank term is
-// added from fp32 epilogue tables (the regular entry point can put it on the
-// tensor cores), so the outputs agree with zoact_pair_forward within the pair
+// added from fp32 epilogue tables, or with few rows by the few-row kernel, which
+// needs no scratch (the regular entry point can put it on the tensor cores from
+// operand tables), so the outputs agree with zoact_pair_forward within the pair
 // forward's tolerance, not bit for bit.
 // It stores P = X U ([rows, r] fp32) and, when room is left, the split-K
 // partials of that projection.  A request with rows * r above

@@ -123,7 +123,7 @@ struct Params {
   int64_t ldy;       // plain mode: row stride of D
   int vec_ok;        // C, C2, P, P2 and ldy allow 16-byte vector access
   int bn;            // N-tile width of pair / plain tiles (multiple of 32, <= BN); gated tiles use BN
-  // INT4 weights of few rows: fp16 scales [d_out, d_in/128]
+  // INT4 weights (few-row kernel): fp16 scales [d_out, d_in/128]
   const __half* Ws;
   const __half* Ws2;
   int* status;
