@@ -248,8 +248,9 @@ constexpr int64_t FEW_ROWS = 256;
 // Row count from which an INT4 pair forward takes row scales and layer groups (the library's contract).
 constexpr int64_t INT4_ROWSCALE_MIN_ROWS = 1024;
 int launch_pair_tc(Ctx* ctx, const PairArgs& a);
-// The few-row kernel can serve fewer than FEW_ROWS rows whose outputs (every block padded to 16 rows) fit one tile; it is
-// chosen where its estimated time is the smaller one.
+// The few-row kernel can serve fewer than FEW_ROWS rows whose outputs (every block padded to 16 rows) fit one tile
+// (possible); it is chosen where its estimated time is the smaller one.
+bool pair_fr_possible(const PairArgs& a);
 bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a);
 int launch_pair_fr(Ctx* ctx, const PairArgs& a);
 // Plain product D[M, N] (fp32) = A[M, K] * B[N, K]^T with 16-bit A, B (K-major), on tcgen05.

@@ -199,14 +199,17 @@ bool one_cta_ready(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
 }  // namespace
 
 // ZOACT_PAIR_KERNEL=few / =1cta: this kernel wherever it can run / never; ZOACT_INT4=staged: not on INT4 weights.
-bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a) {
+bool pair_fr_possible(const PairArgs& a) {
   if (!fr_supported(a)) return false;
   const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
   if (sel && std::strcmp(sel, "1cta") == 0) return false;
-  if (a.wtype == ZOACT_DT_INT4_G128) {
-    const char* isel = std::getenv("ZOACT_INT4");
-    if (isel && std::strcmp(isel, "staged") == 0) return false;
-  }
+  const char* isel = std::getenv("ZOACT_INT4");
+  return !(a.wtype == ZOACT_DT_INT4_G128 && isel && std::strcmp(isel, "staged") == 0);
+}
+
+bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a) {
+  if (!pair_fr_possible(a)) return false;
+  const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
   if (sel && std::strcmp(sel, "few") == 0) return true;
   const OneCta o = one_cta(a);
   // (0.9: about as many calls lose by an error of the estimates one way as the other)

@@ -491,7 +491,11 @@ int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
 
 }  // namespace
 
-int launch_pair_tc(Ctx* ctx, const PairArgs& a) { return pair_tc(ctx, a, true); }
+int launch_pair_tc(Ctx* ctx, const PairArgs& a) {
+  const int st = pair_tc(ctx, a, true);
+  // (few rows whose faster route found no memory for its scratch)
+  return st == ZOACT_ERR_NOMEM && pair_fr_possible(a) ? launch_pair_fr(ctx, a) : st;
+}
 
 int launch_gemm_tc_f32out(Ctx* ctx, const void* A, const void* B, int dtype, int M, int N, int K, float* D) {
   using namespace pairtc;
