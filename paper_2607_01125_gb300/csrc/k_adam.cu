@@ -64,9 +64,9 @@ __device__ __forceinline__ float4 zo_gradient4(const double* __restrict__ a_dev,
   return g;
 }
 
-constexpr int ADAM_UNROLL = 2;           // groups of a thread whose loads are in flight together
-
-template <bool SGD>
+// ADAM_UNROLL: groups of a thread whose loads are in flight together: two where a block has two rounds, else one (65536
+// coefficients after their loss: 18.1 us with the search per group, 16.5 so; 40 registers, as that had, spill: 18.2).
+template <bool SGD, int ADAM_UNROLL>
 __global__ void __launch_bounds__(256)
 zo_update_kernel(float* __restrict__ C, float* __restrict__ m, float* __restrict__ v, const __grid_constant__ AdamTable tab,
                  int64_t g_begin, int64_t g_end, int64_t per_block, const double* __restrict__ a_dev, int nq,
@@ -194,7 +194,9 @@ int launch_adam(Ctx* ctx, float* C, float* m, float* v, const zoact_coeff_block*
     int64_t rounds = (groups + 255) / 256 / cap;
     if (q < 4 || rounds >= 8) rounds = (groups + cap * 256 - 1) / (cap * 256);
     const int64_t per_block = 256 * (rounds < 1 ? 1 : rounds), nb = (groups + per_block - 1) / per_block;
-    ZOACT_CUDA_TRY(launch_pdl(ctx, sgd ? zo_update_kernel<true> : zo_update_kernel<false>, dim3((unsigned)nb),
+    auto kern = per_block > 256 ? (sgd ? zo_update_kernel<true, 2> : zo_update_kernel<false, 2>)
+                                : (sgd ? zo_update_kernel<true, 1> : zo_update_kernel<false, 1>);
+    ZOACT_CUDA_TRY(launch_pdl(ctx, kern, dim3((unsigned)nb),
                               dim3(256), 0, C, m, v, tab, g_begin, g_end, per_block, a, q, qs, lr, b1, b2, adam_eps, step_size,
                               inv_sqrt_bc2, seed, ctx->d_status));
     ++ctx->n_launch;
