@@ -125,7 +125,8 @@ OneCta one_cta(const PairArgs& a) {
   o.nw = a.W2 ? 2 : 1;
   o.stacked = !a.shared || a.r > 32;
   o.rows = o.stacked ? a.nb * a.T : a.T;
-  const int64_t span = o.stacked && a.T % 128 != 0 ? 127 / a.T + 2 : 1;
+  const int64_t tile = o.rows >= FEW_ROWS ? 256 : 128;        // (copies of 256 rows go to CTA pairs)
+  const int64_t span = o.stacked && a.T % tile != 0 ? (tile - 1) / a.T + 2 : 1;
   o.slots = (int)(span < a.nb ? span : a.nb);
   o.ka = aug_cols(a.r) * (a.W2 && a.P2 != a.P ? 2 : 1);
   o.table_rows = (int64_t)o.nw * (o.stacked ? a.nb : 1) * a.d_out;

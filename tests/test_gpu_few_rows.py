@@ -178,6 +178,7 @@ def test_lowrank_term_alone(ctx, monkeypatch, wtype, r, T, shared, gated):
     ("bf16", 64, 64, 100, 64, False, False),        # the other route by its estimate
     ("bf16", 256, 512, 64, 16, False, True),
     ("bf16", 256, 512, 100, 64, True, False),       # ... with copies of the shared input
+    ("bf16", 256, 512, 128, 64, True, False),       # ... 256 copied rows
     ("int4", 128, 64, 100, 64, False, True),        # ... with W expanded
     ("bf16", 4096, 1024, 16, 16, False, False),     # the few-row kernel
     ("int4", 1024, 264, 245, 16, False, False),     # 490 rows: INT4 in pieces of 240 rows and five, without W expanded
