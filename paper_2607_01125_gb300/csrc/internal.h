@@ -252,6 +252,8 @@ int launch_pair_tc(Ctx* ctx, const PairArgs& a);
 // (possible); it is chosen where its estimated time is the smaller one.
 bool pair_fr_possible(const PairArgs& a);
 bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a);
+// Whether the scratch of a call on tiles of 128 or 256 rows (INT4: on W expanded) is there, or may be had now.
+bool tile_route_ready(const Ctx* ctx, const PairArgs& a);
 int launch_pair_fr(Ctx* ctx, const PairArgs& a);
 // Plain product D[M, N] (fp32) = A[M, K] * B[N, K]^T with 16-bit A, B (K-major), on tcgen05.
 // Low-rank term of the tensor-core pair forward (see k_aug.cu):

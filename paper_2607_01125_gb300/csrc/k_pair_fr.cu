@@ -178,25 +178,6 @@ double one_cta_us(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
   return us;
 }
 
-// Whether the other route's scratch is there, or may be had now.
-bool one_cta_ready(const Ctx* ctx, const PairArgs& a, const OneCta& o) {
-  if (!ctx->may_allocate) return true;                              // (its form without scratch)
-  int queries = 0;                                                  // distinct ones of the perturbed blocks
-  for (int b = 0; b < a.nb; ++b) {
-    bool seen = a.coef[b] == 0.f;
-    for (int i = 0; i < b; ++i) seen = seen || (a.coef[i] != 0.f && a.qry[i] == a.qry[b]);
-    queries += !seen;
-  }
-  const int np = a.W2 && a.P2 != a.P ? 2 : 1;
-  const size_t copy = (size_t)a.T * a.d_in * 2 + (size_t)np * a.T * a.r * sizeof(float);
-  const size_t w_bytes = a.wtype == ZOACT_DT_INT4_G128 ? (size_t)a.d_out * a.d_in * 2 : 0;
-  return scratch_ready(ctx, SLOT_AUG_A, (size_t)o.rows * o.slots * o.ka * 2) &&
-         scratch_ready(ctx, SLOT_AUG_B, (size_t)o.table_rows * o.ka * 2) &&
-         (o.stacked || scratch_ready(ctx, SLOT_AUG_Z, (size_t)o.nw * queries * a.r * a.d_out * sizeof(float))) &&
-         (!(a.shared && o.stacked) || scratch_ready(ctx, SLOT_STACKED_X, a.nb * copy + 1024)) &&
-         scratch_ready(ctx, SLOT_WDQ0, w_bytes) && (!a.W2 || scratch_ready(ctx, SLOT_WDQ1, w_bytes));
-}
-
 }  // namespace
 
 // ZOACT_PAIR_KERNEL=few / =1cta: this kernel wherever it can run / never; ZOACT_INT4=staged: not on INT4 weights.
@@ -214,7 +195,39 @@ bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a) {
   if (sel && std::strcmp(sel, "few") == 0) return true;
   const OneCta o = one_cta(a);
   // (0.9: about as many calls lose by an error of the estimates one way as the other)
-  return one_cta_us(ctx, a, o) >= 0.9 * fr_us(ctx, a, fr_plan(ctx, a)) || !one_cta_ready(ctx, a, o);
+  return one_cta_us(ctx, a, o) >= 0.9 * fr_us(ctx, a, fr_plan(ctx, a)) || !tile_route_ready(ctx, a);
+}
+
+// The sizes are launch_pair_tc's.
+bool tile_route_ready(const Ctx* ctx, const PairArgs& a) {
+  if (!ctx->may_allocate) return true;                              // (its form without scratch)
+  const OneCta o = one_cta(a);
+  int queries = 0;                                                  // distinct ones of the perturbed blocks
+  for (int b = 0; b < a.nb; ++b) {
+    bool seen = a.coef[b] == 0.f;
+    for (int i = 0; i < b; ++i) seen = seen || (a.coef[i] != 0.f && a.qry[i] == a.qry[b]);
+    queries += !seen;
+  }
+  const bool one_p = !a.W2 || a.P2 == a.P, pairs_of_ctas = o.rows >= FEW_ROWS;
+  const bool blocks16 = pairs_of_ctas && !o.stacked && a.nb >= 2 && dtype_size(a.ydtype) == 2;
+  const bool mirror = blocks16 && a.nb == 2 && a.qry[0] == a.qry[1] && a.coef[1] == -a.coef[0] && a.coef[0] != 0.f;
+  const int rt = a.r <= 4 ? 4 : a.r <= 8 ? 8 : a.r <= 16 ? 16 : 32;
+  const size_t z = blocks16 && !mirror && one_p ? z_table_words(rt, a.d_out) : (size_t)a.r * a.d_out;
+  const size_t copy = (size_t)a.T * a.d_in * 2 + (size_t)(one_p ? 1 : 2) * a.T * a.r * sizeof(float);
+  const size_t w_bytes = a.wtype == ZOACT_DT_INT4_G128 ? (size_t)a.d_out * a.d_in * 2 : 0;
+  bool ok = scratch_ready(ctx, SLOT_AUG_A, (size_t)o.rows * o.slots * o.ka * 2) &&
+            scratch_ready(ctx, SLOT_AUG_B, (size_t)o.table_rows * o.ka * 2) &&
+            (o.stacked || scratch_ready(ctx, SLOT_AUG_Z, o.nw * queries * z * sizeof(float))) &&
+            (!(a.shared && o.stacked) || scratch_ready(ctx, SLOT_STACKED_X, a.nb * copy + 1024)) &&
+            scratch_ready(ctx, SLOT_WDQ0, w_bytes) && (!a.W2 || scratch_ready(ctx, SLOT_WDQ1, w_bytes));
+  if (pairs_of_ctas) {                                              // a split tail's partials
+    const int64_t pairs = ctx->sm_count / 2, bn = a.W2 ? 128 : 256;
+    const int64_t rem = (o.rows + 255) / 256 * ((a.d_out + bn - 1) / bn) % pairs;
+    const int64_t split = rem > 0 ? (pairs / rem < 4 ? pairs / rem : 4) : 0;
+    if (split >= 2 && ((a.d_in + 63) / 64 + o.slots * (o.ka / 64)) / split >= 4)
+      ok = ok && scratch_ready(ctx, SLOT_SK_PART, (size_t)pairs * 2 * 128 * 256 * sizeof(float));
+  }
+  return ok;
 }
 
 int launch_pair_fr(Ctx* ctx, const PairArgs& a) {

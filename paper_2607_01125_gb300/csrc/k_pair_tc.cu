@@ -220,8 +220,8 @@ int pair_tc(Ctx* ctx, const PairArgs& a, bool few) {
     const size_t bytes = (size_t)a.d_out * a.d_in * 2;
     const bool pieces = a.rows < INT4_ROWSCALE_MIN_ROWS && !one_cta && !(isel && std::strcmp(isel, "staged") == 0) &&
                         a.nseg <= 1 && !a.fuse_loss && !a.in_scale && !a.out_sumsq && a.xdtype == ZOACT_DT_BF16;
-    if (pieces && (!scratch_ready(ctx, SLOT_WDQ0, bytes) || (a.W2 && !scratch_ready(ctx, SLOT_WDQ1, bytes)) ||
-                   !scratch(ctx, SLOT_WDQ0, bytes) || (a.W2 && !scratch(ctx, SLOT_WDQ1, bytes))))
+    if (pieces && (!tile_route_ready(ctx, a) || !scratch(ctx, SLOT_WDQ0, bytes) ||
+                   (a.W2 && !scratch(ctx, SLOT_WDQ1, bytes))))
       return few_row_pieces(ctx, a);
     void* wb = scratch(ctx, SLOT_WDQ0, bytes);
     if (!wb) return ZOACT_ERR_NOMEM;

@@ -215,3 +215,38 @@ def test_first_call_captured(route, wtype, d_in, d_out, T, r, shared, gated):
     a, b = np64(Y[0]), np64(Y[1])
     assert np.linalg.norm(a - b) <= 2.0 ** -8 * np.linalg.norm(b) and np.abs(a).max() > 0
     c.close()
+
+
+@pytest.mark.parametrize("T,shared,r,gated,nb", [(245, False, 16, False, 2), (300, True, 16, True, 2), (300, True, 8, False, 3),
+                                                 (130, False, 40, True, 2)])
+def test_captured_after_a_first_call(T, shared, r, gated, nb):
+    # INT4 from 256 rows on W expanded: with the scratch of a first call there a capture takes the same route, same bits
+    L, W, U, C = _layer(1024, 264, r, "int4", 100, 3)
+    L2 = _layer(1024, 264, r, "int4", 200, 4, U=U)[0]
+    pts = [(0.5, 7), (-0.5, 7)] if nb == 2 else [(0.0, 0), (0.25, 1), (0.25, 2)]
+    X = normal(((T if shared else nb * T), 1024), 5, DEV, dtype=torch.bfloat16)
+    P = X.float() @ U
+    Y = [torch.zeros(nb * T, 264, dtype=torch.bfloat16, device=DEV) for _ in range(2)]
+    torch.cuda.synchronize()
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        c = zo.Context(0)
+        c.sync_stream()
+
+        def run(y):
+            if gated:
+                zo.zoact_multi_forward_gated(c, L, L2, X, T, shared, pts, 1, y, P_gate=P, P_up=P)
+            else:
+                zo.zoact_multi_forward(c, L, X, T, shared, pts, 1, y, P=P)
+
+        run(Y[0])
+        torch.cuda.synchronize()
+        n = c.launch_count()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            run(Y[1])
+        assert c.launch_count() - n == n
+        g.replay()
+        torch.cuda.synchronize()
+    assert torch.equal(Y[0], Y[1])
+    c.close()
