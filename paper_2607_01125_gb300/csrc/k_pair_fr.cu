@@ -193,6 +193,9 @@ bool pair_fr_chosen(const Ctx* ctx, const PairArgs& a) {
   if (!pair_fr_possible(a)) return false;
   const char* sel = std::getenv("ZOACT_PAIR_KERNEL");
   if (sel && std::strcmp(sel, "few") == 0) return true;
+  // fp32 outputs keep this kernel's three-part low-rank term: the other route's two parts leave out 2^-16 of |T||P|, which
+  // a 16-bit output cannot show (its form without scratch sums in fp32)
+  if (a.ydtype == ZOACT_DT_FP32 && ctx->may_allocate) return true;
   const OneCta o = one_cta(a);
   // (0.9: about as many calls lose by an error of the estimates one way as the other)
   return one_cta_us(ctx, a, o) >= 0.9 * fr_us(ctx, a, fr_plan(ctx, a)) || !tile_route_ready(ctx, a);

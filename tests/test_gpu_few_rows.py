@@ -87,19 +87,23 @@ def _ref(W, U, C, X, T, shared, pts, seed, lid, r, int4, split):
     ("int4", 1024, 520, 120, 32, True, 3, True),    # gated, rank 32: one CTA per SM
 ])
 def test_few_rows(ctx, route, wtype, d_in, d_out, T, r, shared, nb, gated):
-    seed, eps, split = 11, 0.5, route != "few"
+    seed, eps = 11, 0.5
     pts = [(eps, 7), (-eps, 7)] if nb == 2 else [(0.0, 0)] + [(eps * (1 + j) / nb, j) for j in range(nb - 1)]
     L, W, U, C = _layer(d_in, d_out, r, wtype, 100, 3)
     dt = torch.float16 if wtype == "fp16" else torch.bfloat16
     X = normal(((T if shared else nb * T), d_in), 5, DEV, dtype=dt)
-    ref, bound = _ref(W, U, C, X, T, shared, pts, seed, 3, r, wtype == "int4", split)
-    if gated:
-        L2, W2, U2, C2 = _layer(d_in, d_out, r, wtype, 200, 4)      # its own basis: a second projection
+    L2, W2, U2, C2 = _layer(d_in, d_out, r, wtype, 200, 4)      # gated: its own basis, a second projection
+
+    def reference(split):
+        ref, bound = _ref(W, U, C, X, T, shared, pts, seed, 3, r, wtype == "int4", split)
+        if not gated:
+            return ref, bound
         u, ub = _ref(W2, U2, C2, X, T, shared, pts, seed, 4, r, wtype == "int4", split)
         g = layers.silu(ref)
-        bound = 1.1 * bound * np.abs(u) + np.abs(g) * ub + 1.1 * bound * ub + 2.0 ** -20 * np.abs(g * u)
-        ref = g * u
+        return g * u, 1.1 * bound * np.abs(u) + np.abs(g) * ub + 1.1 * bound * ub + 2.0 ** -20 * np.abs(g * u)
+
     for ydt in (torch.float32, dt):
+        ref, bound = reference(route == "chosen" and ydt != torch.float32)   # (fp32 outputs keep the few-row kernel)
         outs = []
         for _ in range(2):
             Y = torch.full((nb * T, d_out), float("nan"), dtype=ydt, device=DEV)
